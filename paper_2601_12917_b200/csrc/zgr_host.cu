@@ -64,7 +64,8 @@ struct zgr_ctx {
   std::map<uint64_t, double> ledger;  // seeds whose perturbation is applied to the weights -> sum of the coefficients applied
   uint64_t last_seed = 0;             // most recently swept seed (introspection)
   bool guided_at_init = false;        // b != 0 when the sweep plan was made
-  SplitJob* d_split_jobs = nullptr;   // one job per tensor served by the tcgen05 kernel: rebuild of its operand copy of U
+  SplitJob* d_split_jobs = nullptr;   // one job per tensor served by a tcgen05 kernel: rebuild of its operand copies of U
+  std::vector<int32_t> split_job;     // per tensor: its job, or -1
   int n_split_jobs = 0;
   std::vector<char> frag_stale;       // per tensor: the fragment-order copy of U (legacy tensor-core kernel) lags behind U
   std::vector<Group> groups_multi;    // plan of multi-seed sweeps when it differs from `groups` (legacy tensor-core path only)
@@ -147,15 +148,25 @@ bool make_map_16bit(CUtensorMap* out, const void* base, int64_t rows, int64_t co
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Which tcgen05 kernel serves a tensor: 1 the TMA-staged one (16-bit weights, rank > 8, rows that TMA can address), 2 the
+// tile kernel (everything else with a subspace that the CUDA-core kernel for rank <= 8 does not take), 0 neither.
+int tensor_core_kind(const zgr_tensor& t, bool guided_on) {
+  if (!guided_on || t.rank == 0 || t.rows >= (int64_t{1} << 31) - 256) return 0;
+  const bool vec = (reinterpret_cast<uintptr_t>(t.data) & 15) == 0 && (t.cols % 8 == 0);
+  if (vec && t.rank <= 8) return 0;
+  if (vec && t.dtype != ZGR_F32) return t.cols < (int64_t{1} << 31) - 256 ? 1 : 0;
+  return 2;
+}
+
 bool umma_wanted() {
   const char* e = std::getenv("ZGR_TENSOR_PATH");
   return !(e && std::strcmp(e, "legacy") == 0);
 }
 
-int blocks_per_sm(int path) {
-  switch (path) {
+int blocks_per_sm(const KernelChoice& kc) {
+  switch (kc.path) {
     case PATH_ISO: return 6;
-    case PATH_GENERIC: return 4;
+    case PATH_GENERIC: return kc.kpad > 0 ? 1 : 4;
     case PATH_UMMA: return 1;
     default: return 2;
   }
@@ -205,7 +216,12 @@ void plan(const std::vector<TensorDesc>& descs, const std::vector<int>& which, b
     const bool vec = aligned && (t.cols % 8 == 0);
     int path, kpad, strip, row_step;
     const bool umma_ok = t.umma && kernel_dtype < 0;
-    if (!vec || (t.rank > 8 && t.Ufrag == nullptr) || (multi && t.rank > 8 && !umma_ok)) {
+    const bool tile_ok = t.tile && (kernel_dtype < 0 || kernel_dtype == t.dtype);
+    if (tile_ok) {
+      // fp32 with rank > 8, and rows that are not a multiple of eight elements: sweep_tile_kernel.  (The test hook that
+      // sweeps an fp32 image of a 16-bit tensor keeps the one-element-per-thread kernel below.)
+      path = PATH_GENERIC; kpad = t.kpad; strip = tile_strip_cols(); row_step = 128;
+    } else if (!vec || (t.rank > 8 && t.Ufrag == nullptr) || (multi && t.rank > 8 && !umma_ok)) {
       // (the legacy tensor-core kernel applies one term per sweep; several terms take the fallback)
       path = PATH_GENERIC; kpad = 0; strip = 64; row_step = 1;
     } else if (t.rank <= 8) {
@@ -222,6 +238,8 @@ void plan(const std::vector<TensorDesc>& descs, const std::vector<int>& which, b
       // (the CUDA-core contraction kernel hands its items out dynamically and regenerates its coefficient strip per item:
       //  larger items there; the tcgen05 kernel's items are two tiles wide)
       int64_t nrows = std::max<int64_t>(1, (path == PATH_UMMA || path == PATH_FMA ? 2 * target : target) / ncols);
+      // (the tile kernel builds a 144-column strip per item and 128 columns of weights: about ten items per SM)
+      if (tile_ok) nrows = std::min<int64_t>(std::max<int64_t>(total / (static_cast<int64_t>(sm_count) * 10), 16384), 262144) / strip;
       nrows = ((nrows + row_step - 1) / row_step) * row_step;
       // even out the chunks of this strip
       const int64_t n_chunks = (t.rows + nrows - 1) / nrows;
@@ -235,7 +253,7 @@ void plan(const std::vector<TensorDesc>& descs, const std::vector<int>& which, b
     g.elements = 0;
     for (const WorkItem& w : g.items) g.elements += g.kc.path == PATH_ISO ? w.nrows_or_count : w.nrows_or_count * w.ncols;
   }
-  for (Group& g : out) g.grid = static_cast<int>(std::min<int64_t>(static_cast<int64_t>(g.items.size()), static_cast<int64_t>(sm_count) * blocks_per_sm(g.kc.path)));
+  for (Group& g : out) g.grid = static_cast<int>(std::min<int64_t>(static_cast<int64_t>(g.items.size()), static_cast<int64_t>(sm_count) * blocks_per_sm(g.kc)));
   // tensors were visited in ascending order, so each tensor's items are contiguous within its group
   for (Group& g : out) {
     g.first_item.assign(descs.size() + 1, static_cast<int32_t>(g.items.size()));
@@ -282,9 +300,11 @@ int upload_groups(zgr_ctx* ctx, std::vector<Group>& groups) {
 }
 
 // One sweep  theta <- rnd(theta + sum_q c_q z(seed_q))  over the planned groups (n terms, 1 <= n <= kMaxTerms).
-// t0 <= t1 restricts the sweep to the tensors [t0, t1) (layer-wise sweeps); t1 < 0 means all of them.
+// t0 <= t1 restricts the sweep to the tensors [t0, t1) (layer-wise sweeps); t1 < 0 means all of them.  tmaps: the tensor
+// maps of the first tensor of d_descs (null: the context's own).
 int sweep(zgr_ctx* ctx, std::vector<Group>& groups, const TensorDesc* d_descs, int n, const uint64_t* seeds, const double* c, cudaStream_t st,
-          int32_t t0 = 0, int32_t t1 = -1, bool keep_stats = false) {
+          int32_t t0 = 0, int32_t t1 = -1, bool keep_stats = false, const CUtensorMap* tmaps = nullptr) {
+  if (tmaps == nullptr) tmaps = ctx->d_tmaps;
   SweepParams p;
   std::memset(&p, 0, sizeof(p));
   for (int q = 0; q < n; ++q) {
@@ -312,7 +332,7 @@ int sweep(zgr_ctx* ctx, std::vector<Group>& groups, const TensorDesc* d_descs, i
       p.items = g.d_items + b0;
       p.n_items = b1 - b0;
       p.item_base = b0;
-      grid = static_cast<int>(std::min<int64_t>(p.n_items, static_cast<int64_t>(ctx->sm_count) * blocks_per_sm(g.kc.path)));
+      grid = static_cast<int>(std::min<int64_t>(p.n_items, static_cast<int64_t>(ctx->sm_count) * blocks_per_sm(g.kc)));
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (ctx->profiling && t1 < 0) {
@@ -322,8 +342,9 @@ int sweep(zgr_ctx* ctx, std::vector<Group>& groups, const TensorDesc* d_descs, i
       }
       cudaEventRecord(e0, st);
     }
-    const int rc = check(ctx, g.kc.path == PATH_UMMA ? launch_sweep_umma(g.kc, p, ctx->d_tmaps, ctx->d_err, grid, st)
-                                                     : launch_sweep(g.kc, p, grid, st));
+    const int rc = check(ctx, g.kc.path == PATH_UMMA ? launch_sweep_umma(g.kc, p, tmaps, ctx->d_err, grid, st)
+                              : g.kc.path == PATH_GENERIC && g.kc.kpad > 0 ? launch_sweep_tile(g.kc, p, tmaps, ctx->d_err, grid, st)
+                                                                           : launch_sweep(g.kc, p, grid, st));
     if (rc != ZGR_OK) {
       if (e0) cudaEventDestroy(e0);
       if (e1) cudaEventDestroy(e1);
@@ -361,9 +382,9 @@ int refresh_operands(zgr_ctx* ctx, int32_t tensor, cudaStream_t st) {
       if (rc == ZGR_OK) ctx->launches++;
     }
   }
-  if (rc == ZGR_OK && td.umma) {
-    const int64_t rows_pad = ((td.rows + 127) / 128) * 128;
-    rc = check(ctx, launch_split_subspace_rowmajor(td.U, td.rows, td.rank, td.kpad, rows_pad, td.ushift, td.Uhi, td.Ulo, st));
+  const int32_t job = ctx->split_job[static_cast<size_t>(tensor)];
+  if (rc == ZGR_OK && job >= 0) {
+    rc = check(ctx, launch_split_subspaces(ctx->d_split_jobs + job, 1, st));
     if (rc == ZGR_OK) ctx->launches++;
   }
   return rc;
@@ -538,9 +559,9 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
     td.id = l;
     td.dtype = t.dtype;
     td.umma = 0;
+    td.tile = 0;
     td.ushift = 0;
-    td.Uhi = nullptr;
-    td.Ulo = nullptr;
+    for (void*& copy : td.Ucopy) copy = nullptr;
     const bool vec = (reinterpret_cast<uintptr_t>(t.data) & 15) == 0 && (t.cols % 8 == 0);
     if (guided_on && t.rank > 8 && vec && t.dtype != ZGR_F32) {
       // tensor-core path: library-owned copy of U in A-fragment order
@@ -552,37 +573,44 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
       if (rc == ZGR_OK) rc = check(ctx, launch_split_subspace(t.U, t.rows, t.rank, td.kpad, frag, nullptr));
       if (rc == ZGR_OK) ctx->launches++;
       td.Ufrag = frag;
-      // tcgen05 + TMA path: row-major hi/lo copies of U and three tensor maps
-      if (rc == ZGR_OK && umma_wanted() && encode_tiled_fn() != nullptr && t.rows < (int64_t{1} << 31) - 256 && t.cols < (int64_t{1} << 31) - 256) {
-        const int64_t rows_pad = ((t.rows + 127) / 128) * 128;
-        // entries of an orthonormal U are about 1/sqrt(rows): scaled by 2^ushift they sit between 1 and 2 in size
-        // (capped at 2^12, which leaves fp16 room for entries up to 16 in size)
-        td.ushift = std::min<int32_t>(12, static_cast<int32_t>(std::ceil(0.5 * std::log2(static_cast<double>(t.rows)))));
-        uint16_t *hi = nullptr, *lo = nullptr;
-        rc = dev_alloc(ctx, &hi, static_cast<size_t>(rows_pad) * td.kpad);
-        if (rc == ZGR_OK) rc = dev_alloc(ctx, &lo, static_cast<size_t>(rows_pad) * td.kpad);
-        if (rc == ZGR_OK) rc = check(ctx, launch_split_subspace_rowmajor(t.U, t.rows, t.rank, td.kpad, rows_pad, td.ushift, hi, lo, nullptr));
-        if (rc == ZGR_OK) {
-          ctx->launches++;
-          CUtensorMap* m = &ctx->tmaps[static_cast<size_t>(3 * l)];
-          if (make_map_16bit(m, t.data, t.rows, t.cols, 64) && make_map_16bit(m + 1, hi, rows_pad, td.kpad, td.kpad) &&
-              make_map_16bit(m + 2, lo, rows_pad, td.kpad, td.kpad)) {
-            td.umma = 1;
-            td.Uhi = hi;
-            td.Ulo = lo;
-          }
+    }
+    // tcgen05 kernels: row-major copies of U in parts, and three tensor maps
+    const int kind = tensor_core_kind(t, guided_on);
+    if (rc == ZGR_OK && kind != 0 && umma_wanted() && encode_tiled_fn() != nullptr) {
+      const int parts = kind == 1 ? 2 : 3;
+      const int64_t rows_pad = ((t.rows + 127) / 128) * 128;
+      td.kpad = t.rank <= 16 ? 16 : (t.rank <= 32 ? 32 : 64);
+      // entries of an orthonormal U are about 1/sqrt(rows): scaled by 2^ushift they sit between 1 and 2 in size
+      // (capped at 2^12, which leaves fp16 room for entries up to 16 in size); the bf16 parts need no scaling
+      if (kind == 1) td.ushift = std::min<int32_t>(12, static_cast<int32_t>(std::ceil(0.5 * std::log2(static_cast<double>(t.rows)))));
+      uint16_t* part[3] = {nullptr, nullptr, nullptr};
+      for (int i = 0; i < parts && rc == ZGR_OK; ++i) rc = dev_alloc(ctx, &part[i], static_cast<size_t>(rows_pad) * td.kpad);
+      if (rc == ZGR_OK) {
+        CUtensorMap* m = &ctx->tmaps[static_cast<size_t>(3 * l)];
+        bool maps = kind == 1 ? make_map_16bit(m, t.data, t.rows, t.cols, 64) : true;
+        for (int i = 0; i < parts; ++i) maps = maps && make_map_16bit(m + (kind == 1 ? 1 : 0) + i, part[i], rows_pad, td.kpad, td.kpad);
+        if (maps) {
+          (kind == 1 ? td.umma : td.tile) = 1;
+          for (int i = 0; i < parts; ++i) td.Ucopy[i] = part[i];
         }
       }
     }
   }
+  ctx->split_job.assign(static_cast<size_t>(n), -1);
   if (rc == ZGR_OK) {
     std::vector<SplitJob> jobs;
-    for (const TensorDesc& td : ctx->descs)
-      if (td.umma) jobs.push_back(SplitJob{td.U, td.Uhi, td.Ulo, td.rows, ((td.rows + 127) / 128) * 128, td.rank, td.kpad, td.ushift});
+    for (int32_t l = 0; l < n; ++l) {
+      const TensorDesc& td = ctx->descs[static_cast<size_t>(l)];
+      if (!td.umma && !td.tile) continue;
+      ctx->split_job[static_cast<size_t>(l)] = static_cast<int32_t>(jobs.size());
+      jobs.push_back(SplitJob{td.U, {td.Ucopy[0], td.Ucopy[1], td.Ucopy[2]}, td.rows, ((td.rows + 127) / 128) * 128, td.rank, td.kpad, td.umma ? td.ushift : -1});
+    }
     ctx->n_split_jobs = static_cast<int>(jobs.size());
     if (!jobs.empty()) {
       rc = dev_alloc(ctx, &ctx->d_split_jobs, jobs.size());
       if (rc == ZGR_OK) rc = check(ctx, cudaMemcpy(ctx->d_split_jobs, jobs.data(), jobs.size() * sizeof(SplitJob), cudaMemcpyHostToDevice));
+      if (rc == ZGR_OK) rc = check(ctx, launch_split_subspaces(ctx->d_split_jobs, ctx->n_split_jobs, nullptr));
+      if (rc == ZGR_OK) ctx->launches++;
     }
   }
   if (rc == ZGR_OK) rc = dev_alloc(ctx, &ctx->d_tmaps, ctx->tmaps.size());
@@ -1029,7 +1057,7 @@ int zgr_debug_z(zgr_ctx* ctx, uint64_t seed, int32_t tensor, float* dev_out, voi
   if (rc == ZGR_OK) rc = upload_groups(ctx, groups);
   if (rc == ZGR_OK) rc = check(ctx, cudaMemsetAsync(dev_out, 0, static_cast<size_t>(one[0].rows * one[0].cols) * sizeof(float), st));
   const double one_scale = 1.0;
-  if (rc == ZGR_OK) rc = sweep(ctx, groups, d_one, 1, &seed, &one_scale, st);
+  if (rc == ZGR_OK) rc = sweep(ctx, groups, d_one, 1, &seed, &one_scale, st, 0, -1, false, ctx->d_tmaps + 3 * tensor);
   if (rc == ZGR_OK) rc = check(ctx, cudaStreamSynchronize(st));
   for (size_t i = owned_before; i < ctx->owned.size(); ++i) cudaFree(ctx->owned[i]);
   ctx->owned.resize(owned_before);
@@ -1179,7 +1207,11 @@ int zgr_debug_plan(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, 
       // what zgr_init would have built for this tensor: operand copies for the tensor-core kernels
       td.kpad = t.rank <= 16 ? 16 : (t.rank <= 32 ? 32 : 64);
       td.Ufrag = reinterpret_cast<const uint4*>(uintptr_t{16});   // marker only: never dereferenced by the planner
-      td.umma = (tcgen05 && t.rows < (int64_t{1} << 31) - 256 && t.cols < (int64_t{1} << 31) - 256) ? 1 : 0;
+    }
+    const int kind = tcgen05 ? tensor_core_kind(t, guided_on) : 0;
+    if (kind != 0) {
+      td.kpad = t.rank <= 16 ? 16 : (t.rank <= 32 ? 32 : 64);
+      (kind == 1 ? td.umma : td.tile) = 1;
     }
     all[static_cast<size_t>(l)] = l;
   }
@@ -1199,21 +1231,21 @@ int zgr_debug_plan(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, 
 int zgr_update_subspaces(zgr_ctx* ctx, int32_t n, const int32_t* tensors, const float* const* U_src, int32_t src_is_host, void* stream) {
   if (!ctx || !tensors || n < 1) return ZGR_EINVAL;
   std::vector<char> seen(ctx->descs.size(), 0);
-  int n_umma = 0;
+  int n_jobs = 0;
   for (int32_t i = 0; i < n; ++i) {
     const int32_t l = tensors[i];
     if (l < 0 || l >= static_cast<int32_t>(ctx->descs.size()) || seen[static_cast<size_t>(l)]) return ZGR_EINVAL;
     seen[static_cast<size_t>(l)] = 1;
     if (ctx->descs[static_cast<size_t>(l)].rank == 0) return ZGR_EINVAL;
-    n_umma += ctx->descs[static_cast<size_t>(l)].umma ? 1 : 0;
+    n_jobs += ctx->split_job[static_cast<size_t>(l)] >= 0 ? 1 : 0;
   }
   if (ctx->sticky) return ctx->sticky;
   if (!on_ctx_device(ctx)) return ZGR_EINVAL;
   if (!ctx->ledger.empty()) return ZGR_ESTATE;
   ctx->held_valid = false;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  // every tensor of the tcgen05 path is listed: their operand copies are rebuilt by one launch after the copies
-  const bool fused = n_umma > 0 && n_umma == ctx->n_split_jobs;
+  // every tensor of the tcgen05 paths is listed: their operand copies are rebuilt by one launch after the copies
+  const bool fused = n_jobs > 0 && n_jobs == ctx->n_split_jobs;
   for (int32_t i = 0; i < n; ++i) {
     const int32_t l = tensors[i];
     TensorDesc& td = ctx->descs[static_cast<size_t>(l)];
@@ -1232,15 +1264,15 @@ int zgr_update_subspaces(zgr_ctx* ctx, int32_t n, const int32_t* tensors, const 
         ctx->launches++;
       }
     }
-    if (td.umma && !fused) {
-      const int64_t rows_pad = ((td.rows + 127) / 128) * 128;
-      const int rc = check(ctx, launch_split_subspace_rowmajor(td.U, td.rows, td.rank, td.kpad, rows_pad, td.ushift, td.Uhi, td.Ulo, st));
+    const int32_t job = ctx->split_job[static_cast<size_t>(l)];
+    if (job >= 0 && !fused) {
+      const int rc = check(ctx, launch_split_subspaces(ctx->d_split_jobs + job, 1, st));
       if (rc != ZGR_OK) return rc;
       ctx->launches++;
     }
   }
   if (fused) {
-    const int rc = check(ctx, launch_split_subspace_rowmajor_all(ctx->d_split_jobs, ctx->n_split_jobs, st));
+    const int rc = check(ctx, launch_split_subspaces(ctx->d_split_jobs, ctx->n_split_jobs, st));
     if (rc != ZGR_OK) return rc;
     ctx->launches++;
   }

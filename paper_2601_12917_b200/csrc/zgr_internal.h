@@ -25,8 +25,8 @@ struct TensorDesc {
   int32_t qrows;         // rows of G taken from the codes (Sec. 3.4, proportion omega); rows beyond it are drawn from the seed
   int32_t umma;          // 1: served by the tcgen05 + TMA kernel (tensor maps and row-major hi/lo copies of U exist)
   int32_t ushift;        // the hi/lo copies hold U * 2^ushift (brings a typical entry of an orthonormal U near 1)
-  void* Uhi;             // library-owned, rows_pad x kpad fp16 row-major (TMA source), or null
-  void* Ulo;
+  int32_t tile;          // 1: served by sweep_tile_kernel (tensor maps and the three bf16 parts of U exist)
+  void* Ucopy[3];        // library-owned, rows_pad x kpad row-major (TMA sources): fp16 hi, lo (umma) or three bf16 parts (tile)
 };
 
 // One unit of work of a sweep kernel.

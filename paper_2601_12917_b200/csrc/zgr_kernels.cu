@@ -18,8 +18,6 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
-#include <cmath>
-
 #include "zgr_device.cuh"
 #include "zgr_kernels.h"
 
@@ -489,27 +487,26 @@ __device__ __forceinline__ void split_f16_scaled(float x, float scale, __half& h
   lo = __float2half_rn(y - __half2float(hi));
 }
 
-__global__ void split_subspace_rowmajor_kernel(const float* __restrict__ U, int64_t rows, int r, int kp, int64_t rows_pad, float scale,
-                                               __half* __restrict__ hi, __half* __restrict__ lo) {
-  const int64_t idx = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-  if (idx >= rows_pad * kp) return;
-  const int64_t row = idx / kp;
-  const int k = static_cast<int>(idx % kp);
-  const float x = (row < rows && k < r) ? U[row * r + k] : 0.0f;
-  split_f16_scaled(x, scale, hi[idx], lo[idx]);
-}
-
-__global__ void split_subspace_rowmajor_all_kernel(const SplitJob* __restrict__ jobs) {
+// Row-major operand copies of U for a list of tensors: two fp16 parts of U 2^shift (TMA-staged kernel) or three bf16 parts
+// of U (tile kernel; x = p0 + p1 + p2 exactly).
+__global__ void split_subspaces_kernel(const SplitJob* __restrict__ jobs) {
   const SplitJob j = jobs[blockIdx.y];
   const int64_t n = j.rows_pad * j.kp;
-  __half* hi = static_cast<__half*>(j.hi);
-  __half* lo = static_cast<__half*>(j.lo);
-  const float scale = __int_as_float((127 + j.shift) << 23);
+  const float scale = j.shift >= 0 ? __int_as_float((127 + j.shift) << 23) : 1.0f;
   for (int64_t idx = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; idx < n; idx += static_cast<int64_t>(gridDim.x) * blockDim.x) {
     const int64_t row = idx / j.kp;
     const int k = static_cast<int>(idx % j.kp);
     const float x = (row < j.rows && k < j.r) ? j.U[row * j.r + k] : 0.0f;
-    split_f16_scaled(x, scale, hi[idx], lo[idx]);
+    if (j.shift >= 0) {
+      split_f16_scaled(x, scale, static_cast<__half*>(j.part[0])[idx], static_cast<__half*>(j.part[1])[idx]);
+    } else {
+      const __nv_bfloat16 a = __float2bfloat16_rn(x);
+      const float r1 = x - __bfloat162float(a);
+      const __nv_bfloat16 b = __float2bfloat16_rn(r1);
+      static_cast<__nv_bfloat16*>(j.part[0])[idx] = a;
+      static_cast<__nv_bfloat16*>(j.part[1])[idx] = b;
+      static_cast<__nv_bfloat16*>(j.part[2])[idx] = __float2bfloat16_rn(r1 - __bfloat162float(b));
+    }
   }
 }
 
@@ -644,17 +641,9 @@ cudaError_t launch_split_subspace(const float* U, int64_t rows, int r, int kp, u
   return cudaGetLastError();
 }
 
-cudaError_t launch_split_subspace_rowmajor_all(const SplitJob* d_jobs, int n_jobs, cudaStream_t st) {
+cudaError_t launch_split_subspaces(const SplitJob* d_jobs, int n_jobs, cudaStream_t st) {
   if (n_jobs <= 0) return cudaSuccess;
-  split_subspace_rowmajor_all_kernel<<<dim3(64, static_cast<unsigned>(n_jobs)), 256, 0, st>>>(d_jobs);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_split_subspace_rowmajor(const float* U, int64_t rows, int r, int kp, int64_t rows_pad, int shift, void* hi, void* lo, cudaStream_t st) {
-  const int64_t n = rows_pad * kp;
-  const int block = 256;
-  split_subspace_rowmajor_kernel<<<static_cast<unsigned>((n + block - 1) / block), block, 0, st>>>(
-      U, rows, r, kp, rows_pad, std::ldexp(1.0f, shift), static_cast<__half*>(hi), static_cast<__half*>(lo));
+  split_subspaces_kernel<<<dim3(64, static_cast<unsigned>(n_jobs)), 256, 0, st>>>(d_jobs);
   return cudaGetLastError();
 }
 

@@ -33,17 +33,19 @@ cudaError_t launch_sweep_umma(const KernelChoice& kc, const SweepParams& p, cons
 // Test hook: the sweep kernel with its fp32 results diverted to p.zout (see the ZOUT parameter of the kernel).
 cudaError_t launch_debug_z_umma(const KernelChoice& kc, const SweepParams& p, const CUtensorMap* tmaps, int* error, int grid, cudaStream_t st);
 cudaError_t launch_stats_umma(const KernelChoice& kc, const SweepParams& p, const CUtensorMap* tmaps, int* error, int grid, cudaStream_t st);
-cudaError_t launch_split_subspace_rowmajor(const float* U, int64_t rows, int r, int kp, int64_t rows_pad, int shift, void* hi, void* lo, cudaStream_t st);
-// The same for a device-resident list of tensors in one launch (grid.y = job).
+// Sweep of the other guided tensors (fp32 with rank > 8, rows that are not a multiple of eight elements).  tmaps: the three
+// bf16 parts of U per tensor; kc.kpad = contraction width.
+int tile_strip_cols();
+cudaError_t launch_sweep_tile(const KernelChoice& kc, const SweepParams& p, const CUtensorMap* tmaps, int* error, int grid, cudaStream_t st);
+// Rebuild of the row-major operand copies of U for a device-resident list of tensors in one launch (grid.y = job).
 struct SplitJob {
   const float* U;
-  void* hi;
-  void* lo;
+  void* part[3];   // rows_pad x kp each
   int64_t rows, rows_pad;
   int32_t r, kp;
-  int32_t shift;   // the copies hold U * 2^shift
+  int32_t shift;   // two fp16 parts (hi, lo) of U * 2^shift; -1: three bf16 parts of U
 };
-cudaError_t launch_split_subspace_rowmajor_all(const SplitJob* d_jobs, int n_jobs, cudaStream_t st);
+cudaError_t launch_split_subspaces(const SplitJob* d_jobs, int n_jobs, cudaStream_t st);
 
 cudaError_t launch_stats(int bits, const SweepParams& p, int grid, cudaStream_t st);
 // Norm bookkeeping, second stage: tensor l owns the work items [first, first + count) of the slot array `slots`

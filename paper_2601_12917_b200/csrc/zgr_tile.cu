@@ -1,0 +1,503 @@
+// Sweep with a tensor-core contraction for the guided tensors that the TMA-staged kernel (zgr_umma.cu) cannot take:
+// fp32 storage with rank > 8, and any storage whose rows are not a multiple of eight elements long.
+//     theta <- rnd(theta + c (a Z + b U G))            (Eq. (perturbation) applied as in Algorithm 1)
+//
+// Layout.  Generator blocks run along the flattened tensor, eight elements ("an octet") at a time, so in a tensor whose
+// row length is no multiple of eight the octets of row m start at column  h_m = -(m cols) mod 8  and one of them
+// straddles each row end.  A work item is a strip of 128 columns x a range of rows; within it a row owns the
+// octets whose first element falls into the strip (16 of them, whatever h_m is), plus, in the strip at column 0, the
+// tail of the octet that began in the row before.  An owned octet reaches up to 7 columns beyond the strip, so the
+// product tile is computed 144 columns wide.
+//
+// Pipeline (one CTA per SM, static round-robin over the items):
+//   warp 0   TMA loads of U, 128 rows at a time, pre-split into three bf16 parts
+//   warp 1   tcgen05.mma:  D = c b U G  (128 x 144, fp32) into one of three tensor-memory buffers
+//   warps 2-17  coefficient strips c b G (three bf16 parts, K-major) into shared memory, one item ahead where two strips
+//            fit; then per tile and warp 32 rows x 32 columns: D through a warp-private shared-memory buffer, from one
+//            row per thread (tensor memory) to one octet per thread (global memory: four lanes take 64 / 128
+//            contiguous bytes of a row), and there the weights are loaded, the normals added, the result rounded and stored.
+//
+// Operand precision.  An fp32 number is the sum of three bf16 numbers (8 bits each) without error and without range
+// limits; six of the nine products are formed, the others are below 2^-24 of the result.  The contraction is therefore
+// as accurate as a chain of fp32 multiply-adds.
+//
+// Bank conflicts of the transposition.  Row m of a warp's buffer is `pitch` floats long; lane (m, o) reads
+// D[m][h_m + 8 o + i].  Eight rows x four octets per read: distinct banks if m pitch + h_m = m (pitch - cols) takes
+// eight different values modulo 8, i.e. if pitch - cols is odd.  pitch = 41 for an even, 42 for an odd number of columns
+// (the writes, one float per row, are then at most two-way).  With cols a multiple of 8 every h_m is 0 and both sides
+// use 128-bit accesses with pitch 36.
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
+#include <cuda_runtime.h>
+
+#include <type_traits>
+
+#include "zgr_device.cuh"
+#include "zgr_kernels.h"
+#include "zgr_tcgen05.cuh"
+
+namespace zgr {
+namespace {
+
+constexpr int kTileM = 128, kStrip = 128, kTileN = 144;
+constexpr int kAcc = 3;                        // accumulator buffers: 3 x 144 of the 512 tensor-memory columns
+constexpr int kEpi = 16;                       // epilogue warps: 32 rows x 32 columns of a tile each
+constexpr int kTileThreads = 32 * (2 + kEpi);
+constexpr int kParts = 3;                      // bf16 parts of an operand
+constexpr int kPitchMax = 42;
+constexpr int kXposeBytes = 32 * kPitchMax * 4;   // one warp's buffer
+
+// Shared-memory plan for contraction width kp (16, 32, 64).
+struct TileSmem {
+  int rowb, u_bytes, g_bytes, u_stages, g_stages, total;
+};
+__host__ __device__ inline TileSmem tile_smem(int kp) {
+  TileSmem t;
+  t.rowb = 2 * kp;
+  t.u_bytes = kTileM * t.rowb;
+  t.g_bytes = kTileN * t.rowb;
+  t.u_stages = kp == 64 ? 1 : 2;               // width 64: one U tile and one strip fit beside the buffers
+  t.g_stages = kp == 64 ? 1 : 2;
+  t.total = t.u_stages * kParts * t.u_bytes + t.g_stages * kParts * t.g_bytes + kEpi * kXposeBytes + 256 + 1024;
+  return t;
+}
+
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[40]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,"
+      "%29,%30,%31}, [%32];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]),
+        "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]),
+        "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+      : "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_ld8_tail(uint32_t taddr, uint32_t (&v)[40]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(v[32]), "=r"(v[33]), "=r"(v[34]), "=r"(v[35]), "=r"(v[36]), "=r"(v[37]), "=r"(v[38]), "=r"(v[39])
+               : "r"(taddr)
+               : "memory");
+}
+
+__device__ __forceinline__ void sts16(uint32_t saddr, uint16_t v) { asm volatile("st.shared.b16 [%0], %1;" ::"r"(saddr), "h"(v) : "memory"); }
+
+// x = p0 + p1 + p2 exactly (8 significant bits each)
+__device__ __forceinline__ void split3(float x, uint16_t& p0, uint16_t& p1, uint16_t& p2) {
+  const __nv_bfloat16 a = __float2bfloat16_rn(x);
+  const float r1 = x - __bfloat162float(a);
+  const __nv_bfloat16 b = __float2bfloat16_rn(r1);
+  const __nv_bfloat16 c = __float2bfloat16_rn(r1 - __bfloat162float(b));
+  p0 = __bfloat16_as_ushort(a);
+  p1 = __bfloat16_as_ushort(b);
+  p2 = __bfloat16_as_ushort(c);
+}
+
+// Compressed coefficient of row k, column c, before scale and zero point.
+__device__ __forceinline__ float code1(const TensorDesc& td, int k, int64_t c) {
+  if (td.qbits == 4) {
+    const uint32_t byte = reinterpret_cast<const uint8_t*>(td.q)[static_cast<int64_t>(k) * ((td.cols + 1) >> 1) + (c >> 1)];
+    return static_cast<float>((c & 1) ? (byte >> 4) : (byte & 15u));
+  }
+  return static_cast<float>(td.q[static_cast<int64_t>(k) * td.cols + c]);
+}
+
+// The strip  c b G[0..KP)[col0 .. col0 + 144)  as K-major bf16 operands.  One unit of work is the octet of one row k of G
+// (the octets of G start at other columns in every row when cols is no multiple of 8).
+template <int BITS, bool PRECISE, bool MULTI>
+__device__ __forceinline__ void build_strip(const TensorDesc& td, const SweepParams& p, int64_t col0, int kp, int rowb, int g_bytes, uint32_t g_dst, int et) {
+  constexpr int kOct = kTileN / 8 + 1;
+  const int kp_shift = kp == 64 ? 6 : (kp == 32 ? 5 : 4);
+  const int64_t cols = td.cols;
+  for (int idx = et; idx < (kOct << kp_shift); idx += kEpi * 32) {
+    const int k = idx & (kp - 1), o = idx >> kp_shift;      // consecutive lanes: consecutive k, i.e. neighbouring shared-memory words
+    const int64_t row_e = static_cast<int64_t>(k) * cols;
+    const int64_t e = (((row_e + col0) >> 3) + o) << 3;     // first element of the octet
+    const int64_t c_first = e - row_e;                      // its column (may lie before the strip)
+    const int j0 = static_cast<int>(c_first - col0);        // -7 .. 144
+    float g[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) g[i] = 0.0f;
+    if (k < td.rank && c_first < cols) {
+      if (td.q != nullptr && k < td.qrows) {
+        float cb = p.term[0].cb;
+        if (MULTI)
+          for (int q = 1; q < p.n_terms; ++q) cb += p.term[q].cb;
+        const float lambda = td.qscale[k] * cb;
+        const float delta = td.qzero ? td.qzero[k] : 0.0f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          if (c_first + i >= 0 && c_first + i < cols) g[i] = lambda * (code1(td, k, c_first + i) - delta);
+      } else {
+        normals8<BITS, PRECISE>(p.term[0].keys, static_cast<uint32_t>(td.id), 1u, static_cast<uint64_t>(e), p.unit, g);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) g[i] *= p.term[0].cb;
+        if (MULTI) {
+#pragma unroll 1
+          for (int q = 1; q < p.n_terms; ++q) {
+            float y[8];
+            normals8<BITS, PRECISE>(p.term[q].keys, static_cast<uint32_t>(td.id), 1u, static_cast<uint64_t>(e), p.unit, y);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) g[i] = fmaf(p.term[q].cb, y[i], g[i]);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int j = j0 + i;
+      if (j >= 0 && j < kTileN) {
+        uint16_t q0, q1, q2;
+        split3(c_first + i < cols ? g[i] : 0.0f, q0, q1, q2);
+        const uint32_t at = g_dst + swizzle(static_cast<uint32_t>(j * rowb + 2 * k), rowb);
+        sts16(at, q0);
+        sts16(at + g_bytes, q1);
+        sts16(at + 2 * g_bytes, q2);
+      }
+    }
+  }
+}
+
+// raw storage of an octet: 16 bytes for 16-bit types, 32 for fp32
+template <typename T>
+struct RawOct {
+  static constexpr int N = sizeof(T) == 4 ? 2 : 1;
+  uint4 v[N];
+  __device__ __forceinline__ void load(const T* p) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) v[i] = __ldcs(reinterpret_cast<const uint4*>(p) + i);
+  }
+  __device__ __forceinline__ void unpack(float (&f)[8]) const {
+    if constexpr (sizeof(T) == 4) {
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        f[4 * i] = __uint_as_float(v[i].x);
+        f[4 * i + 1] = __uint_as_float(v[i].y);
+        f[4 * i + 2] = __uint_as_float(v[i].z);
+        f[4 * i + 3] = __uint_as_float(v[i].w);
+      }
+    } else {
+      const uint32_t w[4] = {v[0].x, v[0].y, v[0].z, v[0].w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if constexpr (std::is_same<T, __nv_bfloat16>::value) {
+          f[2 * i] = __uint_as_float(w[i] << 16);
+          f[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
+        } else {
+          const float2 h = __half22float2(*reinterpret_cast<const __half2*>(&w[i]));
+          f[2 * i] = h.x;
+          f[2 * i + 1] = h.y;
+        }
+      }
+    }
+  }
+};
+
+}  // namespace
+
+template <typename T, int BITS, bool PRECISE, bool MULTI, bool SSTATS>
+__global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __grid_constant__ SweepParams p, const CUtensorMap* __restrict__ tmaps,
+                                                                     int* __restrict__ error, const int kp) {
+  extern __shared__ uint8_t smem_raw[];
+  const TileSmem L = tile_smem(kp);
+  const int US = L.u_stages, GS = L.g_stages, rowb = L.rowb;
+  uint8_t* u_base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  uint8_t* g_base = u_base + US * kParts * L.u_bytes;
+  uint8_t* x_base = g_base + GS * kParts * L.g_bytes;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(x_base + kEpi * kXposeBytes);
+  const uint32_t bar0 = smem_u32(bars);
+  auto BAR_ACC_FULL = [&](int b) { return bar0 + 8u * static_cast<uint32_t>(b); };
+  auto BAR_ACC_EMPTY = [&](int b) { return bar0 + 8u * static_cast<uint32_t>(kAcc + b); };
+  auto BAR_U_FULL = [&](int u) { return bar0 + 8u * static_cast<uint32_t>(2 * kAcc + u); };
+  auto BAR_U_FREE = [&](int u) { return bar0 + 8u * static_cast<uint32_t>(2 * kAcc + 2 + u); };
+  auto BAR_G = [&](int g) { return bar0 + 8u * static_cast<uint32_t>(2 * kAcc + 4 + g); };
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kAcc + 6);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+  if (threadIdx.x == 0) {
+    for (int b = 0; b < kAcc; ++b) {
+      mbar_init(BAR_ACC_FULL(b), 1);
+      mbar_init(BAR_ACC_EMPTY(b), kEpi);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(BAR_U_FULL(i), 1);
+      mbar_init(BAR_U_FREE(i), 1);
+      mbar_init(BAR_G(i), kEpi);
+    }
+    *abort_flag = 0;
+    fence_mbar_init();
+  }
+  __syncthreads();
+  if (warp == 1) {
+    tmem_alloc(smem_u32(tmem_slot), 512);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+
+  // All roles walk the same sequence of (item, row tile) pairs; t counts tiles over the life of the CTA.
+  if (warp == 0) {
+    // ------------------------------------------------ U loads
+    if (elect_one()) {
+      int t = 0;
+      bool ok = true;
+      for (int it = blockIdx.x; it < p.n_items && ok; it += gridDim.x) {
+        const WorkItem w = p.items[it];
+        const CUtensorMap* tm = tmaps + 3 * w.tensor;
+        const int row_end = static_cast<int>(w.row0_or_e0 + w.nrows_or_count);
+        for (int row0 = static_cast<int>(w.row0_or_e0); row0 < row_end; row0 += kTileM, ++t) {
+          const int u = t % US;
+          if (t >= US && !mbar_wait<true>(BAR_U_FREE(u), ((t / US) - 1) & 1, abort_flag, error, 21)) { ok = false; break; }
+          const uint32_t dst = smem_u32(u_base + u * kParts * L.u_bytes);
+          mbar_arrive_expect_tx(BAR_U_FULL(u), static_cast<uint32_t>(kParts * L.u_bytes));
+          for (int i = 0; i < kParts; ++i) tma_load_2d(dst + i * L.u_bytes, tm + i, 0, row0, BAR_U_FULL(u));
+        }
+      }
+      // let the last loads land before the CTA gives up its shared memory
+      for (int v = (t > US ? t - US : 0); v < t; ++v) {
+        const unsigned long long t0 = clock64();
+        while (!mbar_try_wait(BAR_U_FULL(v % US), (v / US) & 1) && clock64() - t0 < kWaitLimitCycles) {
+        }
+      }
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------ products
+    if (elect_one()) {
+      const uint32_t idesc = make_idesc(1, kTileN);
+      const uint64_t desc_u0 = make_desc(smem_u32(u_base), rowb);
+      const uint64_t desc_g0 = make_desc(smem_u32(g_base), rowb);
+      const uint64_t u_part = static_cast<uint64_t>(L.u_bytes >> 4), g_part = static_cast<uint64_t>(L.g_bytes >> 4);
+      int t = 0, item_no = 0;
+      bool ok = true;
+      for (int it = blockIdx.x; it < p.n_items && ok; it += gridDim.x, ++item_no) {
+        const WorkItem w = p.items[it];
+        const int g = item_no % GS;
+        if (!mbar_wait<true>(BAR_G(g), (item_no / GS) & 1, abort_flag, error, 22)) break;
+        const uint64_t dg = desc_g0 + static_cast<uint64_t>((g * kParts * L.g_bytes) >> 4);
+        const int row_end = static_cast<int>(w.row0_or_e0 + w.nrows_or_count);
+        for (int row0 = static_cast<int>(w.row0_or_e0); row0 < row_end; row0 += kTileM, ++t) {
+          const int u = t % US, b = t % kAcc;
+          if (!mbar_wait<true>(BAR_U_FULL(u), (t / US) & 1, abort_flag, error, 23)) { ok = false; break; }
+          if (t >= kAcc && !mbar_wait<true>(BAR_ACC_EMPTY(b), ((t / kAcc) - 1) & 1, abort_flag, error, 24)) { ok = false; break; }
+          tc_fence_after();
+          const uint64_t du = desc_u0 + static_cast<uint64_t>((u * kParts * L.u_bytes) >> 4);
+          const uint32_t d = tmem_base + static_cast<uint32_t>(b * kTileN);
+          // smallest products first: (0,2) (2,0) (1,1) (0,1) (1,0) (0,0); part 0 is the leading one
+          uint32_t acc = 0;
+#pragma unroll
+          for (int pr = 0; pr < 6; ++pr) {
+            constexpr int kA[6] = {0, 2, 1, 0, 1, 0}, kB[6] = {2, 0, 1, 1, 0, 0};
+            for (int k = 0; k < kp / 16; ++k) {
+              umma(d, du + kA[pr] * u_part + static_cast<uint64_t>(2 * k), dg + kB[pr] * g_part + static_cast<uint64_t>(2 * k), idesc, acc);
+              acc = 1;
+            }
+          }
+          umma_commit(BAR_ACC_FULL(b));
+          umma_commit(BAR_U_FREE(u));
+        }
+      }
+    }
+  } else {
+    // ------------------------------------------------ epilogue
+    const int e = warp - 2, et = e * 32 + lane;
+    const int quad = warp & 3, cg = e >> 2;                  // tensor-memory lanes 32 quad ..., columns 32 cg ... of the strip
+    const int sub = lane >> 2, o = lane & 3;                 // octet view: row 8 pass + sub, octet o of the 32 columns
+    const uint32_t xbuf = smem_u32(x_base) + static_cast<uint32_t>(e * kXposeBytes);
+    const uint32_t g_s = smem_u32(g_base);
+    const uint32_t tmem_warp = tmem_base + (static_cast<uint32_t>(32 * quad) << 16) + static_cast<uint32_t>(32 * cg);
+    int t = 0, item_no = 0;
+    bool ok = true;
+    auto strip_for = [&](int it, int no) {
+      const WorkItem w = p.items[it];
+      build_strip<BITS, PRECISE, MULTI>(p.tensors[w.tensor], p, w.col0, kp, rowb, L.g_bytes, g_s + static_cast<uint32_t>((no % GS) * kParts * L.g_bytes), et);
+      fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(BAR_G(no % GS));
+    };
+    if (static_cast<int>(blockIdx.x) < p.n_items) strip_for(blockIdx.x, 0);
+    for (int it = blockIdx.x; it < p.n_items && ok; it += gridDim.x, ++item_no) {
+      const WorkItem w = p.items[it];
+      const TensorDesc& td = p.tensors[w.tensor];
+      const uint32_t tid = static_cast<uint32_t>(td.id);
+      const int64_t cols = td.cols;
+      const uint32_t cols8 = static_cast<uint32_t>(cols) & 7u;
+      const bool even8 = cols8 == 0;
+      const int pitch = even8 ? 36 : ((cols & 1) ? 42 : 41);
+      T* const base = static_cast<T*>(td.data);
+      const bool vec = (reinterpret_cast<uintptr_t>(base) & 15) == 0;
+      const int64_t row_end = w.row0_or_e0 + w.nrows_or_count;
+      const int c_chunk = 32 * cg;                           // first column of this warp's chunk within the strip
+      const bool next = it + static_cast<int>(gridDim.x) < p.n_items;
+      double s_iso = 0.0, s_gd = 0.0, s_z = 0.0;             // SSTATS only
+      for (int64_t row0 = w.row0_or_e0; row0 < row_end && ok; row0 += kTileM, ++t) {
+        // the strip of the next item goes into the other buffer before this item's last tile, so that its products run
+        // while this tile is worked on
+        if (GS == 2 && next && row0 + kTileM >= row_end) strip_for(it + gridDim.x, item_no + 1);
+        const int b = t % kAcc;
+        const int64_t wrow = row0 + 32 * quad;               // first row of this warp
+        // one octet per pass: element index of its start, its column, the elements of it that belong to this row
+        const uint32_t h_sub = (0u - static_cast<uint32_t>((wrow + sub) & 7) * cols8) & 7u;   // the same for all passes: rows 8 apart
+        const int64_t e_sub = (wrow + sub) * cols + w.col0 + c_chunk + 8 * o + h_sub;
+        const int64_t c = w.col0 + c_chunk + 8 * o + h_sub;
+        const int n_el = static_cast<int>(min(static_cast<int64_t>(8), cols - c));
+        const bool full = vec && n_el == 8;
+        // weights of the first passes, on their way while the accumulator is waited for (four octets of 16-bit weights fit
+        // the register budget, two of fp32)
+        constexpr int kAhead = sizeof(T) == 4 ? 2 : 4;
+        RawOct<T> raw[kAhead];
+        auto fetch = [&](int pass) {
+          if (full && wrow + 8 * pass + sub < row_end) raw[pass % kAhead].load(base + e_sub + 8 * pass * cols);
+        };
+#pragma unroll
+        for (int pass = 0; pass < kAhead; ++pass) fetch(pass);
+        if (!mbar_wait<false>(BAR_ACC_FULL(b), (t / kAcc) & 1, abort_flag, error, 25)) { ok = false; break; }
+        tc_fence_after();
+        {
+          uint32_t v[40];
+          tmem_ld32(tmem_warp + static_cast<uint32_t>(b * kTileN), v);
+          tmem_ld8_tail(tmem_warp + static_cast<uint32_t>(b * kTileN + 32), v);
+          tmem_ld_wait();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(BAR_ACC_EMPTY(b));
+          const uint32_t xrow = xbuf + static_cast<uint32_t>(lane * pitch * 4);
+          if (even8) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) sts128(xrow + 16u * i, make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
+          } else {
+#pragma unroll
+            for (int i = 0; i < 40; ++i) sts32(xrow + 4u * i, v[i]);
+          }
+        }
+        __syncwarp();
+        auto finish = [&](int64_t el, int i0, int i1, float (&d)[8], bool whole, const RawOct<T>* r) {
+          float th[8], z[8];
+          if (whole) {
+            r->unpack(th);
+          } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) th[i] = (i >= i0 && i < i1) ? Storage<T>::load1(base + el + i) : 0.0f;
+          }
+          if constexpr (!PRECISE && !SSTATS) {
+            const uint64_t oct = static_cast<uint64_t>(el) >> 3;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) z[i] = d[i];
+            normals8_acc<BITS>(p.term[0].keys, tid, static_cast<uint32_t>(oct), static_cast<uint32_t>(oct >> 32), p.term[0].iso, z);
+            if (MULTI) {
+#pragma unroll 1
+              for (int q = 1; q < p.n_terms; ++q)
+                normals8_acc<BITS>(p.term[q].keys, tid, static_cast<uint32_t>(oct), static_cast<uint32_t>(oct >> 32), p.term[q].iso, z);
+            }
+          } else {
+            iso8<BITS, PRECISE, MULTI>(p, tid, static_cast<uint64_t>(el), z);
+            if (SSTATS) {
+              float f_iso = 0.0f, f_gd = 0.0f, f_z = 0.0f;
+#pragma unroll
+              for (int i = 0; i < 8; ++i) {
+                if (whole || (i >= i0 && i < i1)) {
+                  f_iso = fmaf(z[i], z[i], f_iso);
+                  f_gd = fmaf(d[i], d[i], f_gd);
+                  f_z = fmaf(z[i] + d[i], z[i] + d[i], f_z);
+                }
+              }
+              s_iso += static_cast<double>(f_iso);
+              s_gd += static_cast<double>(f_gd);
+              s_z += static_cast<double>(f_z);
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) z[i] += d[i];
+          }
+#pragma unroll
+          for (int i = 0; i < 8; ++i) th[i] += z[i];
+          if (whole) {
+            Storage<T>::store8(base + el, th);
+          } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              if (i >= i0 && i < i1) Storage<T>::store1(base + el + i, th[i]);
+          }
+        };
+#pragma unroll
+        for (int pass = 0; pass < 4; ++pass) {
+          if (n_el > 0 && wrow + 8 * pass + sub < row_end) {
+            float d[8];
+            const uint32_t xat = xbuf + static_cast<uint32_t>(((8 * pass + sub) * pitch + 8 * o + static_cast<int>(h_sub)) * 4);
+            if (even8) {
+              const uint4 d0 = lds128(xat), d1 = lds128(xat + 16);
+              d[0] = __uint_as_float(d0.x); d[1] = __uint_as_float(d0.y); d[2] = __uint_as_float(d0.z); d[3] = __uint_as_float(d0.w);
+              d[4] = __uint_as_float(d1.x); d[5] = __uint_as_float(d1.y); d[6] = __uint_as_float(d1.z); d[7] = __uint_as_float(d1.w);
+            } else {
+#pragma unroll
+              for (int i = 0; i < 8; ++i) d[i] = lds32(xat + 4u * i);
+            }
+            finish(e_sub + 8 * pass * cols, 0, n_el, d, full, &raw[pass % kAhead]);
+          }
+          if (pass + kAhead < 4) fetch(pass + kAhead);
+        }
+        if (!even8 && w.col0 == 0 && cg == 0) {
+          // the columns before the first octet of each row: the tail of an octet that began in the previous row
+          const int64_t row = wrow + lane;
+          const int h = static_cast<int>((0u - static_cast<uint32_t>(row & 7) * cols8) & 7u);
+          if (h > 0 && row < row_end) {
+            float d[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) d[i] = i >= 8 - h ? lds32(xbuf + static_cast<uint32_t>((lane * pitch + i - (8 - h)) * 4)) : 0.0f;
+            finish(row * cols + h - 8, 8 - h, static_cast<int>(min(static_cast<int64_t>(8), 8 - h + cols)), d, false, nullptr);
+          }
+        }
+        __syncwarp();
+      }
+      if (GS == 1 && next && ok) strip_for(it + gridDim.x, item_no + 1);   // every product that read the old strip has completed
+      if constexpr (SSTATS) {
+        if (ok) store_item_stats(p, it, e, s_iso, s_gd, s_z);
+      }
+    }
+  }
+
+  // ---- common exit ----
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, 512);
+  }
+}
+
+namespace {
+template <typename T, int BITS, bool PRECISE, bool MULTI, bool SSTATS>
+cudaError_t launch_tile_one(int kp, const SweepParams& p, const CUtensorMap* tmaps, int* error, int grid, cudaStream_t st) {
+  auto k = sweep_tile_kernel<T, BITS, PRECISE, MULTI, SSTATS>;
+  const int smem = tile_smem(kp).total;
+  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, tile_smem(64).total);
+  if (e != cudaSuccess) return e;
+  k<<<grid, kTileThreads, smem, st>>>(p, tmaps, error, kp);
+  return cudaGetLastError();
+}
+template <typename T, bool PRECISE>
+cudaError_t launch_tile_typed(const KernelChoice& kc, const SweepParams& p, const CUtensorMap* tmaps, int* error, int grid, cudaStream_t st) {
+  if (p.n_terms > 1)
+    return kc.bits == 32 ? launch_tile_one<T, 32, PRECISE, true, false>(kc.kpad, p, tmaps, error, grid, st)
+                         : launch_tile_one<T, 16, PRECISE, true, false>(kc.kpad, p, tmaps, error, grid, st);
+  if (p.item_stats != nullptr)
+    return kc.bits == 32 ? launch_tile_one<T, 32, PRECISE, false, true>(kc.kpad, p, tmaps, error, grid, st)
+                         : launch_tile_one<T, 16, PRECISE, false, true>(kc.kpad, p, tmaps, error, grid, st);
+  return kc.bits == 32 ? launch_tile_one<T, 32, PRECISE, false, false>(kc.kpad, p, tmaps, error, grid, st)
+                       : launch_tile_one<T, 16, PRECISE, false, false>(kc.kpad, p, tmaps, error, grid, st);
+}
+}  // namespace
+
+int tile_strip_cols() { return kStrip; }
+
+cudaError_t launch_sweep_tile(const KernelChoice& kc, const SweepParams& p, const CUtensorMap* tmaps, int* error, int grid, cudaStream_t st) {
+  static_assert(kEpi <= kStatSlots, "one bookkeeping slot per epilogue warp");
+  switch (kc.dtype) {
+    case 0: return launch_tile_typed<float, true>(kc, p, tmaps, error, grid, st);
+    case 1: return launch_tile_typed<__half, false>(kc, p, tmaps, error, grid, st);
+    case 2: return launch_tile_typed<__nv_bfloat16, false>(kc, p, tmaps, error, grid, st);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+}  // namespace zgr
