@@ -65,9 +65,9 @@ struct zgr_ctx {
   uint64_t last_seed = 0;             // most recently swept seed (introspection)
   bool guided_at_init = false;        // b != 0 when the sweep plan was made
   SplitJob* d_split_jobs = nullptr;   // one job per tensor served by a tcgen05 kernel: rebuild of its operand copies of U
+  std::vector<SplitJob> split_jobs;   // the same on the host
   std::vector<int32_t> split_job;     // per tensor: its job, or -1
   int n_split_jobs = 0;
-  std::vector<char> frag_stale;       // per tensor: the fragment-order copy of U (legacy tensor-core kernel) lags behind U
   std::vector<Group> groups_multi;    // plan of multi-seed sweeps when it differs from `groups` (legacy tensor-core path only)
   bool multi_planned = false;
   int sticky = 0;                     // first CUDA failure, returned by every later call
@@ -80,6 +80,7 @@ struct zgr_ctx {
   cudaStream_t aux_stream = nullptr;      // zgr_perturb_layers: odd layers run here, so that one layer's tail overlaps the next one's start
   void* d_qr = nullptr;               // scratch of zgr_build_subspace (grown on demand)
   size_t qr_bytes = 0;
+  int* h_status = nullptr;            // host-mapped status word of zgr_build_subspace
 };
 
 namespace {
@@ -221,7 +222,7 @@ void plan(const std::vector<TensorDesc>& descs, const std::vector<int>& which, b
       // fp32 with rank > 8, and rows that are not a multiple of eight elements: sweep_tile_kernel.  (The test hook that
       // sweeps an fp32 image of a 16-bit tensor keeps the one-element-per-thread kernel below.)
       path = PATH_GENERIC; kpad = t.kpad; strip = tile_strip_cols(); row_step = 128;
-    } else if (!vec || (t.rank > 8 && t.Ufrag == nullptr) || (multi && t.rank > 8 && !umma_ok)) {
+    } else if (!vec || (t.rank > 8 && !umma_ok && (t.Ufrag == nullptr || multi))) {
       // (the legacy tensor-core kernel applies one term per sweep; several terms take the fallback)
       path = PATH_GENERIC; kpad = 0; strip = 64; row_step = 1;
     } else if (t.rank <= 8) {
@@ -368,20 +369,28 @@ int flush_descs(zgr_ctx* ctx, cudaStream_t st) {
 
 bool is_finite(double x) { return std::isfinite(x); }
 
+// Fragment-order copy of U for the mma.sync kernel (made on demand for tensors that the tcgen05 kernel sweeps: only the test
+// hook zgr_debug_z reads it there).
+int make_fragments(zgr_ctx* ctx, TensorDesc& td, cudaStream_t st) {
+  int rc = ZGR_OK;
+  if (td.Ufrag == nullptr) {
+    const size_t n_frag = static_cast<size_t>((td.rows + 15) / 16) * (td.kpad / 16) * 2 * 32;
+    uint4* frag = nullptr;
+    rc = dev_alloc(ctx, &frag, n_frag);
+    if (rc != ZGR_OK) return rc;
+    td.Ufrag = frag;
+  }
+  rc = check(ctx, launch_split_subspace(td.U, td.rows, td.rank, td.kpad, const_cast<uint4*>(td.Ufrag), st));
+  if (rc == ZGR_OK) ctx->launches++;
+  return rc;
+}
+
 // Rebuild the library's operand copies of U for one tensor from the subspace buffer (enqueued on st).
 int refresh_operands(zgr_ctx* ctx, int32_t tensor, cudaStream_t st) {
   TensorDesc& td = ctx->descs[static_cast<size_t>(tensor)];
   int rc = ZGR_OK;
-  if (td.Ufrag != nullptr) {
-    if (td.umma) {
-      // the sweeps of this tensor read the row-major copy below; the fragment-order copy is only needed by
-      // zgr_debug_z and is rebuilt there on demand
-      ctx->frag_stale[static_cast<size_t>(tensor)] = 1;
-    } else {
-      rc = check(ctx, launch_split_subspace(td.U, td.rows, td.rank, td.kpad, const_cast<uint4*>(td.Ufrag), st));
-      if (rc == ZGR_OK) ctx->launches++;
-    }
-  }
+  // (for a tensor of the tcgen05 kernel the fragment-order copy is only read by zgr_debug_z, which rebuilds it)
+  if (td.Ufrag != nullptr && !td.umma) rc = make_fragments(ctx, td, st);
   const int32_t job = ctx->split_job[static_cast<size_t>(tensor)];
   if (rc == ZGR_OK && job >= 0) {
     rc = check(ctx, launch_split_subspaces(ctx->d_split_jobs + job, 1, st));
@@ -536,11 +545,25 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
   }
 
   ctx->descs.resize(static_cast<size_t>(n));
-  ctx->frag_stale.assign(static_cast<size_t>(n), 0);
   ctx->tmaps.resize(static_cast<size_t>(3 * n));
   std::memset(ctx->tmaps.data(), 0, ctx->tmaps.size() * sizeof(CUtensorMap));
   const bool guided_on = ctx->b != 0.0;
   ctx->guided_at_init = guided_on;
+  // one allocation for all operand copies
+  void* operands = nullptr;
+  if (umma_wanted() && encode_tiled_fn() != nullptr) {
+    size_t bytes = 0;
+    for (int32_t l = 0; l < n; ++l) {
+      const int kind = tensor_core_kind(tensors[l], guided_on);
+      const size_t kpad = tensors[l].rank <= 16 ? 16 : (tensors[l].rank <= 32 ? 32 : 64);
+      if (kind != 0) bytes += (kind == 1 ? 2 : 3) * static_cast<size_t>((tensors[l].rows + 127) / 128) * 128 * kpad * 2;
+    }
+    if (bytes > 0) {
+      uint8_t* base = nullptr;
+      rc = dev_alloc(ctx, &base, bytes);
+      operands = base;
+    }
+  }
   for (int32_t l = 0; l < n && rc == ZGR_OK; ++l) {
     const zgr_tensor& t = tensors[l];
     TensorDesc& td = ctx->descs[static_cast<size_t>(l)];
@@ -562,43 +585,38 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
     td.tile = 0;
     td.ushift = 0;
     for (void*& copy : td.Ucopy) copy = nullptr;
-    const bool vec = (reinterpret_cast<uintptr_t>(t.data) & 15) == 0 && (t.cols % 8 == 0);
-    if (guided_on && t.rank > 8 && vec && t.dtype != ZGR_F32) {
-      // tensor-core path: library-owned copy of U in A-fragment order
-      td.kpad = t.rank <= 16 ? 16 : (t.rank <= 32 ? 32 : 64);
-      const int64_t tiles = (t.rows + 15) / 16;
-      const size_t n_frag = static_cast<size_t>(tiles) * (td.kpad / 16) * 2 * 32;
-      uint4* frag = nullptr;
-      rc = dev_alloc(ctx, &frag, n_frag);
-      if (rc == ZGR_OK) rc = check(ctx, launch_split_subspace(t.U, t.rows, t.rank, td.kpad, frag, nullptr));
-      if (rc == ZGR_OK) ctx->launches++;
-      td.Ufrag = frag;
-    }
     // tcgen05 kernels: row-major copies of U in parts, and three tensor maps
     const int kind = tensor_core_kind(t, guided_on);
-    if (rc == ZGR_OK && kind != 0 && umma_wanted() && encode_tiled_fn() != nullptr) {
+    if (kind != 0 && umma_wanted() && encode_tiled_fn() != nullptr) {
       const int parts = kind == 1 ? 2 : 3;
       const int64_t rows_pad = ((t.rows + 127) / 128) * 128;
       td.kpad = t.rank <= 16 ? 16 : (t.rank <= 32 ? 32 : 64);
       // entries of an orthonormal U are about 1/sqrt(rows): scaled by 2^ushift they sit between 1 and 2 in size
       // (capped at 2^12, which leaves fp16 room for entries up to 16 in size); the bf16 parts need no scaling
       if (kind == 1) td.ushift = std::min<int32_t>(12, static_cast<int32_t>(std::ceil(0.5 * std::log2(static_cast<double>(t.rows)))));
-      uint16_t* part[3] = {nullptr, nullptr, nullptr};
-      for (int i = 0; i < parts && rc == ZGR_OK; ++i) rc = dev_alloc(ctx, &part[i], static_cast<size_t>(rows_pad) * td.kpad);
-      if (rc == ZGR_OK) {
-        CUtensorMap* m = &ctx->tmaps[static_cast<size_t>(3 * l)];
-        bool maps = kind == 1 ? make_map_16bit(m, t.data, t.rows, t.cols, 64) : true;
-        for (int i = 0; i < parts; ++i) maps = maps && make_map_16bit(m + (kind == 1 ? 1 : 0) + i, part[i], rows_pad, td.kpad, td.kpad);
-        if (maps) {
-          (kind == 1 ? td.umma : td.tile) = 1;
-          for (int i = 0; i < parts; ++i) td.Ucopy[i] = part[i];
-        }
+      uint8_t* at = static_cast<uint8_t*>(operands);
+      CUtensorMap* m = &ctx->tmaps[static_cast<size_t>(3 * l)];
+      bool maps = kind == 1 ? make_map_16bit(m, t.data, t.rows, t.cols, 64) : true;
+      for (int i = 0; i < parts; ++i) {
+        td.Ucopy[i] = at;
+        maps = maps && make_map_16bit(m + (kind == 1 ? 1 : 0) + i, at, rows_pad, td.kpad, td.kpad);
+        at += static_cast<size_t>(rows_pad) * td.kpad * 2;       // (a multiple of 4096 bytes)
       }
+      if (maps) {
+        (kind == 1 ? td.umma : td.tile) = 1;
+        operands = at;
+      }
+    }
+    const bool vec = (reinterpret_cast<uintptr_t>(t.data) & 15) == 0 && (t.cols % 8 == 0);
+    if (guided_on && t.rank > 8 && vec && t.dtype != ZGR_F32 && !td.umma) {
+      // the mma.sync kernel serves this tensor: copy of U in A-fragment order
+      td.kpad = t.rank <= 16 ? 16 : (t.rank <= 32 ? 32 : 64);
+      rc = make_fragments(ctx, td, nullptr);
     }
   }
   ctx->split_job.assign(static_cast<size_t>(n), -1);
   if (rc == ZGR_OK) {
-    std::vector<SplitJob> jobs;
+    std::vector<SplitJob>& jobs = ctx->split_jobs;
     for (int32_t l = 0; l < n; ++l) {
       const TensorDesc& td = ctx->descs[static_cast<size_t>(l)];
       if (!td.umma && !td.tile) continue;
@@ -1037,12 +1055,9 @@ int zgr_debug_z(zgr_ctx* ctx, uint64_t seed, int32_t tensor, float* dev_out, voi
   if (ctx->sticky) return ctx->sticky;
   if (!on_ctx_device(ctx)) return ZGR_EINVAL;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (ctx->frag_stale[static_cast<size_t>(tensor)]) {
-    const TensorDesc& cur = ctx->descs[static_cast<size_t>(tensor)];
-    const int rcf = check(ctx, launch_split_subspace(cur.U, cur.rows, cur.rank, cur.kpad, const_cast<uint4*>(cur.Ufrag), st));
+  if (ctx->descs[static_cast<size_t>(tensor)].umma) {
+    const int rcf = make_fragments(ctx, ctx->descs[static_cast<size_t>(tensor)], st);
     if (rcf != ZGR_OK) return rcf;
-    ctx->launches++;
-    ctx->frag_stale[static_cast<size_t>(tensor)] = 0;
   }
   // a one-tensor model whose weights are the zeroed output buffer, swept once with scale 1
   std::vector<TensorDesc> one(1, ctx->descs[static_cast<size_t>(tensor)]);
@@ -1155,14 +1170,20 @@ int zgr_build_subspace(zgr_ctx* ctx, int32_t tensor, const float* grads, int32_t
   if (!on_ctx_device(ctx)) return ZGR_EINVAL;
   if (!ctx->ledger.empty()) return ZGR_ESTATE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const size_t need = subspace_scratch_bytes(td.rows, td.rank);
+  const size_t need = subspace_scratch_bytes(td.rows, td.rank, ctx->sm_count);
   if (need > ctx->qr_bytes) {
     void* q = nullptr;
-    const int rc = check(ctx, cudaMalloc(&q, need));
+    int rc = check(ctx, cudaMalloc(&q, need));
     if (rc != ZGR_OK) return rc;
     ctx->owned.push_back(q);          // an outgrown scratch buffer stays owned until zgr_destroy; work enqueued on it may still run
+    rc = check(ctx, cudaMemsetAsync(q, 0, 512, st));
+    if (rc != ZGR_OK) return rc;
     ctx->d_qr = q;
     ctx->qr_bytes = need;
+  }
+  if (!ctx->h_status) {
+    const int rc = check(ctx, cudaHostAlloc(reinterpret_cast<void**>(&ctx->h_status), sizeof(int), cudaHostAllocMapped));
+    if (rc != ZGR_OK) return rc;
   }
   float* U = const_cast<float*>(td.U);
   const float* A = U;                  // NULL source: the gradient directions were written into the subspace buffer itself
@@ -1175,8 +1196,23 @@ int zgr_build_subspace(zgr_ctx* ctx, int32_t tensor, const float* grads, int32_t
       A = grads;
     }
   }
+  ctx->held_valid = false;
+  int rc;
+  if (subspace_fused(td.rows, td.rank, ctx->sm_count)) {
+    const int32_t job = ctx->split_job[static_cast<size_t>(tensor)];
+    *ctx->h_status = -1;
+    rc = check(ctx, launch_basis_fused(A, td.rows, td.rank, U, job >= 0 ? &ctx->split_jobs[static_cast<size_t>(job)] : nullptr, ctx->d_qr, ctx->h_status,
+                                       ctx->sm_count, st));
+    if (rc == ZGR_OK) rc = check(ctx, cudaStreamSynchronize(st));
+    if (rc != ZGR_OK) return rc;
+    ctx->launches++;
+    const int status = *static_cast<volatile int*>(ctx->h_status);
+    if (status < 0) return check(ctx, cudaErrorLaunchTimeout);   // a barrier gave up: the basis may be partly written
+    if (status > 0) return ZGR_EINVAL;                            // linearly dependent directions: nothing was written
+    return td.Ufrag != nullptr && !td.umma ? make_fragments(ctx, td, st) : ZGR_OK;
+  }
   int* d_status = nullptr;
-  int rc = check(ctx, launch_build_subspace(A, td.rows, td.rank, U, ctx->d_qr, &d_status, nullptr, st));
+  rc = check(ctx, launch_build_subspace(A, td.rows, td.rank, U, ctx->d_qr, &d_status, nullptr, st));
   if (rc != ZGR_OK) return rc;
   ctx->launches += 6;
   int status = 0;
@@ -1185,7 +1221,7 @@ int zgr_build_subspace(zgr_ctx* ctx, int32_t tensor, const float* grads, int32_t
   if (rc != ZGR_OK) return rc;
   if (status != 0) return ZGR_EINVAL;  // linearly dependent directions: nothing was written
   // the new basis is in place: refresh the tensor-core operand copies exactly as for a delivered subspace
-  return zgr_update_subspace(ctx, tensor, nullptr, 0, stream);
+  return refresh_operands(ctx, tensor, st);
 }
 
 int zgr_debug_plan(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, int32_t sm_count, int32_t tcgen05, int32_t multi,
@@ -1255,14 +1291,9 @@ int zgr_update_subspaces(zgr_ctx* ctx, int32_t n, const int32_t* tensors, const 
       const int rc = check(ctx, cudaMemcpyAsync(const_cast<float*>(td.U), src, bytes, src_is_host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, st));
       if (rc != ZGR_OK) return rc;
     }
-    if (td.Ufrag != nullptr) {
-      if (td.umma) {
-        ctx->frag_stale[static_cast<size_t>(l)] = 1;
-      } else {
-        const int rc = check(ctx, launch_split_subspace(td.U, td.rows, td.rank, td.kpad, const_cast<uint4*>(td.Ufrag), st));
-        if (rc != ZGR_OK) return rc;
-        ctx->launches++;
-      }
+    if (td.Ufrag != nullptr && !td.umma) {
+      const int rc = make_fragments(ctx, td, st);
+      if (rc != ZGR_OK) return rc;
     }
     const int32_t job = ctx->split_job[static_cast<size_t>(l)];
     if (job >= 0 && !fused) {
@@ -1363,6 +1394,7 @@ void zgr_destroy(zgr_ctx* ctx) {
   for (cudaEvent_t e : ctx->layer_events) cudaEventDestroy(e);
   if (ctx->aux_stream) cudaStreamDestroy(ctx->aux_stream);
   for (void* p : ctx->owned) cudaFree(p);
+  if (ctx->h_status) cudaFreeHost(ctx->h_status);
   delete ctx;
 }
 

@@ -478,17 +478,8 @@ __global__ void split_subspace_kernel(const float* __restrict__ U, int64_t rows,
   out[idx] = make_uint4(regs[0], regs[1], regs[2], regs[3]);
 }
 
-// U (rows x r fp32) -> two row-major fp16 matrices (hi, lo) holding U * 2^shift, rows padded to a multiple of
-// 128 and columns to KP with zeros: the TMA source of the A operand of the tcgen05 kernel.  hi + lo carries
-// 22 significant bits as long as the scaled entry is not far below 1 (lo must stay a normal fp16 number).
-__device__ __forceinline__ void split_f16_scaled(float x, float scale, __half& hi, __half& lo) {
-  const float y = x * scale;                       // power of two: exact
-  hi = __float2half_rn(y);
-  lo = __float2half_rn(y - __half2float(hi));
-}
-
 // Row-major operand copies of U for a list of tensors: two fp16 parts of U 2^shift (TMA-staged kernel) or three bf16 parts
-// of U (tile kernel; x = p0 + p1 + p2 exactly).
+// of U (tile kernel).  Rows are padded to a multiple of 128 and columns to the contraction width with zeros.
 __global__ void split_subspaces_kernel(const SplitJob* __restrict__ jobs) {
   const SplitJob j = jobs[blockIdx.y];
   const int64_t n = j.rows_pad * j.kp;
@@ -497,16 +488,7 @@ __global__ void split_subspaces_kernel(const SplitJob* __restrict__ jobs) {
     const int64_t row = idx / j.kp;
     const int k = static_cast<int>(idx % j.kp);
     const float x = (row < j.rows && k < j.r) ? j.U[row * j.r + k] : 0.0f;
-    if (j.shift >= 0) {
-      split_f16_scaled(x, scale, static_cast<__half*>(j.part[0])[idx], static_cast<__half*>(j.part[1])[idx]);
-    } else {
-      const __nv_bfloat16 a = __float2bfloat16_rn(x);
-      const float r1 = x - __bfloat162float(a);
-      const __nv_bfloat16 b = __float2bfloat16_rn(r1);
-      static_cast<__nv_bfloat16*>(j.part[0])[idx] = a;
-      static_cast<__nv_bfloat16*>(j.part[1])[idx] = b;
-      static_cast<__nv_bfloat16*>(j.part[2])[idx] = __float2bfloat16_rn(r1 - __bfloat162float(b));
-    }
+    split_subspace_entry(j, idx, x, scale);
   }
 }
 

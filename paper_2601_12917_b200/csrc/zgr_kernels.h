@@ -3,6 +3,8 @@
 #define ZGR_KERNELS_H_
 
 #include <cuda.h>
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stddef.h>
 
@@ -45,6 +47,26 @@ struct SplitJob {
   int32_t r, kp;
   int32_t shift;   // two fp16 parts (hi, lo) of U * 2^shift; -1: three bf16 parts of U
 };
+#ifdef __CUDACC__
+// Entry `at` of the copies of job j from the value x of U; scale = 2^shift.
+__device__ __forceinline__ void split_subspace_entry(const SplitJob& j, int64_t at, float x, float scale) {
+  if (j.shift >= 0) {
+    // hi + lo carries 22 significant bits as long as the scaled entry is not far below 1 (lo must stay a normal fp16 number)
+    const float y = x * scale;                       // power of two: exact
+    const __half hi = __float2half_rn(y);
+    static_cast<__half*>(j.part[0])[at] = hi;
+    static_cast<__half*>(j.part[1])[at] = __float2half_rn(y - __half2float(hi));
+  } else {
+    // x = p0 + p1 + p2 exactly
+    const __nv_bfloat16 a = __float2bfloat16_rn(x);
+    const float r1 = x - __bfloat162float(a);
+    const __nv_bfloat16 b = __float2bfloat16_rn(r1);
+    static_cast<__nv_bfloat16*>(j.part[0])[at] = a;
+    static_cast<__nv_bfloat16*>(j.part[1])[at] = b;
+    static_cast<__nv_bfloat16*>(j.part[2])[at] = __float2bfloat16_rn(r1 - __bfloat162float(b));
+  }
+}
+#endif
 cudaError_t launch_split_subspaces(const SplitJob* d_jobs, int n_jobs, cudaStream_t st);
 
 cudaError_t launch_stats(int bits, const SweepParams& p, int grid, cudaStream_t st);

@@ -13,12 +13,24 @@
 // arithmetic, the job is bound by reading A twice and writing U once; tensor cores would add nothing but
 // rounding (their split-bf16 product is good to 2^-16, an orthogonality of 1e-6 needs more).
 //
-// Three kernels per pass:
+// One launch does all of it (basis_kernel): every CTA keeps its rows in shared memory as doubles through both passes, the
+// partial Gram matrices meet in global memory (L2) between barriers, and each CTA factors the r x r sum for itself, since
+// that is cheaper than another barrier.  Up to about a thousand rows per CTA the grid is a single cluster of 8 CTAs, whose
+// barrier is a hardware one and whose 8 partials every CTA adds up directly; larger inputs use one CTA per SM, launched
+// cooperatively, with a counter barrier and the sum of the partials spread over the grid.  The job is bound by latency (a
+// 2048 x 16 input is 131 KB): the six launches, the memset and the copies of the status that it took before were 95 us a
+// tensor.  The last phase also writes the tensor-core operand copies of the new basis.
+// Inputs whose rows do not fit the shared memory of the whole chip (more than about 200,000 rows at rank 16, 53,000 at
+// rank 64) take three kernels per pass instead:
 //   gram_partial   one block per chunk of 128 rows: partial Gram matrix of the chunk, written to scratch
 //   factor         one block: sums the partials in a fixed order, Cholesky factor, inverse of R, status
 //   apply          one block per chunk of 128 rows: Q = A R^-1
 // The summation order is fixed, so the result does not depend on the launch history.
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
+
+#include <algorithm>
 
 #include "zgr_subspace.h"
 
@@ -145,13 +157,311 @@ __global__ void __launch_bounds__(kQrThreads) apply_kernel(const void* __restric
   }
 }
 
+// ---------------------------------------------------------------------------------------------
+// the whole construction in one launch
+// ---------------------------------------------------------------------------------------------
+constexpr int kClusterCtas = 8;
+constexpr double kPivotFloor = 1e-14;   // a pivot below this share of its column's norm is rounding error: the columns are dependent
+constexpr long long kBarrierLimit = 4000000000ll;   // cycles, about 2 s: a barrier that waits longer gives up
+
+struct BasisArgs {
+  const float* A;       // rows x r
+  float* U;             // rows x r, may be A
+  SplitJob copies;      // operand copies to refresh (part[0] null: none)
+  double* partials;     // one RC x RC matrix per CTA (cluster launches: and pass)
+  double* sum;          // RC x RC (grid launches)
+  unsigned* counter;    // grid barrier: arrivals, exits; both zero between launches
+  int* status;          // host-mapped: 0, 1 + dependent column, or -1 if a barrier gave up
+  int64_t rows;
+  int r;
+  int rows_per_cta;
+};
+
+template <bool CLUSTER>
+__device__ __forceinline__ bool basis_barrier(unsigned* counter, int index) {
+  if constexpr (CLUSTER) {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    return true;
+  } else {
+    // barrier number `index` of this launch; the last CTA to leave puts the counter back to zero
+    __shared__ int ok;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      const unsigned target = gridDim.x * static_cast<unsigned>(index + 1);
+      atomicAdd(counter, 1u);
+      const long long t0 = clock64();
+      unsigned seen;
+      do {
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(counter) : "memory");
+      } while (seen < target && clock64() - t0 < kBarrierLimit);
+      ok = seen >= target;
+    }
+    __syncthreads();
+    return ok != 0;
+  }
+}
+
+// RC = r rounded up to 16, 32 or 64.  Thread (ti, tj) of a 16 x 16 arrangement owns the entries (ti + 16 a, tj + 16 b) of
+// the r x r matrices, a <= b (the block upper triangle).
+template <int RC, bool CLUSTER>
+__global__ void __launch_bounds__(kQrThreads) basis_kernel(const BasisArgs p) {
+  constexpr int NB = RC / 16, LD = RC + 1;
+  extern __shared__ double dyn_smem[];
+  double* Rs = dyn_smem;                       // RC x RC: R, row k holds R[k][k..]
+  double* rowbuf = Rs + RC * RC;               // 2 x RC
+  double* inv = rowbuf + 2 * RC;               // 1 / R[k][k]
+  double* diag = inv + RC;                     // diagonal before the factorisation
+  double* X = diag + RC;                       // rows_per_cta x LD
+  const int tid = threadIdx.x, ti = tid >> 4, tj = tid & 15;
+  const int64_t row0 = static_cast<int64_t>(blockIdx.x) * p.rows_per_cta;
+  const int nrows = static_cast<int>(max(static_cast<int64_t>(0), min(static_cast<int64_t>(p.rows_per_cta), p.rows - row0)));
+  const int r = p.r;
+  int status = 0;
+
+  for (int idx = tid; idx < nrows * RC; idx += kQrThreads) {
+    const int i = idx / RC, k = idx % RC;
+    X[i * LD + k] = k < r ? static_cast<double>(p.A[(row0 + i) * r + k]) : 0.0;
+  }
+  __syncthreads();
+
+#pragma unroll 1
+  for (int pass = 0; pass < 2 && status == 0; ++pass) {
+    // ---- Gram matrix of this CTA's rows ----
+    double s[NB][NB];
+    {
+      double acc[NB][NB][2];
+#pragma unroll
+      for (int a = 0; a < NB; ++a)
+#pragma unroll
+        for (int b = 0; b < NB; ++b) acc[a][b][0] = acc[a][b][1] = 0.0;
+      int i = 0;
+      for (; i + 1 < nrows; i += 2) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const double* x = X + (i + h) * LD;
+          double xi[NB], xj[NB];
+#pragma unroll
+          for (int a = 0; a < NB; ++a) { xi[a] = x[ti + 16 * a]; xj[a] = x[tj + 16 * a]; }
+#pragma unroll
+          for (int a = 0; a < NB; ++a)
+#pragma unroll
+            for (int b = a; b < NB; ++b) acc[a][b][h] = fma(xi[a], xj[b], acc[a][b][h]);
+        }
+      }
+      if (i < nrows) {
+        const double* x = X + i * LD;
+#pragma unroll
+        for (int a = 0; a < NB; ++a)
+#pragma unroll
+          for (int b = a; b < NB; ++b) acc[a][b][0] = fma(x[ti + 16 * a], x[tj + 16 * b], acc[a][b][0]);
+      }
+      // (a cluster has one barrier per pass, so the second pass writes its own set)
+      double* out = p.partials + static_cast<int64_t>(blockIdx.x + (CLUSTER ? pass * kClusterCtas : 0)) * RC * RC;
+#pragma unroll
+      for (int a = 0; a < NB; ++a)
+#pragma unroll
+        for (int b = a; b < NB; ++b) out[(ti + 16 * a) * RC + tj + 16 * b] = acc[a][b][0] + acc[a][b][1];
+    }
+    if (!basis_barrier<CLUSTER>(p.counter, 2 * pass)) { status = -1; break; }
+    // ---- their sum, in a fixed order ----
+    if constexpr (CLUSTER) {
+#pragma unroll
+      for (int a = 0; a < NB; ++a)
+#pragma unroll
+        for (int b = a; b < NB; ++b) {
+          double v = 0.0;
+#pragma unroll
+          for (int c = 0; c < kClusterCtas; ++c) v += __ldcg(p.partials + static_cast<int64_t>(c + pass * kClusterCtas) * RC * RC + (ti + 16 * a) * RC + tj + 16 * b);
+          s[a][b] = v;
+        }
+    } else {
+      const int lane = tid & 31, wid = blockIdx.x * (kQrThreads / 32) + (tid >> 5);
+      for (int e = wid; e < RC * RC; e += gridDim.x * (kQrThreads / 32)) {      // one warp per entry
+        if ((e / RC) / 16 > (e % RC) / 16) continue;
+        double v = 0.0;
+        for (int c = lane; c < static_cast<int>(gridDim.x); c += 32) v += __ldcg(p.partials + static_cast<int64_t>(c) * RC * RC + e);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
+        if (lane == 0) p.sum[e] = v;
+      }
+      if (!basis_barrier<CLUSTER>(p.counter, 2 * pass + 1)) { status = -1; break; }
+#pragma unroll
+      for (int a = 0; a < NB; ++a)
+#pragma unroll
+        for (int b = a; b < NB; ++b) s[a][b] = __ldcg(p.sum + (ti + 16 * a) * RC + tj + 16 * b);
+    }
+    // ---- Cholesky factor S = R^T R, one barrier per column; columns >= r are those of the identity ----
+#pragma unroll
+    for (int a = 0; a < NB; ++a)
+      if (ti == tj) {
+        const int k = ti + 16 * a;
+        if (k >= r) s[a][a] = 1.0;
+        diag[k] = s[a][a];
+      }
+#pragma unroll
+    for (int a = 0; a < NB; ++a) {
+#pragma unroll 1
+      for (int kk = 0; kk < 16; ++kk) {
+        const int k = 16 * a + kk;
+        double* row = rowbuf + (k & 1) * RC;
+        if (ti == kk) {
+#pragma unroll
+          for (int b = a; b < NB; ++b) row[tj + 16 * b] = s[a][b];
+        }
+        __syncthreads();
+        const double piv = row[k];
+        if (status == 0 && !(piv > kPivotFloor * diag[k])) status = 1 + k;      // the same decision in every thread of every CTA
+        const double ip = 1.0 / piv;
+        if (tid < RC && tid >= k) {
+          const double rs = sqrt(piv);
+          Rs[k * RC + tid] = row[tid] / rs;
+          if (tid == k) inv[k] = 1.0 / rs;
+        }
+#pragma unroll
+        for (int a2 = a; a2 < NB; ++a2) {
+          const int i = ti + 16 * a2;
+          if (i > k) {
+            const double f = row[i] * ip;
+#pragma unroll
+            for (int b2 = a2; b2 < NB; ++b2) s[a2][b2] -= f * row[tj + 16 * b2];
+          }
+        }
+      }
+    }
+    __syncthreads();
+    if (status != 0) break;
+    // ---- X <- X R^-1, one row per thread, 16 columns at a time ----
+    for (int i = tid; i < nrows; i += kQrThreads) {
+      double* xr = X + i * LD;
+      asm volatile("" ::: "memory");      // R stays in shared memory: hoisted out of the row loop it would fill the register file
+#pragma unroll 1
+      for (int j0 = 0; j0 < RC; j0 += 16) {
+        double x[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) x[j] = xr[j0 + j];
+#pragma unroll 1
+        for (int k = 0; k < j0; ++k) {
+          const double y = xr[k];
+          const double* rk = Rs + k * RC + j0;
+#pragma unroll
+          for (int j = 0; j < 16; ++j) x[j] = fma(-y, rk[j], x[j]);
+        }
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+          x[k] *= inv[j0 + k];
+#pragma unroll
+          for (int j = k + 1; j < 16; ++j) x[j] = fma(-x[k], Rs[(j0 + k) * RC + j0 + j], x[j]);
+        }
+#pragma unroll
+        for (int j = 0; j < 16; ++j) xr[j0 + j] = x[j];
+      }
+    }
+    __syncthreads();
+  }
+
+  if (status == 0) {
+    const SplitJob& c = p.copies;
+    const float scale = c.shift >= 0 ? __int_as_float((127 + c.shift) << 23) : 1.0f;
+    for (int idx = tid; idx < nrows * RC; idx += kQrThreads) {
+      const int i = idx / RC, k = idx % RC;
+      if (k >= r) continue;                    // (the padding of the copies is zero since zgr_init)
+      const float u = static_cast<float>(X[i * LD + k]);
+      p.U[(row0 + i) * r + k] = u;
+      if (c.part[0] != nullptr) split_subspace_entry(c, (row0 + i) * c.kp + k, u, scale);
+    }
+  }
+  if constexpr (!CLUSTER) {
+    if (tid == 0 && atomicInc(p.counter + 1, gridDim.x - 1) == gridDim.x - 1) *p.counter = 0;
+  }
+  if (blockIdx.x == 0 && tid == 0) {
+    *p.status = status;
+    __threadfence_system();
+  }
+}
+
+template <int RC>
+size_t basis_smem(int rows_per_cta) {
+  return (static_cast<size_t>(RC) * RC + 4 * RC + static_cast<size_t>(rows_per_cta) * (RC + 1)) * sizeof(double);
+}
+constexpr size_t kBasisSmemMax = 232448 - 1024;
+
+template <int RC>
+cudaError_t launch_basis(BasisArgs p, int sm_count, cudaStream_t st, bool* served) {
+  *served = true;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  cfg.blockDim = dim3(kQrThreads);
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const int64_t in_cluster = (p.rows + kClusterCtas - 1) / kClusterCtas;
+  if (in_cluster * RC <= 16384) {
+    p.rows_per_cta = static_cast<int>(in_cluster);
+    const size_t smem = basis_smem<RC>(p.rows_per_cta);
+    const cudaError_t e = cudaFuncSetAttribute(basis_kernel<RC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kBasisSmemMax));
+    if (e != cudaSuccess) return e;
+    cfg.gridDim = dim3(kClusterCtas);
+    cfg.dynamicSmemBytes = smem;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kClusterCtas;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    return cudaLaunchKernelEx(&cfg, basis_kernel<RC, true>, p);
+  }
+  const int64_t per_cta = std::max<int64_t>((p.rows + sm_count - 1) / sm_count, 64);
+  if (per_cta > (1 << 20) || basis_smem<RC>(static_cast<int>(per_cta)) > kBasisSmemMax) {
+    *served = false;
+    return cudaSuccess;
+  }
+  p.rows_per_cta = static_cast<int>(per_cta);
+  const cudaError_t e = cudaFuncSetAttribute(basis_kernel<RC, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kBasisSmemMax));
+  if (e != cudaSuccess) return e;
+  cfg.gridDim = dim3(static_cast<unsigned>((p.rows + per_cta - 1) / per_cta));
+  cfg.dynamicSmemBytes = basis_smem<RC>(p.rows_per_cta);
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  return cudaLaunchKernelEx(&cfg, basis_kernel<RC, false>, p);
+}
+
 }  // namespace
 
-size_t subspace_scratch_bytes(int64_t rows, int r) {
+// Scratch layout: [0, 256) status of the three-kernel path, [256, 512) barrier counter, then the matrices.
+size_t subspace_scratch_bytes(int64_t rows, int r, int sm_count) {
   const int64_t n_chunks = (rows + kChunkRows - 1) / kChunkRows;
-  // partial Gram matrices, R^-1, accumulated R, the double image of the first pass's Q, status word
-  return static_cast<size_t>(n_chunks) * r * r * sizeof(double) + 2 * static_cast<size_t>(r) * r * sizeof(double) +
-         static_cast<size_t>(rows) * r * sizeof(double) + 256;
+  // three-kernel path: partial Gram matrices, R^-1, accumulated R, the double image of the first pass's Q
+  const size_t chunked = static_cast<size_t>(n_chunks) * r * r * sizeof(double) + 2 * static_cast<size_t>(r) * r * sizeof(double) +
+                         static_cast<size_t>(rows) * r * sizeof(double);
+  const size_t rc = r <= 16 ? 16 : (r <= 32 ? 32 : 64);
+  const size_t fused = (static_cast<size_t>(std::max(sm_count, 2 * kClusterCtas)) + 1) * rc * rc * sizeof(double);
+  return 512 + (subspace_fused(rows, r, sm_count) ? fused : chunked);
+}
+
+bool subspace_fused(int64_t rows, int r, int sm_count) {
+  const int64_t per_cta = std::max<int64_t>((rows + sm_count - 1) / sm_count, 64);
+  if (per_cta > (1 << 20)) return false;
+  const int n = static_cast<int>(per_cta);
+  return (r <= 16 ? basis_smem<16>(n) : (r <= 32 ? basis_smem<32>(n) : basis_smem<64>(n))) <= kBasisSmemMax;
+}
+
+cudaError_t launch_basis_fused(const float* A, int64_t rows, int r, float* U_out, const SplitJob* copies, void* scratch, int* status, int sm_count,
+                               cudaStream_t st) {
+  if (r < 1 || r > kMaxR || rows < r) return cudaErrorInvalidValue;
+  BasisArgs p = {};
+  p.A = A;
+  p.U = U_out;
+  if (copies) p.copies = *copies;
+  uint8_t* base = static_cast<uint8_t*>(scratch);
+  p.counter = reinterpret_cast<unsigned*>(base + 256);
+  const int rc = r <= 16 ? 16 : (r <= 32 ? 32 : 64);
+  p.sum = reinterpret_cast<double*>(base + 512);
+  p.partials = p.sum + rc * rc;
+  p.status = status;
+  p.rows = rows;
+  p.r = r;
+  bool served = false;
+  const cudaError_t e = rc == 16 ? launch_basis<16>(p, sm_count, st, &served)
+                                 : (rc == 32 ? launch_basis<32>(p, sm_count, st, &served) : launch_basis<64>(p, sm_count, st, &served));
+  return e == cudaSuccess && !served ? cudaErrorInvalidValue : e;
 }
 
 cudaError_t launch_build_subspace(const float* A, int64_t rows, int r, float* U_out, void* scratch, int** status_out, double** r_out, cudaStream_t st) {
@@ -159,7 +469,7 @@ cudaError_t launch_build_subspace(const float* A, int64_t rows, int r, float* U_
   const int n_chunks = static_cast<int>((rows + kChunkRows - 1) / kChunkRows);
   uint8_t* base = static_cast<uint8_t*>(scratch);
   int* status = reinterpret_cast<int*>(base);
-  double* partials = reinterpret_cast<double*>(base + 256);
+  double* partials = reinterpret_cast<double*>(base + 512);
   double* W = partials + static_cast<size_t>(n_chunks) * r * r;
   double* Racc = W + static_cast<size_t>(r) * r;
   double* Q1 = Racc + static_cast<size_t>(r) * r;
