@@ -161,6 +161,9 @@ __global__ void __launch_bounds__(kQrThreads) apply_kernel(const void* __restric
 // the whole construction in one launch
 // ---------------------------------------------------------------------------------------------
 constexpr int kClusterCtas = 8;
+// Entries per CTA up to which one cluster beats the grid (cycles, cluster / grid, at twice that size: 51k / 45k at rank 16,
+// 77k / 60k at rank 32, 121k / 116k at rank 64; the grid pays four barriers of 3k and two more reductions).
+constexpr int kClusterEntries = 4096;
 constexpr double kPivotFloor = 1e-14;   // a pivot below this share of its column's norm is rounding error: the columns are dependent
 constexpr long long kBarrierLimit = 4000000000ll;   // cycles, about 2 s: a barrier that waits longer gives up
 
@@ -176,6 +179,15 @@ struct BasisArgs {
   int r;
   int rows_per_cta;
 };
+
+// 1 / x by two Newton steps on the hardware's approximation (20 bits -> 40 -> working precision): half the latency of a
+// division, and the chain from column to column of the factorisation waits for it.
+__device__ __forceinline__ double reciprocal(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  y = fma(fma(-x, y, 1.0), y, y);
+  return fma(fma(-x, y, 1.0), y, y);
+}
 
 template <bool CLUSTER>
 __device__ __forceinline__ bool basis_barrier(unsigned* counter, int index) {
@@ -202,15 +214,22 @@ __device__ __forceinline__ bool basis_barrier(unsigned* counter, int index) {
   }
 }
 
-// RC = r rounded up to 16, 32 or 64.  Thread (ti, tj) of a 16 x 16 arrangement owns the entries (ti + 16 a, tj + 16 b) of
-// the r x r matrices, a <= b (the block upper triangle).
+// RC = r rounded up to 16, 32 or 64.
+//
+// Gram matrix: four groups of 64 threads take rows in turn; thread (ui, uj) of a group owns the entries (ui + 8 x, uj + 8 y),
+// x <= y, which needs RC/4 shared-memory reads per (RC/8)^2 / 2 multiply-adds (one entry per thread is bound by those reads:
+// 36 cycles per row at RC = 16 against 8).  The groups' sums are added in order.
+// Factorisation: S = L D L^T and, by the same eliminations applied to the identity, M = L^-1; then R^-1 = M^T D^-1/2.
+// Thread (ti, tj) of a 16 x 16 arrangement owns the entries (ti + 16 a, tj + 16 b): a <= b of S, a >= b of M.  One barrier per
+// column; only the reciprocal of the pivot is on the chain from column to column.
+// Product X R^-1: at RC = 16 a thread takes a row, otherwise a warp eight rows, a lane four of them and the columns tj + 16 b.
 template <int RC, bool CLUSTER>
 __global__ void __launch_bounds__(kQrThreads) basis_kernel(const BasisArgs p) {
   constexpr int NB = RC / 16, LD = RC + 1;
   extern __shared__ double dyn_smem[];
-  double* Rs = dyn_smem;                       // RC x RC: R, row k holds R[k][k..]
-  double* rowbuf = Rs + RC * RC;               // 2 x RC
-  double* inv = rowbuf + 2 * RC;               // 1 / R[k][k]
+  double* Ms = dyn_smem;                       // RC x LD: rows of M (before that: the sum of the groups' Gram matrices)
+  double* rowbuf = Ms + RC * LD;               // 2 x RC: current row of D L^T
+  double* inv = rowbuf + 2 * RC;               // D[k], then D[k]^-1/2
   double* diag = inv + RC;                     // diagonal before the factorisation
   double* X = diag + RC;                       // rows_per_cta x LD
   const int tid = threadIdx.x, ti = tid >> 4, tj = tid & 15;
@@ -219,6 +238,7 @@ __global__ void __launch_bounds__(kQrThreads) basis_kernel(const BasisArgs p) {
   const int r = p.r;
   int status = 0;
 
+#pragma unroll 8
   for (int idx = tid; idx < nrows * RC; idx += kQrThreads) {
     const int i = idx / RC, k = idx % RC;
     X[i * LD + k] = k < r ? static_cast<double>(p.A[(row0 + i) * r + k]) : 0.0;
@@ -230,38 +250,46 @@ __global__ void __launch_bounds__(kQrThreads) basis_kernel(const BasisArgs p) {
     // ---- Gram matrix of this CTA's rows ----
     double s[NB][NB];
     {
-      double acc[NB][NB][2];
+      constexpr int B = RC / 8;
+      const int grp = tid >> 6, ui = (tid >> 3) & 7, uj = tid & 7;
+      double acc[B][B];
 #pragma unroll
-      for (int a = 0; a < NB; ++a)
+      for (int x = 0; x < B; ++x)
 #pragma unroll
-        for (int b = 0; b < NB; ++b) acc[a][b][0] = acc[a][b][1] = 0.0;
-      int i = 0;
-      for (; i + 1 < nrows; i += 2) {
+        for (int y = 0; y < B; ++y) acc[x][y] = 0.0;
+#pragma unroll (RC == 64 ? 1 : 4)
+      for (int i = grp; i < nrows; i += 4) {
+        const double* row = X + i * LD;
+        double u[B], v[B];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const double* x = X + (i + h) * LD;
-          double xi[NB], xj[NB];
+        for (int x = 0; x < B; ++x) { u[x] = row[ui + 8 * x]; v[x] = row[uj + 8 * x]; }
 #pragma unroll
-          for (int a = 0; a < NB; ++a) { xi[a] = x[ti + 16 * a]; xj[a] = x[tj + 16 * a]; }
+        for (int x = 0; x < B; ++x)
 #pragma unroll
-          for (int a = 0; a < NB; ++a)
-#pragma unroll
-            for (int b = a; b < NB; ++b) acc[a][b][h] = fma(xi[a], xj[b], acc[a][b][h]);
-        }
+          for (int y = x; y < B; ++y) acc[x][y] = fma(u[x], v[y], acc[x][y]);
       }
-      if (i < nrows) {
-        const double* x = X + i * LD;
+#pragma unroll 1
+      for (int g = 0; g < 4; ++g) {
+        if (grp == g) {
 #pragma unroll
-        for (int a = 0; a < NB; ++a)
+          for (int x = 0; x < B; ++x)
 #pragma unroll
-          for (int b = a; b < NB; ++b) acc[a][b][0] = fma(x[ti + 16 * a], x[tj + 16 * b], acc[a][b][0]);
+            for (int y = x; y < B; ++y) {
+              double* at = Ms + (ui + 8 * x) * RC + uj + 8 * y;
+              *at = g == 0 ? acc[x][y] : *at + acc[x][y];
+            }
+        }
+        __syncthreads();
       }
       // (a cluster has one barrier per pass, so the second pass writes its own set)
       double* out = p.partials + static_cast<int64_t>(blockIdx.x + (CLUSTER ? pass * kClusterCtas : 0)) * RC * RC;
 #pragma unroll
       for (int a = 0; a < NB; ++a)
 #pragma unroll
-        for (int b = a; b < NB; ++b) out[(ti + 16 * a) * RC + tj + 16 * b] = acc[a][b][0] + acc[a][b][1];
+        for (int b = a; b < NB; ++b) {
+          const int i = ti + 16 * a, j = tj + 16 * b;
+          out[i * RC + j] = Ms[min(i, j) * RC + max(i, j)];
+        }
     }
     if (!basis_barrier<CLUSTER>(p.counter, 2 * pass)) { status = -1; break; }
     // ---- their sum, in a fixed order ----
@@ -272,18 +300,31 @@ __global__ void __launch_bounds__(kQrThreads) basis_kernel(const BasisArgs p) {
         for (int b = a; b < NB; ++b) {
           double v = 0.0;
 #pragma unroll
-          for (int c = 0; c < kClusterCtas; ++c) v += __ldcg(p.partials + static_cast<int64_t>(c + pass * kClusterCtas) * RC * RC + (ti + 16 * a) * RC + tj + 16 * b);
+          for (int c = 0; c < kClusterCtas; ++c)
+            v += __ldcg(p.partials + static_cast<int64_t>(c + pass * kClusterCtas) * RC * RC + (ti + 16 * a) * RC + tj + 16 * b);
           s[a][b] = v;
         }
     } else {
-      const int lane = tid & 31, wid = blockIdx.x * (kQrThreads / 32) + (tid >> 5);
-      for (int e = wid; e < RC * RC; e += gridDim.x * (kQrThreads / 32)) {      // one warp per entry
-        if ((e / RC) / 16 > (e % RC) / 16) continue;
-        double v = 0.0;
-        for (int c = lane; c < static_cast<int>(gridDim.x); c += 32) v += __ldcg(p.partials + static_cast<int64_t>(c) * RC * RC + e);
+      // a warp per entry, four entries at a time (entries of the blocks below the diagonal hold nothing and go unused)
+      const int lane = tid & 31, wid = blockIdx.x * (kQrThreads / 32) + (tid >> 5), warps = static_cast<int>(gridDim.x) * (kQrThreads / 32);
+      for (int e0 = wid; e0 < RC * RC; e0 += 4 * warps) {
+        double v[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int c = lane; c < static_cast<int>(gridDim.x); c += 32) {
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
-        if (lane == 0) p.sum[e] = v;
+          for (int q = 0; q < 4; ++q) {
+            const int e = e0 + q * warps;
+            if (e < RC * RC && (e / RC) / 16 <= (e % RC) / 16) v[q] += __ldcg(p.partials + static_cast<int64_t>(c) * RC * RC + e);
+          }
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) v[q] += __shfl_xor_sync(0xFFFFFFFFu, v[q], off);
+        if (lane == 0) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (e0 + q * warps < RC * RC) p.sum[e0 + q * warps] = v[q];
+        }
       }
       if (!basis_barrier<CLUSTER>(p.counter, 2 * pass + 1)) { status = -1; break; }
 #pragma unroll
@@ -291,70 +332,105 @@ __global__ void __launch_bounds__(kQrThreads) basis_kernel(const BasisArgs p) {
 #pragma unroll
         for (int b = a; b < NB; ++b) s[a][b] = __ldcg(p.sum + (ti + 16 * a) * RC + tj + 16 * b);
     }
-    // ---- Cholesky factor S = R^T R, one barrier per column; columns >= r are those of the identity ----
-#pragma unroll
-    for (int a = 0; a < NB; ++a)
-      if (ti == tj) {
-        const int k = ti + 16 * a;
-        if (k >= r) s[a][a] = 1.0;
-        diag[k] = s[a][a];
-      }
+    // ---- S = L D L^T, M = L^-1 ----
+    double m[NB][NB];
 #pragma unroll
     for (int a = 0; a < NB; ++a) {
+#pragma unroll
+      for (int b = 0; b <= a; ++b) m[a][b] = (a == b && ti == tj) ? 1.0 : 0.0;
+      if (ti == tj) diag[ti + 16 * a] = s[a][a];
+    }
+#pragma unroll
+    for (int a = 0; a < NB; ++a) {
+      const int kk_end = min(16, r - 16 * a);
 #pragma unroll 1
-      for (int kk = 0; kk < 16; ++kk) {
+      for (int kk = 0; kk < kk_end; ++kk) {
         const int k = 16 * a + kk;
         double* row = rowbuf + (k & 1) * RC;
         if (ti == kk) {
 #pragma unroll
           for (int b = a; b < NB; ++b) row[tj + 16 * b] = s[a][b];
+#pragma unroll
+          for (int b = 0; b <= a; ++b) Ms[k * LD + tj + 16 * b] = m[a][b];
         }
         __syncthreads();
         const double piv = row[k];
         if (status == 0 && !(piv > kPivotFloor * diag[k])) status = 1 + k;      // the same decision in every thread of every CTA
-        const double ip = 1.0 / piv;
-        if (tid < RC && tid >= k) {
-          const double rs = sqrt(piv);
-          Rs[k * RC + tid] = row[tid] / rs;
-          if (tid == k) inv[k] = 1.0 / rs;
-        }
+        const double ip = reciprocal(piv);
+        if (tid == k) inv[k] = piv;
 #pragma unroll
         for (int a2 = a; a2 < NB; ++a2) {
           const int i = ti + 16 * a2;
           if (i > k) {
             const double f = row[i] * ip;
 #pragma unroll
-            for (int b2 = a2; b2 < NB; ++b2) s[a2][b2] -= f * row[tj + 16 * b2];
+            for (int b2 = a2; b2 < NB; ++b2) s[a2][b2] = fma(-f, row[tj + 16 * b2], s[a2][b2]);
+#pragma unroll
+            for (int b2 = 0; b2 <= a; ++b2) m[a2][b2] = fma(-f, Ms[k * LD + tj + 16 * b2], m[a2][b2]);
           }
         }
       }
     }
     __syncthreads();
     if (status != 0) break;
-    // ---- X <- X R^-1, one row per thread, 16 columns at a time ----
-    for (int i = tid; i < nrows; i += kQrThreads) {
-      double* xr = X + i * LD;
-      asm volatile("" ::: "memory");      // R stays in shared memory: hoisted out of the row loop it would fill the register file
-#pragma unroll 1
-      for (int j0 = 0; j0 < RC; j0 += 16) {
+    if (tid < RC) inv[tid] = tid < r ? 1.0 / sqrt(inv[tid]) : 0.0;
+    for (int idx = tid; idx < (RC - r) * RC; idx += kQrThreads) Ms[(r + idx / RC) * LD + idx % RC] = 0.0;      // rank not a multiple of 16
+    __syncthreads();
+    // ---- X <- X R^-1 = X M^T D^-1/2 ----
+    if constexpr (RC == 16) {
+      // one row per thread: 136 broadcast reads and as many multiply-adds
+      for (int i = tid; i < nrows; i += kQrThreads) {
+        double* xr = X + i * LD;
+        asm volatile("" ::: "memory");      // M stays in shared memory: hoisted out of the row loop it would fill the register file
         double x[16];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) x[j] = xr[j0 + j];
+        for (int k = 0; k < 16; ++k) x[k] = xr[k];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          double q = 0.0;
+#pragma unroll
+          for (int k = 0; k <= j; ++k) q = fma(x[k], Ms[j * LD + k], q);
+          xr[j] = q * inv[j];
+        }
+      }
+    } else {
+      const int warp = tid >> 5, half = (tid >> 4) & 1;
 #pragma unroll 1
-        for (int k = 0; k < j0; ++k) {
-          const double y = xr[k];
-          const double* rk = Rs + k * RC + j0;
+      for (int i0 = 8 * warp; i0 < nrows; i0 += kQrThreads / 4) {
+        const int i1 = i0 + 4 * half;
+        const double* xr[4];
+        double q[4][NB];
 #pragma unroll
-          for (int j = 0; j < 16; ++j) x[j] = fma(-y, rk[j], x[j]);
+        for (int h = 0; h < 4; ++h) {
+          xr[h] = X + min(i1 + h, nrows - 1) * LD;
+#pragma unroll
+          for (int b = 0; b < NB; ++b) q[h][b] = 0.0;
         }
 #pragma unroll
-        for (int k = 0; k < 16; ++k) {
-          x[k] *= inv[j0 + k];
+        for (int kb = 0; kb < NB; ++kb) {
+#pragma unroll 4
+          for (int kk = 0; kk < 16; ++kk) {
+            const int k = 16 * kb + kk;
+            double x[4];
 #pragma unroll
-          for (int j = k + 1; j < 16; ++j) x[j] = fma(-x[k], Rs[(j0 + k) * RC + j0 + j], x[j]);
+            for (int h = 0; h < 4; ++h) x[h] = xr[h][k];
+#pragma unroll
+            for (int b = kb; b < NB; ++b) {
+              const int j = tj + 16 * b;
+              const double w = (b > kb || k <= j) ? Ms[j * LD + k] : 0.0;
+#pragma unroll
+              for (int h = 0; h < 4; ++h) q[h][b] = fma(x[h], w, q[h][b]);
+            }
+          }
         }
+        __syncwarp();
 #pragma unroll
-        for (int j = 0; j < 16; ++j) xr[j0 + j] = x[j];
+        for (int h = 0; h < 4; ++h)
+          if (i1 + h < nrows) {
+#pragma unroll
+            for (int b = 0; b < NB; ++b) X[(i1 + h) * LD + tj + 16 * b] = q[h][b] * inv[tj + 16 * b];
+          }
+        __syncwarp();
       }
     }
     __syncthreads();
@@ -363,6 +439,7 @@ __global__ void __launch_bounds__(kQrThreads) basis_kernel(const BasisArgs p) {
   if (status == 0) {
     const SplitJob& c = p.copies;
     const float scale = c.shift >= 0 ? __int_as_float((127 + c.shift) << 23) : 1.0f;
+#pragma unroll 4
     for (int idx = tid; idx < nrows * RC; idx += kQrThreads) {
       const int i = idx / RC, k = idx % RC;
       if (k >= r) continue;                    // (the padding of the copies is zero since zgr_init)
@@ -382,7 +459,7 @@ __global__ void __launch_bounds__(kQrThreads) basis_kernel(const BasisArgs p) {
 
 template <int RC>
 size_t basis_smem(int rows_per_cta) {
-  return (static_cast<size_t>(RC) * RC + 4 * RC + static_cast<size_t>(rows_per_cta) * (RC + 1)) * sizeof(double);
+  return (static_cast<size_t>(RC) * (RC + 1) + 4 * RC + static_cast<size_t>(rows_per_cta) * (RC + 1)) * sizeof(double);
 }
 constexpr size_t kBasisSmemMax = 232448 - 1024;
 
@@ -396,7 +473,7 @@ cudaError_t launch_basis(BasisArgs p, int sm_count, cudaStream_t st, bool* serve
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   const int64_t in_cluster = (p.rows + kClusterCtas - 1) / kClusterCtas;
-  if (in_cluster * RC <= 16384) {
+  if (in_cluster * RC <= kClusterEntries) {
     p.rows_per_cta = static_cast<int>(in_cluster);
     const size_t smem = basis_smem<RC>(p.rows_per_cta);
     const cudaError_t e = cudaFuncSetAttribute(basis_kernel<RC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kBasisSmemMax));

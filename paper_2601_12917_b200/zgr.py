@@ -11,6 +11,8 @@ import ctypes
 import os
 from typing import List, Optional, Sequence
 
+import torch
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.environ.get("ZGR_LIBRARY", os.path.join(_HERE, "libzgr.so"))   # override: an alternative build of the same ABI
 
@@ -122,15 +124,15 @@ def _check(code: int, what: str) -> None:
 
 
 def _dtype_code(t) -> int:
-    import torch
     return {torch.float32: F32, torch.float16: F16, torch.bfloat16: BF16}[t.dtype]
 
 
 def _stream_ptr(stream) -> Optional[int]:
+    """Raw handle of `stream`, or of the current stream of the current device (asked for without building a Stream object,
+    which costs 3 us a call)."""
     if stream is None:
-        import torch
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return stream.cuda_stream
 
 
 class Zgr:
@@ -239,7 +241,6 @@ class Zgr:
                                       None if ze is None else ze.data_ptr(), None if U is None else U.data_ptr())
         self._keep.append(list(deliveries))
         if copy_stream is None:
-            import torch
             copy_stream = torch.cuda.current_stream()
         _check(lib().zgr_perturb_layers(self._h, seed, scale, nl, (ctypes.c_int32 * nl)(*layer_end), nd, arr, _stream_ptr(stream),
                                         ctypes.c_void_p(copy_stream.cuda_stream)), "zgr_perturb_layers")
@@ -302,13 +303,11 @@ class Zgr:
         _check(lib().zgr_tensor_norms_noalloc(self._h, seed, tensor, out.data_ptr(), _stream_ptr(stream)), "zgr_tensor_norms_noalloc")
 
     def debug_philox(self, seed: int, tensor: int, tag: int, first_block: int, n_blocks: int, stream=None):
-        import torch
         out = torch.empty((n_blocks, 4), dtype=torch.int32, device="cuda")
         _check(lib().zgr_debug_philox(self._h, seed, tensor, tag, first_block, n_blocks, out.data_ptr(), _stream_ptr(stream)), "zgr_debug_philox")
         return out
 
     def debug_z(self, seed: int, tensor: int, stream=None):
-        import torch
         w = self._keep[0][tensor]
         out = torch.empty(w.shape, dtype=torch.float32, device=w.device)
         _check(lib().zgr_debug_z(self._h, seed, tensor, out.data_ptr(), _stream_ptr(stream)), "zgr_debug_z")
@@ -316,7 +315,6 @@ class Zgr:
 
     def debug_z_tcgen05(self, seed: int, tensor: int, stream=None):
         """z of `tensor` in fp32 as the tcgen05 sweep kernel itself computes it (zgr_debug_z_tcgen05)."""
-        import torch
         w = self._keep[0][tensor]
         out = torch.empty(w.shape, dtype=torch.float32, device=w.device)
         _check(lib().zgr_debug_z_tcgen05(self._h, seed, tensor, out.data_ptr(), _stream_ptr(stream)), "zgr_debug_z_tcgen05")
