@@ -407,6 +407,7 @@ __global__ void __launch_bounds__(UmmaCfg<KP>::THREADS, 1) sweep_umma_kernel(con
       const int r = td.rank;
       const uint64_t tcols = static_cast<uint64_t>(td.cols);   // kept in a register: the barriers below force reloads of anything read through td
       const int sh = acc_shift(td, p);
+      const PhiloxPre pre = philox_pre(0u, tid, p.term[0].keys);
       const float gscale = __int_as_float((127 + sh - td.ushift) << 23);   // 2^(s - j): the strips hold c b G 2^(s - j)
       if (GROUPS > 1 && t > 0) {
         // The strips are about to be overwritten.  With two groups this warp may be one tile ahead of the
@@ -476,7 +477,7 @@ __global__ void __launch_bounds__(UmmaCfg<KP>::THREADS, 1) sweep_umma_kernel(con
           const uint32_t out_off = static_cast<uint32_t>(((32 * cgrp) >> 6) * 16384 + row_in_tile * 128);
           if (NS * sub + 32 * cgrp < w.ncols) {
             const uint64_t oct0 = row_oct0 + static_cast<uint64_t>((NS * sub + 32 * cgrp) >> 3);
-            const uint32_t oct0_lo = static_cast<uint32_t>(oct0), oct0_hi = static_cast<uint32_t>(oct0 >> 32);
+            const uint32_t oct0_lo = static_cast<uint32_t>(oct0);     // (the planner keeps tensors of 2^34 elements and more away from here)
             // the row's 128 bytes in the staged tile start on a 128-byte boundary, so the swizzled chunk offset
             // (bits 4..6) can be xor-ed in rather than added: one logic instruction per chunk
             const uint32_t out_box = (theta_s32 + static_cast<uint32_t>(s * Cfg::THETA_BYTES) + out_off) ^ row_xor16;
@@ -492,8 +493,7 @@ __global__ void __launch_bounds__(UmmaCfg<KP>::THREADS, 1) sweep_umma_kernel(con
                 float zi[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) zi[i] = 0.0f;
-                const uint32_t lo = oct0_lo + static_cast<uint32_t>(o);
-                normals8_acc<BITS>(p.term[0].keys, tid, lo, oct0_hi + (lo < oct0_lo ? 1u : 0u), p.term[0].iso, zi);
+                normals8_acc_pre<BITS>(p.term[0].keys, pre, oct0_lo + static_cast<uint32_t>(o), p.term[0].iso, zi);
                 const bool live = row < row_end && NS * sub + 32 * cgrp + 8 * o < w.ncols;
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
@@ -509,14 +509,12 @@ __global__ void __launch_bounds__(UmmaCfg<KP>::THREADS, 1) sweep_umma_kernel(con
               sum_gd += static_cast<double>(f_gd);
               sum_z += static_cast<double>(f_z);
             } else {
-            // four octets per thread, kept independent so that their generator chains interleave
+            if constexpr (SSTATS) {
 #pragma unroll
-            for (int o = 0; o < 4; ++o) {
-              float acc[8];
+              for (int o = 0; o < 4; ++o) {
+                float acc[8];
 #pragma unroll
-              for (int i = 0; i < 8; ++i) acc[i] = __uint_as_float(o < 2 ? h0[8 * (o & 1) + i] : h1[8 * (o & 1) + i]);
-              const uint32_t lo = oct0_lo + static_cast<uint32_t>(o);
-              if constexpr (SSTATS) {
+                for (int i = 0; i < 8; ++i) acc[i] = __uint_as_float(o < 2 ? h0[8 * (o & 1) + i] : h1[8 * (o & 1) + i]);
                 const uint32_t chunk_addr = out_box ^ ((chunk0 + static_cast<uint32_t>(o)) << 4);
                 float th[8];
                 unpack8<T>(lds128(chunk_addr), th);                      // theta, before this thread overwrites it
@@ -526,7 +524,7 @@ __global__ void __launch_bounds__(UmmaCfg<KP>::THREADS, 1) sweep_umma_kernel(con
                   const float gd = acc[i] - th[i];
                   f_gd = fmaf(gd, gd, f_gd);
                 }
-                normals8_acc_rsum<BITS>(p.term[0].keys, tid, lo, oct0_hi + (lo < oct0_lo ? 1u : 0u), p.term[0].iso, acc, f_iso);
+                normals8_acc_rsum<BITS>(p.term[0].keys, tid, oct0_lo + static_cast<uint32_t>(o), 0u, p.term[0].iso, acc, f_iso);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                   const float zc = acc[i] - th[i];
@@ -537,25 +535,43 @@ __global__ void __launch_bounds__(UmmaCfg<KP>::THREADS, 1) sweep_umma_kernel(con
                   sum_gd += static_cast<double>(f_gd);
                   sum_z += static_cast<double>(f_z);
                 }
-              } else
-              normals8_acc<BITS>(p.term[0].keys, tid, lo, oct0_hi + (lo < oct0_lo ? 1u : 0u), p.term[0].iso, acc);
-              if (MULTI) {
-#pragma unroll 1
-                for (int q = 1; q < p.n_terms; ++q)
-                  normals8_acc<BITS>(p.term[q].keys, tid, lo, oct0_hi + (lo < oct0_lo ? 1u : 0u), p.term[q].iso, acc);
+                sts128(chunk_addr, make_uint4(Pack16<T>::pack(acc[0], acc[1]), Pack16<T>::pack(acc[2], acc[3]), Pack16<T>::pack(acc[4], acc[5]),
+                                              Pack16<T>::pack(acc[6], acc[7])));
               }
+            } else {
+              // four octets per thread, kept independent so that their generator chains interleave
+              float acc[4][8];
+#pragma unroll
+              for (int o = 0; o < 4; ++o)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) acc[o][i] = __uint_as_float(o < 2 ? h0[8 * (o & 1) + i] : h1[8 * (o & 1) + i]);
+#pragma unroll
+              for (int o = 0; o < 4; ++o) normals8_acc_pre<BITS>(p.term[0].keys, pre, oct0_lo + static_cast<uint32_t>(o), p.term[0].iso, acc[o]);
+              if (MULTI) {
+                // term by term over all four octets: the keys are fetched once per term, and four chains interleave
+#pragma unroll 1
+                for (int q = 1; q < p.n_terms; ++q) {
+                  const PhiloxKeys& keys = p.term[q].keys;
+                  const PhiloxPre pre_q = philox_pre(0u, tid, keys);
+#pragma unroll
+                  for (int o = 0; o < 4; ++o) normals8_acc_pre<BITS>(keys, pre_q, oct0_lo + static_cast<uint32_t>(o), p.term[q].iso, acc[o]);
+                }
+              }
+#pragma unroll
+            for (int o = 0; o < 4; ++o) {
               if constexpr (ZOUT) {
                 const int col = NS * sub + 32 * cgrp + 8 * o;          // within the item's strip
                 if (row < row_end && col < w.ncols) {
                   float4* dst = reinterpret_cast<float4*>(p.zout + static_cast<uint64_t>(row) * tcols + static_cast<uint64_t>(w.col0 + col));
-                  dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
-                  dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+                  dst[0] = make_float4(acc[o][0], acc[o][1], acc[o][2], acc[o][3]);
+                  dst[1] = make_float4(acc[o][4], acc[o][5], acc[o][6], acc[o][7]);
                 }
               } else {
-                const uint4 q = make_uint4(Pack16<T>::pack(acc[0], acc[1]), Pack16<T>::pack(acc[2], acc[3]), Pack16<T>::pack(acc[4], acc[5]),
-                                           Pack16<T>::pack(acc[6], acc[7]));
+                const uint4 q = make_uint4(Pack16<T>::pack(acc[o][0], acc[o][1]), Pack16<T>::pack(acc[o][2], acc[o][3]),
+                                           Pack16<T>::pack(acc[o][4], acc[o][5]), Pack16<T>::pack(acc[o][6], acc[o][7]));
                 sts128(out_box ^ ((chunk0 + static_cast<uint32_t>(o)) << 4), q);
               }
+            }
             }
             }
           }
