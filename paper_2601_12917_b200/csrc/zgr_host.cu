@@ -28,7 +28,7 @@ struct Group {
   int grid = 0;
   int64_t elements = 0;                                   // weights covered by one launch
   double* d_item_stats = nullptr;                         // kStatSlots x 3 doubles per item (norm bookkeeping), allocated on first use
-  int32_t* d_sched = nullptr;                             // CUDA-core contraction kernel: two item counters (caller's stream, library's second stream)
+  int32_t* d_sched = nullptr;                             // CUDA-core kernels: two item counters (caller's stream, library's second stream)
   std::vector<int32_t> first_item;                        // per tensor l: index of its first item in `items` (size n + 1; items are in tensor order)
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> timed;  // per-launch events while profiling is on
 };
@@ -155,7 +155,8 @@ int tensor_core_kind(const zgr_tensor& t, bool guided_on) {
   if (!guided_on || t.rank == 0 || t.rows >= (int64_t{1} << 31) - 256) return 0;
   const bool vec = (reinterpret_cast<uintptr_t>(t.data) & 15) == 0 && (t.cols % 8 == 0);
   if (vec && t.rank <= 8) return 0;
-  if (vec && t.dtype != ZGR_F32) return t.cols < (int64_t{1} << 31) - 256 ? 1 : 0;
+  // (the TMA-staged kernel keeps the high counter word of the generator fixed: fewer than 2^32 blocks of four elements)
+  if (vec && t.dtype != ZGR_F32 && t.rows * t.cols < (int64_t{1} << 34)) return t.cols < (int64_t{1} << 31) - 256 ? 1 : 0;
   return 2;
 }
 
@@ -164,9 +165,9 @@ bool umma_wanted() {
   return !(e && std::strcmp(e, "legacy") == 0);
 }
 
-int blocks_per_sm(const KernelChoice& kc) {
+int blocks_per_sm(const KernelChoice& kc, bool multi = false, bool stats = false) {
   switch (kc.path) {
-    case PATH_ISO: return 6;
+    case PATH_ISO: return iso_blocks_per_sm(kc.precise != 0, multi, stats);
     case PATH_GENERIC: return kc.kpad > 0 ? 1 : 4;
     case PATH_UMMA: return 1;
     default: return 2;
@@ -209,7 +210,9 @@ void plan(const std::vector<TensorDesc>& descs, const std::vector<int>& which, b
     if (!guided) {
       Group& g = group_for(PATH_ISO, t.dtype, 0);
       const int64_t n = t.rows * t.cols;
-      const int64_t chunk = std::max<int64_t>(8, (target / 8) * 8);
+      // about five items per resident CTA (handed out by a counter), the larger the better for the loads in flight: 405 M bf16
+      // weights take 977 us in items of 8192 elements, 905 in 32768, 890 in 65536
+      const int64_t chunk = std::min<int64_t>(std::max<int64_t>(total / (static_cast<int64_t>(sm_count) * 8 * 5) / 2048 * 2048, 2048), 65536);
       for (int64_t e0 = 0; e0 < n; e0 += chunk)
         g.items.push_back(WorkItem{l, aligned ? 1 : 0, e0, std::min(chunk, n - e0), 0});
       continue;
@@ -289,7 +292,7 @@ int upload_groups(zgr_ctx* ctx, std::vector<Group>& groups) {
     if (rc != ZGR_OK) return rc;
     rc = check(ctx, cudaMemcpy(g.d_items, g.items.data(), g.items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice));
     if (rc != ZGR_OK) return rc;
-    if (g.kc.path == PATH_FMA) {
+    if (g.kc.path == PATH_FMA || g.kc.path == PATH_ISO) {
       rc = dev_alloc(ctx, &g.d_sched, 2);
       if (rc != ZGR_OK) return rc;
       rc = check(ctx, cudaMemset(g.d_sched, 0, 2 * sizeof(int32_t)));
@@ -326,15 +329,14 @@ int sweep(zgr_ctx* ctx, std::vector<Group>& groups, const TensorDesc* d_descs, i
     p.item_stats = keep_stats ? g.d_item_stats : nullptr;
     p.item_base = 0;
     p.sched = g.d_sched ? g.d_sched + (ctx->aux_stream != nullptr && st == ctx->aux_stream ? 1 : 0) : nullptr;
-    int grid = g.grid;
     if (t1 >= 0) {
       const int32_t b0 = g.first_item[static_cast<size_t>(t0)], b1 = g.first_item[static_cast<size_t>(t1)];
       if (b1 <= b0) continue;
       p.items = g.d_items + b0;
       p.n_items = b1 - b0;
       p.item_base = b0;
-      grid = static_cast<int>(std::min<int64_t>(p.n_items, static_cast<int64_t>(ctx->sm_count) * blocks_per_sm(g.kc)));
     }
+    const int grid = static_cast<int>(std::min<int64_t>(p.n_items, static_cast<int64_t>(ctx->sm_count) * blocks_per_sm(g.kc, n > 1, p.item_stats != nullptr)));
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (ctx->profiling && t1 < 0) {
       if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
@@ -385,6 +387,15 @@ int make_fragments(zgr_ctx* ctx, TensorDesc& td, cudaStream_t st) {
   return rc;
 }
 
+// The jobs [first, first + count) of the operand copies, in one launch.
+int split_jobs(zgr_ctx* ctx, int first, int count, cudaStream_t st) {
+  int64_t most = 0;
+  for (int i = first; i < first + count; ++i) most = std::max(most, ctx->split_jobs[static_cast<size_t>(i)].rows_pad * ctx->split_jobs[static_cast<size_t>(i)].kp);
+  const int rc = check(ctx, launch_split_subspaces(ctx->d_split_jobs + first, count, most, st));
+  if (rc == ZGR_OK && count > 0) ctx->launches++;
+  return rc;
+}
+
 // Rebuild the library's operand copies of U for one tensor from the subspace buffer (enqueued on st).
 int refresh_operands(zgr_ctx* ctx, int32_t tensor, cudaStream_t st) {
   TensorDesc& td = ctx->descs[static_cast<size_t>(tensor)];
@@ -392,10 +403,7 @@ int refresh_operands(zgr_ctx* ctx, int32_t tensor, cudaStream_t st) {
   // (for a tensor of the tcgen05 kernel the fragment-order copy is only read by zgr_debug_z, which rebuilds it)
   if (td.Ufrag != nullptr && !td.umma) rc = make_fragments(ctx, td, st);
   const int32_t job = ctx->split_job[static_cast<size_t>(tensor)];
-  if (rc == ZGR_OK && job >= 0) {
-    rc = check(ctx, launch_split_subspaces(ctx->d_split_jobs + job, 1, st));
-    if (rc == ZGR_OK) ctx->launches++;
-  }
+  if (rc == ZGR_OK && job >= 0) rc = split_jobs(ctx, job, 1, st);
   return rc;
 }
 
@@ -627,8 +635,7 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
     if (!jobs.empty()) {
       rc = dev_alloc(ctx, &ctx->d_split_jobs, jobs.size());
       if (rc == ZGR_OK) rc = check(ctx, cudaMemcpy(ctx->d_split_jobs, jobs.data(), jobs.size() * sizeof(SplitJob), cudaMemcpyHostToDevice));
-      if (rc == ZGR_OK) rc = check(ctx, launch_split_subspaces(ctx->d_split_jobs, ctx->n_split_jobs, nullptr));
-      if (rc == ZGR_OK) ctx->launches++;
+      if (rc == ZGR_OK) rc = split_jobs(ctx, 0, static_cast<int>(jobs.size()), nullptr);
     }
   }
   if (rc == ZGR_OK) rc = dev_alloc(ctx, &ctx->d_tmaps, ctx->tmaps.size());
@@ -887,6 +894,7 @@ int zgr_perturb_layers(zgr_ctx* ctx, uint64_t seed, double scale, int32_t n_laye
   // SMs that the previous layer's last blocks have not reached any more.  The library's stream starts behind the
   // work already on the caller's stream, and the caller's stream ends by waiting for it.
   cudaEvent_t ev_begin = ctx->layer_events[static_cast<size_t>(n_layers) + 1];
+  std::vector<int32_t> jobs;
   rc = check(ctx, cudaEventRecord(ev_begin, st));
   if (rc == ZGR_OK) rc = check(ctx, cudaStreamWaitEvent(ctx->aux_stream, ev_begin, 0));
   if (rc != ZGR_OK) return rc;
@@ -895,11 +903,21 @@ int zgr_perturb_layers(zgr_ctx* ctx, uint64_t seed, double scale, int32_t n_laye
     if (n_deliveries > 0 && !by_layer[static_cast<size_t>(L)].empty()) {
       rc = check(ctx, cudaStreamWaitEvent(ls, ctx->layer_events[static_cast<size_t>(L)], 0));
       if (rc != ZGR_OK) return rc;
-      for (int32_t i : by_layer[static_cast<size_t>(L)])
-        if (deliveries[i].U) {
-          rc = refresh_operands(ctx, deliveries[i].tensor, ls);   // the delivered subspace, split for the tensor cores
-          if (rc != ZGR_OK) return rc;
-        }
+      // the delivered subspaces, split for the tensor cores: one launch per run of neighbouring jobs (all of a layer, as a rule)
+      jobs.clear();
+      for (int32_t i : by_layer[static_cast<size_t>(L)]) {
+        TensorDesc& td = ctx->descs[static_cast<size_t>(deliveries[i].tensor)];
+        if (!deliveries[i].U) continue;
+        if (td.Ufrag != nullptr && !td.umma) rc = make_fragments(ctx, td, ls);
+        if (rc != ZGR_OK) return rc;
+        if (ctx->split_job[static_cast<size_t>(deliveries[i].tensor)] >= 0) jobs.push_back(ctx->split_job[static_cast<size_t>(deliveries[i].tensor)]);
+      }
+      std::sort(jobs.begin(), jobs.end());
+      for (size_t i = 0, end; i < jobs.size(); i = end) {
+        for (end = i + 1; end < jobs.size() && jobs[end] == jobs[end - 1] + 1; ++end) {}
+        rc = split_jobs(ctx, jobs[i], static_cast<int>(end - i), ls);
+        if (rc != ZGR_OK) return rc;
+      }
     }
     rc = sweep(ctx, ctx->groups, ctx->d_descs, 1, &seed, &scale, ls, L ? layer_end[L - 1] : 0, layer_end[L], keep);
     if (rc != ZGR_OK) return rc;   // (a failure here leaves the earlier layers swept: the context is sticky-failed by check())
@@ -1297,15 +1315,13 @@ int zgr_update_subspaces(zgr_ctx* ctx, int32_t n, const int32_t* tensors, const 
     }
     const int32_t job = ctx->split_job[static_cast<size_t>(l)];
     if (job >= 0 && !fused) {
-      const int rc = check(ctx, launch_split_subspaces(ctx->d_split_jobs + job, 1, st));
+      const int rc = split_jobs(ctx, job, 1, st);
       if (rc != ZGR_OK) return rc;
-      ctx->launches++;
     }
   }
   if (fused) {
-    const int rc = check(ctx, launch_split_subspaces(ctx->d_split_jobs, ctx->n_split_jobs, st));
+    const int rc = split_jobs(ctx, 0, ctx->n_split_jobs, st);
     if (rc != ZGR_OK) return rc;
-    ctx->launches++;
   }
   return ZGR_OK;
 }

@@ -18,6 +18,9 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <type_traits>
+
 #include "zgr_device.cuh"
 #include "zgr_kernels.h"
 
@@ -37,18 +40,98 @@ constexpr int kWarps = kThreads / 32;
 // SSTATS = true (single-term sweeps only) also accumulates the norm bookkeeping of the sweep: per work item and
 // warp the sums of (c a Z)^2, (c b U G)^2 and (c z)^2 over its elements, stored in the item's slots (the
 // finishing kernel adds them up per tensor in a fixed order; the host divides by c^2).
+// Hands a CTA its work items.  The first one is its own block index; the others come, in order, from a counter in global
+// memory (a fixed assignment leaves the SMs that drew one item fewer idle: with 6 items per CTA a sixth of the sweep).  The
+// fetch is sent when the current item is begun, so its latency is hidden.  Every CTA makes exactly one fetch beyond the end;
+// the last fetch of the launch puts the counter back to zero (launches that share a counter are ordered by their stream).
+// With no more items than CTAs the counter is not touched.
+struct ItemFeed {
+  const SweepParams& p;
+  int* ahead;
+  __device__ __forceinline__ explicit ItemFeed(const SweepParams& params) : p(params) {
+    __shared__ int slot;
+    ahead = &slot;
+  }
+  __device__ __forceinline__ void fetch() {
+    if (threadIdx.x == 0) {
+      int it = p.n_items;
+      if (p.n_items > static_cast<int>(gridDim.x)) {
+        const int t = atomicAdd(p.sched, 1);
+        if (t == p.n_items - 1) *p.sched = 0;
+        it = t + static_cast<int>(gridDim.x);
+      }
+      *ahead = it;
+    }
+  }
+  __device__ __forceinline__ int first() {
+    fetch();
+    return static_cast<int>(blockIdx.x);
+  }
+  __device__ __forceinline__ int next() {       // also a barrier: the readers of the previous item's shared memory are done
+    __syncthreads();
+    const int it = *ahead;
+    __syncthreads();
+    if (it < p.n_items) fetch();
+    return it;
+  }
+};
+
+template <typename T>
+__device__ __forceinline__ void unpack_raw(const uint4& raw, float (&v)[8]) {
+  const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    if constexpr (std::is_same<T, __half>::value) {
+      const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[i]));
+      v[2 * i] = f.x; v[2 * i + 1] = f.y;
+    } else {
+      v[2 * i] = __uint_as_float(w[i] << 16);
+      v[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
+    }
+  }
+}
 template <typename T, int BITS, bool PRECISE, bool MULTI, bool SSTATS = false>
-__global__ void __launch_bounds__(kThreads) sweep_iso_kernel(const __grid_constant__ SweepParams p) {
-  for (int it = blockIdx.x; it < p.n_items; it += gridDim.x) {
+__global__ void __launch_bounds__(kThreads, iso_blocks_per_sm(PRECISE, MULTI, SSTATS)) sweep_iso_kernel(const __grid_constant__ SweepParams p) {
+  ItemFeed feed(p);
+  for (int it = feed.first(); it < p.n_items; it = feed.next()) {
     const WorkItem w = p.items[it];
     const TensorDesc& td = p.tensors[w.tensor];
     T* base = static_cast<T*>(td.data);
     const uint32_t tid = static_cast<uint32_t>(td.id);
     const int64_t e0 = w.row0_or_e0, count = w.nrows_or_count;
     const int64_t n_oct = w.ncols ? count / 8 : 0;  // ncols != 0: 128-bit access is legal for this tensor
+    int64_t n_oct_done = 0;
     double s_iso = 0.0;
+    if constexpr (!PRECISE && !SSTATS) {
+      // the fused transform, with the fixed part of the counter kept as long as its high word does not change
+      const uint64_t b0 = static_cast<uint64_t>(e0) >> (BITS == 32 ? 2 : 3);
+      const uint64_t b1 = static_cast<uint64_t>(e0 + count) >> (BITS == 32 ? 2 : 3);
+      if ((b0 >> 32) == (b1 >> 32)) {
+        const PhiloxPre pre = philox_pre(static_cast<uint32_t>(b0 >> 32), tid, p.term[0].keys);
+        const int n32 = static_cast<int>(n_oct);
+        T* b = base + e0;
+        uint4 raw = {}, nxt = {};
+        if (static_cast<int>(threadIdx.x) < n32) raw = __ldcs(reinterpret_cast<const uint4*>(b) + threadIdx.x);
+        for (int v = threadIdx.x; v < n32; v += kThreads) {
+          const int64_t e = e0 + 8 * static_cast<int64_t>(v);
+          float th[8];
+          if (v + kThreads < n32) nxt = __ldcs(reinterpret_cast<const uint4*>(b) + v + kThreads);
+          unpack_raw<T>(raw, th);
+          raw = nxt;
+          normals8_acc_pre<BITS>(p.term[0].keys, pre, static_cast<uint32_t>(e >> 3), p.term[0].iso, th);
+          if (MULTI) {
+#pragma unroll 1
+            for (int q = 1; q < p.n_terms; ++q)
+              normals8_acc_pre<BITS>(p.term[q].keys, philox_pre(static_cast<uint32_t>(b0 >> 32), tid, p.term[q].keys), static_cast<uint32_t>(e >> 3),
+                                     p.term[q].iso, th);
+          }
+          Storage<T>::store8(base + e, th);
+        }
+        n_oct_done = n_oct;
+      }
+    }
 #pragma unroll 2
-    for (int64_t v = threadIdx.x; v < n_oct; v += kThreads) {
+    for (int64_t v = n_oct_done + threadIdx.x; v < n_oct; v += kThreads) {
       const int64_t e = e0 + 8 * v;
       float th[8], z[8];
       Storage<T>::load8(base + e, th);
@@ -81,22 +164,9 @@ __global__ void __launch_bounds__(kThreads) sweep_iso_kernel(const __grid_consta
 template <typename T, int BITS, bool PRECISE, int R, bool MULTI, bool SSTATS = false>
 __global__ void __launch_bounds__(kThreads, 2) sweep_fma_kernel(const __grid_constant__ SweepParams p) {
   __shared__ float Gs[R][256 + 8];
-  __shared__ int next_item;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (;;) {
-    // Items are handed out in order by a counter in global memory: the models this kernel serves have few items per
-    // CTA (about 18 for a RoBERTa-large-sized set), so a fixed assignment leaves the SMs that drew one item fewer
-    // idle for 3-5 % of the sweep.  Every CTA makes exactly one fetch beyond the end; the last of those puts the
-    // counter back to zero for the next launch (launches that share a counter are ordered by their stream).
-    __syncthreads();  // readers of the previous strip and of next_item are done
-    if (threadIdx.x == 0) {
-      const int t = atomicAdd(p.sched, 1);
-      if (t == p.n_items + static_cast<int>(gridDim.x) - 1) *p.sched = 0;
-      next_item = t;
-    }
-    __syncthreads();
-    const int it = next_item;
-    if (it >= p.n_items) break;
+  ItemFeed feed(p);
+  for (int it = feed.first(); it < p.n_items; it = feed.next()) {
     const WorkItem w = p.items[it];
     const TensorDesc& td = p.tensors[w.tensor];
     T* base = static_cast<T*>(td.data);
@@ -480,15 +550,23 @@ __global__ void split_subspace_kernel(const float* __restrict__ U, int64_t rows,
 
 // Row-major operand copies of U for a list of tensors: two fp16 parts of U 2^shift (TMA-staged kernel) or three bf16 parts
 // of U (tile kernel).  Rows are padded to a multiple of 128 and columns to the contraction width with zeros.
-__global__ void split_subspaces_kernel(const SplitJob* __restrict__ jobs) {
+// A thread makes eight consecutive entries of a row: one 16-byte store per part.
+__global__ void __launch_bounds__(256) split_subspaces_kernel(const SplitJob* __restrict__ jobs) {
   const SplitJob j = jobs[blockIdx.y];
-  const int64_t n = j.rows_pad * j.kp;
+  const int per_row = j.kp / 8;
+  const int64_t n = j.rows_pad * per_row;
   const float scale = j.shift >= 0 ? __int_as_float((127 + j.shift) << 23) : 1.0f;
   for (int64_t idx = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; idx < n; idx += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int64_t row = idx / j.kp;
-    const int k = static_cast<int>(idx % j.kp);
-    const float x = (row < j.rows && k < j.r) ? j.U[row * j.r + k] : 0.0f;
-    split_subspace_entry(j, idx, x, scale);
+    const int64_t row = idx / per_row;
+    const int k0 = static_cast<int>(idx % per_row) * 8;
+    uint16_t out[3][8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float x = (row < j.rows && k0 + i < j.r) ? j.U[row * j.r + k0 + i] : 0.0f;
+      split_subspace_value(j.shift >= 0, x, scale, out[0][i], out[1][i], out[2][i]);
+    }
+    for (int q = 0; q < (j.shift >= 0 ? 2 : 3); ++q)
+      *reinterpret_cast<uint4*>(static_cast<uint16_t*>(j.part[q]) + row * j.kp + k0) = *reinterpret_cast<const uint4*>(out[q]);
   }
 }
 
@@ -623,9 +701,10 @@ cudaError_t launch_split_subspace(const float* U, int64_t rows, int r, int kp, u
   return cudaGetLastError();
 }
 
-cudaError_t launch_split_subspaces(const SplitJob* d_jobs, int n_jobs, cudaStream_t st) {
+cudaError_t launch_split_subspaces(const SplitJob* d_jobs, int n_jobs, int64_t max_entries, cudaStream_t st) {
   if (n_jobs <= 0) return cudaSuccess;
-  split_subspaces_kernel<<<dim3(64, static_cast<unsigned>(n_jobs)), 256, 0, st>>>(d_jobs);
+  const unsigned blocks = static_cast<unsigned>(std::min<int64_t>((max_entries / 8 + 255) / 256, 512));
+  split_subspaces_kernel<<<dim3(blocks, static_cast<unsigned>(n_jobs)), 256, 0, st>>>(d_jobs);
   return cudaGetLastError();
 }
 

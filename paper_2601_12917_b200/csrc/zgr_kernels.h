@@ -23,6 +23,10 @@ struct KernelChoice {
   int precise;  // accurate Gaussian transform (tensors stored in fp32)
 };
 
+// Resident blocks of 256 threads per SM of the isotropic kernel.  Its plain instantiation (fused transform) fits 32 registers:
+// eight blocks, whose loads then cover the DRAM latency (5.74 TB/s standalone against 5.50 with six).
+constexpr int iso_blocks_per_sm(bool precise, bool multi, bool stats) { return !precise && !multi && !stats ? 8 : 5; }
+
 int mma_strip_cols(int kpad);     // columns of a CTA strip on the tensor-core path
 int mma_rows_per_iter(int kpad);  // rows a CTA advances per iteration there
 size_t mma_smem_bytes(int kpad);
@@ -48,26 +52,35 @@ struct SplitJob {
   int32_t shift;   // two fp16 parts (hi, lo) of U * 2^shift; -1: three bf16 parts of U
 };
 #ifdef __CUDACC__
-// Entry `at` of the copies of job j from the value x of U; scale = 2^shift.
-__device__ __forceinline__ void split_subspace_entry(const SplitJob& j, int64_t at, float x, float scale) {
-  if (j.shift >= 0) {
-    // hi + lo carries 22 significant bits as long as the scaled entry is not far below 1 (lo must stay a normal fp16 number)
+// The parts of one entry x of U: fp16 hi + lo of x 2^shift (22 significant bits as long as the scaled entry is not far below 1:
+// lo must stay a normal fp16 number), or three bf16 parts whose sum is x.
+__device__ __forceinline__ void split_subspace_value(bool fp16, float x, float scale, uint16_t& p0, uint16_t& p1, uint16_t& p2) {
+  if (fp16) {
     const float y = x * scale;                       // power of two: exact
     const __half hi = __float2half_rn(y);
-    static_cast<__half*>(j.part[0])[at] = hi;
-    static_cast<__half*>(j.part[1])[at] = __float2half_rn(y - __half2float(hi));
+    p0 = __half_as_ushort(hi);
+    p1 = __half_as_ushort(__float2half_rn(y - __half2float(hi)));
+    p2 = 0;
   } else {
-    // x = p0 + p1 + p2 exactly
     const __nv_bfloat16 a = __float2bfloat16_rn(x);
     const float r1 = x - __bfloat162float(a);
     const __nv_bfloat16 b = __float2bfloat16_rn(r1);
-    static_cast<__nv_bfloat16*>(j.part[0])[at] = a;
-    static_cast<__nv_bfloat16*>(j.part[1])[at] = b;
-    static_cast<__nv_bfloat16*>(j.part[2])[at] = __float2bfloat16_rn(r1 - __bfloat162float(b));
+    p0 = __bfloat16_as_ushort(a);
+    p1 = __bfloat16_as_ushort(b);
+    p2 = __bfloat16_as_ushort(__float2bfloat16_rn(r1 - __bfloat162float(b)));
   }
 }
+// Entry `at` of the copies of job j from the value x of U; scale = 2^shift.
+__device__ __forceinline__ void split_subspace_entry(const SplitJob& j, int64_t at, float x, float scale) {
+  uint16_t p0, p1, p2;
+  split_subspace_value(j.shift >= 0, x, scale, p0, p1, p2);
+  static_cast<uint16_t*>(j.part[0])[at] = p0;
+  static_cast<uint16_t*>(j.part[1])[at] = p1;
+  if (j.shift < 0) static_cast<uint16_t*>(j.part[2])[at] = p2;
+}
 #endif
-cudaError_t launch_split_subspaces(const SplitJob* d_jobs, int n_jobs, cudaStream_t st);
+// max_entries: rows_pad * kp of the largest of the jobs
+cudaError_t launch_split_subspaces(const SplitJob* d_jobs, int n_jobs, int64_t max_entries, cudaStream_t st);
 
 cudaError_t launch_stats(int bits, const SweepParams& p, int grid, cudaStream_t st);
 // Norm bookkeeping, second stage: tensor l owns the work items [first, first + count) of the slot array `slots`

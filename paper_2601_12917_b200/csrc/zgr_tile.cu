@@ -81,17 +81,6 @@ __device__ __forceinline__ void tmem_ld8_tail(uint32_t taddr, uint32_t (&v)[40])
 
 __device__ __forceinline__ void sts16(uint32_t saddr, uint16_t v) { asm volatile("st.shared.b16 [%0], %1;" ::"r"(saddr), "h"(v) : "memory"); }
 
-// x = p0 + p1 + p2 exactly (8 significant bits each)
-__device__ __forceinline__ void split3(float x, uint16_t& p0, uint16_t& p1, uint16_t& p2) {
-  const __nv_bfloat16 a = __float2bfloat16_rn(x);
-  const float r1 = x - __bfloat162float(a);
-  const __nv_bfloat16 b = __float2bfloat16_rn(r1);
-  const __nv_bfloat16 c = __float2bfloat16_rn(r1 - __bfloat162float(b));
-  p0 = __bfloat16_as_ushort(a);
-  p1 = __bfloat16_as_ushort(b);
-  p2 = __bfloat16_as_ushort(c);
-}
-
 // Compressed coefficient of row k, column c, before scale and zero point.
 __device__ __forceinline__ float code1(const TensorDesc& td, int k, int64_t c) {
   if (td.qbits == 4) {
@@ -147,7 +136,7 @@ __device__ __forceinline__ void build_strip(const TensorDesc& td, const SweepPar
       const int j = j0 + i;
       if (j >= 0 && j < kTileN) {
         uint16_t q0, q1, q2;
-        split3(c_first + i < cols ? g[i] : 0.0f, q0, q1, q2);
+        split_subspace_value(false, c_first + i < cols ? g[i] : 0.0f, 1.0f, q0, q1, q2);
         const uint32_t at = g_dst + swizzle(static_cast<uint32_t>(j * rowb + 2 * k), rowb);
         sts16(at, q0);
         sts16(at + g_bytes, q1);
