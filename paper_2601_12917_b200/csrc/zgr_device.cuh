@@ -16,6 +16,22 @@
 namespace zgr {
 
 // ---------------------------------------------------------------------------------------------
+// Programmatic dependent launch.  A sweep is one kernel per family of tensors and a step is three sweeps, so on small models
+// the gaps between launches are most of the time.  Every sweep kernel is launched with the programmatic-serialisation
+// attribute: its CTAs may start while the kernel before it in the stream still runs.  The first kernel of a sweep waits for
+// that kernel to complete (dependency_begin with late = 0) and then lets its successor start.  The other kernels of the same sweep
+// work on other tensors, and everything older had completed before the first one let them start: they begin at once
+// (late = 1) and wait at their end, so that their completion implies that of the kernels before them.
+// ---------------------------------------------------------------------------------------------
+__device__ __forceinline__ void dependency_begin(const SweepParams& p) {
+  if (!p.late) asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void dependency_end(const SweepParams& p) {
+  if (p.late) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// ---------------------------------------------------------------------------------------------
 // Philox4x32-10 (Salmon et al., SC'11).  The paper asks only that client and edge server
 // regenerate the same perturbation from a shared seed (Algorithm 1); a counter-based generator
 // makes every element a pure function of (seed, tensor, stream tag, element index), so any tiling
@@ -383,6 +399,32 @@ __device__ __forceinline__ void normals8_acc_pre(const PhiloxKeys& keys, const P
       for (int w = 0; w < 4; w += 2) box_muller_acc2(field16a(x[w]), field16b(x[w]), field16a(x[w + 1]), field16b(x[w + 1]), ns, acc, 2 * w);
     }
   }
+}
+
+// The same by the accurate transform.
+template <int BITS>
+__device__ __forceinline__ void normals8_acc_accurate_pre(const PhiloxKeys& keys, const PhiloxPre& pre, uint32_t oct_lo, const NormalScale& ns,
+                                                          float (&acc)[8]) {
+  uint32_t x[4];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    if (BITS == 32 || h == 0) philox4x32_10_pre(BITS == 32 ? 2 * oct_lo + h : oct_lo, pre, keys, x);
+    uint64_t n0, n1;
+    if (BITS == 32) box_muller_accurate2(field23(x[0]), field23(x[1]), field23(x[2]), field23(x[3]), ns, n0, n1);
+    else box_muller_accurate2(field16a(x[2 * h]), field16b(x[2 * h]), field16a(x[2 * h + 1]), field16b(x[2 * h + 1]), ns, n0, n1);
+    float a0, a1, b0, b1;
+    unpack2(n0, a0, b0);
+    unpack2(n1, a1, b1);
+    acc[4 * h] += a0;
+    acc[4 * h + 1] += a1;
+    acc[4 * h + 2] += b0;
+    acc[4 * h + 3] += b1;
+  }
+}
+template <int BITS, bool PRECISE>
+__device__ __forceinline__ void normals8_add(const PhiloxKeys& keys, const PhiloxPre& pre, uint32_t oct_lo, const NormalScale& ns, float (&acc)[8]) {
+  if constexpr (PRECISE) normals8_acc_accurate_pre<BITS>(keys, pre, oct_lo, ns, acc);
+  else normals8_acc_pre<BITS>(keys, pre, oct_lo, ns, acc);
 }
 
 // normals8_acc that also returns the energy of its eight normals (sum of their squares) in rsum.

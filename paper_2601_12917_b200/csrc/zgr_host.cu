@@ -7,8 +7,10 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <new>
+#include <queue>
 #include <vector>
 
 #include "zgr.h"
@@ -174,6 +176,114 @@ int blocks_per_sm(const KernelChoice& kc, bool multi = false, bool stats = false
   }
 }
 
+struct Member {
+  int tensor, strip, row_step;
+};
+
+// Append the items of one tensor: strips of `strip` columns, each cut into even chunks of at most about nrows rows.
+void cut_tensor(const TensorDesc& t, int l, int strip, int row_step, int64_t nrows_for_strip(int64_t, int), int64_t arg, std::vector<WorkItem>& items) {
+  for (int64_t c0 = 0; c0 < t.cols; c0 += strip) {
+    const int ncols = static_cast<int>(std::min<int64_t>(strip, t.cols - c0));
+    int64_t nrows = std::max<int64_t>(1, nrows_for_strip(arg, ncols));
+    nrows = ((nrows + row_step - 1) / row_step) * row_step;
+    const int64_t n_chunks = (t.rows + nrows - 1) / nrows;
+    nrows = (t.rows + n_chunks - 1) / n_chunks;
+    nrows = ((nrows + row_step - 1) / row_step) * row_step;
+    for (int64_t r0 = 0; r0 < t.rows; r0 += nrows) items.push_back(WorkItem{l, ncols, r0, std::min(nrows, t.rows - r0), c0});
+  }
+}
+
+// Work items of one group.  An item is a strip of columns x a range of rows; it costs its tiles and, once, its coefficient
+// strip, so few tall items are cheap but divide badly over the SMs.  `target`: elements per item for about 16 rounds.
+void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>& members, int sm_count, int64_t target, Group& g) {
+  const auto by_elements = [](int64_t elements, int ncols) { return elements / ncols; };
+  const auto by_rows = [](int64_t rows, int) { return rows; };
+  const bool tile = g.kc.path == PATH_GENERIC && g.kc.kpad > 0;
+  if (g.kc.path == PATH_FMA) {
+    // handed out by a counter: nine items per CTA on large sets; down to as many rows as make the strip half of an item's
+    // generator work when there is too little to go round
+    int64_t total = 0;
+    for (const Member& m : members) total += descs[m.tensor].rows * descs[m.tensor].cols;
+    const int64_t least = std::min<int64_t>(256 * 2 * g.kc.kpad, 16384);
+    const int64_t per = std::min<int64_t>(std::max<int64_t>(total / (static_cast<int64_t>(sm_count) * 2 * 8), least), 1048576);
+    for (const Member& m : members) cut_tensor(descs[m.tensor], m.tensor, m.strip, m.row_step, by_elements, per, g.items);
+    return;
+  }
+  int64_t tiles = 0;
+  if (tile) {
+    // Handed out by a counter to one CTA per SM.  Tall items are cheap (an item costs its 128 x 128 tiles and, per 512 octets of
+    // its strip, 0.2 to 0.6 of a tile: fp32 rank 32 took 451 us a sweep in items of one tile, 344 in items of eight), small ones
+    // finish evenly: the height for the first two thirds of the work and that for the last third are those that the list
+    // scheduling of the items, replayed here, ends with first.  Half of a last item is added, because the tiles do not take
+    // equally long in fact (119 M bf16 weights in rows of 1234: 565 us a step with 8 and 8 tiles, 536 with 8 and 2).  Below a
+    // dozen tiles per SM one height serves all (12.5 M fp32 weights, rank 32: 522 us with a smaller second height, 400 without).
+    for (const Member& m : members) tiles += ((descs[m.tensor].rows + 127) / 128) * ((descs[m.tensor].cols + 127) / 128);
+    const double item_cost = 0.15 + (0.2 + 0.2 * g.kc.precise + (g.kc.precise && g.kc.bits == 32 ? 0.2 : 0.0)) * ((19 * g.kc.kpad + 511) / 512) +
+                             (g.kc.kpad == 64 ? 0.3 : 0.0);
+    const bool few = tiles < 12 * static_cast<int64_t>(sm_count);
+    double best = 0.0;
+    std::vector<WorkItem> trial;
+    for (int64_t big : {16, 12, 8, 6, 4, 3, 2, 1})
+      for (int64_t small : {big, std::max<int64_t>(big / 4, 1)}) {
+        if (few && small != big) continue;
+        if (best > 0.0 && (small == big ? tiles / big > 40 * static_cast<int64_t>(sm_count) : big == 1)) continue;
+        trial.clear();
+        int64_t done = 0;
+        for (const Member& m : members) {
+          cut_tensor(descs[m.tensor], m.tensor, m.strip, m.row_step, by_rows, 128 * (3 * done < 2 * tiles ? big : small), trial);
+          done += ((descs[m.tensor].rows + 127) / 128) * ((descs[m.tensor].cols + 127) / 128);
+        }
+        std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
+        double end = 0.0;
+        for (const WorkItem& w : trial) {
+          double at = 0.0;
+          if (free_at.size() >= static_cast<size_t>(sm_count)) {
+            at = free_at.top();
+            free_at.pop();
+          }
+          at += static_cast<double>((w.nrows_or_count + 127) / 128) + item_cost;
+          free_at.push(at);
+          end = std::max(end, at);
+        }
+        if (!few) end += 0.5 * (static_cast<double>(small) + item_cost);
+        if (best == 0.0 || end < best) {
+          best = end;
+          g.items = trial;
+        }
+      }
+    return;
+  }
+  for (const Member& m : members) tiles += ((descs[m.tensor].rows + 127) / 128) * ((descs[m.tensor].cols + 127) / 128);
+  if (g.kc.path != PATH_UMMA || tiles >= 24 * static_cast<int64_t>(sm_count)) {
+    for (const Member& m : members)
+      cut_tensor(descs[m.tensor], m.tensor, m.strip, m.row_step, by_elements, g.kc.path == PATH_UMMA ? 2 * target : target, g.items);
+    return;
+  }
+  // The TMA-staged kernel deals its items out in a fixed round-robin over one CTA per SM.  On sets of fewer than two dozen
+  // tiles per SM the item shape is the one whose busiest CTA has the least to do, in units of a 128 x 128 tile: a strip costs
+  // about kpad/50 tiles (coefficients generated, split and written with little to overlap) and an item 0.7 for filling its
+  // pipeline.
+  const double strip_cost = g.kc.kpad / 50.0, item_cost = 0.7;
+  double best = 0.0;
+  std::vector<WorkItem> trial;
+  for (int narrow = 0; narrow < (members.empty() || members[0].strip <= 128 ? 1 : 2); ++narrow)
+    for (int64_t rows = 128; rows <= 8192; rows *= 2) {
+      if (tiles / (rows / 128) < sm_count / 2 && best > 0.0) break;
+      trial.clear();
+      for (const Member& m : members) cut_tensor(descs[m.tensor], m.tensor, narrow ? 128 : m.strip, m.row_step, by_rows, rows, trial);
+      std::vector<double> busy(static_cast<size_t>(sm_count), 0.0);
+      for (size_t i = 0; i < trial.size(); ++i) {
+        const double wide = (trial[i].ncols + 127) / 128;
+        busy[i % busy.size()] += wide * (static_cast<double>((trial[i].nrows_or_count + 127) / 128) + strip_cost) + item_cost;
+      }
+      const double most = *std::max_element(busy.begin(), busy.end());
+      if (best == 0.0 || most < best) {
+        best = most;
+        g.items = trial;
+      }
+    }
+}
+
 // Split the tensors listed in `which` into work items, grouped by the kernel that serves them.
 // The kernel family follows the tensor's own storage type (fp32 tensors take the accurate transform and
 // an exact fp32 contraction); `kernel_dtype` >= 0 overrides only the type the kernel reads and writes,
@@ -203,6 +313,7 @@ void plan(const std::vector<TensorDesc>& descs, const std::vector<int>& which, b
     return out[it->second];
   };
 
+  std::vector<std::vector<Member>> members;   // per group: the tensors it serves with strips of columns
   for (int l : which) {
     const TensorDesc& t = descs[l];
     const bool aligned = (reinterpret_cast<uintptr_t>(t.data) & 15) == 0;
@@ -237,22 +348,13 @@ void plan(const std::vector<TensorDesc>& descs, const std::vector<int>& which, b
       strip = mma_strip_cols(kpad); row_step = mma_rows_per_iter(kpad);
     }
     Group& g = group_for(path, t.dtype, kpad);
-    for (int64_t c0 = 0; c0 < t.cols; c0 += strip) {
-      const int ncols = static_cast<int>(std::min<int64_t>(strip, t.cols - c0));
-      // (the CUDA-core contraction kernel hands its items out dynamically and regenerates its coefficient strip per item:
-      //  larger items there; the tcgen05 kernel's items are two tiles wide)
-      int64_t nrows = std::max<int64_t>(1, (path == PATH_UMMA || path == PATH_FMA ? 2 * target : target) / ncols);
-      // (the tile kernel builds a 144-column strip per item and 128 columns of weights: about ten items per SM)
-      if (tile_ok) nrows = std::min<int64_t>(std::max<int64_t>(total / (static_cast<int64_t>(sm_count) * 10), 16384), 262144) / strip;
-      nrows = ((nrows + row_step - 1) / row_step) * row_step;
-      // even out the chunks of this strip
-      const int64_t n_chunks = (t.rows + nrows - 1) / nrows;
-      nrows = (t.rows + n_chunks - 1) / n_chunks;
-      nrows = ((nrows + row_step - 1) / row_step) * row_step;
-      for (int64_t r0 = 0; r0 < t.rows; r0 += nrows)
-        g.items.push_back(WorkItem{l, ncols, r0, std::min(nrows, t.rows - r0), c0});
-    }
+    const size_t gi = static_cast<size_t>(&g - out.data());
+    if (members.size() <= gi) members.resize(gi + 1);
+    members[gi].push_back(Member{l, strip, row_step});
   }
+  members.resize(out.size());
+  for (size_t gi = 0; gi < out.size(); ++gi)
+    if (out[gi].kc.path != PATH_ISO) plan_tiles(descs, members[gi], sm_count, target, out[gi]);
   for (Group& g : out) {
     g.elements = 0;
     for (const WorkItem& w : g.items) g.elements += g.kc.path == PATH_ISO ? w.nrows_or_count : w.nrows_or_count * w.ncols;
@@ -292,7 +394,7 @@ int upload_groups(zgr_ctx* ctx, std::vector<Group>& groups) {
     if (rc != ZGR_OK) return rc;
     rc = check(ctx, cudaMemcpy(g.d_items, g.items.data(), g.items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice));
     if (rc != ZGR_OK) return rc;
-    if (g.kc.path == PATH_FMA || g.kc.path == PATH_ISO) {
+    if (g.kc.path == PATH_FMA || g.kc.path == PATH_ISO || (g.kc.path == PATH_GENERIC && g.kc.kpad > 0)) {
       rc = dev_alloc(ctx, &g.d_sched, 2);
       if (rc != ZGR_OK) return rc;
       rc = check(ctx, cudaMemset(g.d_sched, 0, 2 * sizeof(int32_t)));
@@ -322,6 +424,7 @@ int sweep(zgr_ctx* ctx, std::vector<Group>& groups, const TensorDesc* d_descs, i
   double cb_total = 0.0;
   for (int q = 0; q < n; ++q) cb_total += std::fabs(c[q] * ctx->b);
   p.kshift = kshift_for(cb_total);
+  bool first = true;     // the first kernel of the sweep waits for earlier work, the others rely on it
   for (Group& g : groups) {
     if (g.items.empty()) continue;
     p.items = g.d_items;
@@ -337,6 +440,8 @@ int sweep(zgr_ctx* ctx, std::vector<Group>& groups, const TensorDesc* d_descs, i
       p.item_base = b0;
     }
     const int grid = static_cast<int>(std::min<int64_t>(p.n_items, static_cast<int64_t>(ctx->sm_count) * blocks_per_sm(g.kc, n > 1, p.item_stats != nullptr)));
+    p.late = first ? 0 : 1;
+    first = false;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (ctx->profiling && t1 < 0) {
       if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {

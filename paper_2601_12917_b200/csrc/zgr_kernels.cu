@@ -92,6 +92,7 @@ __device__ __forceinline__ void unpack_raw(const uint4& raw, float (&v)[8]) {
 }
 template <typename T, int BITS, bool PRECISE, bool MULTI, bool SSTATS = false>
 __global__ void __launch_bounds__(kThreads, iso_blocks_per_sm(PRECISE, MULTI, SSTATS)) sweep_iso_kernel(const __grid_constant__ SweepParams p) {
+  dependency_begin(p);
   ItemFeed feed(p);
   for (int it = feed.first(); it < p.n_items; it = feed.next()) {
     const WorkItem w = p.items[it];
@@ -153,18 +154,22 @@ __global__ void __launch_bounds__(kThreads, iso_blocks_per_sm(PRECISE, MULTI, SS
     }
     if (SSTATS) store_item_stats(p, it, threadIdx.x >> 5, s_iso, 0.0, s_iso);
   }
+  dependency_end(p);
 }
 
 // ---------------------------------------------------------------------------------------------
 // rank <= R (R = 4 or 8): CUDA-core contraction.
-// A CTA owns a strip of up to 256 columns; lane l of every warp owns the octet of columns
-// [8l, 8l+8) of the strip and keeps its R x 8 coefficients in registers; the eight warps walk
-// the rows of the item in an interleaved fashion, each row being one 128-bit access per lane.
+// A CTA owns a strip of up to 256 columns.  A warp works on one row of a strip of more than 128 columns at a time, on two
+// rows of a narrower one, on four up to 64 and on eight up to 32: lane l owns the octet l mod L of columns, L = 32, 16, 8
+// or 4, and keeps its R x 8 coefficients in registers, so that narrow tensors and last strips do not leave lanes idle
+// (8.3 M bf16 weights 128 columns wide, rank 4: 50 us a sweep with L = 32).  The eight warps walk the rows in turn, each row
+// being one 128-bit access per lane.
 // ---------------------------------------------------------------------------------------------
 template <typename T, int BITS, bool PRECISE, int R, bool MULTI, bool SSTATS = false>
 __global__ void __launch_bounds__(kThreads, 2) sweep_fma_kernel(const __grid_constant__ SweepParams p) {
   __shared__ float Gs[R][256 + 8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  dependency_begin(p);
   ItemFeed feed(p);
   for (int it = feed.first(); it < p.n_items; it = feed.next()) {
     const WorkItem w = p.items[it];
@@ -188,21 +193,24 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_fma_kernel(const __grid_con
       }
     }
     __syncthreads();
-    const bool active = 8 * lane < w.ncols;
+    const int lanes_log2 = w.ncols > 128 ? 5 : (w.ncols > 64 ? 4 : (w.ncols > 32 ? 3 : 2));
+    const int oct = lane & ((1 << lanes_log2) - 1);
+    const bool active = 8 * oct < w.ncols;
     float g[R][8];
 #pragma unroll
     for (int k = 0; k < R; ++k)
 #pragma unroll
-      for (int i = 0; i < 8; ++i) g[k][i] = active ? Gs[k][8 * lane + i] : 0.0f;
+      for (int i = 0; i < 8; ++i) g[k][i] = active ? Gs[k][8 * oct + i] : 0.0f;
     const bool u_vec = (r == R) && ((reinterpret_cast<uintptr_t>(td.U) & 15) == 0);
     const int64_t row_end = w.row0_or_e0 + w.nrows_or_count;
     double s_iso = 0.0, s_gd = 0.0, s_z = 0.0;   // SSTATS only
-    for (int64_t row = w.row0_or_e0 + warp; row < row_end; row += kWarps) {
+    const int64_t step = kWarps << (5 - lanes_log2);
+    for (int64_t row = w.row0_or_e0 + (warp << (5 - lanes_log2)) + (lane >> lanes_log2); row < row_end; row += step) {
 #if ZGR_FMA_PREFETCH
       // this warp's row after next: start it on its way from HBM to L2 now (each lane asks for its own 8 elements);
       // with four warps per scheduler there is not enough other work to cover a full DRAM round trip otherwise
-      if (active && row + ZGR_FMA_PREFETCH * kWarps < row_end) {
-        const T* nxt = base + (row + ZGR_FMA_PREFETCH * kWarps) * cols + w.col0 + 8 * lane;
+      if (active && row + ZGR_FMA_PREFETCH * step < row_end) {
+        const T* nxt = base + (row + ZGR_FMA_PREFETCH * step) * cols + w.col0 + 8 * oct;
         asm volatile("prefetch.global.L2 [%0];" ::"l"(nxt));
       }
 #endif
@@ -218,7 +226,7 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_fma_kernel(const __grid_con
         for (int k = 0; k < R; ++k) u[k] = k < r ? __ldg(td.U + row * r + k) : 0.0f;
       }
       if (active) {
-        const int64_t e = row * cols + w.col0 + 8 * lane;
+        const int64_t e = row * cols + w.col0 + 8 * oct;
         float th[8], z[8];
         Storage<T>::load8(base + e, th);
         iso8<BITS, PRECISE, MULTI>(p, tid, static_cast<uint64_t>(e), z);
@@ -246,6 +254,7 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_fma_kernel(const __grid_con
     }
     if (SSTATS) store_item_stats(p, it, warp, s_iso, s_gd, s_z);
   }
+  dependency_end(p);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -585,18 +594,21 @@ __global__ void philox_blocks_kernel(PhiloxKeys keys, uint32_t tensor, uint32_t 
 // ---------------------------------------------------------------------------------------------
 namespace {
 
+// The kernels that handle programmatic dependencies themselves
+cudaError_t launch_dependent(void (*k)(SweepParams), const SweepParams& p, int grid, cudaStream_t st) {
+  return launch_sweep_kernel(k, grid, kThreads, 0, st, p);
+}
+
 template <typename T, int BITS, bool PRECISE, bool MULTI>
 cudaError_t launch_typed(const KernelChoice& kc, const SweepParams& p, int grid, cudaStream_t st) {
   if constexpr (!MULTI) {
     if (p.item_stats != nullptr) {      // the sweep also accumulates the norm bookkeeping
       switch (kc.path) {
         case PATH_ISO:
-          sweep_iso_kernel<T, BITS, PRECISE, false, true><<<grid, kThreads, 0, st>>>(p);
-          return cudaGetLastError();
+          return launch_dependent(sweep_iso_kernel<T, BITS, PRECISE, false, true>, p, grid, st);
         case PATH_FMA:
-          if (kc.kpad == 4) sweep_fma_kernel<T, BITS, PRECISE, 4, false, true><<<grid, kThreads, 0, st>>>(p);
-          else sweep_fma_kernel<T, BITS, PRECISE, 8, false, true><<<grid, kThreads, 0, st>>>(p);
-          return cudaGetLastError();
+          if (kc.kpad == 4) return launch_dependent(sweep_fma_kernel<T, BITS, PRECISE, 4, false, true>, p, grid, st);
+          return launch_dependent(sweep_fma_kernel<T, BITS, PRECISE, 8, false, true>, p, grid, st);
         case PATH_GENERIC:
           sweep_generic_kernel<T, BITS, PRECISE, false, true><<<grid, kThreads, 0, st>>>(p);
           return cudaGetLastError();
@@ -607,12 +619,10 @@ cudaError_t launch_typed(const KernelChoice& kc, const SweepParams& p, int grid,
   }
   switch (kc.path) {
     case PATH_ISO:
-      sweep_iso_kernel<T, BITS, PRECISE, MULTI><<<grid, kThreads, 0, st>>>(p);
-      break;
+      return launch_dependent(sweep_iso_kernel<T, BITS, PRECISE, MULTI>, p, grid, st);
     case PATH_FMA:
-      if (kc.kpad == 4) sweep_fma_kernel<T, BITS, PRECISE, 4, MULTI><<<grid, kThreads, 0, st>>>(p);
-      else sweep_fma_kernel<T, BITS, PRECISE, 8, MULTI><<<grid, kThreads, 0, st>>>(p);
-      break;
+      if (kc.kpad == 4) return launch_dependent(sweep_fma_kernel<T, BITS, PRECISE, 4, MULTI>, p, grid, st);
+      return launch_dependent(sweep_fma_kernel<T, BITS, PRECISE, 8, MULTI>, p, grid, st);
     case PATH_GENERIC:
       sweep_generic_kernel<T, BITS, PRECISE, MULTI><<<grid, kThreads, 0, st>>>(p);
       break;

@@ -31,6 +31,23 @@ int mma_strip_cols(int kpad);     // columns of a CTA strip on the tensor-core p
 int mma_rows_per_iter(int kpad);  // rows a CTA advances per iteration there
 size_t mma_smem_bytes(int kpad);
 
+// Launch of a kernel that handles programmatic dependencies (dependency_begin / dependency_end): it may start before the
+// kernel ahead of it in the stream has completed.
+template <typename... Params, typename... Args>
+cudaError_t launch_sweep_kernel(void (*kernel)(Params...), int grid, int threads, size_t smem, cudaStream_t st, const Args&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = dim3(static_cast<unsigned>(grid));
+  cfg.blockDim = dim3(static_cast<unsigned>(threads));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
 cudaError_t launch_sweep(const KernelChoice& kc, const SweepParams& p, int grid, cudaStream_t st);
 // tcgen05 + TMA sweep (16-bit weights, rank > 8).  tmaps: three tensor maps per tensor (theta, U hi, U lo).
 int umma_strip_cols(int kpad);

@@ -9,8 +9,8 @@
 // tail of the octet that began in the row before.  An owned octet reaches up to 7 columns beyond the strip, so the
 // product tile is computed 144 columns wide.
 //
-// Pipeline (one CTA per SM, static round-robin over the items):
-//   warp 0   TMA loads of U, 128 rows at a time, pre-split into three bf16 parts
+// Pipeline (one CTA per SM; the first item of a CTA is its own index, the others come from a counter in global memory):
+//   warp 0   hands out the items through a ring of four, TMA loads of U, 128 rows at a time, pre-split into three bf16 parts
 //   warp 1   tcgen05.mma:  D = c b U G  (128 x 144, fp32) into one of three tensor-memory buffers
 //   warps 2-17  coefficient strips c b G (three bf16 parts, K-major) into shared memory, one item ahead where two strips
 //            fit; then per tile and warp 32 rows x 32 columns: D through a warp-private shared-memory buffer, from one
@@ -44,7 +44,11 @@ constexpr int kAcc = 3;                        // accumulator buffers: 3 x 144 o
 constexpr int kEpi = 16;                       // epilogue warps: 32 rows x 32 columns of a tile each
 constexpr int kTileThreads = 32 * (2 + kEpi);
 constexpr int kParts = 3;                      // bf16 parts of an operand
+constexpr int kRing = 4;                       // items published ahead
 constexpr int kPitchMax = 42;
+#ifndef ZGR_PF
+#define ZGR_PF (sizeof(T) == 4)
+#endif
 constexpr int kXposeBytes = 32 * kPitchMax * 4;   // one warp's buffer
 
 // Shared-memory plan for contraction width kp (16, 32, 64).
@@ -199,8 +203,16 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
   auto BAR_U_FULL = [&](int u) { return bar0 + 8u * static_cast<uint32_t>(2 * kAcc + u); };
   auto BAR_U_FREE = [&](int u) { return bar0 + 8u * static_cast<uint32_t>(2 * kAcc + 2 + u); };
   auto BAR_G = [&](int g) { return bar0 + 8u * static_cast<uint32_t>(2 * kAcc + 4 + g); };
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kAcc + 6);
+  auto BAR_ITEM = [&](int i) { return bar0 + 8u * static_cast<uint32_t>(2 * kAcc + 6 + i); };            // item published
+  auto BAR_ITEM_READ = [&](int i) { return bar0 + 8u * static_cast<uint32_t>(2 * kAcc + 6 + kRing + i); };   // read by the other roles
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kAcc + 6 + 2 * kRing);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  volatile int* ring = abort_flag + 1;
+  // Number of the CTA's n-th item, or n_items at the end (and when a wait gave up); called once per n by each reading thread or warp.
+  auto item = [&](int n) -> int {
+    if (!mbar_wait<false>(BAR_ITEM(n % kRing), (n / kRing) & 1, abort_flag, error, 26)) return p.n_items;
+    return ring[n % kRing];
+  };
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
@@ -212,6 +224,10 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
       mbar_init(BAR_U_FULL(i), 1);
       mbar_init(BAR_U_FREE(i), 1);
       mbar_init(BAR_G(i), kEpi);
+    }
+    for (int i = 0; i < kRing; ++i) {
+      mbar_init(BAR_ITEM(i), 1);
+      mbar_init(BAR_ITEM_READ(i), 1 + kEpi);
     }
     *abort_flag = 0;
     fence_mbar_init();
@@ -225,6 +241,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  dependency_begin(p);
 
   // All roles walk the same sequence of (item, row tile) pairs; t counts tiles over the life of the CTA.
   if (warp == 0) {
@@ -232,8 +249,21 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
     if (elect_one()) {
       int t = 0;
       bool ok = true;
-      for (int it = blockIdx.x; it < p.n_items && ok; it += gridDim.x) {
+      int it = blockIdx.x;
+      for (int n = 0; ok; ++n) {
+        if (n >= kRing && !mbar_wait<true>(BAR_ITEM_READ(n % kRing), ((n / kRing) - 1) & 1, abort_flag, error, 20)) break;
+        ring[n % kRing] = it;
+        mbar_arrive(BAR_ITEM(n % kRing));
+        if (it >= p.n_items) break;
+        // the next item (as in ItemFeed of the CUDA-core kernels: one fetch beyond the end per CTA, the last one resets)
+        int after = p.n_items;
+        if (p.n_items > static_cast<int>(gridDim.x)) {
+          const int f = atomicAdd(p.sched, 1);
+          if (f == p.n_items - 1) *p.sched = 0;
+          after = f + static_cast<int>(gridDim.x);
+        }
         const WorkItem w = p.items[it];
+        it = after;
         const CUtensorMap* tm = tmaps + 3 * w.tensor;
         const int row_end = static_cast<int>(w.row0_or_e0 + w.nrows_or_count);
         for (int row0 = static_cast<int>(w.row0_or_e0); row0 < row_end; row0 += kTileM, ++t) {
@@ -258,9 +288,12 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
       const uint64_t desc_u0 = make_desc(smem_u32(u_base), rowb);
       const uint64_t desc_g0 = make_desc(smem_u32(g_base), rowb);
       const uint64_t u_part = static_cast<uint64_t>(L.u_bytes >> 4), g_part = static_cast<uint64_t>(L.g_bytes >> 4);
-      int t = 0, item_no = 0;
+      int t = 0;
       bool ok = true;
-      for (int it = blockIdx.x; it < p.n_items && ok; it += gridDim.x, ++item_no) {
+      for (int item_no = 0; ok; ++item_no) {
+        const int it = item(item_no);
+        mbar_arrive(BAR_ITEM_READ(item_no % kRing));
+        if (it >= p.n_items) break;
         const WorkItem w = p.items[it];
         const int g = item_no % GS;
         if (!mbar_wait<true>(BAR_G(g), (item_no / GS) & 1, abort_flag, error, 22)) break;
@@ -305,8 +338,16 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
       __syncwarp();
       if (lane == 0) mbar_arrive(BAR_G(no % GS));
     };
-    if (static_cast<int>(blockIdx.x) < p.n_items) strip_for(blockIdx.x, 0);
-    for (int it = blockIdx.x; it < p.n_items && ok; it += gridDim.x, ++item_no) {
+    auto take = [&](int n) -> int {
+      const int it = item(n);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(BAR_ITEM_READ(n % kRing));
+      return it;
+    };
+    int it = take(0);
+    if (it < p.n_items) strip_for(it, 0);
+    for (int it_next; it < p.n_items && ok; it = it_next, ++item_no) {
+      it_next = p.n_items;
       const WorkItem w = p.items[it];
       const TensorDesc& td = p.tensors[w.tensor];
       const uint32_t tid = static_cast<uint32_t>(td.id);
@@ -318,12 +359,14 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
       const bool vec = (reinterpret_cast<uintptr_t>(base) & 15) == 0;
       const int64_t row_end = w.row0_or_e0 + w.nrows_or_count;
       const int c_chunk = 32 * cg;                           // first column of this warp's chunk within the strip
-      const bool next = it + static_cast<int>(gridDim.x) < p.n_items;
       double s_iso = 0.0, s_gd = 0.0, s_z = 0.0;             // SSTATS only
       for (int64_t row0 = w.row0_or_e0; row0 < row_end && ok; row0 += kTileM, ++t) {
         // the strip of the next item goes into the other buffer before this item's last tile, so that its products run
         // while this tile is worked on
-        if (GS == 2 && next && row0 + kTileM >= row_end) strip_for(it + gridDim.x, item_no + 1);
+        if (row0 + kTileM >= row_end) {
+          it_next = take(item_no + 1);
+          if (GS == 2 && it_next < p.n_items) strip_for(it_next, item_no + 1);
+        }
         const int b = t % kAcc;
         const int64_t wrow = row0 + 32 * quad;               // first row of this warp
         // one octet per pass: element index of its start, its column, the elements of it that belong to this row
@@ -335,12 +378,22 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
         // weights of the first passes, on their way while the accumulator is waited for (four octets of 16-bit weights fit
         // the register budget, two of fp32)
         constexpr int kAhead = sizeof(T) == 4 ? 2 : 4;
+        constexpr bool kPrefetchNext = ZGR_PF;
         RawOct<T> raw[kAhead];
         auto fetch = [&](int pass) {
           if (full && wrow + 8 * pass + sub < row_end) raw[pass % kAhead].load(base + e_sub + 8 * pass * cols);
         };
 #pragma unroll
         for (int pass = 0; pass < kAhead; ++pass) fetch(pass);
+        if constexpr (kPrefetchNext) {
+          // the same octets of the next row tile: on their way from HBM to L2 while this one is worked on
+          if (n_el > 0) {
+#pragma unroll
+            for (int pass = 0; pass < 4; ++pass)
+              if (wrow + kTileM + 8 * pass + sub < row_end)
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(base + e_sub + (kTileM + 8 * pass) * cols));
+          }
+        }
         if (!mbar_wait<false>(BAR_ACC_FULL(b), (t / kAcc) & 1, abort_flag, error, 25)) { ok = false; break; }
         tc_fence_after();
         {
@@ -361,10 +414,11 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
           }
         }
         __syncwarp();
-        auto finish = [&](int64_t el, int i0, int i1, float (&d)[8], bool whole, const RawOct<T>* r) {
+        auto finish = [&](int64_t el, int i0, int i1, float (&d)[8]) {
+          const bool whole = vec && i0 == 0 && i1 == 8;
           float th[8], z[8];
           if (whole) {
-            r->unpack(th);
+            Storage<T>::load8(base + el, th);
           } else {
 #pragma unroll
             for (int i = 0; i < 8; ++i) th[i] = (i >= i0 && i < i1) ? Storage<T>::load1(base + el + i) : 0.0f;
@@ -408,22 +462,64 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
               if (i >= i0 && i < i1) Storage<T>::store1(base + el + i, th[i]);
           }
         };
+        auto read_d = [&](int pass, float (&d)[8]) {
+          const uint32_t xat = xbuf + static_cast<uint32_t>(((8 * pass + sub) * pitch + 8 * o + static_cast<int>(h_sub)) * 4);
+          if (even8) {
+            const uint4 d0 = lds128(xat), d1 = lds128(xat + 16);
+            d[0] = __uint_as_float(d0.x); d[1] = __uint_as_float(d0.y); d[2] = __uint_as_float(d0.z); d[3] = __uint_as_float(d0.w);
+            d[4] = __uint_as_float(d1.x); d[5] = __uint_as_float(d1.y); d[6] = __uint_as_float(d1.z); d[7] = __uint_as_float(d1.w);
+          } else {
 #pragma unroll
+            for (int i = 0; i < 8; ++i) d[i] = lds32(xat + 4u * i);
+          }
+        };
+        // All octets of the warp whole and under one high counter word (nearly always): straight-line code, several octets
+        // per thread whose generator chains interleave.  Otherwise (row ends, last rows, the bookkeeping) one octet after the other.
+        constexpr int kShift = BITS == 32 ? 34 : 35;       // element index -> high word of its block number
+        const uint32_t hi0 = static_cast<uint32_t>(static_cast<uint64_t>(e_sub) >> kShift);
+        const bool fast = !SSTATS && __all_sync(0xFFFFFFFFu, full && wrow + 24 + sub < row_end &&
+                                                                 hi0 == static_cast<uint32_t>(static_cast<uint64_t>(e_sub + 24 * cols) >> kShift));
+        if (fast) {
+          const PhiloxPre pre = philox_pre(hi0, tid, p.term[0].keys);
+          constexpr int kWide = sizeof(T) == 4 ? 2 : 4;
+#pragma unroll
+          for (int p0 = 0; p0 < 4; p0 += kWide) {
+            float z[kWide][8];
+            uint32_t oct[kWide];
+#pragma unroll
+            for (int x = 0; x < kWide; ++x) {
+              read_d(p0 + x, z[x]);
+              oct[x] = static_cast<uint32_t>(static_cast<uint64_t>(e_sub + 8 * (p0 + x) * cols) >> 3);
+            }
+#pragma unroll
+            for (int x = 0; x < kWide; ++x) normals8_add<BITS, PRECISE>(p.term[0].keys, pre, oct[x], p.term[0].iso, z[x]);
+            if (MULTI) {
+#pragma unroll 1
+              for (int q = 1; q < p.n_terms; ++q) {
+                const PhiloxPre pre_q = philox_pre(hi0, tid, p.term[q].keys);
+#pragma unroll
+                for (int x = 0; x < kWide; ++x) normals8_add<BITS, PRECISE>(p.term[q].keys, pre_q, oct[x], p.term[q].iso, z[x]);
+              }
+            }
+#pragma unroll
+            for (int x = 0; x < kWide; ++x) {
+              float th[8];
+              raw[(p0 + x) % kAhead].unpack(th);
+#pragma unroll
+              for (int i = 0; i < 8; ++i) th[i] += z[x][i];
+              Storage<T>::store8(base + e_sub + 8 * (p0 + x) * cols, th);
+              if (p0 + x + kAhead < 4) fetch(p0 + x + kAhead);
+            }
+          }
+        } else {
+#pragma unroll 1
         for (int pass = 0; pass < 4; ++pass) {
           if (n_el > 0 && wrow + 8 * pass + sub < row_end) {
             float d[8];
-            const uint32_t xat = xbuf + static_cast<uint32_t>(((8 * pass + sub) * pitch + 8 * o + static_cast<int>(h_sub)) * 4);
-            if (even8) {
-              const uint4 d0 = lds128(xat), d1 = lds128(xat + 16);
-              d[0] = __uint_as_float(d0.x); d[1] = __uint_as_float(d0.y); d[2] = __uint_as_float(d0.z); d[3] = __uint_as_float(d0.w);
-              d[4] = __uint_as_float(d1.x); d[5] = __uint_as_float(d1.y); d[6] = __uint_as_float(d1.z); d[7] = __uint_as_float(d1.w);
-            } else {
-#pragma unroll
-              for (int i = 0; i < 8; ++i) d[i] = lds32(xat + 4u * i);
-            }
-            finish(e_sub + 8 * pass * cols, 0, n_el, d, full, &raw[pass % kAhead]);
+            read_d(pass, d);
+            finish(e_sub + 8 * pass * cols, 0, n_el, d);
           }
-          if (pass + kAhead < 4) fetch(pass + kAhead);
+        }
         }
         if (!even8 && w.col0 == 0 && cg == 0) {
           // the columns before the first octet of each row: the tail of an octet that began in the previous row
@@ -433,12 +529,12 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
             float d[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) d[i] = i >= 8 - h ? lds32(xbuf + static_cast<uint32_t>((lane * pitch + i - (8 - h)) * 4)) : 0.0f;
-            finish(row * cols + h - 8, 8 - h, static_cast<int>(min(static_cast<int64_t>(8), 8 - h + cols)), d, false, nullptr);
+            finish(row * cols + h - 8, 8 - h, static_cast<int>(min(static_cast<int64_t>(8), 8 - h + cols)), d);
           }
         }
         __syncwarp();
       }
-      if (GS == 1 && next && ok) strip_for(it + gridDim.x, item_no + 1);   // every product that read the old strip has completed
+      if (GS == 1 && it_next < p.n_items && ok) strip_for(it_next, item_no + 1);   // every product that read the old strip has completed
       if constexpr (SSTATS) {
         if (ok) store_item_stats(p, it, e, s_iso, s_gd, s_z);
       }
@@ -446,6 +542,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
   }
 
   // ---- common exit ----
+  dependency_end(p);
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
@@ -461,8 +558,7 @@ cudaError_t launch_tile_one(int kp, const SweepParams& p, const CUtensorMap* tma
   const int smem = tile_smem(kp).total;
   const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, tile_smem(64).total);
   if (e != cudaSuccess) return e;
-  k<<<grid, kTileThreads, smem, st>>>(p, tmaps, error, kp);
-  return cudaGetLastError();
+  return launch_sweep_kernel(k, grid, kTileThreads, static_cast<size_t>(smem), st, p, tmaps, error, kp);
 }
 template <typename T, bool PRECISE>
 cudaError_t launch_tile_typed(const KernelChoice& kc, const SweepParams& p, const CUtensorMap* tmaps, int* error, int grid, cudaStream_t st) {

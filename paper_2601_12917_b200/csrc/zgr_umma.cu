@@ -235,6 +235,7 @@ __global__ void __launch_bounds__(UmmaCfg<KP>::THREADS, 1) sweep_umma_kernel(con
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  dependency_begin(p);
 
   // The three roles walk the same sequence of (item, row block, tile) triples; t counts tiles and
   // rb counts row blocks over the whole life of the CTA, which fixes every ring slot and phase.
@@ -592,6 +593,7 @@ __global__ void __launch_bounds__(UmmaCfg<KP>::THREADS, 1) sweep_umma_kernel(con
   }
 
   // ---- common exit ----
+  dependency_end(p);
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
@@ -615,13 +617,12 @@ cudaError_t launch_umma_kp(int kpad, const SweepParams& p, const CUtensorMap* tm
     auto k = sweep_umma_kernel<T, BITS, KPV, STATS, MULTI, ZOUT, SSTATS>;                                                 \
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, UmmaCfg<KPV>::SMEM_BYTES); \
     if (e != cudaSuccess) return e;                                                                                \
-    k<<<grid, UmmaCfg<KPV>::THREADS, UmmaCfg<KPV>::SMEM_BYTES, st>>>(p, tmaps, error);                                      \
+    return launch_sweep_kernel(k, grid, UmmaCfg<KPV>::THREADS, UmmaCfg<KPV>::SMEM_BYTES, st, p, tmaps, error);                \
   }
   if (kpad == 16) ZGR_LAUNCH_UMMA(16)
   else if (kpad == 32) ZGR_LAUNCH_UMMA(32)
   else ZGR_LAUNCH_UMMA(64)
 #undef ZGR_LAUNCH_UMMA
-  return cudaGetLastError();
 }
 }  // namespace
 
