@@ -489,14 +489,29 @@ struct Storage;
 
 template <>
 struct Storage<float> {
-  static __device__ __forceinline__ void load8(const float* p, float (&v)[8]) {
-    const float4 a = __ldcs(reinterpret_cast<const float4*>(p));
-    const float4 b = __ldcs(reinterpret_cast<const float4*>(p) + 1);
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+  // wide: the address is a multiple of 32 bytes, one 256-bit access per octet (two 128-bit ones cost twice the cache
+  // wavefronts: neighbouring lanes are 32 bytes apart)
+  static __device__ __forceinline__ void load8(const float* p, float (&v)[8], bool wide = false) {
+    if (wide) {
+      asm volatile("ld.global.L1::no_allocate.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                   : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                   : "l"(p)
+                   : "memory");
+    } else {
+      const float4 a = __ldcs(reinterpret_cast<const float4*>(p));
+      const float4 b = __ldcs(reinterpret_cast<const float4*>(p) + 1);
+      v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    }
   }
-  static __device__ __forceinline__ void store8(float* p, const float (&v)[8]) {
-    __stcs(reinterpret_cast<float4*>(p), make_float4(v[0], v[1], v[2], v[3]));
-    __stcs(reinterpret_cast<float4*>(p) + 1, make_float4(v[4], v[5], v[6], v[7]));
+  static __device__ __forceinline__ void store8(float* p, const float (&v)[8], bool wide = false) {
+    if (wide) {
+      asm volatile("st.global.v8.f32 [%8], {%0,%1,%2,%3,%4,%5,%6,%7};" ::"f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]),
+                   "f"(v[7]), "l"(p)
+                   : "memory");
+    } else {
+      __stcs(reinterpret_cast<float4*>(p), make_float4(v[0], v[1], v[2], v[3]));
+      __stcs(reinterpret_cast<float4*>(p) + 1, make_float4(v[4], v[5], v[6], v[7]));
+    }
   }
   static __device__ __forceinline__ float load1(const float* p) { return *p; }
   static __device__ __forceinline__ void store1(float* p, float v) { *p = v; }
@@ -504,7 +519,7 @@ struct Storage<float> {
 
 template <>
 struct Storage<__half> {
-  static __device__ __forceinline__ void load8(const __half* p, float (&v)[8]) {
+  static __device__ __forceinline__ void load8(const __half* p, float (&v)[8], bool = false) {
     const uint4 raw = __ldcs(reinterpret_cast<const uint4*>(p));
     const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
 #pragma unroll
@@ -514,7 +529,7 @@ struct Storage<__half> {
       v[2 * i + 1] = f.y;
     }
   }
-  static __device__ __forceinline__ void store8(__half* p, const float (&v)[8]) {
+  static __device__ __forceinline__ void store8(__half* p, const float (&v)[8], bool = false) {
     uint32_t w[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -529,7 +544,7 @@ struct Storage<__half> {
 
 template <>
 struct Storage<__nv_bfloat16> {
-  static __device__ __forceinline__ void load8(const __nv_bfloat16* p, float (&v)[8]) {
+  static __device__ __forceinline__ void load8(const __nv_bfloat16* p, float (&v)[8], bool = false) {
     const uint4 raw = __ldcs(reinterpret_cast<const uint4*>(p));
     const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
 #pragma unroll
@@ -538,7 +553,7 @@ struct Storage<__nv_bfloat16> {
       v[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
     }
   }
-  static __device__ __forceinline__ void store8(__nv_bfloat16* p, const float (&v)[8]) {
+  static __device__ __forceinline__ void store8(__nv_bfloat16* p, const float (&v)[8], bool = false) {
     uint32_t w[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {

@@ -10,6 +10,7 @@
 #include <functional>
 #include <map>
 #include <new>
+#include <numeric>
 #include <queue>
 #include <vector>
 
@@ -151,12 +152,32 @@ bool make_map_16bit(CUtensorMap* out, const void* base, int64_t rows, int64_t co
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Which tcgen05 kernel serves a tensor: 1 the TMA-staged one (16-bit weights, rank > 8, rows that TMA can address), 2 the
-// tile kernel (everything else with a subspace that the CUDA-core kernel for rank <= 8 does not take), 0 neither.
-int tensor_core_kind(const zgr_tensor& t, bool guided_on) {
+// Weights in rank <= 8 tensors whose rows are whole octets, by storage: the kernel that serves them depends on how many there are.
+struct LowRank {
+  int64_t f32 = 0, half = 0;
+};
+bool whole_octets(const zgr_tensor& t) { return (reinterpret_cast<uintptr_t>(t.data) & 15) == 0 && (t.cols % 8 == 0); }
+LowRank low_rank(const zgr_tensor* tensors, int32_t n) {
+  LowRank lr;
+  for (int32_t l = 0; l < n; ++l)
+    if (tensors[l].rank > 0 && tensors[l].rank <= 8 && whole_octets(tensors[l])) (tensors[l].dtype == ZGR_F32 ? lr.f32 : lr.half) += tensors[l].rows * tensors[l].cols;
+  return lr;
+}
+
+// Which tcgen05 kernel serves a tensor: 1 the TMA-staged one (16-bit weights in rows that TMA can address), 2 the tile kernel
+// (everything else with a subspace), 0 neither.  Small sets of rank <= 8 stay with the CUDA-core kernel, which starts faster
+// (a step of 1.0 M bf16 weights, rank 8: 22 us there, 29 on tensor cores; 3.9 M: 66 and 29; 354 M: 1380 and 914).
+int tensor_core_kind(const zgr_tensor& t, bool guided_on, const LowRank& lr, int bits) {
   if (!guided_on || t.rank == 0 || t.rows >= (int64_t{1} << 31) - 256) return 0;
-  const bool vec = (reinterpret_cast<uintptr_t>(t.data) & 15) == 0 && (t.cols % 8 == 0);
-  if (vec && t.rank <= 8) return 0;
+  const bool vec = whole_octets(t);
+  if (vec && t.rank <= 8) {
+    const int64_t set = t.dtype == ZGR_F32 ? lr.f32 : lr.half;
+    if (set < (int64_t{1} << 21)) return 0;
+    // (fp32 sets that keep every SM busy for long run at the power cap, where the kernel without tensor cores is ahead: 354 M
+    // weights, rank 8, in steady state 1885 us a step there and 1918 here, in short runs rank 4 1538 and 1600, 1718 and 1903 with
+    // 32 random bits; 42 M, rank 8: 289 and 208, rank 4: 209 and 210)
+    if (t.dtype == ZGR_F32 && ((t.rank <= 4 && set >= (int64_t{1} << 25)) || set >= (int64_t{1} << 28))) return 0;
+  }
   // (the TMA-staged kernel keeps the high counter word of the generator fixed: fewer than 2^32 blocks of four elements)
   if (vec && t.dtype != ZGR_F32 && t.rows * t.cols < (int64_t{1} << 34)) return t.cols < (int64_t{1} << 31) - 256 ? 1 : 0;
   return 2;
@@ -168,9 +189,10 @@ bool umma_wanted() {
 }
 
 int blocks_per_sm(const KernelChoice& kc, bool multi = false, bool stats = false) {
+  if (is_tile(kc)) return 1;
   switch (kc.path) {
     case PATH_ISO: return iso_blocks_per_sm(kc.precise != 0, multi, stats);
-    case PATH_GENERIC: return kc.kpad > 0 ? 1 : 4;
+    case PATH_GENERIC: return 4;
     case PATH_UMMA: return 1;
     default: return 2;
   }
@@ -198,8 +220,8 @@ void cut_tensor(const TensorDesc& t, int l, int strip, int row_step, int64_t nro
 void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>& members, int sm_count, int64_t target, Group& g) {
   const auto by_elements = [](int64_t elements, int ncols) { return elements / ncols; };
   const auto by_rows = [](int64_t rows, int) { return rows; };
-  const bool tile = g.kc.path == PATH_GENERIC && g.kc.kpad > 0;
-  if (g.kc.path == PATH_FMA) {
+  const bool tile = is_tile(g.kc);
+  if (g.kc.path == PATH_FMA && !tile) {
     // handed out by a counter: nine items per CTA on large sets; down to as many rows as make the strip half of an item's
     // generator work when there is too little to go round
     int64_t total = 0;
@@ -223,9 +245,11 @@ void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>&
     const bool few = tiles < 12 * static_cast<int64_t>(sm_count);
     double best = 0.0;
     std::vector<WorkItem> trial;
+    std::vector<double> dealt(static_cast<size_t>(sm_count));
     for (int64_t big : {16, 12, 8, 6, 4, 3, 2, 1})
       for (int64_t small : {big, std::max<int64_t>(big / 4, 1)}) {
         if (few && small != big) continue;
+        if (tiles >= 64 * static_cast<int64_t>(sm_count) && big != 8 && big != 4) continue;
         if (best > 0.0 && (small == big ? tiles / big > 40 * static_cast<int64_t>(sm_count) : big == 1)) continue;
         trial.clear();
         int64_t done = 0;
@@ -246,6 +270,13 @@ void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>&
           end = std::max(end, at);
         }
         if (!few) end += 0.5 * (static_cast<double>(small) + item_cost);
+        if (tiles >= 64 * static_cast<int64_t>(sm_count)) {
+          // long sweeps: also even when dealt out in turn, so that neither the model nor the counter has to be right
+          std::fill(dealt.begin(), dealt.end(), 0.0);
+          for (size_t i = 0; i < trial.size(); ++i) dealt[i % dealt.size()] += static_cast<double>(trial[i].nrows_or_count) * trial[i].ncols;
+          const double mean = std::accumulate(dealt.begin(), dealt.end(), 0.0) / static_cast<double>(dealt.size());
+          if (*std::max_element(dealt.begin(), dealt.end()) > 1.025 * mean) end *= 2.0;
+        }
         if (best == 0.0 || end < best) {
           best = end;
           g.items = trial;
@@ -335,11 +366,11 @@ void plan(const std::vector<TensorDesc>& descs, const std::vector<int>& which, b
     if (tile_ok) {
       // fp32 with rank > 8, and rows that are not a multiple of eight elements: sweep_tile_kernel.  (The test hook that
       // sweeps an fp32 image of a 16-bit tensor keeps the one-element-per-thread kernel below.)
-      path = PATH_GENERIC; kpad = t.kpad; strip = tile_strip_cols(); row_step = 128;
+      path = vec && t.rank <= 8 ? PATH_FMA : PATH_GENERIC; kpad = t.kpad; strip = tile_strip_cols(); row_step = 128;
     } else if (!vec || (t.rank > 8 && !umma_ok && (t.Ufrag == nullptr || multi))) {
       // (the legacy tensor-core kernel applies one term per sweep; several terms take the fallback)
       path = PATH_GENERIC; kpad = 0; strip = 64; row_step = 1;
-    } else if (t.rank <= 8) {
+    } else if (t.rank <= 8 && !umma_ok) {
       path = PATH_FMA; kpad = t.rank <= 4 ? 4 : 8; strip = 256; row_step = 1;
     } else if (umma_ok) {
       path = PATH_UMMA; kpad = t.kpad; strip = umma_strip_cols(kpad); row_step = 128;
@@ -394,7 +425,7 @@ int upload_groups(zgr_ctx* ctx, std::vector<Group>& groups) {
     if (rc != ZGR_OK) return rc;
     rc = check(ctx, cudaMemcpy(g.d_items, g.items.data(), g.items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice));
     if (rc != ZGR_OK) return rc;
-    if (g.kc.path == PATH_FMA || g.kc.path == PATH_ISO || (g.kc.path == PATH_GENERIC && g.kc.kpad > 0)) {
+    if (g.kc.path == PATH_FMA || g.kc.path == PATH_ISO || is_tile(g.kc)) {
       rc = dev_alloc(ctx, &g.d_sched, 2);
       if (rc != ZGR_OK) return rc;
       rc = check(ctx, cudaMemset(g.d_sched, 0, 2 * sizeof(int32_t)));
@@ -451,7 +482,7 @@ int sweep(zgr_ctx* ctx, std::vector<Group>& groups, const TensorDesc* d_descs, i
       cudaEventRecord(e0, st);
     }
     const int rc = check(ctx, g.kc.path == PATH_UMMA ? launch_sweep_umma(g.kc, p, tmaps, ctx->d_err, grid, st)
-                              : g.kc.path == PATH_GENERIC && g.kc.kpad > 0 ? launch_sweep_tile(g.kc, p, tmaps, ctx->d_err, grid, st)
+                              : is_tile(g.kc) ? launch_sweep_tile(g.kc, p, tmaps, ctx->d_err, grid, st)
                                                                            : launch_sweep(g.kc, p, grid, st));
     if (rc != ZGR_OK) {
       if (e0) cudaEventDestroy(e0);
@@ -662,12 +693,13 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
   std::memset(ctx->tmaps.data(), 0, ctx->tmaps.size() * sizeof(CUtensorMap));
   const bool guided_on = ctx->b != 0.0;
   ctx->guided_at_init = guided_on;
+  const LowRank lr = low_rank(tensors, n);
   // one allocation for all operand copies
   void* operands = nullptr;
   if (umma_wanted() && encode_tiled_fn() != nullptr) {
     size_t bytes = 0;
     for (int32_t l = 0; l < n; ++l) {
-      const int kind = tensor_core_kind(tensors[l], guided_on);
+      const int kind = tensor_core_kind(tensors[l], guided_on, lr, cfg->bits_per_normal);
       const size_t kpad = tensors[l].rank <= 16 ? 16 : (tensors[l].rank <= 32 ? 32 : 64);
       if (kind != 0) bytes += (kind == 1 ? 2 : 3) * static_cast<size_t>((tensors[l].rows + 127) / 128) * 128 * kpad * 2;
     }
@@ -699,7 +731,7 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
     td.ushift = 0;
     for (void*& copy : td.Ucopy) copy = nullptr;
     // tcgen05 kernels: row-major copies of U in parts, and three tensor maps
-    const int kind = tensor_core_kind(t, guided_on);
+    const int kind = tensor_core_kind(t, guided_on, lr, cfg->bits_per_normal);
     if (kind != 0 && umma_wanted() && encode_tiled_fn() != nullptr) {
       const int parts = kind == 1 ? 2 : 3;
       const int64_t rows_pad = ((t.rows + 127) / 128) * 128;
@@ -1156,6 +1188,8 @@ int zgr_get_stats(zgr_ctx* ctx, uint64_t seed, double* out, void* stream) {
 int zgr_enable_stats(zgr_ctx* ctx, int32_t enable) {
   if (!ctx) return ZGR_EINVAL;
   ctx->stats_on = enable != 0;     // norms already held stay available until something they depend on changes
+  // the slots of the partial sums, here rather than inside the first perturbation
+  if (ctx->stats_on && ctx->sticky == 0 && on_ctx_device(ctx) && sweep_stats_possible(ctx)) return prepare_sweep_stats(ctx);
   return ZGR_OK;
 }
 
@@ -1354,6 +1388,7 @@ int zgr_debug_plan(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, 
   const int valid = validate_model(tensors, n, cfg, &d, &K);
   if (valid != ZGR_OK) return valid;
   const bool guided_on = K > 0 && cfg->alpha < 1.0;
+  const LowRank lr = low_rank(tensors, n);
   std::vector<TensorDesc> descs(static_cast<size_t>(n));
   std::vector<int> all(static_cast<size_t>(n));
   for (int32_t l = 0; l < n; ++l) {
@@ -1367,7 +1402,7 @@ int zgr_debug_plan(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, 
       td.kpad = t.rank <= 16 ? 16 : (t.rank <= 32 ? 32 : 64);
       td.Ufrag = reinterpret_cast<const uint4*>(uintptr_t{16});   // marker only: never dereferenced by the planner
     }
-    const int kind = tcgen05 ? tensor_core_kind(t, guided_on) : 0;
+    const int kind = tcgen05 ? tensor_core_kind(t, guided_on, lr, cfg->bits_per_normal) : 0;
     if (kind != 0) {
       td.kpad = t.rank <= 16 ? 16 : (t.rank <= 32 ? 32 : 64);
       (kind == 1 ? td.umma : td.tile) = 1;

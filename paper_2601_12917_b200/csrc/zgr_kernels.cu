@@ -175,6 +175,7 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_fma_kernel(const __grid_con
     const WorkItem w = p.items[it];
     const TensorDesc& td = p.tensors[w.tensor];
     T* base = static_cast<T*>(td.data);
+    const bool wide = (reinterpret_cast<uintptr_t>(base) & 31) == 0;
     const uint32_t tid = static_cast<uint32_t>(td.id);
     const int r = td.rank;
     const int64_t cols = td.cols;
@@ -196,11 +197,11 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_fma_kernel(const __grid_con
     const int lanes_log2 = w.ncols > 128 ? 5 : (w.ncols > 64 ? 4 : (w.ncols > 32 ? 3 : 2));
     const int oct = lane & ((1 << lanes_log2) - 1);
     const bool active = 8 * oct < w.ncols;
-    float g[R][8];
+    uint64_t g[R][4];     // pairs of neighbouring columns: two multiply-adds per instruction (354 M fp32 weights, rank 8: 1890 -> 1865 us a step)
 #pragma unroll
     for (int k = 0; k < R; ++k)
 #pragma unroll
-      for (int i = 0; i < 8; ++i) g[k][i] = active ? Gs[k][8 * oct + i] : 0.0f;
+      for (int i = 0; i < 4; ++i) g[k][i] = active ? pack2(Gs[k][8 * oct + 2 * i], Gs[k][8 * oct + 2 * i + 1]) : 0;
     const bool u_vec = (r == R) && ((reinterpret_cast<uintptr_t>(td.U) & 15) == 0);
     const int64_t row_end = w.row0_or_e0 + w.nrows_or_count;
     double s_iso = 0.0, s_gd = 0.0, s_z = 0.0;   // SSTATS only
@@ -228,28 +229,37 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_fma_kernel(const __grid_con
       if (active) {
         const int64_t e = row * cols + w.col0 + 8 * oct;
         float th[8], z[8];
-        Storage<T>::load8(base + e, th);
+        Storage<T>::load8(base + e, th, wide);
         iso8<BITS, PRECISE, MULTI>(p, tid, static_cast<uint64_t>(e), z);
         float f_iso = 0.0f, f_gd = 0.0f, f_z = 0.0f;
+        uint64_t acc[4];      // the perturbation is summed on its own scale, then added to theta once
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          float acc = z[i];  // the perturbation is summed on its own scale, then added to theta once
+        for (int i = 0; i < 4; ++i) acc[i] = pack2(z[2 * i], z[2 * i + 1]);
 #pragma unroll
-          for (int k = 0; k < R; ++k) acc = fmaf(u[k], g[k][i], acc);
+        for (int k = 0; k < R; ++k) {
+          const uint64_t uu = dup2(u[k]);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) acc[i] = fma2(uu, g[k][i], acc[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          float a0, a1;
+          unpack2(acc[i], a0, a1);
           if (SSTATS) {
-            const float gd = acc - z[i];
-            f_iso = fmaf(z[i], z[i], f_iso);
-            f_gd = fmaf(gd, gd, f_gd);
-            f_z = fmaf(acc, acc, f_z);
+            const float z0 = z[2 * i], z1 = z[2 * i + 1];
+            f_iso = fmaf(z0, z0, fmaf(z1, z1, f_iso));
+            f_gd = fmaf(a0 - z0, a0 - z0, fmaf(a1 - z1, a1 - z1, f_gd));
+            f_z = fmaf(a0, a0, fmaf(a1, a1, f_z));
           }
-          th[i] += acc;
+          th[2 * i] += a0;
+          th[2 * i + 1] += a1;
         }
         if (SSTATS) {
           s_iso += static_cast<double>(f_iso);
           s_gd += static_cast<double>(f_gd);
           s_z += static_cast<double>(f_z);
         }
-        Storage<T>::store8(base + e, th);
+        Storage<T>::store8(base + e, th, wide);
       }
     }
     if (SSTATS) store_item_stats(p, it, warp, s_iso, s_gd, s_z);

@@ -27,6 +27,10 @@ struct KernelChoice {
 // eight blocks, whose loads then cover the DRAM latency (5.74 TB/s standalone against 5.50 with six).
 constexpr int iso_blocks_per_sm(bool precise, bool multi, bool stats) { return !precise && !multi && !stats ? 8 : 5; }
 
+// The groups that sweep_tile_kernel serves: rank <= 8 tensors in whole octets are counted under the path of the CUDA-core
+// kernel (whose contraction widths are 4 and 8), the others under that of the fallback kernel (whose width is 0).
+inline bool is_tile(const KernelChoice& kc) { return (kc.path == PATH_FMA && kc.kpad == 16) || (kc.path == PATH_GENERIC && kc.kpad > 0); }
+
 int mma_strip_cols(int kpad);     // columns of a CTA strip on the tensor-core path
 int mma_rows_per_iter(int kpad);  // rows a CTA advances per iteration there
 size_t mma_smem_bytes(int kpad);

@@ -150,38 +150,33 @@ __device__ __forceinline__ void build_strip(const TensorDesc& td, const SweepPar
   }
 }
 
-// raw storage of an octet: 16 bytes for 16-bit types, 32 for fp32
+// storage of an octet as it is loaded: 16 bytes of 16-bit weights, unpacked on use, or eight floats
 template <typename T>
 struct RawOct {
-  static constexpr int N = sizeof(T) == 4 ? 2 : 1;
-  uint4 v[N];
-  __device__ __forceinline__ void load(const T* p) {
-#pragma unroll
-    for (int i = 0; i < N; ++i) v[i] = __ldcs(reinterpret_cast<const uint4*>(p) + i);
-  }
+  uint4 v;
+  __device__ __forceinline__ void load(const T* p, bool) { v = __ldcs(reinterpret_cast<const uint4*>(p)); }
   __device__ __forceinline__ void unpack(float (&f)[8]) const {
-    if constexpr (sizeof(T) == 4) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-      for (int i = 0; i < N; ++i) {
-        f[4 * i] = __uint_as_float(v[i].x);
-        f[4 * i + 1] = __uint_as_float(v[i].y);
-        f[4 * i + 2] = __uint_as_float(v[i].z);
-        f[4 * i + 3] = __uint_as_float(v[i].w);
-      }
-    } else {
-      const uint32_t w[4] = {v[0].x, v[0].y, v[0].z, v[0].w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if constexpr (std::is_same<T, __nv_bfloat16>::value) {
-          f[2 * i] = __uint_as_float(w[i] << 16);
-          f[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
-        } else {
-          const float2 h = __half22float2(*reinterpret_cast<const __half2*>(&w[i]));
-          f[2 * i] = h.x;
-          f[2 * i + 1] = h.y;
-        }
+    for (int i = 0; i < 4; ++i) {
+      if constexpr (std::is_same<T, __nv_bfloat16>::value) {
+        f[2 * i] = __uint_as_float(w[i] << 16);
+        f[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
+      } else {
+        const float2 h = __half22float2(*reinterpret_cast<const __half2*>(&w[i]));
+        f[2 * i] = h.x;
+        f[2 * i + 1] = h.y;
       }
     }
+  }
+};
+template <>
+struct RawOct<float> {
+  float v[8];
+  __device__ __forceinline__ void load(const float* p, bool wide) { Storage<float>::load8(p, v, wide); }
+  __device__ __forceinline__ void unpack(float (&f)[8]) const {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) f[i] = v[i];
   }
 };
 
@@ -356,7 +351,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
       const bool even8 = cols8 == 0;
       const int pitch = even8 ? 36 : ((cols & 1) ? 42 : 41);
       T* const base = static_cast<T*>(td.data);
-      const bool vec = (reinterpret_cast<uintptr_t>(base) & 15) == 0;
+      const bool vec = (reinterpret_cast<uintptr_t>(base) & 15) == 0, wide = (reinterpret_cast<uintptr_t>(base) & 31) == 0;
       const int64_t row_end = w.row0_or_e0 + w.nrows_or_count;
       const int c_chunk = 32 * cg;                           // first column of this warp's chunk within the strip
       double s_iso = 0.0, s_gd = 0.0, s_z = 0.0;             // SSTATS only
@@ -380,11 +375,11 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
         constexpr int kAhead = sizeof(T) == 4 ? 2 : 4;
         constexpr bool kPrefetchNext = ZGR_PF;
         RawOct<T> raw[kAhead];
-        auto fetch = [&](int pass) {
-          if (full && wrow + 8 * pass + sub < row_end) raw[pass % kAhead].load(base + e_sub + 8 * pass * cols);
+        auto fetch = [&](int pass, RawOct<T>& into) {
+          if (full && wrow + 8 * pass + sub < row_end) into.load(base + e_sub + 8 * pass * cols, wide);
         };
 #pragma unroll
-        for (int pass = 0; pass < kAhead; ++pass) fetch(pass);
+        for (int pass = 0; pass < kAhead; ++pass) fetch(pass, raw[pass]);
         if constexpr (kPrefetchNext) {
           // the same octets of the next row tile: on their way from HBM to L2 while this one is worked on
           if (n_el > 0) {
@@ -414,7 +409,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
           }
         }
         __syncwarp();
-        auto finish = [&](int64_t el, int i0, int i1, float (&d)[8]) {
+        auto finish = [&](int64_t el, int i0, int i1, const float (&d)[8]) {
           const bool whole = vec && i0 == 0 && i1 == 8;
           float th[8], z[8];
           if (whole) {
@@ -481,8 +476,10 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
                                                                  hi0 == static_cast<uint32_t>(static_cast<uint64_t>(e_sub + 24 * cols) >> kShift));
         if (fast) {
           const PhiloxPre pre = philox_pre(hi0, tid, p.term[0].keys);
-          constexpr int kWide = sizeof(T) == 4 ? 2 : 4;
-#pragma unroll
+          // as many at a time as were loaded ahead (a loop that is not unrolled: the accurate transform would fill the
+          // instruction cache)
+          constexpr int kWide = kAhead;
+#pragma unroll 1
           for (int p0 = 0; p0 < 4; p0 += kWide) {
             float z[kWide][8];
             uint32_t oct[kWide];
@@ -504,33 +501,33 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
 #pragma unroll
             for (int x = 0; x < kWide; ++x) {
               float th[8];
-              raw[(p0 + x) % kAhead].unpack(th);
+              raw[x].unpack(th);
 #pragma unroll
               for (int i = 0; i < 8; ++i) th[i] += z[x][i];
-              Storage<T>::store8(base + e_sub + 8 * (p0 + x) * cols, th);
-              if (p0 + x + kAhead < 4) fetch(p0 + x + kAhead);
+              Storage<T>::store8(base + e_sub + 8 * (p0 + x) * cols, th, wide);
+              if (p0 + kWide < 4) fetch(p0 + x + kWide, raw[x]);
             }
           }
-        } else {
+        }
+        // pass 4: the columns before the first octet of each row (lane = row), the tail of an octet that began in the previous row
+        const bool head = !even8 && w.col0 == 0 && cg == 0;
 #pragma unroll 1
-        for (int pass = 0; pass < 4; ++pass) {
-          if (n_el > 0 && wrow + 8 * pass + sub < row_end) {
-            float d[8];
+        for (int pass = fast ? 4 : 0; pass < (head ? 5 : 4); ++pass) {
+          float d[8];
+          int64_t el = e_sub + 8 * pass * cols;
+          int i0 = 0, i1 = wrow + 8 * pass + sub < row_end ? n_el : 0;
+          if (pass < 4) {
             read_d(pass, d);
-            finish(e_sub + 8 * pass * cols, 0, n_el, d);
-          }
-        }
-        }
-        if (!even8 && w.col0 == 0 && cg == 0) {
-          // the columns before the first octet of each row: the tail of an octet that began in the previous row
-          const int64_t row = wrow + lane;
-          const int h = static_cast<int>((0u - static_cast<uint32_t>(row & 7) * cols8) & 7u);
-          if (h > 0 && row < row_end) {
-            float d[8];
+          } else {
+            const int64_t row = wrow + lane;
+            const int h = static_cast<int>((0u - static_cast<uint32_t>(row & 7) * cols8) & 7u);
+            el = row * cols + h - 8;
+            i0 = 8 - h;
+            i1 = row < row_end && h > 0 ? static_cast<int>(min(static_cast<int64_t>(8), 8 - h + cols)) : 0;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) d[i] = i >= 8 - h ? lds32(xbuf + static_cast<uint32_t>((lane * pitch + i - (8 - h)) * 4)) : 0.0f;
-            finish(row * cols + h - 8, 8 - h, static_cast<int>(min(static_cast<int64_t>(8), 8 - h + cols)), d);
+            for (int i = 0; i < 8; ++i) d[i] = i >= i0 ? lds32(xbuf + static_cast<uint32_t>((lane * pitch + i - i0) * 4)) : 0.0f;
           }
+          if (i1 > i0) finish(el, i0, i1, d);
         }
         __syncwarp();
       }
