@@ -41,6 +41,7 @@ constexpr int kChunkRows = 128;
 constexpr int kLd = 65;               // leading dimension of the shared-memory matrices (64 + 1: no bank conflicts down a column)
 constexpr int kQrThreads = 256;
 constexpr int kMaxR = 64;
+constexpr double kPivotFloor = 1e-14;   // a pivot below this share of its column's squared norm is rounding error: the columns are dependent
 
 // Partial Gram matrix of rows [chunk*128, +128) of X (rows x r).  X is fp32 (SRC_DOUBLE = false) or double.
 template <bool SRC_DOUBLE>
@@ -81,18 +82,20 @@ __global__ void __launch_bounds__(kQrThreads) factor_kernel(const double* __rest
   double (*Winv)[kLd] = reinterpret_cast<double (*)[kLd]>(dyn_smem + kMaxR * kLd);
   double (*Old)[kLd] = reinterpret_cast<double (*)[kLd]>(dyn_smem + 2 * kMaxR * kLd);
   __shared__ int bad;
+  __shared__ double norm2[kMaxR];        // diagonal before the factorisation: the columns' squared norms
   if (threadIdx.x == 0) bad = 0;
   for (int idx = threadIdx.x; idx < r * r; idx += kQrThreads) {
     double s = 0.0;
     for (int c = 0; c < n_chunks; ++c) s += partials[static_cast<int64_t>(c) * r * r + idx];
     S[idx / r][idx % r] = s;
+    if (idx / r == idx % r) norm2[idx / r] = s;
   }
   __syncthreads();
   // Cholesky, column by column (right-looking), upper triangular factor kept in the upper triangle of S
   for (int k = 0; k < r; ++k) {
     if (threadIdx.x == 0) {
       const double p = S[k][k];
-      if (!(p > 0.0) && bad == 0) bad = 1 + k;
+      if (!(p > kPivotFloor * norm2[k]) && bad == 0) bad = 1 + k;
       S[k][k] = p > 0.0 ? sqrt(p) : 1.0;
     }
     __syncthreads();
@@ -164,7 +167,6 @@ constexpr int kClusterCtas = 8;
 // Entries per CTA up to which one cluster beats the grid (cycles, cluster / grid, at twice that size: 51k / 45k at rank 16,
 // 77k / 60k at rank 32, 121k / 116k at rank 64; the grid pays four barriers of 3k and two more reductions).
 constexpr int kClusterEntries = 4096;
-constexpr double kPivotFloor = 1e-14;   // a pivot below this share of its column's norm is rounding error: the columns are dependent
 constexpr long long kBarrierLimit = 4000000000ll;   // cycles, about 2 s: a barrier that waits longer gives up
 
 struct BasisArgs {

@@ -1,0 +1,106 @@
+"""The kernels that are chosen by size, type and row length, at the sizes where they can go wrong (needs a B200):
+edges of tiles and octets in the tile kernel, low ranks on the tensor-core kernels, more items than blocks, bases on
+either side of the cluster and grid launches.  Every call against the oracle, with the tolerances of helpers.py."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2601_12917_b200 import synth, zgr
+
+from helpers import Pair
+
+pytestmark = pytest.mark.gpu
+
+
+# Octets straddle row ends when the row length is no multiple of eight: lengths below, at and above one octet, one strip of
+# 128 columns and its overlap of 16, row counts around a warp's 32 and a tile's 128 rows, every contraction width.
+@pytest.mark.parametrize("dtype,bits", [("f32", 32), ("f32", 16), ("bf16", 16), ("f16", 32)])
+@pytest.mark.parametrize("rows,cols,rank", [(5, 3, 2), (33, 7, 16), (128, 9, 4), (31, 127, 17), (129, 129, 9), (127, 137, 33), (257, 150, 64), (300, 1285, 16),
+                                            (64, 263, 1)])
+def test_rows_that_are_no_multiple_of_eight(rows, cols, rank, dtype, bits):
+    p = Pair([(rows, cols), (1, 37)], [rank, 0], dtype, bits=bits, seed=rows + cols)
+    p.lib.profile(True)
+    reports = p.step(seed=17, lp=2.4, lm=1.7, lr=1e-4)
+    assert {k["path"] for k in p.lib.profile_read()} == {"generic", "iso"}
+    assert all(rep["moved"] > 0.3 for call in reports[:2] for rep in call)
+    assert p.lib.device_status() == 0
+
+
+# fp32 with rank above 8 in whole octets: one short strip, exact tiles, ragged last rows and strip; several tensors, so that
+# a block works on items of different tensors and widths.
+@pytest.mark.parametrize("bits", [16, 32])
+@pytest.mark.parametrize("shapes,ranks", [([(40, 8), (1, 9)], [9, 0]), ([(128, 128), (1, 9)], [16, 0]), ([(130, 264), (385, 136), (1, 9)], [32, 24, 0]),
+                                          ([(200, 520), (96, 72), (1, 9)], [64, 40, 0])])
+def test_fp32_above_rank_8(shapes, ranks, bits):
+    p = Pair(shapes, ranks, "f32", bits=bits, seed=5)
+    p.step(seed=3, lp=1.8, lm=2.3, lr=1e-4)
+    assert p.lib.device_status() == 0
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_tile_kernel_norms_codes_and_several_seeds(dtype):
+    shapes, ranks = [(150, 203), (70, 136), (1, 25)], [20, 12, 0]
+    p = Pair(shapes, ranks, dtype, bits=16, seed=8, stats=True, alpha=0.4)
+    G = oracle.coeffs(9, 0, 16, 20, 203)
+    q, sc, ze = oracle.dtc_quantise_int4(G)
+    p.set_dtc(0, q, sc, ze, bits=4)
+    p.step(seed=31, lp=2.2, lm=1.9, lr=1e-4)
+    got = p.lib.get_stats(31)
+    for l in range(3):
+        np.testing.assert_allclose(got[l], oracle.stats_tensor(p.oracle_tensor(l), 31, l, 16, p.a, p.b), rtol=2e-5, atol=1e-9)
+    p.lib.enable_stats(False)
+    seeds, lp, lm = [41, 42, 43], [2.1, 1.6, 2.4], [1.9, 2.0, 1.8]
+    coeffs = [oracle.update_coefficient(0.0, a, b, p.eps, 1e-4) for a, b in zip(lp, lm)]
+    p.call_and_check_multi(seeds, coeffs, lambda: p.lib.restore_update_multi(seeds, lp, lm, 1e-4), "three seeds")
+
+
+# Low ranks: sets of 2^21 weights and more leave the CUDA-core kernel (narrow and ragged last strips of it are in the parity tests).
+@pytest.mark.parametrize("dtype,path", [("bf16", "umma"), ("f16", "umma"), ("f32", "fma")])
+@pytest.mark.parametrize("rank", [1, 4, 8])
+def test_low_rank_sets_of_some_size(dtype, path, rank):
+    p = Pair([(1030, 2056), (1, 40), (140, 72)], [rank, 0, rank], dtype, bits=16, seed=2)
+    p.lib.profile(True)
+    p.step(seed=6, lp=2.0, lm=1.7, lr=1e-4)
+    assert {k["path"]: k["kpad"] for k in p.lib.profile_read()} == {path: 16, "iso": 0}
+    assert p.lib.device_status() == 0
+
+
+# Strips of the CUDA-core kernel of at most 32, 64 and 128 columns: 8, 4 and 2 rows per warp.
+@pytest.mark.parametrize("cols", [8, 32, 40, 64, 72, 128, 136, 392])
+def test_narrow_strips(cols):
+    p = Pair([(77, cols), (9, cols), (1, 8)], [8, 3, 0], "f32", bits=32, seed=cols)
+    p.step(seed=12, lp=2.0, lm=1.6, lr=1e-4)
+
+
+# More items than resident blocks: the item counter is used and put back to zero (three sweeps of one context in a row).
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_isotropic_sweeps_with_more_items_than_blocks(dtype):
+    p = Pair([(1201, 2569), (3, 5)], [0, 0], dtype, bits=16, seed=4, alpha=1.0)
+    p.step(seed=8, lp=2.3, lm=1.6, lr=1e-4)
+    p.step(seed=9, lp=1.9, lm=2.2, lr=1e-4)
+
+
+# 4096 entries per block of a cluster, then one block per SM; ranks that are padded; a short last block.  The last two
+# exceed the shared memory of the whole chip and take the three-kernel path.
+@pytest.mark.parametrize("rows,r", [(1, 1), (16, 16), (2048, 16), (2049, 16), (1025, 17), (513, 33), (9000, 64), (20001, 5), (60000, 64), (230000, 2)])
+def test_basis_on_either_side_of_the_launch_shapes(rows, r):
+    w = torch.zeros(rows, 8, device="cuda", dtype=torch.float32)
+    z = zgr.Zgr([w], [torch.zeros(rows, r, device="cuda")], 0.5, 1e-3)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(rows)
+    A = torch.randn(rows, r, generator=gen, device="cuda") * torch.logspace(0, -3, r, device="cuda")
+    for _ in range(2):                                     # the barrier counter is back at zero for the second call
+        z.build_subspace(0, A.contiguous())
+    U = z._keep[1][0].double()
+    assert (U.T @ U - torch.eye(r, device="cuda", dtype=torch.float64)).abs().max() <= 1e-6
+    Q, R = torch.linalg.qr(A.double())
+    Q = Q * torch.sign(torch.diagonal(R))
+    assert (U - Q).abs().max() <= 1e-5
+    if r > 1:                                              # dependent columns are refused whatever the launch, and nothing is written
+        B = A.clone()
+        B[:, r - 1] = B[:, 0]
+        with pytest.raises(zgr.ZgrError) as e:
+            z.build_subspace(0, B.contiguous())
+        assert e.value.code == zgr.EINVAL
+        assert torch.equal(z._keep[1][0].double(), U)
