@@ -28,6 +28,8 @@ struct Group {
   KernelChoice kc;
   std::vector<WorkItem> items;
   WorkItem* d_items = nullptr;
+  std::vector<int32_t> starts;                            // small tensor-core groups: first item of every CTA's share, and the end (else empty)
+  int32_t* d_starts = nullptr;
   int grid = 0;
   int64_t elements = 0;                                   // weights covered by one launch
   double* d_item_stats = nullptr;                         // kStatSlots x 3 doubles per item (norm bookkeeping), allocated on first use
@@ -215,6 +217,47 @@ void cut_tensor(const TensorDesc& t, int l, int strip, int row_step, int64_t nro
   }
 }
 
+// Small sets on the tensor-core kernels: the strips, one after the other, are cut into one contiguous share per CTA, all shares
+// costing the same (in units of a 128 x 128 tile: the tiles, `strip_cost` times the rank for every 128 columns of a strip
+// begun, `item_cost` for every item begun).  A CTA then builds one or two strips instead of one per item.  Returns the cost of a share.
+double share_out(const std::vector<TensorDesc>& descs, const std::vector<Member>& members, int strip_cols, int sm_count, double strip_cost, double item_cost,
+                 std::vector<WorkItem>& items, std::vector<int32_t>& starts) {
+  const auto fill = [&](double share, bool emit) -> int {
+    int cta = 0;
+    double room = share;
+    if (emit) starts.assign(1, 0);
+    for (const Member& m : members) {
+      const TensorDesc& t = descs[m.tensor];
+      const int64_t blocks = (t.rows + 127) / 128;
+      for (int64_t c0 = 0; c0 < t.cols; c0 += strip_cols) {
+        const int ncols = static_cast<int>(std::min<int64_t>(strip_cols, t.cols - c0));
+        const double wide = (ncols + 127) / 128, begin = strip_cost * t.rank * wide + item_cost;
+        for (int64_t at = 0, take; at < blocks; at += take) {
+          if (room < begin + wide && room < share) {
+            ++cta;
+            room = share;
+            if (emit) starts.push_back(static_cast<int32_t>(items.size()));
+          }
+          take = std::min<int64_t>(std::max<int64_t>(static_cast<int64_t>((room - begin) / wide + 1e-9), 1), blocks - at);
+          room -= begin + wide * static_cast<double>(take);
+          if (emit) items.push_back(WorkItem{m.tensor, ncols, 128 * at, std::min<int64_t>(128 * take, t.rows - 128 * at), c0});
+        }
+      }
+    }
+    if (emit) starts.push_back(static_cast<int32_t>(items.size()));
+    return cta + 1;
+  };
+  double low = 0.0, high = 1.0;
+  while (fill(high, false) > sm_count) high *= 2.0;
+  for (int i = 0; i < 20; ++i) {
+    const double mid = 0.5 * (low + high);
+    (fill(mid, false) <= sm_count ? high : low) = mid;
+  }
+  items.clear();
+  fill(high, true);
+  return high;
+}
+
 // Work items of one group.  An item is a strip of columns x a range of rows; it costs its tiles and, once, its coefficient
 // strip, so few tall items are cheap but divide badly over the SMs.  `target`: elements per item for about 16 rounds.
 void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>& members, int sm_count, int64_t target, Group& g) {
@@ -232,84 +275,72 @@ void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>&
     return;
   }
   int64_t tiles = 0;
-  if (tile) {
-    // Handed out by a counter to one CTA per SM.  Tall items are cheap (an item costs its 128 x 128 tiles and, per 512 octets of
-    // its strip, 0.2 to 0.6 of a tile: fp32 rank 32 took 451 us a sweep in items of one tile, 344 in items of eight), small ones
-    // finish evenly: the height for the first two thirds of the work and that for the last third are those that the list
-    // scheduling of the items, replayed here, ends with first.  Half of a last item is added, because the tiles do not take
-    // equally long in fact (119 M bf16 weights in rows of 1234: 565 us a step with 8 and 8 tiles, 536 with 8 and 2).  Below a
-    // dozen tiles per SM one height serves all (12.5 M fp32 weights, rank 32: 522 us with a smaller second height, 400 without).
-    for (const Member& m : members) tiles += ((descs[m.tensor].rows + 127) / 128) * ((descs[m.tensor].cols + 127) / 128);
-    const double item_cost = 0.15 + (0.2 + 0.2 * g.kc.precise + (g.kc.precise && g.kc.bits == 32 ? 0.2 : 0.0)) * ((19 * g.kc.kpad + 511) / 512) +
-                             (g.kc.kpad == 64 ? 0.3 : 0.0);
-    const bool few = tiles < 12 * static_cast<int64_t>(sm_count);
-    double best = 0.0;
-    std::vector<WorkItem> trial;
-    std::vector<double> dealt(static_cast<size_t>(sm_count));
-    for (int64_t big : {16, 12, 8, 6, 4, 3, 2, 1})
-      for (int64_t small : {big, std::max<int64_t>(big / 4, 1)}) {
-        if (few && small != big) continue;
-        if (tiles >= 64 * static_cast<int64_t>(sm_count) && big != 8 && big != 4) continue;
-        if (best > 0.0 && (small == big ? tiles / big > 40 * static_cast<int64_t>(sm_count) : big == 1)) continue;
-        trial.clear();
-        int64_t done = 0;
-        for (const Member& m : members) {
-          cut_tensor(descs[m.tensor], m.tensor, m.strip, m.row_step, by_rows, 128 * (3 * done < 2 * tiles ? big : small), trial);
-          done += ((descs[m.tensor].rows + 127) / 128) * ((descs[m.tensor].cols + 127) / 128);
-        }
-        std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
-        double end = 0.0;
-        for (const WorkItem& w : trial) {
-          double at = 0.0;
-          if (free_at.size() >= static_cast<size_t>(sm_count)) {
-            at = free_at.top();
-            free_at.pop();
-          }
-          at += static_cast<double>((w.nrows_or_count + 127) / 128) + item_cost;
-          free_at.push(at);
-          end = std::max(end, at);
-        }
-        if (!few) end += 0.5 * (static_cast<double>(small) + item_cost);
-        if (tiles >= 64 * static_cast<int64_t>(sm_count)) {
-          // long sweeps: also even when dealt out in turn, so that neither the model nor the counter has to be right
-          std::fill(dealt.begin(), dealt.end(), 0.0);
-          for (size_t i = 0; i < trial.size(); ++i) dealt[i % dealt.size()] += static_cast<double>(trial[i].nrows_or_count) * trial[i].ncols;
-          const double mean = std::accumulate(dealt.begin(), dealt.end(), 0.0) / static_cast<double>(dealt.size());
-          if (*std::max_element(dealt.begin(), dealt.end()) > 1.025 * mean) end *= 2.0;
-        }
-        if (best == 0.0 || end < best) {
-          best = end;
-          g.items = trial;
-        }
+  for (const Member& m : members) tiles += ((descs[m.tensor].rows + 127) / 128) * ((descs[m.tensor].cols + 127) / 128);
+  const int64_t sms = sm_count;
+  if (tile ? tiles < 12 * sms : g.kc.path == PATH_UMMA && tiles < 24 * sms) {
+    // per 128 columns and rank about a hundredth of a tile for the strip, twice that for fp32 (anything from 1/60 to 1/200 gives the
+    // same times); an item has a pipeline to fill, which the tile kernel does ahead where two strips fit
+    const double strip_cost = g.kc.precise ? 0.02 : 0.01;
+    const double item_cost = tile && g.kc.kpad < 64 ? 0.3 : 0.7;
+    const int widest = members.empty() ? 128 : members[0].strip;
+    double best = share_out(descs, members, widest, sm_count, strip_cost, item_cost, g.items, g.starts);
+    if (widest > 128) {
+      std::vector<WorkItem> items;
+      std::vector<int32_t> starts;
+      if (share_out(descs, members, 128, sm_count, strip_cost, item_cost, items, starts) < best) {
+        g.items.swap(items);
+        g.starts.swap(starts);
       }
+    }
     return;
   }
-  for (const Member& m : members) tiles += ((descs[m.tensor].rows + 127) / 128) * ((descs[m.tensor].cols + 127) / 128);
-  if (g.kc.path != PATH_UMMA || tiles >= 24 * static_cast<int64_t>(sm_count)) {
+  if (!tile) {
     for (const Member& m : members)
       cut_tensor(descs[m.tensor], m.tensor, m.strip, m.row_step, by_elements, g.kc.path == PATH_UMMA ? 2 * target : target, g.items);
     return;
   }
-  // The TMA-staged kernel deals its items out in a fixed round-robin over one CTA per SM.  On sets of fewer than two dozen
-  // tiles per SM the item shape is the one whose busiest CTA has the least to do, in units of a 128 x 128 tile: a strip costs
-  // about kpad/50 tiles (coefficients generated, split and written with little to overlap) and an item 0.7 for filling its
-  // pipeline.
-  const double strip_cost = g.kc.kpad / 50.0, item_cost = 0.7;
+  // Handed out by a counter to one CTA per SM.  Tall items are cheap (an item costs its 128 x 128 tiles and, per 512 octets of
+  // its strip, 0.2 to 0.6 of a tile: fp32 rank 32 took 451 us a sweep in items of one tile, 344 in items of eight), small ones
+  // finish evenly: the height for the first two thirds of the work and that for the last third are those that the list
+  // scheduling of the items, replayed here, ends with first.  Half of a last item is added, because the tiles do not take
+  // equally long in fact (119 M bf16 weights in rows of 1234: 565 us a step with 8 and 8 tiles, 536 with 8 and 2).
+  const double item_cost = 0.15 + (0.2 + 0.2 * g.kc.precise + (g.kc.precise && g.kc.bits == 32 ? 0.2 : 0.0)) * ((19 * g.kc.kpad + 511) / 512) +
+                           (g.kc.kpad == 64 ? 0.3 : 0.0);
   double best = 0.0;
   std::vector<WorkItem> trial;
-  for (int narrow = 0; narrow < (members.empty() || members[0].strip <= 128 ? 1 : 2); ++narrow)
-    for (int64_t rows = 128; rows <= 8192; rows *= 2) {
-      if (tiles / (rows / 128) < sm_count / 2 && best > 0.0) break;
+  std::vector<double> dealt(static_cast<size_t>(sm_count));
+  for (int64_t big : {16, 12, 8, 6, 4, 3, 2, 1})
+    for (int64_t small : {big, std::max<int64_t>(big / 4, 1)}) {
+      if (tiles >= 64 * sms && big != 8 && big != 4) continue;
+      if (best > 0.0 && (small == big ? tiles / big > 40 * sms : big == 1)) continue;
       trial.clear();
-      for (const Member& m : members) cut_tensor(descs[m.tensor], m.tensor, narrow ? 128 : m.strip, m.row_step, by_rows, rows, trial);
-      std::vector<double> busy(static_cast<size_t>(sm_count), 0.0);
-      for (size_t i = 0; i < trial.size(); ++i) {
-        const double wide = (trial[i].ncols + 127) / 128;
-        busy[i % busy.size()] += wide * (static_cast<double>((trial[i].nrows_or_count + 127) / 128) + strip_cost) + item_cost;
+      int64_t done = 0;
+      for (const Member& m : members) {
+        cut_tensor(descs[m.tensor], m.tensor, m.strip, m.row_step, by_rows, 128 * (3 * done < 2 * tiles ? big : small), trial);
+        done += ((descs[m.tensor].rows + 127) / 128) * ((descs[m.tensor].cols + 127) / 128);
       }
-      const double most = *std::max_element(busy.begin(), busy.end());
-      if (best == 0.0 || most < best) {
-        best = most;
+      std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
+      double end = 0.0;
+      for (const WorkItem& w : trial) {
+        double at = 0.0;
+        if (free_at.size() >= static_cast<size_t>(sm_count)) {
+          at = free_at.top();
+          free_at.pop();
+        }
+        at += static_cast<double>((w.nrows_or_count + 127) / 128) + item_cost;
+        free_at.push(at);
+        end = std::max(end, at);
+      }
+      end += 0.5 * (static_cast<double>(small) + item_cost);
+      if (tiles >= 64 * sms) {
+        // long sweeps: also even when dealt out in turn, so that neither the model nor the counter has to be right
+        std::fill(dealt.begin(), dealt.end(), 0.0);
+        for (size_t i = 0; i < trial.size(); ++i) dealt[i % dealt.size()] += static_cast<double>(trial[i].nrows_or_count) * trial[i].ncols;
+        const double mean = std::accumulate(dealt.begin(), dealt.end(), 0.0) / static_cast<double>(dealt.size());
+        if (*std::max_element(dealt.begin(), dealt.end()) > 1.025 * mean) end *= 2.0;
+      }
+      if (best == 0.0 || end < best) {
+        best = end;
         g.items = trial;
       }
     }
@@ -390,7 +421,8 @@ void plan(const std::vector<TensorDesc>& descs, const std::vector<int>& which, b
     g.elements = 0;
     for (const WorkItem& w : g.items) g.elements += g.kc.path == PATH_ISO ? w.nrows_or_count : w.nrows_or_count * w.ncols;
   }
-  for (Group& g : out) g.grid = static_cast<int>(std::min<int64_t>(static_cast<int64_t>(g.items.size()), static_cast<int64_t>(sm_count) * blocks_per_sm(g.kc)));
+  for (Group& g : out)
+    g.grid = !g.starts.empty() ? static_cast<int>(g.starts.size()) - 1 : static_cast<int>(std::min<int64_t>(static_cast<int64_t>(g.items.size()), static_cast<int64_t>(sm_count) * blocks_per_sm(g.kc)));
   // tensors were visited in ascending order, so each tensor's items are contiguous within its group
   for (Group& g : out) {
     g.first_item.assign(descs.size() + 1, static_cast<int32_t>(g.items.size()));
@@ -425,6 +457,11 @@ int upload_groups(zgr_ctx* ctx, std::vector<Group>& groups) {
     if (rc != ZGR_OK) return rc;
     rc = check(ctx, cudaMemcpy(g.d_items, g.items.data(), g.items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice));
     if (rc != ZGR_OK) return rc;
+    if (!g.starts.empty()) {
+      rc = dev_alloc(ctx, &g.d_starts, g.starts.size());
+      if (rc == ZGR_OK) rc = check(ctx, cudaMemcpy(g.d_starts, g.starts.data(), g.starts.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+      if (rc != ZGR_OK) return rc;
+    }
     if (g.kc.path == PATH_FMA || g.kc.path == PATH_ISO || is_tile(g.kc)) {
       rc = dev_alloc(ctx, &g.d_sched, 2);
       if (rc != ZGR_OK) return rc;
@@ -470,7 +507,9 @@ int sweep(zgr_ctx* ctx, std::vector<Group>& groups, const TensorDesc* d_descs, i
       p.n_items = b1 - b0;
       p.item_base = b0;
     }
-    const int grid = static_cast<int>(std::min<int64_t>(p.n_items, static_cast<int64_t>(ctx->sm_count) * blocks_per_sm(g.kc, n > 1, p.item_stats != nullptr)));
+    p.starts = t1 >= 0 ? nullptr : g.d_starts;
+    const int grid = p.starts ? g.grid
+                              : static_cast<int>(std::min<int64_t>(p.n_items, static_cast<int64_t>(ctx->sm_count) * blocks_per_sm(g.kc, n > 1, p.item_stats != nullptr)));
     p.late = first ? 0 : 1;
     first = false;
     cudaEvent_t e0 = nullptr, e1 = nullptr;

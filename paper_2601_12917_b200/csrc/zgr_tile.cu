@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  dependency_begin(p);
+  if (warp == 1) dependency_begin(p);     // (warp 0: after the first item is out; the epilogue warps: after the first strip)
 
   // All roles walk the same sequence of (item, row tile) pairs; t counts tiles over the life of the CTA.
   if (warp == 0) {
@@ -244,15 +244,19 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
     if (elect_one()) {
       int t = 0;
       bool ok = true;
-      int it = blockIdx.x;
+      int it = p.starts ? p.starts[blockIdx.x] : static_cast<int>(blockIdx.x);
+      const int share_end = p.starts ? p.starts[blockIdx.x + 1] : 0;
       for (int n = 0; ok; ++n) {
         if (n >= kRing && !mbar_wait<true>(BAR_ITEM_READ(n % kRing), ((n / kRing) - 1) & 1, abort_flag, error, 20)) break;
         ring[n % kRing] = it;
         mbar_arrive(BAR_ITEM(n % kRing));
+        if (n == 0) dependency_begin(p);
         if (it >= p.n_items) break;
         // the next item (as in ItemFeed of the CUDA-core kernels: one fetch beyond the end per CTA, the last one resets)
         int after = p.n_items;
-        if (p.n_items > static_cast<int>(gridDim.x)) {
+        if (p.starts) {
+          if (it + 1 < share_end) after = it + 1;
+        } else if (p.n_items > static_cast<int>(gridDim.x)) {
           const int f = atomicAdd(p.sched, 1);
           if (f == p.n_items - 1) *p.sched = 0;
           after = f + static_cast<int>(gridDim.x);
@@ -340,7 +344,11 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
       return it;
     };
     int it = take(0);
+    // the first strip is made of the seed alone, unless codes are delivered for it, which may come from earlier work in the stream
+    const bool codes = it < p.n_items && p.tensors[p.items[it].tensor].q != nullptr;
+    if (codes) dependency_begin(p);
     if (it < p.n_items) strip_for(it, 0);
+    if (!codes) dependency_begin(p);
     for (int it_next; it < p.n_items && ok; it = it_next, ++item_no) {
       it_next = p.n_items;
       const WorkItem w = p.items[it];

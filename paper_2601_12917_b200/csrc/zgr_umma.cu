@@ -235,7 +235,10 @@ __global__ void __launch_bounds__(UmmaCfg<KP>::THREADS, 1) sweep_umma_kernel(con
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  dependency_begin(p);
+  if (warp < 2) dependency_begin(p);      // (the epilogue warps: after the first strip, which is made of the seed alone)
+  // this CTA's items: a contiguous share, or every gridDim.x-th one
+  const int it_first = p.starts ? p.starts[blockIdx.x] : static_cast<int>(blockIdx.x);
+  const int it_end = p.starts ? p.starts[blockIdx.x + 1] : p.n_items, it_step = p.starts ? 1 : static_cast<int>(gridDim.x);
 
   // The three roles walk the same sequence of (item, row block, tile) triples; t counts tiles and
   // rb counts row blocks over the whole life of the CTA, which fixes every ring slot and phase.
@@ -252,7 +255,7 @@ __global__ void __launch_bounds__(UmmaCfg<KP>::THREADS, 1) sweep_umma_kernel(con
         for (int c = 0; c * 64 < o.ncols; ++c) tma_store_2d(tm, o.col0 + 64 * c, o.row0, src + c * 16384);
         tma_commit();
       };
-      for (int it = blockIdx.x; it < p.n_items && ok; it += gridDim.x) {
+      for (int it = it_first; it < it_end && ok; it += it_step) {
         const WorkItem w = p.items[it];
         const CUtensorMap* tm = tmaps + 3 * w.tensor;
         const int row_end = static_cast<int>(w.row0_or_e0 + w.nrows_or_count);
@@ -318,7 +321,7 @@ __global__ void __launch_bounds__(UmmaCfg<KP>::THREADS, 1) sweep_umma_kernel(con
       const uint64_t desc_g0 = make_desc(smem_u32(g_base), ROWB);
       int t = 0, rb = 0, item_no = 0;
       bool ok = true;
-      for (int it = blockIdx.x; it < p.n_items && ok; it += gridDim.x, ++item_no) {
+      for (int it = it_first; it < it_end && ok; it += it_step, ++item_no) {
         const WorkItem w = p.items[it];
         const int sh = acc_shift(p.tensors[w.tensor], p);
         if (!mbar_wait<true>(BAR_G, item_no & 1, abort_flag, error, 3)) break;
@@ -401,7 +404,7 @@ __global__ void __launch_bounds__(UmmaCfg<KP>::THREADS, 1) sweep_umma_kernel(con
     const uint32_t g_s32 = smem_u32(g_base);
     int t = 0, item_no = 0;
     bool ok = true;
-    for (int it = blockIdx.x; it < p.n_items && ok; it += gridDim.x, ++item_no) {
+    for (int it = it_first; it < it_end && ok; it += it_step, ++item_no) {
       const WorkItem w = p.items[it];
       const TensorDesc& td = p.tensors[w.tensor];
       const uint32_t tid = static_cast<uint32_t>(td.id);
@@ -417,6 +420,8 @@ __global__ void __launch_bounds__(UmmaCfg<KP>::THREADS, 1) sweep_umma_kernel(con
         const int tp = t - 1;
         if (!mbar_wait<false>(BAR_ACC_FULL(tp % NACC), (tp / NACC) & 1, abort_flag, error, 11)) break;
       }
+      // (codes that earlier work in the stream delivers may only be read behind it)
+      if (item_no == 0 && td.q != nullptr) dependency_begin(p);
       // ---- coefficient strips c b G -> K-major hi/lo operands, one per tile of a row block ----
       for (int idx = et; idx < (KP / 2) * (NSUB * NS / 8); idx += kEpiWarps * 32) {
         // consecutive lanes take consecutive pairs of rows k of the same columns: their 32-bit stores below then
@@ -452,6 +457,7 @@ __global__ void __launch_bounds__(UmmaCfg<KP>::THREADS, 1) sweep_umma_kernel(con
       fence_proxy_async();
       __syncwarp();
       if (lane == 0) mbar_arrive(BAR_G);
+      if (item_no == 0 && td.q == nullptr) dependency_begin(p);
       // The epilogue warps of a scheduler run the same instruction stream from the same starting
       // point: first the integer rounds of the generator, then the special-function half of the
       // transform.  Holding every other column group back once per item puts half of each scheduler's
