@@ -312,7 +312,7 @@ void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>&
   for (int64_t big : {16, 12, 8, 6, 4, 3, 2, 1})
     for (int64_t small : {big, std::max<int64_t>(big / 4, 1)}) {
       if (tiles >= 64 * sms && big != 8 && big != 4) continue;
-      if (best > 0.0 && (small == big ? tiles / big > 40 * sms : big == 1)) continue;
+      if (best > 0.0 && (small == big ? tiles / big > 16 * sms : tiles / big > 10 * sms || big == 1)) continue;
       trial.clear();
       int64_t done = 0;
       for (const Member& m : members) {
@@ -383,9 +383,9 @@ void plan(const std::vector<TensorDesc>& descs, const std::vector<int>& which, b
     if (!guided) {
       Group& g = group_for(PATH_ISO, t.dtype, 0);
       const int64_t n = t.rows * t.cols;
-      // about five items per resident CTA (handed out by a counter), the larger the better for the loads in flight: 405 M bf16
+      // about three items per resident CTA (handed out by a counter), the larger the better for the loads in flight: 405 M bf16
       // weights take 977 us in items of 8192 elements, 905 in 32768, 890 in 65536
-      const int64_t chunk = std::min<int64_t>(std::max<int64_t>(total / (static_cast<int64_t>(sm_count) * 8 * 5) / 2048 * 2048, 2048), 65536);
+      const int64_t chunk = std::min<int64_t>(std::max<int64_t>(total / (static_cast<int64_t>(sm_count) * 8 * 3) / 2048 * 2048, 2048), 65536);
       for (int64_t e0 = 0; e0 < n; e0 += chunk)
         g.items.push_back(WorkItem{l, aligned ? 1 : 0, e0, std::min(chunk, n - e0), 0});
       continue;
@@ -1396,13 +1396,18 @@ int zgr_build_subspace(zgr_ctx* ctx, int32_t tensor, const float* grads, int32_t
   int rc;
   if (subspace_fused(td.rows, td.rank, ctx->sm_count)) {
     const int32_t job = ctx->split_job[static_cast<size_t>(tensor)];
-    *ctx->h_status = -1;
+    constexpr int kPending = INT32_MIN;
+    volatile int* const h_status = ctx->h_status;
+    *h_status = kPending;
     rc = check(ctx, launch_basis_fused(A, td.rows, td.rank, U, job >= 0 ? &ctx->split_jobs[static_cast<size_t>(job)] : nullptr, ctx->d_qr, ctx->h_status,
                                        ctx->sm_count, st));
-    if (rc == ZGR_OK) rc = check(ctx, cudaStreamSynchronize(st));
+    // The kernel writes the word when everything it does is visible, some microseconds before the driver would report the
+    // stream idle; if it has not come after a while (a long queue, or a failed launch) the driver is asked.
+    for (int spin = 0; rc == ZGR_OK && *h_status == kPending && spin < 1000000; ++spin) {}
+    if (rc == ZGR_OK && *h_status == kPending) rc = check(ctx, cudaStreamSynchronize(st));
     if (rc != ZGR_OK) return rc;
     ctx->launches++;
-    const int status = *static_cast<volatile int*>(ctx->h_status);
+    const int status = *h_status;
     if (status < 0) return check(ctx, cudaErrorLaunchTimeout);   // a barrier gave up: the basis may be partly written
     if (status > 0) return ZGR_EINVAL;                            // linearly dependent directions: nothing was written
     return td.Ufrag != nullptr && !td.umma ? make_fragments(ctx, td, st) : ZGR_OK;

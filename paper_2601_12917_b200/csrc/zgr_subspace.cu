@@ -15,8 +15,8 @@
 //
 // One launch does all of it (basis_kernel): every CTA keeps its rows in shared memory as doubles through both passes, the
 // partial Gram matrices meet in global memory (L2) between barriers, and each CTA factors the r x r sum for itself, since
-// that is cheaper than another barrier.  Up to about a thousand rows per CTA the grid is a single cluster of 8 CTAs, whose
-// barrier is a hardware one and whose 8 partials every CTA adds up directly; larger inputs use one CTA per SM, launched
+// that is cheaper than another barrier.  Up to about a thousand rows per CTA the grid is a single cluster of 8 or 16 CTAs, whose
+// barrier is a hardware one and whose partials every CTA adds up directly; larger inputs use one CTA per SM, launched
 // cooperatively, with a counter barrier and the sum of the partials spread over the grid.  The job is bound by latency (a
 // 2048 x 16 input is 131 KB): the six launches, the memset and the copies of the status that it took before were 95 us a
 // tensor.  The last phase also writes the tensor-core operand copies of the new basis.
@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(kQrThreads) apply_kernel(const void* __restric
 // ---------------------------------------------------------------------------------------------
 // the whole construction in one launch
 // ---------------------------------------------------------------------------------------------
-constexpr int kClusterCtas = 8;
+__host__ __device__ constexpr int cluster_ctas(int rc) { return rc == 16 ? 16 : 8; }
 // Entries per CTA up to which one cluster beats the grid (cycles, cluster / grid, at twice that size: 51k / 45k at rank 16,
 // 77k / 60k at rank 32, 121k / 116k at rank 64; the grid pays four barriers of 3k and two more reductions).
 constexpr int kClusterEntries = 4096;
@@ -176,7 +176,7 @@ struct BasisArgs {
   double* partials;     // one RC x RC matrix per CTA (cluster launches: and pass)
   double* sum;          // RC x RC (grid launches)
   unsigned* counter;    // grid barrier: arrivals, exits; both zero between launches
-  int* status;          // host-mapped: 0, 1 + dependent column, or -1 if a barrier gave up
+  volatile int* status; // host-mapped: 0, 1 + dependent column, or -1 if a barrier gave up
   int64_t rows;
   int r;
   int rows_per_cta;
@@ -218,16 +218,17 @@ __device__ __forceinline__ bool basis_barrier(unsigned* counter, int index) {
 
 // RC = r rounded up to 16, 32 or 64.
 //
-// Gram matrix: four groups of 64 threads take rows in turn; thread (ui, uj) of a group owns the entries (ui + 8 x, uj + 8 y),
+// Gram matrix: groups of 64 threads take rows in turn; thread (ui, uj) of a group owns the entries (ui + 8 x, uj + 8 y),
 // x <= y, which needs RC/4 shared-memory reads per (RC/8)^2 / 2 multiply-adds (one entry per thread is bound by those reads:
 // 36 cycles per row at RC = 16 against 8).  The groups' sums are added in order.
 // Factorisation: S = L D L^T and, by the same eliminations applied to the identity, M = L^-1; then R^-1 = M^T D^-1/2.
 // Thread (ti, tj) of a 16 x 16 arrangement owns the entries (ti + 16 a, tj + 16 b): a <= b of S, a >= b of M.  One barrier per
-// column; only the reciprocal of the pivot is on the chain from column to column.
+// column; only the reciprocal of the pivot is on the chain from column to column.  (512 threads at RC = 64: 73 us a call
+// instead of 58, the barriers cost more than the shorter updates save.)
 // Product X R^-1: at RC = 16 a thread takes a row, otherwise a warp eight rows, a lane four of them and the columns tj + 16 b.
 template <int RC, bool CLUSTER>
 __global__ void __launch_bounds__(kQrThreads) basis_kernel(const BasisArgs p) {
-  constexpr int NB = RC / 16, LD = RC + 1;
+  constexpr int kT = kQrThreads, NB = RC / 16, LD = RC + 1, CL = cluster_ctas(RC);
   extern __shared__ double dyn_smem[];
   double* Ms = dyn_smem;                       // RC x LD: rows of M (before that: the sum of the groups' Gram matrices)
   double* rowbuf = Ms + RC * LD;               // 2 x RC: current row of D L^T
@@ -241,7 +242,7 @@ __global__ void __launch_bounds__(kQrThreads) basis_kernel(const BasisArgs p) {
   int status = 0;
 
 #pragma unroll 8
-  for (int idx = tid; idx < nrows * RC; idx += kQrThreads) {
+  for (int idx = tid; idx < nrows * RC; idx += kT) {
     const int i = idx / RC, k = idx % RC;
     X[i * LD + k] = k < r ? static_cast<double>(p.A[(row0 + i) * r + k]) : 0.0;
   }
@@ -260,7 +261,7 @@ __global__ void __launch_bounds__(kQrThreads) basis_kernel(const BasisArgs p) {
 #pragma unroll
         for (int y = 0; y < B; ++y) acc[x][y] = 0.0;
 #pragma unroll (RC == 64 ? 1 : 4)
-      for (int i = grp; i < nrows; i += 4) {
+      for (int i = grp; i < nrows; i += kT / 64) {
         const double* row = X + i * LD;
         double u[B], v[B];
 #pragma unroll
@@ -271,7 +272,7 @@ __global__ void __launch_bounds__(kQrThreads) basis_kernel(const BasisArgs p) {
           for (int y = x; y < B; ++y) acc[x][y] = fma(u[x], v[y], acc[x][y]);
       }
 #pragma unroll 1
-      for (int g = 0; g < 4; ++g) {
+      for (int g = 0; g < kT / 64; ++g) {
         if (grp == g) {
 #pragma unroll
           for (int x = 0; x < B; ++x)
@@ -284,7 +285,7 @@ __global__ void __launch_bounds__(kQrThreads) basis_kernel(const BasisArgs p) {
         __syncthreads();
       }
       // (a cluster has one barrier per pass, so the second pass writes its own set)
-      double* out = p.partials + static_cast<int64_t>(blockIdx.x + (CLUSTER ? pass * kClusterCtas : 0)) * RC * RC;
+      double* out = p.partials + static_cast<int64_t>(blockIdx.x + (CLUSTER ? pass * CL : 0)) * RC * RC;
 #pragma unroll
       for (int a = 0; a < NB; ++a)
 #pragma unroll
@@ -302,13 +303,13 @@ __global__ void __launch_bounds__(kQrThreads) basis_kernel(const BasisArgs p) {
         for (int b = a; b < NB; ++b) {
           double v = 0.0;
 #pragma unroll
-          for (int c = 0; c < kClusterCtas; ++c)
-            v += __ldcg(p.partials + static_cast<int64_t>(c + pass * kClusterCtas) * RC * RC + (ti + 16 * a) * RC + tj + 16 * b);
+          for (int c = 0; c < CL; ++c)
+            v += __ldcg(p.partials + static_cast<int64_t>(c + pass * CL) * RC * RC + (ti + 16 * a) * RC + tj + 16 * b);
           s[a][b] = v;
         }
     } else {
       // a warp per entry, four entries at a time (entries of the blocks below the diagonal hold nothing and go unused)
-      const int lane = tid & 31, wid = blockIdx.x * (kQrThreads / 32) + (tid >> 5), warps = static_cast<int>(gridDim.x) * (kQrThreads / 32);
+      const int lane = tid & 31, wid = blockIdx.x * (kT / 32) + (tid >> 5), warps = static_cast<int>(gridDim.x) * (kT / 32);
       for (int e0 = wid; e0 < RC * RC; e0 += 4 * warps) {
         double v[4] = {0.0, 0.0, 0.0, 0.0};
         for (int c = lane; c < static_cast<int>(gridDim.x); c += 32) {
@@ -337,11 +338,13 @@ __global__ void __launch_bounds__(kQrThreads) basis_kernel(const BasisArgs p) {
     // ---- S = L D L^T, M = L^-1 ----
     double m[NB][NB];
 #pragma unroll
-    for (int a = 0; a < NB; ++a) {
+    for (int a = 0; a < NB; ++a)
 #pragma unroll
-      for (int b = 0; b <= a; ++b) m[a][b] = (a == b && ti == tj) ? 1.0 : 0.0;
-      if (ti == tj) diag[ti + 16 * a] = s[a][a];
-    }
+      for (int b = 0; b <= a; ++b) {
+        const bool on_diagonal = a == b && ti == tj;
+        m[a][b] = on_diagonal ? 1.0 : 0.0;
+        if (on_diagonal) diag[ti + 16 * a] = s[a][a];
+      }
 #pragma unroll
     for (int a = 0; a < NB; ++a) {
       const int kk_end = min(16, r - 16 * a);
@@ -376,12 +379,12 @@ __global__ void __launch_bounds__(kQrThreads) basis_kernel(const BasisArgs p) {
     __syncthreads();
     if (status != 0) break;
     if (tid < RC) inv[tid] = tid < r ? 1.0 / sqrt(inv[tid]) : 0.0;
-    for (int idx = tid; idx < (RC - r) * RC; idx += kQrThreads) Ms[(r + idx / RC) * LD + idx % RC] = 0.0;      // rank not a multiple of 16
+    for (int idx = tid; idx < (RC - r) * RC; idx += kT) Ms[(r + idx / RC) * LD + idx % RC] = 0.0;      // rank not a multiple of 16
     __syncthreads();
     // ---- X <- X R^-1 = X M^T D^-1/2 ----
     if constexpr (RC == 16) {
       // one row per thread: 136 broadcast reads and as many multiply-adds
-      for (int i = tid; i < nrows; i += kQrThreads) {
+      for (int i = tid; i < nrows; i += kT) {
         double* xr = X + i * LD;
         asm volatile("" ::: "memory");      // M stays in shared memory: hoisted out of the row loop it would fill the register file
         double x[16];
@@ -398,7 +401,7 @@ __global__ void __launch_bounds__(kQrThreads) basis_kernel(const BasisArgs p) {
     } else {
       const int warp = tid >> 5, half = (tid >> 4) & 1;
 #pragma unroll 1
-      for (int i0 = 8 * warp; i0 < nrows; i0 += kQrThreads / 4) {
+      for (int i0 = 8 * warp; i0 < nrows; i0 += kT / 4) {
         const int i1 = i0 + 4 * half;
         const double* xr[4];
         double q[4][NB];
@@ -442,7 +445,7 @@ __global__ void __launch_bounds__(kQrThreads) basis_kernel(const BasisArgs p) {
     const SplitJob& c = p.copies;
     const float scale = c.shift >= 0 ? __int_as_float((127 + c.shift) << 23) : 1.0f;
 #pragma unroll 4
-    for (int idx = tid; idx < nrows * RC; idx += kQrThreads) {
+    for (int idx = tid; idx < nrows * RC; idx += kT) {
       const int i = idx / RC, k = idx % RC;
       if (k >= r) continue;                    // (the padding of the copies is zero since zgr_init)
       const float u = static_cast<float>(X[i * LD + k]);
@@ -450,12 +453,21 @@ __global__ void __launch_bounds__(kQrThreads) basis_kernel(const BasisArgs p) {
       if (c.part[0] != nullptr) split_subspace_entry(c, (row0 + i) * c.kp + k, u, scale);
     }
   }
-  if constexpr (!CLUSTER) {
-    if (tid == 0 && atomicInc(p.counter + 1, gridDim.x - 1) == gridDim.x - 1) *p.counter = 0;
-  }
-  if (blockIdx.x == 0 && tid == 0) {
-    *p.status = status;
-    __threadfence_system();
+  // The host polls the status word: it is written once every CTA's results are visible.
+  __threadfence();
+  if constexpr (CLUSTER) {
+    basis_barrier<CLUSTER>(p.counter, 0);
+    if (blockIdx.x == 0 && tid == 0) {
+      __threadfence_system();
+      *p.status = status;
+    }
+  } else {
+    __syncthreads();
+    if (tid == 0 && atomicInc(p.counter + 1, gridDim.x - 1) == gridDim.x - 1) {
+      *p.counter = 0;
+      __threadfence_system();
+      *p.status = status;
+    }
   }
 }
 
@@ -474,16 +486,18 @@ cudaError_t launch_basis(BasisArgs p, int sm_count, cudaStream_t st, bool* serve
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const int64_t in_cluster = (p.rows + kClusterCtas - 1) / kClusterCtas;
+  constexpr int CL = cluster_ctas(RC);
+  const int64_t in_cluster = (p.rows + CL - 1) / CL;
   if (in_cluster * RC <= kClusterEntries) {
     p.rows_per_cta = static_cast<int>(in_cluster);
     const size_t smem = basis_smem<RC>(p.rows_per_cta);
-    const cudaError_t e = cudaFuncSetAttribute(basis_kernel<RC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kBasisSmemMax));
+    cudaError_t e = cudaFuncSetAttribute(basis_kernel<RC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kBasisSmemMax));
+    if (e == cudaSuccess && CL > 8) e = cudaFuncSetAttribute(basis_kernel<RC, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
-    cfg.gridDim = dim3(kClusterCtas);
+    cfg.gridDim = dim3(CL);
     cfg.dynamicSmemBytes = smem;
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = kClusterCtas;
+    attr[0].val.clusterDim.x = CL;
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     return cudaLaunchKernelEx(&cfg, basis_kernel<RC, true>, p);
   }
@@ -511,7 +525,7 @@ size_t subspace_scratch_bytes(int64_t rows, int r, int sm_count) {
   const size_t chunked = static_cast<size_t>(n_chunks) * r * r * sizeof(double) + 2 * static_cast<size_t>(r) * r * sizeof(double) +
                          static_cast<size_t>(rows) * r * sizeof(double);
   const size_t rc = r <= 16 ? 16 : (r <= 32 ? 32 : 64);
-  const size_t fused = (static_cast<size_t>(std::max(sm_count, 2 * kClusterCtas)) + 1) * rc * rc * sizeof(double);
+  const size_t fused = (static_cast<size_t>(std::max(sm_count, 32)) + 1) * rc * rc * sizeof(double);
   return 512 + (subspace_fused(rows, r, sm_count) ? fused : chunked);
 }
 
