@@ -336,19 +336,6 @@ __device__ __forceinline__ void box_muller_acc(uint32_t m1, uint32_t m2, const N
   acc1 = fmaf(rho, sin_approx(phi), acc1);
 }
 
-// The same, also adding the squared radius of the pair to rsum: (s rho cos)^2 + (s rho sin)^2 = s^2 rho^2 is the
-// argument of the square root, so the energy of the two normals costs one addition.
-__device__ __forceinline__ void box_muller_acc_rsum(uint32_t m1, uint32_t m2, const NormalScale& ns, float& acc0, float& acc1, float& rsum) {
-  const float u1 = __uint_as_float(m1) + ns.u1_off;
-  const float t2 = __uint_as_float(m2);
-  const float x = fabsf(ns.kr * lg2_approx(u1));
-  rsum += x;
-  const float rho = sqrt_approx(x);
-  const float phi = fmaf(t2, 6.28318530717958647692f, ns.phase);
-  acc0 = fmaf(rho, cos_approx(phi), acc0);
-  acc1 = fmaf(rho, sin_approx(phi), acc1);
-}
-
 // acc[0..7] += the eight scaled normals of octet number `oct` (= element index / 8, as two 32-bit
 // halves) of stream (tensor, tag 0).  Hardware-approximation transform only.
 template <int BITS>
@@ -374,10 +361,15 @@ __device__ __forceinline__ void normals8_acc(const PhiloxKeys& keys, uint32_t te
 // (the adjacent accumulators of a pair are the two halves of one operation).  Generator alone: 0.69 instead of 0.75 cycles per
 // element and scheduler with four warps each; in the TMA-staged sweep -3 % on OPT-1.3B-shaped fp16 rank 16 (3518 -> 3405 us
 // a step), -2 % on rank 64 and with 32 random bits, -0.8 % at rank 32, where the board is at its power cap.
-__device__ __forceinline__ void box_muller_acc2(uint32_t ma1, uint32_t ma2, uint32_t mb1, uint32_t mb2, const NormalScale& ns, float (&acc)[8], int at) {
+// RSUM: also adds the squared radii to rsum: (s rho cos)^2 + (s rho sin)^2 = s^2 rho^2 is the argument of the square root, so the
+// energy of the normals costs an addition per pair.
+template <bool RSUM>
+__device__ __forceinline__ void box_muller_acc2(uint32_t ma1, uint32_t ma2, uint32_t mb1, uint32_t mb2, const NormalScale& ns, float (&acc)[8], int at,
+                                                float& rsum) {
   float ua, ub, la, lb, pa, pb;
   unpack2(add2(pack2(__uint_as_float(ma1), __uint_as_float(mb1)), dup2(ns.u1_off)), ua, ub);
   unpack2(mul2(pack2(lg2_approx(ua), lg2_approx(ub)), dup2(ns.kr)), la, lb);
+  if (RSUM) rsum += fabsf(la) + fabsf(lb);
   const float ra = sqrt_approx(fabsf(la)), rb = sqrt_approx(fabsf(lb));
   unpack2(fma2(pack2(__uint_as_float(ma2), __uint_as_float(mb2)), dup2(6.28318530717958647692f), dup2(ns.phase)), pa, pb);
   unpack2(fma2(dup2(ra), pack2(cos_approx(pa), sin_approx(pa)), pack2(acc[at], acc[at + 1])), acc[at], acc[at + 1]);
@@ -386,19 +378,26 @@ __device__ __forceinline__ void box_muller_acc2(uint32_t ma1, uint32_t ma2, uint
 
 // acc[0..7] += the eight scaled normals of octet number `oct` (low word; the high word and the tensor are in `pre`, made
 // for the high word of the octet's block number: 2 oct in 32-bit mode).
-template <int BITS>
-__device__ __forceinline__ void normals8_acc_pre(const PhiloxKeys& keys, const PhiloxPre& pre, uint32_t oct_lo, const NormalScale& ns, float (&acc)[8]) {
+template <int BITS, bool RSUM>
+__device__ __forceinline__ void normals8_acc_pre_rsum(const PhiloxKeys& keys, const PhiloxPre& pre, uint32_t oct_lo, const NormalScale& ns, float (&acc)[8],
+                                                      float& rsum) {
   uint32_t x[4];
 #pragma unroll
   for (int h = 0; h < (BITS == 32 ? 2 : 1); ++h) {
     philox4x32_10_pre(BITS == 32 ? 2 * oct_lo + h : oct_lo, pre, keys, x);
     if (BITS == 32) {
-      box_muller_acc2(field23(x[0]), field23(x[1]), field23(x[2]), field23(x[3]), ns, acc, 4 * h);
+      box_muller_acc2<RSUM>(field23(x[0]), field23(x[1]), field23(x[2]), field23(x[3]), ns, acc, 4 * h, rsum);
     } else {
 #pragma unroll
-      for (int w = 0; w < 4; w += 2) box_muller_acc2(field16a(x[w]), field16b(x[w]), field16a(x[w + 1]), field16b(x[w + 1]), ns, acc, 2 * w);
+      for (int w = 0; w < 4; w += 2)
+        box_muller_acc2<RSUM>(field16a(x[w]), field16b(x[w]), field16a(x[w + 1]), field16b(x[w + 1]), ns, acc, 2 * w, rsum);
     }
   }
+}
+template <int BITS>
+__device__ __forceinline__ void normals8_acc_pre(const PhiloxKeys& keys, const PhiloxPre& pre, uint32_t oct_lo, const NormalScale& ns, float (&acc)[8]) {
+  float none = 0.0f;
+  normals8_acc_pre_rsum<BITS, false>(keys, pre, oct_lo, ns, acc, none);
 }
 
 // The same by the accurate transform.
@@ -425,26 +424,6 @@ template <int BITS, bool PRECISE>
 __device__ __forceinline__ void normals8_add(const PhiloxKeys& keys, const PhiloxPre& pre, uint32_t oct_lo, const NormalScale& ns, float (&acc)[8]) {
   if constexpr (PRECISE) normals8_acc_accurate_pre<BITS>(keys, pre, oct_lo, ns, acc);
   else normals8_acc_pre<BITS>(keys, pre, oct_lo, ns, acc);
-}
-
-// normals8_acc that also returns the energy of its eight normals (sum of their squares) in rsum.
-template <int BITS>
-__device__ __forceinline__ void normals8_acc_rsum(const PhiloxKeys& keys, uint32_t tensor, uint32_t oct_lo, uint32_t oct_hi, const NormalScale& ns,
-                                                  float (&acc)[8], float& rsum) {
-  uint32_t x[4];
-  if (BITS == 32) {
-    const uint32_t b_lo = oct_lo << 1, b_hi = (oct_hi << 1) | (oct_lo >> 31);
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      philox4x32_10(b_lo + h, b_hi, tensor, 0u, keys, x);
-      box_muller_acc_rsum(field23(x[0]), field23(x[1]), ns, acc[4 * h + 0], acc[4 * h + 1], rsum);
-      box_muller_acc_rsum(field23(x[2]), field23(x[3]), ns, acc[4 * h + 2], acc[4 * h + 3], rsum);
-    }
-  } else {
-    philox4x32_10(oct_lo, oct_hi, tensor, 0u, keys, x);
-#pragma unroll
-    for (int w = 0; w < 4; ++w) box_muller_acc_rsum(field16a(x[w]), field16b(x[w]), ns, acc[2 * w], acc[2 * w + 1], rsum);
-  }
 }
 
 // Partial sums of the norm bookkeeping of one warp for one work item: reduce over the lanes in a fixed order and

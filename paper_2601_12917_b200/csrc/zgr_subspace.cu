@@ -488,7 +488,7 @@ cudaError_t launch_basis(BasisArgs p, int sm_count, cudaStream_t st, bool* serve
   cfg.numAttrs = 1;
   constexpr int CL = cluster_ctas(RC);
   const int64_t in_cluster = (p.rows + CL - 1) / CL;
-  if (in_cluster * RC <= kClusterEntries) {
+  if (in_cluster * RC <= (RC == 64 ? 2 : 1) * kClusterEntries) {
     p.rows_per_cta = static_cast<int>(in_cluster);
     const size_t smem = basis_smem<RC>(p.rows_per_cta);
     cudaError_t e = cudaFuncSetAttribute(basis_kernel<RC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kBasisSmemMax));

@@ -477,10 +477,10 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
           }
         };
         // All octets of the warp whole and under one high counter word (nearly always): straight-line code, several octets
-        // per thread whose generator chains interleave.  Otherwise (row ends, last rows, the bookkeeping) one octet after the other.
+        // per thread whose generator chains interleave.  Otherwise (row ends, last rows) one octet after the other.
         constexpr int kShift = BITS == 32 ? 34 : 35;       // element index -> high word of its block number
         const uint32_t hi0 = static_cast<uint32_t>(static_cast<uint64_t>(e_sub) >> kShift);
-        const bool fast = !SSTATS && __all_sync(0xFFFFFFFFu, full && wrow + 24 + sub < row_end &&
+        const bool fast = __all_sync(0xFFFFFFFFu, full && wrow + 24 + sub < row_end &&
                                                                  hi0 == static_cast<uint32_t>(static_cast<uint64_t>(e_sub + 24 * cols) >> kShift));
         if (fast) {
           const PhiloxPre pre = philox_pre(hi0, tid, p.term[0].keys);
@@ -496,8 +496,31 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
               read_d(p0 + x, z[x]);
               oct[x] = static_cast<uint32_t>(static_cast<uint64_t>(e_sub + 8 * (p0 + x) * cols) >> 3);
             }
+            if constexpr (SSTATS) {
 #pragma unroll
-            for (int x = 0; x < kWide; ++x) normals8_add<BITS, PRECISE>(p.term[0].keys, pre, oct[x], p.term[0].iso, z[x]);
+              for (int x = 0; x < kWide; ++x) {
+                float d[8], f_iso = 0.0f, f_gd = 0.0f, f_z = 0.0f;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                  d[i] = z[x][i];
+                  z[x][i] = 0.0f;
+                }
+                normals8_add<BITS, PRECISE>(p.term[0].keys, pre, oct[x], p.term[0].iso, z[x]);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                  f_iso = fmaf(z[x][i], z[x][i], f_iso);
+                  f_gd = fmaf(d[i], d[i], f_gd);
+                  z[x][i] += d[i];
+                  f_z = fmaf(z[x][i], z[x][i], f_z);
+                }
+                s_iso += static_cast<double>(f_iso);
+                s_gd += static_cast<double>(f_gd);
+                s_z += static_cast<double>(f_z);
+              }
+            } else {
+#pragma unroll
+              for (int x = 0; x < kWide; ++x) normals8_add<BITS, PRECISE>(p.term[0].keys, pre, oct[x], p.term[0].iso, z[x]);
+            }
             if (MULTI) {
 #pragma unroll 1
               for (int q = 1; q < p.n_terms; ++q) {

@@ -531,7 +531,7 @@ __global__ void __launch_bounds__(UmmaCfg<KP>::THREADS, 1) sweep_umma_kernel(con
                   const float gd = acc[i] - th[i];
                   f_gd = fmaf(gd, gd, f_gd);
                 }
-                normals8_acc_rsum<BITS>(p.term[0].keys, tid, oct0_lo + static_cast<uint32_t>(o), 0u, p.term[0].iso, acc, f_iso);
+                normals8_acc_pre_rsum<BITS, true>(p.term[0].keys, pre, oct0_lo + static_cast<uint32_t>(o), p.term[0].iso, acc, f_iso);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                   const float zc = acc[i] - th[i];
