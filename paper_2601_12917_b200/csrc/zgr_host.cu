@@ -53,6 +53,11 @@ struct zgr_ctx {
   bool descs_dirty = false;
   std::vector<void*> owned;           // device allocations made by the library
   std::vector<Group> groups;          // sweep plan
+  // Small sets: the items of the CUDA-core contraction group with those of the isotropic group behind them, for one launch of the
+  // contraction kernel instead of two (not while the kernels are timed or keep the norm bookkeeping, nor layer by layer).
+  int merged_fma = -1, merged_iso = -1;
+  WorkItem* d_merged = nullptr;
+  int32_t n_merged = 0;
   std::vector<WorkItem> stats_items;  // plan of the norm kernel (tensors not served by the tcgen05 kernel)
   bool stats_planned = false;
   WorkItem* d_stats_items = nullptr;
@@ -473,6 +478,27 @@ int upload_groups(zgr_ctx* ctx, std::vector<Group>& groups) {
   return check(ctx, cudaDeviceSynchronize());
 }
 
+// The isotropic elements that may ride along: up to 2^20, a few microseconds of one launch.
+int merge_small_groups(zgr_ctx* ctx) {
+  for (size_t i = 0; i < ctx->groups.size(); ++i)
+    for (size_t j = 0; j < ctx->groups.size(); ++j) {
+      const Group &f = ctx->groups[i], &g = ctx->groups[j];
+      if (f.kc.path != PATH_FMA || is_tile(f.kc) || g.kc.path != PATH_ISO || f.kc.dtype != g.kc.dtype || f.kc.precise != g.kc.precise || g.items.empty() ||
+          f.items.empty() || g.elements > (1 << 20))
+        continue;
+      std::vector<WorkItem> items(f.items);
+      items.insert(items.end(), g.items.begin(), g.items.end());
+      int rc = dev_alloc(ctx, &ctx->d_merged, items.size());
+      if (rc == ZGR_OK) rc = check(ctx, cudaMemcpy(ctx->d_merged, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice));
+      if (rc != ZGR_OK) return rc;
+      ctx->n_merged = static_cast<int32_t>(items.size());
+      ctx->merged_fma = static_cast<int>(i);
+      ctx->merged_iso = static_cast<int>(j);
+      return ZGR_OK;
+    }
+  return ZGR_OK;
+}
+
 // One sweep  theta <- rnd(theta + sum_q c_q z(seed_q))  over the planned groups (n terms, 1 <= n <= kMaxTerms).
 // t0 <= t1 restricts the sweep to the tensors [t0, t1) (layer-wise sweeps); t1 < 0 means all of them.  tmaps: the tensor
 // maps of the first tensor of d_descs (null: the context's own).
@@ -493,12 +519,19 @@ int sweep(zgr_ctx* ctx, std::vector<Group>& groups, const TensorDesc* d_descs, i
   for (int q = 0; q < n; ++q) cb_total += std::fabs(c[q] * ctx->b);
   p.kshift = kshift_for(cb_total);
   bool first = true;     // the first kernel of the sweep waits for earlier work, the others rely on it
+  const bool merge = ctx->d_merged != nullptr && &groups == &ctx->groups && !ctx->profiling && t1 < 0 && !keep_stats;
   for (Group& g : groups) {
     if (g.items.empty()) continue;
+    const int index = static_cast<int>(&g - groups.data());
+    if (merge && index == ctx->merged_iso) continue;
     p.items = g.d_items;
     p.n_items = static_cast<int32_t>(g.items.size());
     p.item_stats = keep_stats ? g.d_item_stats : nullptr;
     p.item_base = 0;
+    if (merge && index == ctx->merged_fma) {
+      p.items = ctx->d_merged;
+      p.n_items = ctx->n_merged;
+    }
     p.sched = g.d_sched ? g.d_sched + (ctx->aux_stream != nullptr && st == ctx->aux_stream ? 1 : 0) : nullptr;
     if (t1 >= 0) {
       const int32_t b0 = g.first_item[static_cast<size_t>(t0)], b1 = g.first_item[static_cast<size_t>(t1)];
@@ -826,6 +859,7 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
     plan(ctx->descs, all, guided_on, cfg->bits_per_normal, ctx->sm_count, ctx->groups);
     rc = upload_groups(ctx, ctx->groups);
   }
+  if (rc == ZGR_OK) rc = merge_small_groups(ctx);
   if (rc == ZGR_OK) rc = dev_alloc(ctx, &ctx->d_stats, static_cast<size_t>(3 * n));
   if (rc == ZGR_OK) rc = check(ctx, cudaDeviceSynchronize());  // the subspace copies are complete
   if (rc != ZGR_OK) {

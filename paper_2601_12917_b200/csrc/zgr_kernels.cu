@@ -90,6 +90,35 @@ __device__ __forceinline__ void unpack_raw(const uint4& raw, float (&v)[8]) {
     }
   }
 }
+// The octets [first, n_oct) and the ragged end of the elements [e0, e0 + count) of one tensor, by the threads of a block.
+// Returns the sum of the squared normals (SSTATS).
+template <typename T, int BITS, bool PRECISE, bool MULTI, bool SSTATS>
+__device__ __forceinline__ double iso_elements(const SweepParams& p, T* base, uint32_t tid, int64_t e0, int64_t count, int64_t first, int64_t n_oct) {
+  double s_iso = 0.0;
+#pragma unroll 2
+  for (int64_t v = first + threadIdx.x; v < n_oct; v += kThreads) {
+    const int64_t e = e0 + 8 * v;
+    float th[8], z[8];
+    Storage<T>::load8(base + e, th);
+    iso8<BITS, PRECISE, MULTI>(p, tid, static_cast<uint64_t>(e), z);
+    if (SSTATS) {
+      float f = 0.0f;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) f = fmaf(z[i], z[i], f);
+      s_iso += static_cast<double>(f);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) th[i] += z[i];
+    Storage<T>::store8(base + e, th);
+  }
+  for (int64_t e = e0 + 8 * n_oct + threadIdx.x; e < e0 + count; e += kThreads) {
+    const float z = iso1<BITS, PRECISE, MULTI>(p, tid, static_cast<uint64_t>(e));
+    if (SSTATS) s_iso += static_cast<double>(z) * z;
+    Storage<T>::store1(base + e, Storage<T>::load1(base + e) + z);
+  }
+  return s_iso;
+}
+
 template <typename T, int BITS, bool PRECISE, bool MULTI, bool SSTATS = false>
 __global__ void __launch_bounds__(kThreads, iso_blocks_per_sm(PRECISE, MULTI, SSTATS)) sweep_iso_kernel(const __grid_constant__ SweepParams p) {
   dependency_begin(p);
@@ -102,8 +131,7 @@ __global__ void __launch_bounds__(kThreads, iso_blocks_per_sm(PRECISE, MULTI, SS
     const int64_t e0 = w.row0_or_e0, count = w.nrows_or_count;
     const int64_t n_oct = w.ncols ? count / 8 : 0;  // ncols != 0: 128-bit access is legal for this tensor
     int64_t n_oct_done = 0;
-    double s_iso = 0.0;
-    if constexpr (!PRECISE && !SSTATS) {
+    if constexpr (!PRECISE && !SSTATS && sizeof(T) == 2) {
       // the fused transform, with the fixed part of the counter kept as long as its high word does not change
       const uint64_t b0 = static_cast<uint64_t>(e0) >> (BITS == 32 ? 2 : 3);
       const uint64_t b1 = static_cast<uint64_t>(e0 + count) >> (BITS == 32 ? 2 : 3);
@@ -131,27 +159,7 @@ __global__ void __launch_bounds__(kThreads, iso_blocks_per_sm(PRECISE, MULTI, SS
         n_oct_done = n_oct;
       }
     }
-#pragma unroll 2
-    for (int64_t v = n_oct_done + threadIdx.x; v < n_oct; v += kThreads) {
-      const int64_t e = e0 + 8 * v;
-      float th[8], z[8];
-      Storage<T>::load8(base + e, th);
-      iso8<BITS, PRECISE, MULTI>(p, tid, static_cast<uint64_t>(e), z);
-      if (SSTATS) {
-        float f = 0.0f;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) f = fmaf(z[i], z[i], f);
-        s_iso += static_cast<double>(f);
-      }
-#pragma unroll
-      for (int i = 0; i < 8; ++i) th[i] += z[i];
-      Storage<T>::store8(base + e, th);
-    }
-    for (int64_t e = e0 + 8 * n_oct + threadIdx.x; e < e0 + count; e += kThreads) {
-      const float z = iso1<BITS, PRECISE, MULTI>(p, tid, static_cast<uint64_t>(e));
-      if (SSTATS) s_iso += static_cast<double>(z) * z;
-      Storage<T>::store1(base + e, Storage<T>::load1(base + e) + z);
-    }
+    const double s_iso = iso_elements<T, BITS, PRECISE, MULTI, SSTATS>(p, base, tid, e0, count, n_oct_done, n_oct);
     if (SSTATS) store_item_stats(p, it, threadIdx.x >> 5, s_iso, 0.0, s_iso);
   }
   dependency_end(p);
@@ -169,12 +177,24 @@ template <typename T, int BITS, bool PRECISE, int R, bool MULTI, bool SSTATS = f
 __global__ void __launch_bounds__(kThreads, 2) sweep_fma_kernel(const __grid_constant__ SweepParams p) {
   __shared__ float Gs[R][256 + 8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  dependency_begin(p);
   ItemFeed feed(p);
-  for (int it = feed.first(); it < p.n_items; it = feed.next()) {
+  for (int it = blockIdx.x, first = 1; it < p.n_items; it = feed.next(), first = 0) {
     const WorkItem w = p.items[it];
     const TensorDesc& td = p.tensors[w.tensor];
+    // the first strip is made of the seed alone, before the wait for the previous kernel, unless codes are delivered for it
+    // (they may come from earlier work in the stream)
+    if (first && td.q != nullptr) dependency_begin(p);
     T* base = static_cast<T*>(td.data);
+    if (!SSTATS && td.rank == 0) {
+      // a small set's 1-D tensors ride along (items as in the isotropic kernel): on such sets a launch costs more than they do
+      if (first) {
+        dependency_begin(p);
+        feed.fetch();
+      }
+      iso_elements<T, BITS, PRECISE, MULTI, false>(p, base, static_cast<uint32_t>(td.id), w.row0_or_e0, w.nrows_or_count, 0,
+                                                   w.ncols ? w.nrows_or_count / 8 : 0);
+      continue;
+    }
     const bool wide = (reinterpret_cast<uintptr_t>(base) & 31) == 0;
     const uint32_t tid = static_cast<uint32_t>(td.id);
     const int r = td.rank;
@@ -192,6 +212,10 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_fma_kernel(const __grid_con
 #pragma unroll
         for (int i = 0; i < 8; ++i) Gs[k][8 * o + i] = g[i];
       }
+    }
+    if (first) {
+      if (td.q == nullptr) dependency_begin(p);
+      feed.fetch();
     }
     __syncthreads();
     const int lanes_log2 = w.ncols > 128 ? 5 : (w.ncols > 64 ? 4 : (w.ncols > 32 ? 3 : 2));

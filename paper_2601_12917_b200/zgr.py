@@ -167,10 +167,10 @@ class Zgr:
 
     # -- the three calls of a step --------------------------------------------------------------
     def perturb(self, seed: int, scale: float, stream=None) -> None:
-        _check(lib().zgr_perturb(self._h, seed, scale, _stream_ptr(stream)), "zgr_perturb")
+        _check(_lib.zgr_perturb(self._h, seed, scale, _stream_ptr(stream)), "zgr_perturb")
 
     def restore_update(self, seed: int, loss_plus: float, loss_minus: float, lr: float, stream=None) -> None:
-        _check(lib().zgr_restore_update(self._h, seed, loss_plus, loss_minus, lr, _stream_ptr(stream)), "zgr_restore_update")
+        _check(_lib.zgr_restore_update(self._h, seed, loss_plus, loss_minus, lr, _stream_ptr(stream)), "zgr_restore_update")
 
     # -- several seeds in one sweep ---------------------------------------------------------------
     def sweep_multi(self, seeds: Sequence[int], coeffs: Sequence[float], stream=None) -> None:

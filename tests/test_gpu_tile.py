@@ -73,6 +73,26 @@ def test_narrow_strips(cols):
     p.step(seed=12, lp=2.0, lm=1.6, lr=1e-4)
 
 
+# z of a 16-bit tensor without a subspace (the hook sweeps an fp32 image with the hardware-approximation transform).
+@pytest.mark.parametrize("bits", [16, 32])
+def test_z_of_a_16_bit_tensor_without_a_subspace(bits):
+    p = Pair([(70, 264), (1, 5001)], [9, 0], "bf16", bits=bits, seed=6)
+    z = oracle.z_tensor(p.oracle_tensor(1), 77, 1, bits, p.a, p.b).ravel()
+    assert np.abs(p.lib.debug_z(77, 1).double().cpu().numpy().ravel() - z).max() <= 1e-5
+
+
+# 1-D tensors in the launch of the CUDA-core kernel (small sets): aligned, ragged and unaligned ones, one and several seeds.
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_one_dimensional_tensors_ride_along(dtype):
+    p = Pair([(96, 256), (1, 1), (1, 9), (1, 5003), (40, 72), (1, 4096)], [4, 0, 0, 0, 8, 0], dtype, bits=16, seed=3)
+    launches = p.lib.launch_count()
+    p.step(seed=5, lp=2.1, lm=1.7, lr=1e-4)
+    assert p.lib.launch_count() - launches == 6              # three sweeps, one kernel per contraction width
+    seeds, lp, lm = [41, 42], [2.1, 1.6], [1.9, 2.0]
+    coeffs = [oracle.update_coefficient(0.0, a, b, p.eps, 1e-4) for a, b in zip(lp, lm)]
+    p.call_and_check_multi(seeds, coeffs, lambda: p.lib.restore_update_multi(seeds, lp, lm, 1e-4), "two seeds")
+
+
 # More items than resident blocks: the item counter is used and put back to zero (three sweeps of one context in a row).
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_isotropic_sweeps_with_more_items_than_blocks(dtype):
