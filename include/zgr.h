@@ -63,10 +63,11 @@ typedef struct zgr_ctx zgr_ctx; /* opaque; created by zgr_init, released by zgr_
 /* One weight tensor.  1-D tensors are given as rows = 1, cols = length, U = NULL, rank = 0. */
 typedef struct {
   void* data;       /* device; rows*cols elements of `dtype`, row-major, contiguous, updated in place.
-                       Must be aligned to the element size; 16-byte alignment and cols a multiple of
-                       16 bytes' worth of elements select the vectorised kernels.  fp32 storage with
-                       rank > 8 is served by the one-element-per-thread fallback kernel (exact fp32
-                       contraction; none of the paper-shaped configurations needs it) */
+                       Must be aligned to the element size.  16-byte alignment and cols a multiple of
+                       eight elements select the kernels that stage whole tiles; other shapes, and fp32
+                       storage with rank > 8, are served by a tile kernel that works on octets across
+                       row ends (tensor-core contraction with three bf16 parts per operand, as accurate
+                       as fp32 multiply-adds) */
   int64_t rows;     /* m_l >= 1 */
   int64_t cols;     /* n_l >= 1 */
   int32_t dtype;    /* ZGR_F32 | ZGR_F16 | ZGR_BF16 */
@@ -231,7 +232,7 @@ int zgr_update_subspaces(zgr_ctx* ctx, int32_t n, const int32_t* tensors, const 
  * spanning, with the columns before it, the first k + 1 directions.  It overwrites that subspace buffer, and the
  * library's operand copies are rebuilt as by zgr_update_subspace.  Cholesky QR applied twice, carried in double:
  * orthonormal to about 1e-7 for inputs whose condition number is below about 1e6.  Allocates scratch on
- * first use (and when a larger tensor comes); synchronises `stream`.
+ * first use (and when a larger tensor comes); returns when the basis is in place and visible to every stream.
  * ZGR_EINVAL: bad index, tensor without subspace, fewer rows than rank, misaligned pointer, or directions that
  * are linearly dependent to working precision (nothing is written then).  ZGR_ESTATE: a perturbation is active. */
 int zgr_build_subspace(zgr_ctx* ctx, int32_t tensor, const float* grads, int32_t src_is_host, void* stream);
@@ -286,15 +287,16 @@ int zgr_debug_check_device(int32_t ctx_device, int32_t current_device);
  * of the tensor with coefficient 1, and its fp32 result for every element, taken just before the rounding
  * to the storage type, is written to dev_out (device, rows*cols fp32, 16-byte aligned).  The weights are
  * not touched.  Allocates and frees the image; synchronises `stream`.
- * ZGR_ESTATE: the sweeps do not serve this tensor with the tcgen05 kernel (fp32 storage, rank <= 8,
- * unaligned data, alpha = 1 at zgr_init, or the legacy tensor-core path was selected). */
+ * ZGR_ESTATE: the sweeps do not serve this tensor with that kernel (fp32 storage, rank 0, rank <= 8 in a model with
+ * few such weights, unaligned data or rows, alpha = 1 at zgr_init, or the legacy tensor-core path was selected). */
 int zgr_debug_z_tcgen05(zgr_ctx* ctx, uint64_t seed, int32_t tensor, float* dev_out, void* stream);
 
 /* The work plan of a sweep, computed on the host alone (no device is needed or touched): which kernel
  * family serves which part of which tensor.  Test hook for the planner: the items of a plan must cover
  * every element of every tensor exactly once.  path: 0 isotropic (elements [row0_or_e0, +nrows_or_count) of
- * the tensor), otherwise rows [row0_or_e0, +nrows_or_count) x columns [col0, +ncols): 1 CUDA-core rank <= 8,
- * 2 legacy tensor-core, 3 fallback, 4 tcgen05.  `tensors[].data / U` are only inspected for alignment and
+ * the tensor), otherwise rows [row0_or_e0, +nrows_or_count) x columns [col0, +ncols): 1 rank <= 8,
+ * 2 legacy tensor-core, 3 any shape, 4 tcgen05 with TMA-staged weights.  kpad > 8 on paths 1 and 3 is the tile kernel's contraction
+ * width (an item's last octet of a row may reach into the next strip there).  `tensors[].data / U` are only inspected for alignment and
  * null-ness.  tcgen05 != 0 plans as on a device where tensor maps can be made; multi != 0 gives the plan of
  * the multi-seed sweeps.  Up to max_items items are written to out; *n_items receives the full count.
  * Errors as zgr_init (ZGR_EINVAL), plus sm_count < 1 or a null n_items. */
@@ -307,8 +309,8 @@ int zgr_debug_plan(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, 
 
 /* Per-kernel timing.  While enabled, every sweep launch is bracketed by CUDA events on its stream.
  * zgr_profile_read synchronises the device, writes one entry per kernel family that ran since the
- * last read (up to max_entries) and clears the record.  path: 0 isotropic, 1 CUDA-core rank<=8,
- * 2 tensor-core, 3 fallback; elements = weights covered by one launch. */
+ * last read (up to max_entries) and clears the record.  path, kpad: as in zgr_plan_item; elements = weights covered by one
+ * launch.  While enabled every kernel family is launched by itself (1-D tensors of small models otherwise ride along with path 1). */
 typedef struct {
   int32_t path, dtype, kpad, launches;
   int64_t elements;
