@@ -1,4 +1,4 @@
-// Blackwell-native sweep for 16-bit weights with a rank > 8 subspace:
+// Blackwell-native sweep for 16-bit weights with a subspace (rank > 8, and lower ranks in models of some size):
 //     theta <- rnd(theta + c (a Z + b U G))            (Eq. (perturbation) applied as in Algorithm 1)
 //
 // The generator and the Gaussian transform alone fill about 80 % of an SM's issue slots at the rate
@@ -546,14 +546,18 @@ __global__ void __launch_bounds__(UmmaCfg<KP>::THREADS, 1) sweep_umma_kernel(con
                                               Pack16<T>::pack(acc[6], acc[7])));
               }
             } else {
-              // four octets per thread, kept independent so that their generator chains interleave
+              // four octets per thread, kept independent so that their generator chains interleave (one after the other with 32
+              // random bits per normal, where an octet is two generator blocks: 3615 -> 3540 us on four LLaMA-7B-shaped layers)
               float acc[4][8];
 #pragma unroll
               for (int o = 0; o < 4; ++o)
 #pragma unroll
                 for (int i = 0; i < 8; ++i) acc[o][i] = __uint_as_float(o < 2 ? h0[8 * (o & 1) + i] : h1[8 * (o & 1) + i]);
 #pragma unroll
-              for (int o = 0; o < 4; ++o) normals8_acc_pre<BITS>(p.term[0].keys, pre, oct0_lo + static_cast<uint32_t>(o), p.term[0].iso, acc[o]);
+              for (int o = 0; o < 4; ++o) {
+                normals8_acc_pre<BITS>(p.term[0].keys, pre, oct0_lo + static_cast<uint32_t>(o), p.term[0].iso, acc[o]);
+                if (BITS == 32) asm volatile("" ::: "memory");
+              }
               if (MULTI) {
                 // term by term over all four octets: the keys are fetched once per term, and four chains interleave
 #pragma unroll 1
