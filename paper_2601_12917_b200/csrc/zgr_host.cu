@@ -324,9 +324,16 @@ void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>&
         cut_tensor(descs[m.tensor], m.tensor, m.strip, m.row_step, by_rows, 128 * (3 * done < 2 * tiles ? big : small), trial);
         done += ((descs[m.tensor].rows + 127) / 128) * ((descs[m.tensor].cols + 127) / 128);
       }
+      // No schedule ends before the mean load: heights that cannot win are not replayed, nor replayed to their end (the search
+      // is most of the time that setting up such a set takes).
+      const double last = 0.5 * (static_cast<double>(small) + item_cost);
+      double load = 0.0;
+      for (const WorkItem& w : trial) load += static_cast<double>((w.nrows_or_count + 127) / 128) + item_cost;
+      if (best > 0.0 && load / static_cast<double>(sm_count) * (1.0 - 1e-9) + last >= best) continue;
       std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
       double end = 0.0;
       for (const WorkItem& w : trial) {
+        if (best > 0.0 && end + last >= best) break;
         double at = 0.0;
         if (free_at.size() >= static_cast<size_t>(sm_count)) {
           at = free_at.top();
@@ -336,7 +343,7 @@ void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>&
         free_at.push(at);
         end = std::max(end, at);
       }
-      end += 0.5 * (static_cast<double>(small) + item_cost);
+      end += last;
       if (tiles >= 64 * sms) {
         // long sweeps: also even when dealt out in turn, so that neither the model nor the counter has to be right
         std::fill(dealt.begin(), dealt.end(), 0.0);

@@ -46,9 +46,6 @@ constexpr int kTileThreads = 32 * (2 + kEpi);
 constexpr int kParts = 3;                      // bf16 parts of an operand
 constexpr int kRing = 4;                       // items published ahead
 constexpr int kPitchMax = 42;
-#ifndef ZGR_PF
-#define ZGR_PF (sizeof(T) == 4)
-#endif
 constexpr int kXposeBytes = 32 * kPitchMax * 4;   // one warp's buffer
 
 // Shared-memory plan for contraction width kp (16, 32, 64).
@@ -381,7 +378,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
         // weights of the first passes, on their way while the accumulator is waited for (four octets of 16-bit weights fit
         // the register budget, two of fp32)
         constexpr int kAhead = sizeof(T) == 4 ? 2 : 4;
-        constexpr bool kPrefetchNext = ZGR_PF;
+        constexpr bool kPrefetchNext = sizeof(T) == 4;
         RawOct<T> raw[kAhead];
         auto fetch = [&](int pass, RawOct<T>& into) {
           if (full && wrow + 8 * pass + sub < row_end) into.load(base + e_sub + 8 * pass * cols, wide);
