@@ -287,8 +287,7 @@ int zgr_debug_check_device(int32_t ctx_device, int32_t current_device);
  * of the tensor with coefficient 1, and its fp32 result for every element, taken just before the rounding
  * to the storage type, is written to dev_out (device, rows*cols fp32, 16-byte aligned).  The weights are
  * not touched.  Allocates and frees the image; synchronises `stream`.
- * ZGR_ESTATE: the sweeps do not serve this tensor with that kernel (fp32 storage, rank 0, rank <= 8 in a model with
- * few such weights, unaligned data or rows, alpha = 1 at zgr_init, or the legacy tensor-core path was selected). */
+ * ZGR_ESTATE: the sweeps do not serve this tensor with that kernel (fp32 storage, rank <= 8, unaligned data or rows, alpha = 1 at zgr_init, or the legacy tensor-core path was selected). */
 int zgr_debug_z_tcgen05(zgr_ctx* ctx, uint64_t seed, int32_t tensor, float* dev_out, void* stream);
 
 /* The work plan of a sweep, computed on the host alone (no device is needed or touched): which kernel

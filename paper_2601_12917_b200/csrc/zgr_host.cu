@@ -171,9 +171,12 @@ LowRank low_rank(const zgr_tensor* tensors, int32_t n) {
   return lr;
 }
 
-// Which tcgen05 kernel serves a tensor: 1 the TMA-staged one (16-bit weights in rows that TMA can address), 2 the tile kernel
-// (everything else with a subspace), 0 neither.  Small sets of rank <= 8 stay with the CUDA-core kernel, which starts faster
-// (a step of 1.0 M bf16 weights, rank 8: 22 us there, 29 on tensor cores; 3.9 M: 66 and 29; 354 M: 1380 and 914).
+// Which tcgen05 kernel serves a tensor: 1 the TMA-staged one (16-bit weights in rows that TMA can address, rank > 8), 2 the tile
+// kernel (everything else with a subspace), 0 neither.  Small sets of rank <= 8 stay with the CUDA-core kernel, which starts
+// faster and cuts finer (a step of 2.0 M bf16 weights, rank 8: 25 us there; 4.0 M: 42, 28 on the tile kernel; 300 M: 1163, 1018).
+// Rank <= 8 takes no operand copies in two fp16 parts: those hold 22 bits of entries up to 2^16 2^-ushift, and the fp32
+// multiply-adds of the CUDA-core kernel, which serves the same tensors in a smaller set, have neither limit (the TMA-staged kernel:
+// 776 us at 300 M).
 int tensor_core_kind(const zgr_tensor& t, bool guided_on, const LowRank& lr, int bits) {
   if (!guided_on || t.rank == 0 || t.rows >= (int64_t{1} << 31) - 256) return 0;
   const bool vec = whole_octets(t);
@@ -184,6 +187,7 @@ int tensor_core_kind(const zgr_tensor& t, bool guided_on, const LowRank& lr, int
     // weights, rank 8, in steady state 1885 us a step there and 1918 here, in short runs rank 4 1538 and 1600, 1718 and 1903 with
     // 32 random bits; 42 M, rank 8: 289 and 208, rank 4: 209 and 210)
     if (t.dtype == ZGR_F32 && ((t.rank <= 4 && set >= (int64_t{1} << 25)) || set >= (int64_t{1} << 28))) return 0;
+    return 2;
   }
   // (the TMA-staged kernel keeps the high counter word of the generator fixed: fewer than 2^32 blocks of four elements)
   if (vec && t.dtype != ZGR_F32 && t.rows * t.cols < (int64_t{1} << 34)) return t.cols < (int64_t{1} << 31) - 256 ? 1 : 0;

@@ -1,4 +1,4 @@
-// Blackwell-native sweep for 16-bit weights with a subspace (rank > 8, and lower ranks in models of some size):
+// Blackwell-native sweep for 16-bit weights with a rank > 8 subspace:
 //     theta <- rnd(theta + c (a Z + b U G))            (Eq. (perturbation) applied as in Algorithm 1)
 //
 // The generator and the Gaussian transform alone fill about 80 % of an SM's issue slots at the rate

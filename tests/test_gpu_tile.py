@@ -55,8 +55,9 @@ def test_tile_kernel_norms_codes_and_several_seeds(dtype):
     p.call_and_check_multi(seeds, coeffs, lambda: p.lib.restore_update_multi(seeds, lp, lm, 1e-4), "three seeds")
 
 
-# Low ranks: sets of 2^21 weights and more leave the CUDA-core kernel (narrow and ragged last strips of it are in the parity tests).
-@pytest.mark.parametrize("dtype,path", [("bf16", "umma"), ("f16", "umma"), ("f32", "fma")])
+# Low ranks: sets of 2^21 weights and more leave the CUDA-core kernel for the tile kernel, which is reported under the same path with its
+# contraction width (narrow and ragged last strips of the CUDA-core kernel are in the parity tests).
+@pytest.mark.parametrize("dtype,path", [("bf16", "fma"), ("f16", "fma"), ("f32", "fma")])
 @pytest.mark.parametrize("rank", [1, 4, 8])
 def test_low_rank_sets_of_some_size(dtype, path, rank):
     p = Pair([(1030, 2056), (1, 40), (140, 72)], [rank, 0, rank], dtype, bits=16, seed=2)
@@ -64,6 +65,21 @@ def test_low_rank_sets_of_some_size(dtype, path, rank):
     p.step(seed=6, lp=2.0, lm=1.7, lr=1e-4)
     assert {k["path"]: k["kpad"] for k in p.lib.profile_read()} == {path: 16, "iso": 0}
     assert p.lib.device_status() == 0
+
+
+# A subspace that is not normalised: entries up to 2^12 in size, which two fp16 parts cannot hold at any rows' scale.  On either side of
+# 2^21 weights the same model gives the same z; the tolerances are those of helpers.check_sweep for a z that is `size` times larger.
+@pytest.mark.parametrize("dtype", ["bf16", "f16"])
+@pytest.mark.parametrize("rows", [500, 1030])
+def test_low_rank_subspace_of_any_size(rows, dtype):
+    size = 2.0 ** 15
+    p = Pair([(rows, 2056), (1, 40)], [8, 0], dtype, bits=16, seed=2)
+    p.U[0] *= size
+    p.lib.update_subspace(0)
+    p.z_unit, p.sigma_z = (lambda: size), (lambda l: float(np.sqrt(p.a ** 2 + (p.b * size) ** 2 * 8 / rows)) if l == 0 else p.a)
+    assert float(p.U[0].abs().max()) > 2.0 ** 11
+    p.call_and_check(3, 1e-3 / size, lambda: p.lib.perturb(3, 1e-3 / size), "perturb")
+    p.call_and_check(3, -1e-3 / size, lambda: p.lib.restore_update(3, 2.0, 2.0, 0.0), "restore")
 
 
 # Strips of the CUDA-core kernel of at most 32, 64 and 128 columns: 8, 4 and 2 rows per warp.
