@@ -16,16 +16,17 @@
 namespace zgr {
 
 // ---------------------------------------------------------------------------------------------
-// Programmatic dependent launch.  A sweep is one kernel per family of tensors and a step is three sweeps, so on small models
-// the gaps between launches are most of the time.  Every sweep kernel is launched with the programmatic-serialisation
-// attribute: its CTAs may start while the kernel before it in the stream still runs.  The first kernel of a sweep waits for
-// that kernel to complete (dependency_begin with late = 0) and then lets its successor start.  The other kernels of the same sweep
-// work on other tensors, and everything older had completed before the first one let them start: they begin at once
-// (late = 1) and wait at their end, so that their completion implies that of the kernels before them.
+// Programmatic dependent launch.  A sweep is one kernel per family of tensors.  Every sweep kernel is launched with the
+// programmatic-serialisation attribute, and all but the last of a sweep let the kernel behind them start early (early = 1).
+// The last one does not: the kernel behind it is the caller's, who may launch it with the same attribute and load weights
+// before its own wait, as for constants.  The first kernel of a sweep waits for the kernel before it to complete
+// (dependency_begin with late = 0).  The other kernels of the same sweep work on other tensors, and everything older had
+// completed before the first one let them start: they begin at once (late = 1) and wait at their end, so that their
+// completion implies that of the kernels before them.
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void dependency_begin(const SweepParams& p) {
   if (!p.late) asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (p.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 __device__ __forceinline__ void dependency_end(const SweepParams& p) {
   if (p.late) asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -531,10 +531,16 @@ int sweep(zgr_ctx* ctx, std::vector<Group>& groups, const TensorDesc* d_descs, i
   p.kshift = kshift_for(cb_total);
   bool first = true;     // the first kernel of the sweep waits for earlier work, the others rely on it
   const bool merge = ctx->d_merged != nullptr && &groups == &ctx->groups && !ctx->profiling && t1 < 0 && !keep_stats;
+  const auto has_work = [&](const Group& g) {
+    if (g.items.empty() || (merge && &g - groups.data() == ctx->merged_iso)) return false;
+    return t1 < 0 || g.first_item[static_cast<size_t>(t1)] > g.first_item[static_cast<size_t>(t0)];
+  };
+  const Group* last = nullptr;
+  for (const Group& g : groups)
+    if (has_work(g)) last = &g;
   for (Group& g : groups) {
-    if (g.items.empty()) continue;
+    if (!has_work(g)) continue;
     const int index = static_cast<int>(&g - groups.data());
-    if (merge && index == ctx->merged_iso) continue;
     p.items = g.d_items;
     p.n_items = static_cast<int32_t>(g.items.size());
     p.item_stats = keep_stats ? g.d_item_stats : nullptr;
@@ -546,7 +552,6 @@ int sweep(zgr_ctx* ctx, std::vector<Group>& groups, const TensorDesc* d_descs, i
     p.sched = g.d_sched ? g.d_sched + (ctx->aux_stream != nullptr && st == ctx->aux_stream ? 1 : 0) : nullptr;
     if (t1 >= 0) {
       const int32_t b0 = g.first_item[static_cast<size_t>(t0)], b1 = g.first_item[static_cast<size_t>(t1)];
-      if (b1 <= b0) continue;
       p.items = g.d_items + b0;
       p.n_items = b1 - b0;
       p.item_base = b0;
@@ -555,6 +560,7 @@ int sweep(zgr_ctx* ctx, std::vector<Group>& groups, const TensorDesc* d_descs, i
     const int grid = p.starts ? g.grid
                               : static_cast<int>(std::min<int64_t>(p.n_items, static_cast<int64_t>(ctx->sm_count) * blocks_per_sm(g.kc, n > 1, p.item_stats != nullptr)));
     p.late = first ? 0 : 1;
+    p.early = &g != last ? 1 : 0;
     first = false;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (ctx->profiling && t1 < 0) {

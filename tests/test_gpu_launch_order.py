@@ -1,0 +1,73 @@
+"""Order of the sweeps' kernels with the caller's (needs a B200): the kernels are launched with programmatic dependencies, which must
+not show outside a sweep."""
+import pytest
+import torch
+
+from paper_2601_12917_b200 import zgr
+
+pytestmark = pytest.mark.gpu
+
+READER = b"""extern "C" __global__ void reader(const unsigned* w, unsigned* out) {
+  const unsigned v = w[threadIdx.x];
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  out[threadIdx.x] = v;
+}"""
+
+
+def _checked(r):
+    assert int(r[0]) == 0, r[0]
+    return r[1] if len(r) > 1 else None
+
+
+def _early_reader():
+    """A kernel that is launched with the programmatic attribute and loads 256 words before its own wait, as kernels do with weights
+    that they take for constants."""
+    from cuda.bindings import driver, nvrtc
+    prog = _checked(nvrtc.nvrtcCreateProgram(READER, b"reader.cu", 0, [], []))
+    _checked(nvrtc.nvrtcCompileProgram(prog, 1, [b"--gpu-architecture=sm_100a"]))
+    cubin = b" " * _checked(nvrtc.nvrtcGetCUBINSize(prog))
+    _checked(nvrtc.nvrtcGetCUBIN(prog, cubin))
+    module = _checked(driver.cuModuleLoadData(cubin))
+    fn = _checked(driver.cuModuleGetFunction(module, b"reader"))
+
+    def launch(words, out):
+        import ctypes
+        cfg = driver.CUlaunchConfig()
+        cfg.gridDimX = cfg.gridDimY = cfg.gridDimZ = 1
+        cfg.blockDimX, cfg.blockDimY, cfg.blockDimZ = 256, 1, 1
+        cfg.hStream = driver.CUstream(torch.cuda.current_stream().cuda_stream)
+        attr = driver.CUlaunchAttribute()
+        attr.id = driver.CUlaunchAttributeID.CU_LAUNCH_ATTRIBUTE_PROGRAMMATIC_STREAM_SERIALIZATION
+        attr.value.programmaticStreamSerializationAllowed = 1
+        cfg.attrs, cfg.numAttrs = [attr], 1
+        _checked(driver.cuLaunchKernelEx(cfg, fn, ((words, out), (ctypes.c_void_p, ctypes.c_void_p)), 0))
+    launch.module = module
+    return launch
+
+
+# The last 256 words of the last matrix, i.e. of the work that a sweep comes to last, for every kernel family: TMA-staged, tile
+# (ragged, fp32), CUDA-core, isotropic, the last in one and in two launches a sweep.
+@pytest.mark.parametrize("dtype,cols,rank,alpha", [("bfloat16", 4096, 32, 0.5), ("bfloat16", 4098, 16, 0.5), ("float32", 4096, 24, 0.5), ("float32", 4096, 4, 0.5),
+                                                   ("float16", 4096, 0, 1.0)])
+@pytest.mark.parametrize("vector", [False, True])
+def test_a_kernel_behind_a_sweep_sees_its_weights(dtype, cols, rank, alpha, vector):
+    rows = 16384
+    w = [torch.zeros(rows, cols, device="cuda", dtype=getattr(torch, dtype))]
+    U = [torch.randn(rows, rank, device="cuda") / rows ** 0.5 if rank else None]
+    if vector:
+        w.append(torch.zeros(100, device="cuda", dtype=w[0].dtype))
+        U.append(None)
+    z = zgr.Zgr(w, U, alpha, 1e-3, zgr.SCALE_UNIT, 16)
+    launch = _early_reader()
+    words = w[0].view(torch.int32).view(-1)[-256:]
+    out = torch.zeros(256, device="cuda", dtype=torch.int32)
+    for i in range(8):
+        seed = i // 2 + 1
+        if i % 2 == 0:
+            z.perturb(seed, 1.0)
+        else:
+            z.restore_update(seed, 2.0, 1.0, 1e-3)
+        launch(words.data_ptr(), out.data_ptr())
+        torch.cuda.synchronize()
+        assert torch.equal(out, words), f"sweep {i}"
+    assert z.device_status() == 0
