@@ -22,6 +22,8 @@
  *     enqueued on it and return without synchronising.  The sweeps of one context must be ordered
  *     with respect to each other (one stream, or streams that the caller orders): they write the
  *     same weights and share the library's work-item counters.
+ *   - Tensors that share storage (tied weights listed twice) are swept one after the other if different
+ *     kernel families (zgr_debug_plan) serve them, in the order of each family's first tensor.  Tensors of one family must not overlap.
  *   - "device" pointers are CUDA device addresses on the current device; the library never
  *     dereferences them on the host and never frees them.  They are borrowed for the life of the
  *     context.

@@ -17,19 +17,16 @@ namespace zgr {
 
 // ---------------------------------------------------------------------------------------------
 // Programmatic dependent launch.  A sweep is one kernel per family of tensors.  Every sweep kernel is launched with the
-// programmatic-serialisation attribute, and all but the last of a sweep let the kernel behind them start early (early = 1).
-// The last one does not: the kernel behind it is the caller's, who may launch it with the same attribute and load weights
-// before its own wait, as for constants.  The first kernel of a sweep waits for the kernel before it to complete
-// (dependency_begin with late = 0).  The other kernels of the same sweep work on other tensors, and everything older had
-// completed before the first one let them start: they begin at once (late = 1) and wait at their end, so that their
-// completion implies that of the kernels before them.
+// programmatic-serialisation attribute, and all but the last of a sweep let the kernel behind them start early (early = 1):
+// its CTAs set up their barriers and tensor memory and make their first strip while the last items of this one are worked on.
+// Every kernel waits for the one before it before it reads or writes anything that earlier work may have written: only the
+// kernel that waits is promised that it sees those writes, and the tensors of two families may share storage.  The last kernel
+// does not trigger: the kernel behind it is the caller's, who may launch it with the same attribute and load weights before
+// its own wait, as for constants.
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void dependency_begin(const SweepParams& p) {
-  if (!p.late) asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   if (p.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-__device__ __forceinline__ void dependency_end(const SweepParams& p) {
-  if (p.late) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -51,6 +51,7 @@ struct zgr_ctx {
   std::vector<TensorDesc> descs;      // host mirror of the device table
   TensorDesc* d_descs = nullptr;
   bool descs_dirty = false;
+  bool descs_fresh = false;           // copied to the device since the last sweep
   std::vector<void*> owned;           // device allocations made by the library
   std::vector<Group> groups;          // sweep plan
   // Small sets: the items of the CUDA-core contraction group with those of the isotropic group behind them, for one launch of the
@@ -489,13 +490,42 @@ int upload_groups(zgr_ctx* ctx, std::vector<Group>& groups) {
   return check(ctx, cudaDeviceSynchronize());
 }
 
+// Do tensors of one group share storage with tensors of the other?  (Kernels of different families run one after the other.)
+bool share_storage(const std::vector<TensorDesc>& descs, const Group& f, const Group& g) {
+  std::vector<std::pair<uintptr_t, uintptr_t>> range[2];
+  for (size_t l = 0; l < descs.size(); ++l)
+    for (int i = 0; i < 2; ++i) {
+      const Group& in = i == 0 ? f : g;
+      const uintptr_t at = reinterpret_cast<uintptr_t>(descs[l].data);
+      if (in.first_item[l + 1] > in.first_item[l]) range[i].emplace_back(at, at + static_cast<uintptr_t>(descs[l].rows * descs[l].cols * dtype_bytes(descs[l].dtype)));
+    }
+  std::sort(range[0].begin(), range[0].end());
+  std::sort(range[1].begin(), range[1].end());
+  uintptr_t reach[2] = {0, 0};               // end of the ranges that begin before the current one
+  for (size_t i = 0, j = 0; i < range[0].size() || j < range[1].size();) {
+    const int side = j == range[1].size() || (i < range[0].size() && range[0][i] < range[1][j]) ? 0 : 1;
+    const auto& r = side == 0 ? range[0][i++] : range[1][j++];
+    if (r.first < reach[1 - side]) return true;
+    reach[side] = std::max(reach[side], r.second);
+  }
+  return false;
+}
+
+// The isotropic families go first: they are a few microseconds as a rule, during which the CTAs of the next kernel set up and make
+// their first strip.  (Families that share storage with a matrix keep their place.)
+void order_groups(const std::vector<TensorDesc>& descs, std::vector<Group>& groups) {
+  for (size_t i = 1; i < groups.size(); ++i)
+    for (size_t j = i; j > 0 && groups[j].kc.path == PATH_ISO && groups[j - 1].kc.path != PATH_ISO && !share_storage(descs, groups[j - 1], groups[j]); --j)
+      std::swap(groups[j - 1], groups[j]);
+}
+
 // The isotropic elements that may ride along: up to 2^20, a few microseconds of one launch.
 int merge_small_groups(zgr_ctx* ctx) {
   for (size_t i = 0; i < ctx->groups.size(); ++i)
     for (size_t j = 0; j < ctx->groups.size(); ++j) {
       const Group &f = ctx->groups[i], &g = ctx->groups[j];
       if (f.kc.path != PATH_FMA || is_tile(f.kc) || g.kc.path != PATH_ISO || f.kc.dtype != g.kc.dtype || f.kc.precise != g.kc.precise || g.items.empty() ||
-          f.items.empty() || g.elements > (1 << 20))
+          f.items.empty() || g.elements > (1 << 20) || share_storage(ctx->descs, f, g))
         continue;
       std::vector<WorkItem> items(f.items);
       items.insert(items.end(), g.items.begin(), g.items.end());
@@ -529,7 +559,6 @@ int sweep(zgr_ctx* ctx, std::vector<Group>& groups, const TensorDesc* d_descs, i
   double cb_total = 0.0;
   for (int q = 0; q < n; ++q) cb_total += std::fabs(c[q] * ctx->b);
   p.kshift = kshift_for(cb_total);
-  bool first = true;     // the first kernel of the sweep waits for earlier work, the others rely on it
   const bool merge = ctx->d_merged != nullptr && &groups == &ctx->groups && !ctx->profiling && t1 < 0 && !keep_stats;
   const auto has_work = [&](const Group& g) {
     if (g.items.empty() || (merge && &g - groups.data() == ctx->merged_iso)) return false;
@@ -538,6 +567,8 @@ int sweep(zgr_ctx* ctx, std::vector<Group>& groups, const TensorDesc* d_descs, i
   const Group* last = nullptr;
   for (const Group& g : groups)
     if (has_work(g)) last = &g;
+  const bool early = !ctx->descs_fresh;      // (the kernels read the tensor table before they wait)
+  ctx->descs_fresh = false;
   for (Group& g : groups) {
     if (!has_work(g)) continue;
     const int index = static_cast<int>(&g - groups.data());
@@ -559,9 +590,7 @@ int sweep(zgr_ctx* ctx, std::vector<Group>& groups, const TensorDesc* d_descs, i
     p.starts = t1 >= 0 ? nullptr : g.d_starts;
     const int grid = p.starts ? g.grid
                               : static_cast<int>(std::min<int64_t>(p.n_items, static_cast<int64_t>(ctx->sm_count) * blocks_per_sm(g.kc, n > 1, p.item_stats != nullptr)));
-    p.late = first ? 0 : 1;
-    p.early = &g != last ? 1 : 0;
-    first = false;
+    p.early = early && &g != last ? 1 : 0;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (ctx->profiling && t1 < 0) {
       if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
@@ -590,7 +619,10 @@ int sweep(zgr_ctx* ctx, std::vector<Group>& groups, const TensorDesc* d_descs, i
 int flush_descs(zgr_ctx* ctx, cudaStream_t st) {
   if (!ctx->descs_dirty) return ZGR_OK;
   const int rc = check(ctx, cudaMemcpyAsync(ctx->d_descs, ctx->descs.data(), ctx->descs.size() * sizeof(TensorDesc), cudaMemcpyHostToDevice, st));
-  if (rc == ZGR_OK) ctx->descs_dirty = false;
+  if (rc == ZGR_OK) {
+    ctx->descs_dirty = false;
+    ctx->descs_fresh = true;
+  }
   return rc;
 }
 
@@ -874,6 +906,7 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
     std::vector<int> all(static_cast<size_t>(n));
     for (int32_t l = 0; l < n; ++l) all[static_cast<size_t>(l)] = l;
     plan(ctx->descs, all, guided_on, cfg->bits_per_normal, ctx->sm_count, ctx->groups);
+    order_groups(ctx->descs, ctx->groups);
     rc = upload_groups(ctx, ctx->groups);
   }
   if (rc == ZGR_OK) rc = merge_small_groups(ctx);

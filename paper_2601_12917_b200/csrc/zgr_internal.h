@@ -76,7 +76,6 @@ struct SweepParams {
   int32_t n_items;
   const int32_t* starts; // tensor-core kernels: CTA b works on the items [starts[b], starts[b + 1]); null: dealt out
   int32_t early;         // 1: the next kernel in the stream belongs to the same sweep and may start early (see dependency_begin)
-  int32_t late;          // 0: wait for the stream's earlier work before anything else; 1: only before finishing (see dependency_begin)
   float* zout;           // rows x cols fp32 image of the one tensor swept (test hook of the tcgen05 kernel only)
   double* item_stats;    // norm bookkeeping: kStatSlots x 3 doubles per work item of the group (partial sums per warp), or null
   int32_t item_base;     // index of items[0] in the group's full item list (layer-wise launches start in the middle)

@@ -121,6 +121,10 @@ __device__ __forceinline__ double iso_elements(const SweepParams& p, T* base, ui
 
 template <typename T, int BITS, bool PRECISE, bool MULTI, bool SSTATS = false>
 __global__ void __launch_bounds__(kThreads, iso_blocks_per_sm(PRECISE, MULTI, SSTATS)) sweep_iso_kernel(const __grid_constant__ SweepParams p) {
+  {                                                  // the tables' first entries on their way during the wait
+    const TensorDesc& td = p.tensors[p.items[blockIdx.x].tensor];
+    asm volatile("" ::"l"(td.data), "r"(td.id));
+  }
   dependency_begin(p);
   ItemFeed feed(p);
   for (int it = feed.first(); it < p.n_items; it = feed.next()) {
@@ -162,7 +166,6 @@ __global__ void __launch_bounds__(kThreads, iso_blocks_per_sm(PRECISE, MULTI, SS
     const double s_iso = iso_elements<T, BITS, PRECISE, MULTI, SSTATS>(p, base, tid, e0, count, n_oct_done, n_oct);
     if (SSTATS) store_item_stats(p, it, threadIdx.x >> 5, s_iso, 0.0, s_iso);
   }
-  dependency_end(p);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -288,7 +291,6 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_fma_kernel(const __grid_con
     }
     if (SSTATS) store_item_stats(p, it, warp, s_iso, s_gd, s_z);
   }
-  dependency_end(p);
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -35,7 +35,7 @@ int mma_strip_cols(int kpad);     // columns of a CTA strip on the tensor-core p
 int mma_rows_per_iter(int kpad);  // rows a CTA advances per iteration there
 size_t mma_smem_bytes(int kpad);
 
-// Launch of a kernel that handles programmatic dependencies (dependency_begin / dependency_end): it may start before the
+// Launch of a kernel that handles programmatic dependencies (dependency_begin): it may start before the
 // kernel ahead of it in the stream has completed.
 template <typename... Params, typename... Args>
 cudaError_t launch_sweep_kernel(void (*kernel)(Params...), int grid, int threads, size_t smem, cudaStream_t st, const Args&... args) {

@@ -567,7 +567,6 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
   }
 
   // ---- common exit ----
-  dependency_end(p);
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {

@@ -603,7 +603,6 @@ __global__ void __launch_bounds__(UmmaCfg<KP>::THREADS, 1) sweep_umma_kernel(con
   }
 
   // ---- common exit ----
-  dependency_end(p);
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {

@@ -1,9 +1,13 @@
 """Order of the sweeps' kernels with the caller's (needs a B200): the kernels are launched with programmatic dependencies, which must
 not show outside a sweep."""
+import numpy as np
 import pytest
 import torch
 
-from paper_2601_12917_b200 import zgr
+import oracle
+from paper_2601_12917_b200 import synth, zgr
+
+from helpers import ORACLE_DTYPE, from_double, to_double, to_storage, ulp
 
 pytestmark = pytest.mark.gpu
 
@@ -70,4 +74,31 @@ def test_a_kernel_behind_a_sweep_sees_its_weights(dtype, cols, rank, alpha, vect
         launch(words.data_ptr(), out.data_ptr())
         torch.cuda.synchronize()
         assert torch.equal(out, words), f"sweep {i}"
+    assert z.device_status() == 0
+
+
+# One buffer listed twice, as a matrix with a subspace and as a vector without one (or as matrices of two ranks): the kernel
+# families run one after the other, so both perturbations arrive.  c z is several times the weights: a lost one shows.
+@pytest.mark.parametrize("dtype,rows,cols,ranks", [("f32", 96, 256, (4, 0)), ("bf16", 96, 256, (8, 0)), ("bf16", 256, 1024, (32, 0)), ("bf16", 250, 1025, (16, 0)),
+                                                   ("f32", 256, 1024, (4, 8)), ("f32", 256, 1024, (24, 0)), ("f16", 2048, 1032, (16, 8))])
+def test_storage_shared_by_two_kernel_families(dtype, rows, cols, ranks):
+    ot = ORACLE_DTYPE[dtype]
+    w = from_double(oracle.round_to(synth.weights_host(synth.TensorSpec("t", rows, cols, 0), 1).ravel(), ot), dtype, (rows, cols), "cuda")
+    views = [w, w if ranks[1] else w.view(-1)]
+    U = [torch.from_numpy(synth.subspace(rows, r, 5 + r)).cuda() if r else None for r in ranks]
+    z = zgr.Zgr(views, U, 0.5, 1e-3, zgr.SCALE_UNIT, 16)
+    a, b = z.scalars()
+    for seed, c in ((1, 0.1), (1, -0.2), (2, 0.15)):
+        theta = to_storage(w)
+        for l, r in enumerate(ranks):
+            m, n = (rows, cols) if r else (1, rows * cols)
+            t = oracle.OracleTensor(theta=theta, rows=m, cols=n, dtype=ot, U=None if U[l] is None else U[l].cpu().numpy(), q=None, scale=None, zero=None)
+            oracle.sweep_tensor(t, seed, l, 16, a, b, c)
+            theta = t.theta
+        z.sweep_multi([seed], [c])
+        torch.cuda.synchronize()
+        exp, got = oracle.decode(theta, ot), to_double(w)
+        # per sweep 1 ulp of the largest operand (16 bits) or 1e-6 of the largest weight (fp32), as in helpers.check_sweep; two sweeps
+        allowed = 2e-6 * np.abs(exp).max() if dtype == "f32" else 2 * ulp(np.full(1, np.abs(exp).max()), dtype)[0]
+        assert np.abs(got - exp).max() <= allowed
     assert z.device_status() == 0
