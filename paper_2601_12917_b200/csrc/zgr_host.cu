@@ -1494,7 +1494,9 @@ int zgr_build_subspace(zgr_ctx* ctx, int32_t tensor, const float* grads, int32_t
     const int status = *h_status;
     if (status < 0) return check(ctx, cudaErrorLaunchTimeout);   // a barrier gave up: the basis may be partly written
     if (status > 0) return ZGR_EINVAL;                            // linearly dependent directions: nothing was written
-    return td.Ufrag != nullptr && !td.umma ? make_fragments(ctx, td, st) : ZGR_OK;
+    if (td.Ufrag == nullptr || td.umma) return ZGR_OK;
+    rc = make_fragments(ctx, td, st);
+    return rc == ZGR_OK ? check(ctx, cudaStreamSynchronize(st)) : rc;
   }
   int* d_status = nullptr;
   rc = check(ctx, launch_build_subspace(A, td.rows, td.rank, U, ctx->d_qr, &d_status, nullptr, st));
@@ -1505,8 +1507,10 @@ int zgr_build_subspace(zgr_ctx* ctx, int32_t tensor, const float* grads, int32_t
   if (rc == ZGR_OK) rc = check(ctx, cudaStreamSynchronize(st));
   if (rc != ZGR_OK) return rc;
   if (status != 0) return ZGR_EINVAL;  // linearly dependent directions: nothing was written
-  // the new basis is in place: refresh the tensor-core operand copies exactly as for a delivered subspace
-  return refresh_operands(ctx, tensor, st);
+  // the new basis is in place: refresh the tensor-core operand copies exactly as for a delivered subspace (only now that the
+  // status is known: a refused input leaves them alone too), and wait for them, which sweeps on any stream may read next
+  rc = refresh_operands(ctx, tensor, st);
+  return rc == ZGR_OK ? check(ctx, cudaStreamSynchronize(st)) : rc;
 }
 
 int zgr_debug_plan(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, int32_t sm_count, int32_t tcgen05, int32_t multi,

@@ -13,7 +13,7 @@ import torch
 import oracle
 from paper_2601_12917_b200 import synth, zgr
 
-from helpers import Pair, to_double
+from helpers import Pair, check_sweep, to_double
 
 pytestmark = pytest.mark.gpu
 
@@ -56,6 +56,29 @@ def test_device_built_basis_matches_householder(rows, cols, r, dtype, src):
     # a ZGR step with the device-built basis, every call against the oracle (which reads the same U back)
     reports = p.step(seed=4, lp=2.2, lm=1.9, lr=1e-4)
     assert all(rep["moved"] > 0.3 for call in reports[:2] for rep in call)
+
+
+# The call returns when the basis and the operand copies made of it are visible to every stream: built on a side stream, swept on
+# another one without an event between them, through the one-launch construction, the three-kernel one and the mma.sync operands.
+@pytest.mark.parametrize("rows,r,path", [(4096, 64, ""), (60000, 64, ""), (4096, 64, "legacy"), (60000, 64, "legacy")])
+def test_a_basis_is_visible_to_every_stream(rows, r, path, monkeypatch):
+    if path:
+        monkeypatch.setenv("ZGR_TENSOR_PATH", path)
+    p = Pair([(rows, 64), (1, 24)], [r, 0], "bf16", bits=16, seed=2)
+    side, other = torch.cuda.Stream(), torch.cuda.Stream()
+    for seed in (4, 5, 6):
+        A = torch.from_numpy(_directions(rows, r, seed=seed)).cuda()
+        theta = p.oracle_tensor(0).theta
+        torch.cuda.synchronize()
+        p.lib.build_subspace(0, A, stream=side)
+        p.lib.perturb(seed, p.eps, stream=other)
+        torch.cuda.synchronize()
+        t = p.oracle_tensor(0)                          # the new basis ...
+        t.theta = theta                                 # ... under the weights as they were
+        before = oracle.decode(theta, t.dtype)
+        oracle.sweep_tensor(t, seed, 0, 16, p.a, p.b, p.eps)
+        check_sweep(to_double(p.theta[0]), oracle.decode(t.theta, t.dtype), before, "bf16", 1.0, f"basis {seed}", operand=p.eps * p.sigma_z(0))
+        p.lib.restore_update(seed, 2.0, 2.0, 0.0)
 
 
 def test_dependent_directions_are_refused_and_leave_the_basis_alone():
