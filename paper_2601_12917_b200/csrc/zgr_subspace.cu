@@ -569,17 +569,13 @@ cudaError_t launch_build_subspace(const float* A, int64_t rows, int r, float* U_
   constexpr int kGramSmem = kChunkRows * kLd * sizeof(double);
   constexpr int kFactorSmem = 3 * kMaxR * kLd * sizeof(double);
   constexpr int kApplySmem = (kChunkRows + kMaxR) * kLd * sizeof(double);
-  static bool attributes_set = false;   // per process; setting them again is harmless
-  if (!attributes_set) {
-    cudaError_t a = cudaFuncSetAttribute(gram_partial_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGramSmem);
-    if (a == cudaSuccess) a = cudaFuncSetAttribute(gram_partial_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGramSmem);
-    if (a == cudaSuccess) a = cudaFuncSetAttribute(factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFactorSmem);
-    if (a == cudaSuccess) a = cudaFuncSetAttribute(apply_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kApplySmem);
-    if (a == cudaSuccess) a = cudaFuncSetAttribute(apply_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kApplySmem);
-    if (a != cudaSuccess) return a;
-    attributes_set = true;
-  }
-  cudaError_t e = cudaMemsetAsync(status, 0, sizeof(int), st);
+  // (on every call: the attributes belong to the current device, and a context may live on any)
+  cudaError_t e = cudaFuncSetAttribute(gram_partial_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGramSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(gram_partial_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGramSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFactorSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(apply_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kApplySmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(apply_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kApplySmem);
+  if (e == cudaSuccess) e = cudaMemsetAsync(status, 0, sizeof(int), st);
   if (e != cudaSuccess) return e;
   // pass 1: A (fp32) -> Q1 (double)
   gram_partial_kernel<false><<<n_chunks, kQrThreads, kGramSmem, st>>>(A, rows, r, partials);
