@@ -32,6 +32,7 @@
 
 #include <algorithm>
 
+#include "zgr_grid_exit.h"
 #include "zgr_subspace.h"
 
 namespace zgr {
@@ -175,7 +176,7 @@ struct BasisArgs {
   SplitJob copies;      // operand copies to refresh (part[0] null: none)
   double* partials;     // one RC x RC matrix per CTA (cluster launches: and pass)
   double* sum;          // RC x RC (grid launches)
-  unsigned* counter;    // grid barrier: arrivals, exits; both zero between launches
+  unsigned* counter;    // grid barrier: arrivals, exits, a CTA gave up; all zero between launches
   volatile int* status; // host-mapped: 0, 1 + dependent column, or -1 if a barrier gave up
   int64_t rows;
   int r;
@@ -215,6 +216,19 @@ __device__ __forceinline__ bool basis_barrier(unsigned* counter, int index) {
     return ok != 0;
   }
 }
+
+// The words of `counter` for leave_grid
+struct ExitWords {
+  unsigned* counter;
+  __device__ __forceinline__ void fail() { atomicExch(counter + 2, 1u); }
+  __device__ __forceinline__ bool count_out(unsigned n) {
+    __threadfence();
+    const bool last = atomicInc(counter + 1, n - 1) == n - 1;
+    __threadfence();
+    return last;
+  }
+  __device__ __forceinline__ bool take_failed() { return atomicExch(counter + 2, 0u) != 0; }
+};
 
 // RC = r rounded up to 16, 32 or 64.
 //
@@ -463,7 +477,8 @@ __global__ void __launch_bounds__(kQrThreads) basis_kernel(const BasisArgs p) {
     }
   } else {
     __syncthreads();
-    if (tid == 0 && atomicInc(p.counter + 1, gridDim.x - 1) == gridDim.x - 1) {
+    ExitWords words{p.counter};
+    if (tid == 0 && leave_grid(words, gridDim.x, status)) {
       *p.counter = 0;
       __threadfence_system();
       *p.status = status;
