@@ -596,6 +596,10 @@ __global__ void split_subspace_kernel(const float* __restrict__ U, int64_t rows,
 // Row-major operand copies of U for a list of tensors: two fp16 parts of U 2^shift (TMA-staged kernel) or three bf16 parts
 // of U (tile kernel).  Rows are padded to a multiple of 128 and columns to the contraction width with zeros.
 // A thread makes eight consecutive entries of a row: one 16-byte store per part.
+struct alignas(16) SplitRow {
+  uint16_t v[8];
+};
+static_assert(sizeof(SplitRow) == 16 && alignof(SplitRow) == 16, "one aligned 16-byte store, wherever the entries are kept");
 __global__ void __launch_bounds__(256) split_subspaces_kernel(const SplitJob* __restrict__ jobs) {
   const SplitJob j = jobs[blockIdx.y];
   const int per_row = j.kp / 8;
@@ -604,14 +608,15 @@ __global__ void __launch_bounds__(256) split_subspaces_kernel(const SplitJob* __
   for (int64_t idx = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; idx < n; idx += static_cast<int64_t>(gridDim.x) * blockDim.x) {
     const int64_t row = idx / per_row;
     const int k0 = static_cast<int>(idx % per_row) * 8;
-    uint16_t out[3][8];
+    SplitRow out[3];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const float x = (row < j.rows && k0 + i < j.r) ? j.U[row * j.r + k0 + i] : 0.0f;
-      split_subspace_value(j.shift >= 0, x, scale, out[0][i], out[1][i], out[2][i]);
+      split_subspace_value(j.shift >= 0, x, scale, out[0].v[i], out[1].v[i], out[2].v[i]);
     }
-    for (int q = 0; q < (j.shift >= 0 ? 2 : 3); ++q)
-      *reinterpret_cast<uint4*>(static_cast<uint16_t*>(j.part[q]) + row * j.kp + k0) = *reinterpret_cast<const uint4*>(out[q]);
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+      if (q < 2 || j.shift < 0) *reinterpret_cast<SplitRow*>(static_cast<uint16_t*>(j.part[q]) + row * j.kp + k0) = out[q];
   }
 }
 
