@@ -42,7 +42,10 @@ constexpr int kChunkRows = 128;
 constexpr int kLd = 65;               // leading dimension of the shared-memory matrices (64 + 1: no bank conflicts down a column)
 constexpr int kQrThreads = 256;
 constexpr int kMaxR = 64;
-constexpr double kPivotFloor = 1e-14;   // a pivot below this share of its column's squared norm is rounding error: the columns are dependent
+// A pivot below this share of its column's squared norm means dependent columns: an angle of 4.5e-8 to the span of the earlier
+// ones.  The fp32 rounding of an exact linear combination leaves up to about 3e-8 (8e-16 here), the sums in double below 5e-16 when
+// exact; directions at 5e-8 and more give a basis that is right to 3e-8 and are accepted.
+constexpr double kPivotFloor = 2e-15;
 
 // Partial Gram matrix of rows [chunk*128, +128) of X (rows x r).  X is fp32 (SRC_DOUBLE = false) or double.
 template <bool SRC_DOUBLE>
@@ -86,8 +89,15 @@ __global__ void __launch_bounds__(kQrThreads) factor_kernel(const double* __rest
   __shared__ double norm2[kMaxR];        // diagonal before the factorisation: the columns' squared norms
   if (threadIdx.x == 0) bad = 0;
   for (int idx = threadIdx.x; idx < r * r; idx += kQrThreads) {
-    double s = 0.0;
-    for (int c = 0; c < n_chunks; ++c) s += partials[static_cast<int64_t>(c) * r * r + idx];
+    // (with the rounding errors of the additions kept and added last: 60,000 rows are 469 chunks, whose plain sum is off by as
+    // much as the pivot of directions 3e-8 apart)
+    double s = 0.0, lost = 0.0;
+    for (int c = 0; c < n_chunks; ++c) {
+      const double x = partials[static_cast<int64_t>(c) * r * r + idx], t = s + x, back = t - s;
+      lost += (s - (t - back)) + (x - back);
+      s = t;
+    }
+    s += lost;
     S[idx / r][idx % r] = s;
     if (idx / r == idx % r) norm2[idx / r] = s;
   }

@@ -140,3 +140,25 @@ def test_basis_on_either_side_of_the_launch_shapes(rows, r):
             z.build_subspace(0, B.contiguous())
         assert e.value.code == zgr.EINVAL
         assert torch.equal(z._keep[1][0].double(), U)
+
+
+# Nearly parallel directions are independent down to an angle of 4.5e-8, whatever the launch: the basis of directions 6e-8 apart, one fp32
+# rounding, is delivered as right as any (bounds as above), and an exact copy is refused.
+@pytest.mark.parametrize("rows,r", [(2048, 2), (9000, 2), (20001, 33), (60000, 64), (230000, 2)])
+def test_nearly_parallel_directions(rows, r):
+    z = zgr.Zgr([torch.zeros(rows, 8, device="cuda")], [torch.zeros(rows, r, device="cuda")], 0.5, 1e-3)
+    gen = torch.Generator(device="cuda")
+    for seed in range(6):
+        gen.manual_seed(seed)
+        A = torch.randn(rows, r, generator=gen, device="cuda").double()
+        A[:, r - 1] = A[:, 0] + 6e-8 * torch.randn(rows, generator=gen, device="cuda").double()
+        A = A.float().contiguous()
+        z.build_subspace(0, A)
+        U = z._keep[1][0].double()
+        assert (U.T @ U - torch.eye(r, device="cuda", dtype=torch.float64)).abs().max() <= 1e-6
+        Q, R = torch.linalg.qr(A.double())
+        assert (U - Q * torch.sign(torch.diagonal(R))).abs().max() <= 1e-5
+        A[:, r - 1] = A[:, 0]
+        with pytest.raises(zgr.ZgrError) as e:
+            z.build_subspace(0, A)
+        assert e.value.code == zgr.EINVAL
