@@ -151,12 +151,18 @@ __global__ void __launch_bounds__(kThreads, iso_blocks_per_sm(PRECISE, MULTI, SS
           if (v + kThreads < n32) nxt = __ldcs(reinterpret_cast<const uint4*>(b) + v + kThreads);
           unpack_raw<T>(raw, th);
           raw = nxt;
-          normals8_acc_pre<BITS>(p.term[0].keys, pre, static_cast<uint32_t>(e >> 3), p.term[0].iso, th);
-          if (MULTI) {
+          if constexpr (MULTI) {
+            // the terms are summed on their own scale and added to theta once: one rounding at the size of the weight, not one a term
+            float z[8] = {};
+            normals8_acc_pre<BITS>(p.term[0].keys, pre, static_cast<uint32_t>(e >> 3), p.term[0].iso, z);
 #pragma unroll 1
             for (int q = 1; q < p.n_terms; ++q)
               normals8_acc_pre<BITS>(p.term[q].keys, philox_pre(static_cast<uint32_t>(b0 >> 32), tid, p.term[q].keys), static_cast<uint32_t>(e >> 3),
-                                     p.term[q].iso, th);
+                                     p.term[q].iso, z);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) th[i] += z[i];
+          } else {
+            normals8_acc_pre<BITS>(p.term[0].keys, pre, static_cast<uint32_t>(e >> 3), p.term[0].iso, th);
           }
           Storage<T>::store8(base + e, th);
         }

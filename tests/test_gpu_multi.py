@@ -59,6 +59,25 @@ def test_eight_terms_in_one_pass():
     assert all(r["moved"] > 0.3 for r in reports)
 
 
+@pytest.mark.parametrize("bits", [32, 16])
+def test_terms_of_an_isotropic_tensor_are_summed_before_they_meet_the_weight(bits):
+    """Eight terms of 5e-4 on fp16 weights in [1, 2).  Summed on their own scale they are exact to 1e-10, and adding the sum rounds once
+    to fp32, as here; a rounding per term at the size of the weight (2^-25 on average, seven more of them) would flip the rounding to
+    fp16 (steps of 2^-10) in some 5e-5 to 7e-5 of the elements."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(3)
+    w = (1 + torch.rand(1 << 23, generator=gen, device="cuda")).half().clamp_(1, 1.99)
+    z = zgr.Zgr([w], [None], 1.0, 1e-3, zgr.SCALE_UNIT, bits)
+    seeds, coeffs = list(range(20, 28)), [5e-4 * (-1) ** (i // 3) for i in range(8)]
+    exp = w.double()
+    for s, c in zip(seeds, coeffs):
+        exp += c * z.debug_z(s, 0).double()
+    before = w.clone()
+    z.sweep_multi(seeds, coeffs)
+    assert float((w != before).double().mean()) > 0.5
+    assert float((w != exp.float().half()).double().mean()) <= 1e-5
+
+
 @pytest.mark.parametrize("dtype,bits", [("bf16", 16), ("f32", 32)])
 def test_deferred_schedule_of_a_four_query_step(dtype, bits):
     """2Q+1 sweeps: each restore is fused with the next query's perturbation, one final multi-seed update."""
