@@ -9,6 +9,7 @@
 #include <cstring>
 #include <functional>
 #include <map>
+#include <mutex>
 #include <new>
 #include <numeric>
 #include <queue>
@@ -39,6 +40,49 @@ struct Group {
 };
 
 int dtype_bytes(int dt) { return dt == ZGR_F32 ? 4 : 2; }
+
+// Host-mapped status words of zgr_build_subspace, one per context that has called it, from one 16 KB page per process: pinning
+// memory takes 1.2 to 2.8 ms, ten times a first call without it.  A word goes back when its context ends (no kernel writes it
+// any more: the call waits for its kernel).  Beyond the page's 256 words a context pins its own.
+class StatusWords {
+  static constexpr int kWords = 256, kStride = 64 / sizeof(int);
+  std::mutex mutex_;
+  int* page_ = nullptr;
+  bool used_[kWords] = {};
+
+ public:
+  cudaError_t take(int** word, bool* own) {
+    const std::lock_guard<std::mutex> lock(mutex_);
+    *own = false;
+    if (page_ == nullptr) {
+      void* page = nullptr;
+      const cudaError_t e = cudaHostAlloc(&page, kWords * kStride * sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable);
+      if (e != cudaSuccess) return e;
+      page_ = static_cast<int*>(page);
+    }
+    for (int i = 0; i < kWords; ++i)
+      if (!used_[i]) {
+        used_[i] = true;
+        *word = page_ + i * kStride;
+        return cudaSuccess;
+      }
+    *own = true;
+    return cudaHostAlloc(reinterpret_cast<void**>(word), sizeof(int), cudaHostAllocMapped);
+  }
+  void give_back(int* word, bool own) {
+    if (word == nullptr) return;
+    if (own) {
+      cudaFreeHost(word);
+      return;
+    }
+    const std::lock_guard<std::mutex> lock(mutex_);
+    used_[(word - page_) / kStride] = false;
+  }
+};
+StatusWords& status_words() {
+  static StatusWords words;
+  return words;
+}
 
 }  // namespace
 
@@ -91,7 +135,8 @@ struct zgr_ctx {
   cudaStream_t aux_stream = nullptr;      // zgr_perturb_layers: odd layers run here, so that one layer's tail overlaps the next one's start
   void* d_qr = nullptr;               // scratch of zgr_build_subspace (grown on demand)
   size_t qr_bytes = 0;
-  int* h_status = nullptr;            // host-mapped status word of zgr_build_subspace
+  int* h_status = nullptr;            // host-mapped status word of zgr_build_subspace (see StatusWords)
+  bool h_status_own = false;
 };
 
 namespace {
@@ -1462,7 +1507,7 @@ int zgr_build_subspace(zgr_ctx* ctx, int32_t tensor, const float* grads, int32_t
     ctx->qr_bytes = need;
   }
   if (!ctx->h_status) {
-    const int rc = check(ctx, cudaHostAlloc(reinterpret_cast<void**>(&ctx->h_status), sizeof(int), cudaHostAllocMapped));
+    const int rc = check(ctx, status_words().take(&ctx->h_status, &ctx->h_status_own));
     if (rc != ZGR_OK) return rc;
   }
   float* U = const_cast<float*>(td.U);
@@ -1682,7 +1727,7 @@ void zgr_destroy(zgr_ctx* ctx) {
   for (cudaEvent_t e : ctx->layer_events) cudaEventDestroy(e);
   if (ctx->aux_stream) cudaStreamDestroy(ctx->aux_stream);
   for (void* p : ctx->owned) cudaFree(p);
-  if (ctx->h_status) cudaFreeHost(ctx->h_status);
+  status_words().give_back(ctx->h_status, ctx->h_status_own);
   delete ctx;
 }
 

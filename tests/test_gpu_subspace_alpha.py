@@ -147,3 +147,26 @@ def test_adaptive_alpha_balances_the_energies(scale_mode):
     p.lib.perturb(1, 1e-3)
     assert L.zgr_adapt_alpha(p.lib._h, arr, 0.1, 0.9, 1.0, ctypes.byref(out)) == zgr.ESTATE
     p.lib.restore_update(1, 2.0, 2.0, 0.0)
+
+
+def test_bases_of_more_contexts_than_shared_status_words():
+    """Contexts take their status words from a page of 256 that outlives them, beyond that their own, and give them back: twice 258
+    contexts at once, every one with a call that succeeds and one that is refused."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(4)
+    A = torch.randn(64, 4, generator=gen, device="cuda")
+    Q, R = torch.linalg.qr(A.double())
+    Q = (Q * torch.sign(torch.diagonal(R))).float()
+    B = A.clone()
+    B[:, 2] = B[:, 0]
+    w = torch.zeros(64, 8, device="cuda")
+    for _ in range(2):
+        contexts = [zgr.Zgr([w], [torch.zeros(64, 4, device="cuda")], 0.5, 1e-3) for _ in range(258)]
+        for c in contexts:
+            c.build_subspace(0, A)
+        for c in contexts:
+            with pytest.raises(zgr.ZgrError):
+                c.build_subspace(0, B)
+        assert all(float((c._keep[1][0] - Q).abs().max()) <= 1e-6 for c in contexts)
+        for c in contexts:
+            c.close()
