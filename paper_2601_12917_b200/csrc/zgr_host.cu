@@ -7,12 +7,10 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
-#include <functional>
 #include <map>
 #include <mutex>
 #include <new>
 #include <numeric>
-#include <queue>
 #include <vector>
 
 #include "zgr.h"
@@ -102,7 +100,7 @@ struct zgr_ctx {
   // contraction kernel instead of two (not while the kernels are timed or keep the norm bookkeeping, nor layer by layer).
   int merged_fma = -1, merged_iso = -1;
   WorkItem* d_merged = nullptr;
-  int32_t n_merged = 0;
+  std::vector<WorkItem> merged;
   std::vector<WorkItem> stats_items;  // plan of the norm kernel (tensors not served by the tcgen05 kernel)
   bool stats_planned = false;
   WorkItem* d_stats_items = nullptr;
@@ -302,9 +300,14 @@ double share_out(const std::vector<TensorDesc>& descs, const std::vector<Member>
     if (emit) starts.push_back(static_cast<int32_t>(items.size()));
     return cta + 1;
   };
-  double low = 0.0, high = 1.0;
-  while (fill(high, false) > sm_count) high *= 2.0;
-  for (int i = 0; i < 20; ++i) {
+  double tiles = 0.0;
+  for (const Member& m : members) tiles += static_cast<double>((descs[m.tensor].rows + 127) / 128 * ((descs[m.tensor].cols + 127) / 128));
+  double low = tiles / sm_count, high = 1.25 * low + 1.0;     // (the tiles alone take `low`)
+  while (fill(high, false) > sm_count) {
+    low = high;
+    high *= 1.5;
+  }
+  for (int i = 0; i < 10; ++i) {
     const double mid = 0.5 * (low + high);
     (fill(mid, false) <= sm_count ? high : low) = mid;
   }
@@ -363,34 +366,43 @@ void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>&
                            (g.kc.kpad == 64 ? 0.3 : 0.0);
   double best = 0.0;
   std::vector<WorkItem> trial;
-  std::vector<double> dealt(static_cast<size_t>(sm_count));
+  std::vector<double> dealt(static_cast<size_t>(sm_count)), free_at(static_cast<size_t>(sm_count));
   for (int64_t big : {16, 12, 8, 6, 4, 3, 2, 1})
     for (int64_t small : {big, std::max<int64_t>(big / 4, 1)}) {
       if (tiles >= 64 * sms && big != 8 && big != 4) continue;
       if (best > 0.0 && (small == big ? tiles / big > 16 * sms : tiles / big > 10 * sms || big == 1)) continue;
+      // No schedule ends before the mean load: heights that cannot win are not cut into items, nor replayed to their end (the
+      // search is a fourth of the time that setting up such a set takes).
+      const double last = 0.5 * (static_cast<double>(small) + item_cost);
+      if (best > 0.0) {
+        int64_t done = 0, n_items = 0;
+        for (const Member& m : members) {
+          const int64_t strips = (descs[m.tensor].cols + 127) / 128, blocks = (descs[m.tensor].rows + 127) / 128, h = 3 * done < 2 * tiles ? big : small;
+          const int64_t chunks = (descs[m.tensor].rows + 128 * h - 1) / (128 * h), even = (blocks + chunks - 1) / chunks;
+          n_items += strips * ((blocks + even - 1) / even);
+          done += blocks * strips;
+        }
+        const double load = static_cast<double>(tiles) + static_cast<double>(n_items) * item_cost;
+        if (load / static_cast<double>(sm_count) * (1.0 - 1e-9) + last >= best) continue;
+      }
       trial.clear();
       int64_t done = 0;
       for (const Member& m : members) {
         cut_tensor(descs[m.tensor], m.tensor, m.strip, m.row_step, by_rows, 128 * (3 * done < 2 * tiles ? big : small), trial);
         done += ((descs[m.tensor].rows + 127) / 128) * ((descs[m.tensor].cols + 127) / 128);
       }
-      // No schedule ends before the mean load: heights that cannot win are not replayed, nor replayed to their end (the search
-      // is most of the time that setting up such a set takes).
-      const double last = 0.5 * (static_cast<double>(small) + item_cost);
-      double load = 0.0;
-      for (const WorkItem& w : trial) load += static_cast<double>((w.nrows_or_count + 127) / 128) + item_cost;
-      if (best > 0.0 && load / static_cast<double>(sm_count) * (1.0 - 1e-9) + last >= best) continue;
-      std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
+      std::fill(free_at.begin(), free_at.end(), 0.0);      // heap with the CTA that is free first at [0]
       double end = 0.0;
       for (const WorkItem& w : trial) {
         if (best > 0.0 && end + last >= best) break;
-        double at = 0.0;
-        if (free_at.size() >= static_cast<size_t>(sm_count)) {
-          at = free_at.top();
-          free_at.pop();
+        const double at = free_at[0] + static_cast<double>((w.nrows_or_count + 127) / 128) + item_cost;
+        size_t i = 0;
+        for (size_t c; (c = 2 * i + 1) < free_at.size(); i = c) {
+          if (c + 1 < free_at.size() && free_at[c + 1] < free_at[c]) ++c;
+          if (free_at[c] >= at) break;
+          free_at[i] = free_at[c];
         }
-        at += static_cast<double>((w.nrows_or_count + 127) / 128) + item_cost;
-        free_at.push(at);
+        free_at[i] = at;
         end = std::max(end, at);
       }
       end += last;
@@ -512,27 +524,53 @@ int dev_alloc(zgr_ctx* ctx, T** p, size_t count) {
   return ZGR_OK;
 }
 
-int upload_groups(zgr_ctx* ctx, std::vector<Group>& groups) {
-  for (Group& g : groups) {
-    if (g.items.empty()) continue;
-    int rc = dev_alloc(ctx, &g.d_items, g.items.size());
-    if (rc != ZGR_OK) return rc;
-    rc = check(ctx, cudaMemcpy(g.d_items, g.items.data(), g.items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice));
-    if (rc != ZGR_OK) return rc;
-    if (!g.starts.empty()) {
-      rc = dev_alloc(ctx, &g.d_starts, g.starts.size());
-      if (rc == ZGR_OK) rc = check(ctx, cudaMemcpy(g.d_starts, g.starts.data(), g.starts.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
-      if (rc != ZGR_OK) return rc;
-    }
-    if (g.kc.path == PATH_FMA || g.kc.path == PATH_ISO || is_tile(g.kc)) {
-      rc = dev_alloc(ctx, &g.d_sched, 2);
-      if (rc != ZGR_OK) return rc;
-      rc = check(ctx, cudaMemset(g.d_sched, 0, 2 * sizeof(int32_t)));
-      if (rc != ZGR_OK) return rc;
-    }
+// Device tables of a context, one allocation and one copy for all of them (an allocation takes about 0.4 ms when it needs fresh
+// pages).  The sources are read by copy(), so that tables may hold addresses that place() gave.
+class Tables {
+  struct Part {
+    void** at;
+    const void* src;      // null: zeros
+    size_t offset, bytes;
+  };
+  std::vector<Part> parts_;
+  size_t image_ = 0;
+  uint8_t* base_ = nullptr;
+
+ public:
+  template <typename T>
+  void add(T** p, const T* src, size_t count) {
+    parts_.push_back(Part{reinterpret_cast<void**>(p), src, image_, count * sizeof(T)});
+    image_ += (std::max<size_t>(count, 1) * sizeof(T) + 255) / 256 * 256;
   }
-  // the copies and the zeroing above are not ordered with launches on the caller's (possibly non-blocking) streams
-  return check(ctx, cudaDeviceSynchronize());
+  void add(Group& g) {
+    if (g.items.empty()) return;
+    add(&g.d_items, g.items.data(), g.items.size());
+    if (!g.starts.empty()) add(&g.d_starts, g.starts.data(), g.starts.size());
+    if (g.kc.path == PATH_FMA || g.kc.path == PATH_ISO || is_tile(g.kc)) add(&g.d_sched, static_cast<const int32_t*>(nullptr), 2);
+  }
+  // `extra` bytes behind the tables are not copied to.
+  int place(zgr_ctx* ctx, size_t extra, uint8_t** extra_at) {
+    const int rc = dev_alloc(ctx, &base_, image_ + extra);
+    if (rc != ZGR_OK) return rc;
+    for (const Part& t : parts_) *t.at = base_ + t.offset;
+    if (extra_at) *extra_at = base_ + image_;
+    return ZGR_OK;
+  }
+  int copy(zgr_ctx* ctx) {
+    std::vector<uint8_t> image(image_, 0);
+    for (const Part& t : parts_)
+      if (t.src != nullptr && t.bytes > 0) std::memcpy(image.data() + t.offset, t.src, t.bytes);
+    const int rc = check(ctx, cudaMemcpy(base_, image.data(), image_, cudaMemcpyHostToDevice));
+    // the copy is not ordered with launches on the caller's (possibly non-blocking) streams
+    return rc == ZGR_OK ? check(ctx, cudaDeviceSynchronize()) : rc;
+  }
+};
+
+int upload_groups(zgr_ctx* ctx, std::vector<Group>& groups) {
+  Tables tables;
+  for (Group& g : groups) tables.add(g);
+  const int rc = tables.place(ctx, 0, nullptr);
+  return rc == ZGR_OK ? tables.copy(ctx) : rc;
 }
 
 // Do tensors of one group share storage with tensors of the other?  (Kernels of different families run one after the other.)
@@ -565,24 +603,19 @@ void order_groups(const std::vector<TensorDesc>& descs, std::vector<Group>& grou
 }
 
 // The isotropic elements that may ride along: up to 2^20, a few microseconds of one launch.
-int merge_small_groups(zgr_ctx* ctx) {
+void merge_small_groups(zgr_ctx* ctx) {
   for (size_t i = 0; i < ctx->groups.size(); ++i)
     for (size_t j = 0; j < ctx->groups.size(); ++j) {
       const Group &f = ctx->groups[i], &g = ctx->groups[j];
       if (f.kc.path != PATH_FMA || is_tile(f.kc) || g.kc.path != PATH_ISO || f.kc.dtype != g.kc.dtype || f.kc.precise != g.kc.precise || g.items.empty() ||
           f.items.empty() || g.elements > (1 << 20) || share_storage(ctx->descs, f, g))
         continue;
-      std::vector<WorkItem> items(f.items);
-      items.insert(items.end(), g.items.begin(), g.items.end());
-      int rc = dev_alloc(ctx, &ctx->d_merged, items.size());
-      if (rc == ZGR_OK) rc = check(ctx, cudaMemcpy(ctx->d_merged, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice));
-      if (rc != ZGR_OK) return rc;
-      ctx->n_merged = static_cast<int32_t>(items.size());
+      ctx->merged = f.items;
+      ctx->merged.insert(ctx->merged.end(), g.items.begin(), g.items.end());
       ctx->merged_fma = static_cast<int>(i);
       ctx->merged_iso = static_cast<int>(j);
-      return ZGR_OK;
+      return;
     }
-  return ZGR_OK;
 }
 
 // One sweep  theta <- rnd(theta + sum_q c_q z(seed_q))  over the planned groups (n terms, 1 <= n <= kMaxTerms).
@@ -623,7 +656,7 @@ int sweep(zgr_ctx* ctx, std::vector<Group>& groups, const TensorDesc* d_descs, i
     p.item_base = 0;
     if (merge && index == ctx->merged_fma) {
       p.items = ctx->d_merged;
-      p.n_items = ctx->n_merged;
+      p.n_items = static_cast<int32_t>(ctx->merged.size());
     }
     p.sched = g.d_sched ? g.d_sched + (ctx->aux_stream != nullptr && st == ctx->aux_stream ? 1 : 0) : nullptr;
     if (t1 >= 0) {
@@ -860,21 +893,7 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
   const bool guided_on = ctx->b != 0.0;
   ctx->guided_at_init = guided_on;
   const LowRank lr = low_rank(tensors, n);
-  // one allocation for all operand copies
-  void* operands = nullptr;
-  if (umma_wanted() && encode_tiled_fn() != nullptr) {
-    size_t bytes = 0;
-    for (int32_t l = 0; l < n; ++l) {
-      const int kind = tensor_core_kind(tensors[l], guided_on, lr, cfg->bits_per_normal);
-      const size_t kpad = tensors[l].rank <= 16 ? 16 : (tensors[l].rank <= 32 ? 32 : 64);
-      if (kind != 0) bytes += (kind == 1 ? 2 : 3) * static_cast<size_t>((tensors[l].rows + 127) / 128) * 128 * kpad * 2;
-    }
-    if (bytes > 0) {
-      uint8_t* base = nullptr;
-      rc = dev_alloc(ctx, &base, bytes);
-      operands = base;
-    }
-  }
+  size_t operand_bytes = 0;
   for (int32_t l = 0; l < n && rc == ZGR_OK; ++l) {
     const zgr_tensor& t = tensors[l];
     TensorDesc& td = ctx->descs[static_cast<size_t>(l)];
@@ -896,27 +915,15 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
     td.tile = 0;
     td.ushift = 0;
     for (void*& copy : td.Ucopy) copy = nullptr;
-    // tcgen05 kernels: row-major copies of U in parts, and three tensor maps
-    const int kind = tensor_core_kind(t, guided_on, lr, cfg->bits_per_normal);
-    if (kind != 0 && umma_wanted() && encode_tiled_fn() != nullptr) {
-      const int parts = kind == 1 ? 2 : 3;
-      const int64_t rows_pad = ((t.rows + 127) / 128) * 128;
+    // tcgen05 kernels: row-major copies of U in parts, and three tensor maps (those of the copies once these have their place)
+    const int kind = umma_wanted() && encode_tiled_fn() != nullptr ? tensor_core_kind(t, guided_on, lr, cfg->bits_per_normal) : 0;
+    if (kind == 2 || (kind == 1 && make_map_16bit(&ctx->tmaps[static_cast<size_t>(3 * l)], t.data, t.rows, t.cols, 64))) {
       td.kpad = t.rank <= 16 ? 16 : (t.rank <= 32 ? 32 : 64);
       // entries of an orthonormal U are about 1/sqrt(rows): scaled by 2^ushift they sit between 1 and 2 in size
       // (capped at 2^12, which leaves fp16 room for entries up to 16 in size); the bf16 parts need no scaling
       if (kind == 1) td.ushift = std::min<int32_t>(12, static_cast<int32_t>(std::ceil(0.5 * std::log2(static_cast<double>(t.rows)))));
-      uint8_t* at = static_cast<uint8_t*>(operands);
-      CUtensorMap* m = &ctx->tmaps[static_cast<size_t>(3 * l)];
-      bool maps = kind == 1 ? make_map_16bit(m, t.data, t.rows, t.cols, 64) : true;
-      for (int i = 0; i < parts; ++i) {
-        td.Ucopy[i] = at;
-        maps = maps && make_map_16bit(m + (kind == 1 ? 1 : 0) + i, at, rows_pad, td.kpad, td.kpad);
-        at += static_cast<size_t>(rows_pad) * td.kpad * 2;       // (a multiple of 4096 bytes)
-      }
-      if (maps) {
-        (kind == 1 ? td.umma : td.tile) = 1;
-        operands = at;
-      }
+      (kind == 1 ? td.umma : td.tile) = 1;
+      operand_bytes += (kind == 1 ? 2 : 3) * static_cast<size_t>((t.rows + 127) / 128) * 128 * static_cast<size_t>(td.kpad) * 2;
     }
     const bool vec = (reinterpret_cast<uintptr_t>(t.data) & 15) == 0 && (t.cols % 8 == 0);
     if (guided_on && t.rank > 8 && vec && t.dtype != ZGR_F32 && !td.umma) {
@@ -928,34 +935,40 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
   ctx->split_job.assign(static_cast<size_t>(n), -1);
   if (rc == ZGR_OK) {
     std::vector<SplitJob>& jobs = ctx->split_jobs;
-    for (int32_t l = 0; l < n; ++l) {
-      const TensorDesc& td = ctx->descs[static_cast<size_t>(l)];
-      if (!td.umma && !td.tile) continue;
-      ctx->split_job[static_cast<size_t>(l)] = static_cast<int32_t>(jobs.size());
-      jobs.push_back(SplitJob{td.U, {td.Ucopy[0], td.Ucopy[1], td.Ucopy[2]}, td.rows, ((td.rows + 127) / 128) * 128, td.rank, td.kpad, td.umma ? td.ushift : -1});
-    }
-    ctx->n_split_jobs = static_cast<int>(jobs.size());
-    if (!jobs.empty()) {
-      rc = dev_alloc(ctx, &ctx->d_split_jobs, jobs.size());
-      if (rc == ZGR_OK) rc = check(ctx, cudaMemcpy(ctx->d_split_jobs, jobs.data(), jobs.size() * sizeof(SplitJob), cudaMemcpyHostToDevice));
-      if (rc == ZGR_OK) rc = split_jobs(ctx, 0, static_cast<int>(jobs.size()), nullptr);
-    }
-  }
-  if (rc == ZGR_OK) rc = dev_alloc(ctx, &ctx->d_tmaps, ctx->tmaps.size());
-  if (rc == ZGR_OK) rc = check(ctx, cudaMemcpy(ctx->d_tmaps, ctx->tmaps.data(), ctx->tmaps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice));
-  if (rc == ZGR_OK) rc = dev_alloc(ctx, &ctx->d_err, 1);
-  if (rc == ZGR_OK) rc = check(ctx, cudaMemset(ctx->d_err, 0, sizeof(int)));
-  if (rc == ZGR_OK) rc = dev_alloc(ctx, &ctx->d_descs, ctx->descs.size());
-  if (rc == ZGR_OK) rc = check(ctx, cudaMemcpy(ctx->d_descs, ctx->descs.data(), ctx->descs.size() * sizeof(TensorDesc), cudaMemcpyHostToDevice));
-  if (rc == ZGR_OK) {
+    for (int32_t l = 0; l < n; ++l)
+      if (ctx->descs[static_cast<size_t>(l)].umma || ctx->descs[static_cast<size_t>(l)].tile) ctx->split_job[static_cast<size_t>(l)] = ctx->n_split_jobs++;
+    jobs.resize(static_cast<size_t>(ctx->n_split_jobs));
     std::vector<int> all(static_cast<size_t>(n));
     for (int32_t l = 0; l < n; ++l) all[static_cast<size_t>(l)] = l;
     plan(ctx->descs, all, guided_on, cfg->bits_per_normal, ctx->sm_count, ctx->groups);
     order_groups(ctx->descs, ctx->groups);
-    rc = upload_groups(ctx, ctx->groups);
+    merge_small_groups(ctx);
+    Tables tables;
+    tables.add(&ctx->d_split_jobs, jobs.data(), jobs.size());
+    tables.add(&ctx->d_tmaps, ctx->tmaps.data(), ctx->tmaps.size());
+    tables.add(&ctx->d_descs, ctx->descs.data(), ctx->descs.size());
+    tables.add(&ctx->d_err, static_cast<const int*>(nullptr), 1);
+    tables.add(&ctx->d_stats, static_cast<const double*>(nullptr), static_cast<size_t>(3 * n));
+    for (Group& g : ctx->groups) tables.add(g);
+    if (!ctx->merged.empty()) tables.add(&ctx->d_merged, ctx->merged.data(), ctx->merged.size());
+    uint8_t* at = nullptr;
+    rc = tables.place(ctx, operand_bytes, &at);
+    for (int32_t l = 0; l < n && rc == ZGR_OK; ++l) {
+      TensorDesc& td = ctx->descs[static_cast<size_t>(l)];
+      const int32_t job = ctx->split_job[static_cast<size_t>(l)];
+      if (job < 0) continue;
+      const int64_t rows_pad = ((td.rows + 127) / 128) * 128;
+      CUtensorMap* m = &ctx->tmaps[static_cast<size_t>(3 * l)] + (td.umma ? 1 : 0);
+      for (int i = 0; i < (td.umma ? 2 : 3); ++i) {
+        td.Ucopy[i] = at;
+        if (!make_map_16bit(m + i, at, rows_pad, td.kpad, td.kpad)) rc = check(ctx, cudaErrorUnknown);
+        at += static_cast<size_t>(rows_pad) * td.kpad * 2;       // (a multiple of 4096 bytes)
+      }
+      jobs[static_cast<size_t>(job)] = SplitJob{td.U, {td.Ucopy[0], td.Ucopy[1], td.Ucopy[2]}, td.rows, rows_pad, td.rank, td.kpad, td.umma ? td.ushift : -1};
+    }
+    if (rc == ZGR_OK) rc = tables.copy(ctx);
+    if (rc == ZGR_OK) rc = split_jobs(ctx, 0, ctx->n_split_jobs, nullptr);
   }
-  if (rc == ZGR_OK) rc = merge_small_groups(ctx);
-  if (rc == ZGR_OK) rc = dev_alloc(ctx, &ctx->d_stats, static_cast<size_t>(3 * n));
   if (rc == ZGR_OK) rc = check(ctx, cudaDeviceSynchronize());  // the subspace copies are complete
   if (rc != ZGR_OK) {
     zgr_destroy(ctx);
