@@ -244,7 +244,10 @@ __device__ __forceinline__ uint32_t field16b(uint32_t x) { return and_or(__funne
 // so a single fold replaces the quadrant logic and the only sign is xor-ed into the radius.  The polynomials are fitted
 // on [-1/4, 1/4] (least squares reweighted towards the minimax solution); their leading terms 4 x and 1 - 16 x^2 are
 // added last, which keeps the rounding error of the sum near half an ulp: 8.9e-8 and 7.8e-8 maximum absolute error in
-// fp32 arithmetic (2.0e-8 and 2.5e-8 rms), as much as the quarter-turn form.  Logarithm as in neg2_log.
+// fp32 arithmetic (3.2e-8 and 2.6e-8 rms; 1.9e-8 in the quarter-turn form).  Logarithm as in neg2_log, except that its constant is
+// the next float away from zero: hardware logarithm and square root lean towards zero, by half an ulp of the radius together,
+// which this takes back for the most part.  Against 64 bits the normals are off by 6.8e-8 rms, 8.4e-7 at most (9.3e-8 and 1.1e-6
+// with the nearest float to 2 ln 2; 6.6e-8 and 1.0e-6 one ulp further; box_muller<true> 7.2e-8 and 8.9e-7).
 //
 // The generator with this transform runs at 0.96 cycles per element and scheduler against 1.03-1.09 with two calls of
 // box_muller<true> (free-running loop, 16 random bits per normal).
@@ -263,7 +266,7 @@ __device__ __forceinline__ void box_muller_accurate2(uint32_t ma1, uint32_t ma2,
   q = fma2(q, v, dup2(1.0f));
   q = fma2(q, v, dup2(2.0f));
   unpack2(mul2(q, v), na, nb);
-  unpack2(mul2(pack2(lg2_approx(ua), lg2_approx(ub)), dup2(-1.3862943611f)), ga, gb);
+  unpack2(mul2(pack2(lg2_approx(ua), lg2_approx(ub)), dup2(-1.3862944841f)), ga, gb);      // -2 ln 2, next float
   const uint64_t rho = mul2(pack2(sqrt_approx(va <= 0.0625f ? na : ga), sqrt_approx(vb <= 0.0625f ? nb : gb)), dup2(ns.s));
   const uint64_t w = add2(add2(pack2(__uint_as_float(ma2), __uint_as_float(mb2)), off), dup2(-0.5f));
   float wa, wb;
