@@ -618,7 +618,7 @@ __global__ void __launch_bounds__(256) split_subspaces_kernel(const SplitJob* __
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const float x = (row < j.rows && k0 + i < j.r) ? j.U[row * j.r + k0 + i] : 0.0f;
-      split_subspace_value(j.shift >= 0, x, scale, out[0].v[i], out[1].v[i], out[2].v[i]);
+      split_subspace_value(j.shift >= 0, x, scale, truncation_lean(j.kp), out[0].v[i], out[1].v[i], out[2].v[i]);
     }
 #pragma unroll
     for (int q = 0; q < 3; ++q)

@@ -18,8 +18,9 @@
 //            contiguous bytes of a row), and there the weights are loaded, the normals added, the result rounded and stored.
 //
 // Operand precision.  An fp32 number is the sum of three bf16 numbers (8 bits each) without error and without range
-// limits; six of the nine products are formed, the others are below 2^-24 of the result.  The contraction is therefore
-// as accurate as a chain of fp32 multiply-adds.
+// limits; six of the nine products are formed, the others are below 2^-24 of the result.  With the copies of U leaning against
+// the truncation of the tensor cores (truncation_lean) the contraction is as accurate as a chain of fp32 multiply-adds, from
+// rank 2 on more so.
 //
 // Bank conflicts of the transposition.  Row m of a warp's buffer is `pitch` floats long; lane (m, o) reads
 // D[m][h_m + 8 o + i].  Eight rows x four octets per read: distinct banks if m pitch + h_m = m (pitch - cols) takes
@@ -137,7 +138,7 @@ __device__ __forceinline__ void build_strip(const TensorDesc& td, const SweepPar
       const int j = j0 + i;
       if (j >= 0 && j < kTileN) {
         uint16_t q0, q1, q2;
-        split_subspace_value(false, c_first + i < cols ? g[i] : 0.0f, 1.0f, q0, q1, q2);
+        split_subspace_value(false, c_first + i < cols ? g[i] : 0.0f, 1.0f, 0.0f, q0, q1, q2);
         const uint32_t at = g_dst + swizzle(static_cast<uint32_t>(j * rowb + 2 * k), rowb);
         sts16(at, q0);
         sts16(at + g_bytes, q1);

@@ -172,3 +172,26 @@ def test_normals_of_fp32_tensors(bits):
     p = Pair([(2048, 1536)], [0], "f32", bits=bits, seed=1, alpha=1.0)
     err = p.lib.debug_z(5, 0).double().cpu().numpy().ravel() - oracle.z_tensor(p.oracle_tensor(0), 5, 0, bits, p.a, p.b).ravel()
     assert np.sqrt(np.mean(err ** 2)) <= 7.2e-8 and np.abs(err).max() <= 9e-7
+
+
+# Accuracy of the tile kernel's contraction against 64 bits, alone (alpha = 0) and on coefficients with all 24 bits (codes minus an odd zero
+# point, formed here as the kernel forms them): not behind a chain of fp32 multiply-adds, whose error is given first (one fp32
+# rounding is 2.5e-8, the truncation of the tensor cores alone 4.6e-8 to 7.7e-8).
+@pytest.mark.parametrize("cols", [1536, 1537])
+@pytest.mark.parametrize("rank,chain", [(2, 3.4e-8), (4, 4.0e-8), (8, 5.0e-8), (16, 7.6e-8), (32, 1.0e-7), (64, 1.5e-7)])
+def test_contraction_of_fp32_tensors(rank, chain, cols):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(rank)
+    w = torch.zeros(2048, cols, device="cuda")
+    U = torch.linalg.qr(torch.randn(2048, rank, generator=gen, device="cuda"))[0].contiguous()
+    q = torch.randint(-127, 128, (rank, cols), generator=gen, device="cuda").to(torch.int8)
+    scale, zero = (torch.rand(rank, generator=gen, device="cuda") + 0.5) / 64, 2 * torch.rand(rank, generator=gen, device="cuda") - 1
+    z = zgr.Zgr([w], [U], 0.0, 1e-3, zgr.SCALE_PAPER, 16)
+    z.set_coeffs_dtc(0, q, scale, zero)
+    z.perturb(1, 1e-3)                                     # (also brings the codes into the device's table)
+    z.restore_update(1, 2.0, 2.0, 0.0)
+    b = torch.tensor(z.scalars()[1], dtype=torch.float64, device="cuda").float()
+    exact = U.double() @ ((scale * b)[:, None] * (q.float() - zero[:, None])).double()
+    err = z.debug_z(1, 0).double() - exact
+    assert float(err.norm() / exact.norm()) <= chain
+    assert abs(float((err * exact.sign()).sum() / exact.abs().sum())) <= 1e-8      # and no lean
