@@ -233,8 +233,8 @@ int zgr_update_subspaces(zgr_ctx* ctx, int32_t n, const int32_t* tensors, const 
  * the orthonormal basis of their span that a QR factorisation with a positive diagonal of R gives, column k
  * spanning, with the columns before it, the first k + 1 directions.  It overwrites that subspace buffer, and the
  * library's operand copies are rebuilt as by zgr_update_subspace.  Cholesky QR applied twice, carried in double:
- * orthonormal to about 1e-7 for inputs whose condition number is below about 1e6.  Allocates scratch on
- * first use (and when a larger tensor comes); returns when the basis is in place and visible to every stream.
+ * orthonormal to about 1e-7 for inputs whose condition number is below about 1e6.  Scratch beyond
+ * 2 MB is allocated on first use (and when a larger tensor comes); returns when the basis is in place and visible to every stream.
  * ZGR_EINVAL: bad index, tensor without subspace, fewer rows than rank, misaligned pointer, or directions that
  * are linearly dependent to working precision (nothing is written then).  ZGR_ESTATE: a perturbation is active. */
 int zgr_build_subspace(zgr_ctx* ctx, int32_t tensor, const float* grads, int32_t src_is_host, void* stream);

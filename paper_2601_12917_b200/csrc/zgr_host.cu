@@ -951,8 +951,24 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
     tables.add(&ctx->d_stats, static_cast<const double*>(nullptr), static_cast<size_t>(3 * n));
     for (Group& g : ctx->groups) tables.add(g);
     if (!ctx->merged.empty()) tables.add(&ctx->d_merged, ctx->merged.data(), ctx->merged.size());
-    uint8_t* at = nullptr;
-    rc = tables.place(ctx, operand_bytes, &at);
+    // Scratch of zgr_build_subspace, up to 2 MB (every rank up to 32, and rank 64 in one cluster): as an allocation of its own inside the
+    // first call it would be most of that call.  Its first 512 bytes are the last of the zeroed tables.
+    size_t scratch = 0;
+    for (int32_t l = 0; l < n; ++l) {
+      const zgr_tensor& t = tensors[l];
+      if (t.rank == 0 || t.rows < t.rank || !subspace_fused(t.rows, t.rank, ctx->sm_count)) continue;
+      const size_t need = subspace_scratch_bytes(t.rows, t.rank, ctx->sm_count);
+      if (need <= (size_t{2} << 20)) scratch = std::max(scratch, need);
+    }
+    uint8_t *at = nullptr, *qr = nullptr;
+    if (scratch > 0) tables.add(&qr, static_cast<const uint8_t*>(nullptr), 512);
+    const size_t behind = scratch > 0 ? (scratch - 512 + 255) / 256 * 256 : 0;
+    rc = tables.place(ctx, behind + operand_bytes, &at);
+    if (rc == ZGR_OK) {
+      at += behind;
+      ctx->d_qr = qr;
+      ctx->qr_bytes = scratch;
+    }
     for (int32_t l = 0; l < n && rc == ZGR_OK; ++l) {
       TensorDesc& td = ctx->descs[static_cast<size_t>(l)];
       const int32_t job = ctx->split_job[static_cast<size_t>(l)];

@@ -178,6 +178,7 @@ __host__ __device__ constexpr int cluster_ctas(int rc) { return rc == 16 ? 16 : 
 // Entries per CTA up to which one cluster beats the grid (cycles, cluster / grid, at twice that size: 51k / 45k at rank 16,
 // 77k / 60k at rank 32, 121k / 116k at rank 64; the grid pays four barriers of 3k and two more reductions).
 constexpr int kClusterEntries = 4096;
+inline bool in_cluster(int64_t rows, int rc) { return (rows + cluster_ctas(rc) - 1) / cluster_ctas(rc) * rc <= (rc == 64 ? 2 : 1) * kClusterEntries; }
 constexpr long long kBarrierLimit = 4000000000ll;   // cycles, about 2 s: a barrier that waits longer gives up
 
 struct BasisArgs {
@@ -512,9 +513,8 @@ cudaError_t launch_basis(BasisArgs p, int sm_count, cudaStream_t st, bool* serve
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   constexpr int CL = cluster_ctas(RC);
-  const int64_t in_cluster = (p.rows + CL - 1) / CL;
-  if (in_cluster * RC <= (RC == 64 ? 2 : 1) * kClusterEntries) {
-    p.rows_per_cta = static_cast<int>(in_cluster);
+  if (in_cluster(p.rows, RC)) {
+    p.rows_per_cta = static_cast<int>((p.rows + CL - 1) / CL);
     const size_t smem = basis_smem<RC>(p.rows_per_cta);
     cudaError_t e = cudaFuncSetAttribute(basis_kernel<RC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kBasisSmemMax));
     if (e == cudaSuccess && CL > 8) e = cudaFuncSetAttribute(basis_kernel<RC, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -549,8 +549,9 @@ size_t subspace_scratch_bytes(int64_t rows, int r, int sm_count) {
   // three-kernel path: partial Gram matrices, R^-1, accumulated R, the double image of the first pass's Q
   const size_t chunked = static_cast<size_t>(n_chunks) * r * r * sizeof(double) + 2 * static_cast<size_t>(r) * r * sizeof(double) +
                          static_cast<size_t>(rows) * r * sizeof(double);
-  const size_t rc = r <= 16 ? 16 : (r <= 32 ? 32 : 64);
-  const size_t fused = (static_cast<size_t>(std::max(sm_count, 32)) + 1) * rc * rc * sizeof(double);
+  const int rc = r <= 16 ? 16 : (r <= 32 ? 32 : 64);
+  const size_t matrices = 1 + static_cast<size_t>(in_cluster(rows, rc) ? 2 * cluster_ctas(rc) : sm_count);
+  const size_t fused = matrices * static_cast<size_t>(rc * rc) * sizeof(double);
   return 512 + (subspace_fused(rows, r, sm_count) ? fused : chunked);
 }
 
