@@ -12,6 +12,7 @@ import oracle
 from paper_2601_12917_b200 import synth, zgr
 
 from helpers import Pair
+from test_plan import plan
 
 pytestmark = pytest.mark.gpu
 
@@ -161,9 +162,9 @@ def test_layer_table_and_delivery_errors():
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_layerwise_sweeps_of_low_rank_tensors_on_both_streams(dtype):
     """Every layer holds tensors of rank <= 8, so consecutive layers run the CUDA-core contraction kernel on the two
-    alternating streams at the same time; that kernel hands its work items out through a counter per stream, which
-    each launch must leave at zero for the next one.  Many layers of different sizes, layer-wise and whole-model
-    sweeps in turn, every call against the oracle and against a context that only ever sweeps the whole model."""
+    alternating streams at the same time.  Many layers of different sizes, layer-wise and whole-model sweeps in turn, every
+    call against the oracle and against a context that only ever sweeps the whole model.  (A layer has fewer items than
+    there are blocks here, so nothing is handed out; the test of the item counters below exceeds them.)"""
     shapes, ranks, ends = [], [], []
     for L in range(9):
         shapes += [(96 + 40 * L, 264 + 256 * (L % 3)), (1, 72 + 8 * L), (64 + 8 * L, 520)]
@@ -187,3 +188,32 @@ def test_layerwise_sweeps_of_low_rank_tensors_on_both_streams(dtype):
         for l in range(len(shapes)):
             assert torch.equal(a.theta[l], b.theta[l]), f"step {step} tensor {l}"
     assert a.lib.device_status() == 0 and a.lib.state()[0] is False
+
+
+# Layers with more items than resident blocks (CUDA-core kernel 2 per SM, isotropic kernel 5 or 8, tile kernel 1), so that every
+# layer draws on the item counter of its stream and has to leave it at zero for the next sweep.  (Path 0 is the
+# isotropic family, 1 the CUDA-core and 3 the tile kernel; the plan says that the layers are large enough.)
+@pytest.mark.parametrize("dtype,shapes,ranks,ends,path,blocks", [
+    ("f32", [(2000, 520), (1, 3_000_000)] * 2, [4, 0] * 2, [2, 4], 1, 2), ("bf16", [(2000, 520), (1, 3_000_000)] * 2, [4, 0] * 2, [2, 4], 1, 2),
+    ("bf16", [(2000, 5001)] * 3, [16] * 3, [1, 2, 3], 3, 1), ("f32", [(1500, 10248)] * 2, [24] * 2, [1, 2], 3, 1)])
+def test_layerwise_item_counters_of_both_streams(dtype, shapes, ranks, ends, path, blocks):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    items = plan(shapes, ranks, [{"f32": zgr.F32, "bf16": zgr.BF16}[dtype]] * len(shapes), sm_count=sms)
+    for begin, end in zip([0] + ends[:-1], ends):
+        assert sum(it.path == path and begin <= it.tensor < end for it in items) > blocks * sms
+        if path == 1:
+            assert sum(it.path == 0 and begin <= it.tensor < end for it in items) > 8 * sms
+    a, b = (Pair(shapes, ranks, dtype, bits=16, seed=6) for _ in range(2))
+    eps = 1e-3
+    for seed in (5, 6):
+        b.lib.perturb(seed, eps)
+        if seed == 5:
+            a.call_and_check(seed, eps, lambda: a.lib.perturb_layers(seed, eps, ends), "perturb_layers(+eps)")
+        else:
+            a.lib.perturb_layers(seed, eps, ends)
+        for p in (a, b):
+            (p.lib.perturb_layers(seed, -2 * eps, ends) if p is a else p.lib.perturb(seed, -2 * eps))
+            p.lib.restore_update(seed, 2.3, 1.8, 1e-4)
+        torch.cuda.synchronize()
+        assert all(torch.equal(x, y) for x, y in zip(a.theta, b.theta))
+    assert a.lib.device_status() == 0

@@ -9,6 +9,7 @@ import oracle
 from paper_2601_12917_b200 import synth, zgr
 
 from helpers import Pair
+from test_plan import plan
 
 pytestmark = pytest.mark.gpu
 
@@ -53,6 +54,22 @@ def test_tile_kernel_norms_codes_and_several_seeds(dtype):
     seeds, lp, lm = [41, 42, 43], [2.1, 1.6, 2.4], [1.9, 2.0, 1.8]
     coeffs = [oracle.update_coefficient(0.0, a, b, p.eps, 1e-4) for a, b in zip(lp, lm)]
     p.call_and_check_multi(seeds, coeffs, lambda: p.lib.restore_update_multi(seeds, lp, lm, 1e-4), "three seeds")
+
+
+# Sets with more items than SMs: the tile kernel draws on its item counter (below about 29 M weights each block has a share of its own),
+# in items of the two heights that the planner chose, and puts the counter back to zero: five sweeps of one context in a row.
+@pytest.mark.parametrize("dtype,shapes,ranks", [("bf16", [(4000, 5001), (2000, 5001), (1, 77)], [16, 16, 0]),
+                                                 ("f32", [(4000, 5128), (2000, 5128), (1, 77)], [24, 24, 0])])
+def test_tile_items_from_the_counter(dtype, shapes, ranks):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    items = [it for it in plan(shapes, ranks, [{"f32": zgr.F32, "bf16": zgr.BF16}[dtype]] * 3, sm_count=sms) if it.path == 3]
+    assert len(items) > sms and (32 + 16) * 40 >= 12 * sms        # more items than blocks, and enough tiles for the counter
+    assert len({(it.nrows_or_count + 127) // 128 for it in items}) > 1
+    p = Pair(shapes, ranks, dtype, bits=16, seed=9)
+    p.step(seed=3, lp=2.3, lm=1.7, lr=1e-4)
+    p.call_and_check(4, 1e-3, lambda: p.lib.perturb(4, 1e-3), "perturb")
+    p.call_and_check(4, -1e-3, lambda: p.lib.restore_update(4, 2.0, 2.0, 0.0), "restore")
+    assert p.lib.device_status() == 0
 
 
 # Low ranks: sets of 2^21 weights and more leave the CUDA-core kernel for the tile kernel, which is reported under the same path with its

@@ -127,6 +127,21 @@ def test_full_size_configurations(name):
         assert per_cta.max() / per_cta.mean() < 1.03
 
 
+# The tile kernel's large sets, whose item heights come from a replay of the hand-out: ragged rows in 16 bits, fp32 above rank 8, and
+# rank 8 on either side of the sizes between which fp32 sets take it; shares of small sets beside them.
+@pytest.mark.parametrize("sm_count", [148, 132, 1])
+@pytest.mark.parametrize("shapes,ranks,dtype,path", [
+    ([(1234, 4937), (4937, 1234), (1, 1234)] * 12, [16, 16, 0] * 12, zgr.BF16, 3), ([(6000, 5001)], [33], zgr.F16, 3),
+    ([(4096, 1024), (1024, 4096), (50265, 1024)] * 3, [32] * 9, zgr.F32, 3), ([(2000, 5128)] * 3, [64, 24, 9], zgr.F32, 3),
+    ([(1024, 2040)], [8], zgr.F32, 1), ([(1024, 2056)], [8], zgr.F32, 1), ([(8192, 4096)] * 3, [8] * 3, zgr.F32, 1), ([(8192, 8192)] * 4, [8] * 4, zgr.F32, 1),
+    ([(300, 2051)] * 7, [16] * 7, zgr.BF16, 3)])
+def test_large_sets_of_the_tile_kernel(shapes, ranks, dtype, path, sm_count):
+    for multi in (0, 1):
+        items = plan(shapes, ranks, [dtype] * len(shapes), sm_count=sm_count, multi=multi)
+        check_exact_cover(items, shapes)
+        assert {it.path for it in items if ranks[it.tensor] > 0} == {path}
+
+
 def test_alpha_one_plans_everything_as_isotropic_and_errors_are_reported():
     items = plan([(64, 256), (1, 100)], [8, 0], [zgr.BF16, zgr.BF16], alpha=1.0)
     assert {it.path for it in items} == {0}
