@@ -109,7 +109,9 @@ __device__ __forceinline__ void build_strip(const TensorDesc& td, const SweepPar
 #pragma unroll
     for (int i = 0; i < 8; ++i) g[i] = 0.0f;
     if (k < td.rank && c_first < cols) {
-      if (td.q != nullptr && k < td.qrows) {
+      if (td.q != nullptr && k < td.qrows && (cols & 7) == 0) {
+        guided8<BITS, PRECISE, MULTI>(td, p, k, c_first, g);      // eight codes of one row in one load
+      } else if (td.q != nullptr && k < td.qrows) {
         float cb = p.term[0].cb;
         if (MULTI)
           for (int q = 1; q < p.n_terms; ++q) cb += p.term[q].cb;

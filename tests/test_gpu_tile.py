@@ -56,6 +56,21 @@ def test_tile_kernel_norms_codes_and_several_seeds(dtype):
     p.call_and_check_multi(seeds, coeffs, lambda: p.lib.restore_update_multi(seeds, lp, lm, 1e-4), "three seeds")
 
 
+# Codes for rows of whole octets, which the strip reads eight at a time, all rows of the tensor coded or the first seven; one and two seeds.
+@pytest.mark.parametrize("code_bits", [8, 4])
+@pytest.mark.parametrize("n_rows", [None, 7])
+def test_tile_kernel_codes_in_whole_octets(code_bits, n_rows):
+    p = Pair([(150, 264), (1, 25)], [12, 0], "f32", bits=16, seed=8)
+    if code_bits == 8:
+        p.set_dtc(0, *synth.dtc_payload(12, 264, seed=3), bits=8, n_rows=n_rows)
+    else:
+        p.set_dtc(0, *oracle.dtc_quantise_int4(oracle.coeffs(9, 0, 16, 12, 264)), bits=4, n_rows=n_rows)
+    p.step(seed=31, lp=2.2, lm=1.9, lr=1e-4)
+    seeds, lp, lm = [41, 42], [2.1, 1.6], [1.9, 2.0]
+    coeffs = [oracle.update_coefficient(0.0, a, b, p.eps, 1e-4) for a, b in zip(lp, lm)]
+    p.call_and_check_multi(seeds, coeffs, lambda: p.lib.restore_update_multi(seeds, lp, lm, 1e-4), "two seeds")
+
+
 # Sets with more items than SMs: the tile kernel draws on its item counter (below about 29 M weights each block has a share of its own),
 # in items of the two heights that the planner chose, and puts the counter back to zero: five sweeps of one context in a row.
 @pytest.mark.parametrize("dtype,shapes,ranks", [("bf16", [(4000, 5001), (2000, 5001), (1, 77)], [16, 16, 0]),
