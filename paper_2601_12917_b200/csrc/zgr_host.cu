@@ -221,16 +221,18 @@ LowRank low_rank(const zgr_tensor* tensors, int32_t n) {
 // Rank <= 8 takes no operand copies in two fp16 parts: those hold 22 bits of entries up to 2^16 2^-ushift, and the fp32
 // multiply-adds of the CUDA-core kernel, which serves the same tensors in a smaller set, have neither limit (the TMA-staged kernel:
 // 776 us at 300 M).
-int tensor_core_kind(const zgr_tensor& t, bool guided_on, const LowRank& lr, int bits) {
+int tensor_core_kind(const zgr_tensor& t, bool guided_on, const LowRank& lr) {
   if (!guided_on || t.rank == 0 || t.rows >= (int64_t{1} << 31) - 256) return 0;
   const bool vec = whole_octets(t);
   if (vec && t.rank <= 8) {
     const int64_t set = t.dtype == ZGR_F32 ? lr.f32 : lr.half;
     if (set < (int64_t{1} << 21)) return 0;
-    // (fp32 sets that keep every SM busy for long run at the power cap, where the kernel without tensor cores is ahead: 354 M
-    // weights, rank 8, in steady state 1885 us a step there and 1918 here, in short runs rank 4 1538 and 1600, 1718 and 1903 with
-    // 32 random bits; 42 M, rank 8: 289 and 208, rank 4: 209 and 210)
-    if (t.dtype == ZGR_F32 && ((t.rank <= 4 && set >= (int64_t{1} << 25)) || set >= (int64_t{1} << 28))) return 0;
+    // (fp32 sets that keep every SM busy for long run at the power cap, where the kernel without tensor cores catches up, the sooner
+    // the narrower its contraction and the fewer of it are padding.  us a step on CUDA cores / on the tile kernel, 16 random bits:
+    // rank 4  24 M 151 / 140, 42 M 209 / 210;  rank 5  64 M 388 / 361, 128 M 721 / 701, 160 M 892 / 892;  rank 8  48 M 290 / 260,
+    // 64 M 361 / 361, 96 M 511 / 530, 160 M 837 / 875, 354 M 1885 / 1918; with 32 bits rank 8 48 M 332 / 298, 64 M 405 / 416)
+    const int64_t line = int64_t{1} << (t.rank <= 4 ? 25 : (t.rank == 8 ? 26 : 28));
+    if (t.dtype == ZGR_F32 && set >= line) return 0;
     return 2;
   }
   // (the TMA-staged kernel keeps the high counter word of the generator fixed: fewer than 2^32 blocks of four elements)
@@ -916,7 +918,7 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
     td.ushift = 0;
     for (void*& copy : td.Ucopy) copy = nullptr;
     // tcgen05 kernels: row-major copies of U in parts, and three tensor maps (those of the copies once these have their place)
-    const int kind = umma_wanted() && encode_tiled_fn() != nullptr ? tensor_core_kind(t, guided_on, lr, cfg->bits_per_normal) : 0;
+    const int kind = umma_wanted() && encode_tiled_fn() != nullptr ? tensor_core_kind(t, guided_on, lr) : 0;
     if (kind == 2 || (kind == 1 && make_map_16bit(&ctx->tmaps[static_cast<size_t>(3 * l)], t.data, t.rows, t.cols, 64))) {
       td.kpad = t.rank <= 16 ? 16 : (t.rank <= 32 ? 32 : 64);
       // entries of an orthonormal U are about 1/sqrt(rows): scaled by 2^ushift they sit between 1 and 2 in size
@@ -1608,7 +1610,7 @@ int zgr_debug_plan(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, 
       td.kpad = t.rank <= 16 ? 16 : (t.rank <= 32 ? 32 : 64);
       td.Ufrag = reinterpret_cast<const uint4*>(uintptr_t{16});   // marker only: never dereferenced by the planner
     }
-    const int kind = tcgen05 ? tensor_core_kind(t, guided_on, lr, cfg->bits_per_normal) : 0;
+    const int kind = tcgen05 ? tensor_core_kind(t, guided_on, lr) : 0;
     if (kind != 0) {
       td.kpad = t.rank <= 16 ? 16 : (t.rank <= 32 ? 32 : 64);
       (kind == 1 ? td.umma : td.tile) = 1;
