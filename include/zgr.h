@@ -65,11 +65,11 @@ typedef struct zgr_ctx zgr_ctx; /* opaque; created by zgr_init, released by zgr_
 /* One weight tensor.  1-D tensors are given as rows = 1, cols = length, U = NULL, rank = 0. */
 typedef struct {
   void* data;       /* device; rows*cols elements of `dtype`, row-major, contiguous, updated in place.
-                       Must be aligned to the element size.  16-byte alignment and cols a multiple of
-                       eight elements select the kernels that stage whole tiles; other shapes, and fp32
-                       storage with rank > 8, are served by a tile kernel that works on octets across
-                       row ends (tensor-core contraction with three bf16 parts per operand, as accurate
-                       as fp32 multiply-adds) */
+                       Must be aligned to the element size.  16-bit storage with rank > 8, 16-byte alignment
+                       and cols a multiple of eight elements is staged in whole tiles; all else with a
+                       subspace, except small sets of rank <= 8 and large fp32 ones, is served by a tile
+                       kernel that works on octets across row ends (tensor-core contraction with three bf16
+                       parts per operand, as accurate as fp32 multiply-adds) */
   int64_t rows;     /* m_l >= 1 */
   int64_t cols;     /* n_l >= 1 */
   int32_t dtype;    /* ZGR_F32 | ZGR_F16 | ZGR_BF16 */

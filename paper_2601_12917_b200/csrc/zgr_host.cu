@@ -32,7 +32,7 @@ struct Group {
   int grid = 0;
   int64_t elements = 0;                                   // weights covered by one launch
   double* d_item_stats = nullptr;                         // kStatSlots x 3 doubles per item (norm bookkeeping), allocated on first use
-  int32_t* d_sched = nullptr;                             // CUDA-core kernels: two item counters (caller's stream, library's second stream)
+  int32_t* d_sched = nullptr;                             // CUDA-core and tile kernels: two item counters (caller's stream, library's second stream)
   std::vector<int32_t> first_item;                        // per tensor l: index of its first item in `items` (size n + 1; items are in tensor order)
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> timed;  // per-launch events while profiling is on
 };

@@ -6,11 +6,11 @@
 // in registers / shared memory and never stored.
 //
 //   sweep_iso      tensors without a subspace (1-D tensors, rank 0) or with b = 0
-//   sweep_fma      rank <= 8 on small or large fp32 sets: U G on CUDA-core FMAs in fp32, G strip in shared memory and registers
+//   sweep_fma      rank <= 8, small sets and large fp32 ones: U G on CUDA-core FMAs in fp32, G strip in shared memory and registers
 //   sweep_mma      rank  > 8, fallback of the tcgen05 kernels: mma.sync, bf16 hi/lo split operands (three products per
 //                  tile, fp32 accumulate), accumulators initialised with theta
 //   sweep_generic  any shape or alignment, one element per thread (fallback of the tile kernel)
-// The tcgen05 kernels are in zgr_umma.cu (weights staged by TMA) and zgr_tile.cu (fp32 and ragged rows).
+// The tcgen05 kernels are in zgr_umma.cu (weights staged by TMA) and zgr_tile.cu (fp32, ragged rows, rank <= 8).
 //
 // All kernels are persistent over a device-resident list of work items, so a sweep over a model with hundreds of tensors is
 // a handful of launches.

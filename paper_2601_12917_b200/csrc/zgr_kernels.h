@@ -18,7 +18,7 @@ enum Path { PATH_ISO = 0, PATH_FMA = 1, PATH_MMA = 2, PATH_GENERIC = 3, PATH_UMM
 struct KernelChoice {
   int path;   // Path
   int dtype;  // ZGR_F32 | ZGR_F16 | ZGR_BF16
-  int kpad;   // FMA: 4 or 8;  MMA: 16, 32 or 64;  otherwise 0
+  int kpad;   // contraction width.  FMA: 4 or 8;  MMA, UMMA and the tile kernel (see is_tile): 16, 32 or 64;  otherwise 0
   int bits;   // 32 or 16 random bits per normal
   int precise;  // accurate Gaussian transform (tensors stored in fp32)
 };
@@ -28,7 +28,7 @@ struct KernelChoice {
 constexpr int iso_blocks_per_sm(bool precise, bool multi, bool stats) { return !precise && !multi && !stats ? 8 : 5; }
 
 // The groups that sweep_tile_kernel serves: rank <= 8 tensors in whole octets are counted under the path of the CUDA-core
-// kernel (whose contraction widths are 4 and 8), the others under that of the fallback kernel (whose width is 0).
+// kernel (whose own widths are 4 and 8), the others under that of the fallback kernel (whose own width is 0).
 inline bool is_tile(const KernelChoice& kc) { return (kc.path == PATH_FMA && kc.kpad == 16) || (kc.path == PATH_GENERIC && kc.kpad > 0); }
 
 int mma_strip_cols(int kpad);     // columns of a CTA strip on the tensor-core path
@@ -60,8 +60,8 @@ cudaError_t launch_sweep_umma(const KernelChoice& kc, const SweepParams& p, cons
 // Test hook: the sweep kernel with its fp32 results diverted to p.zout (see the ZOUT parameter of the kernel).
 cudaError_t launch_debug_z_umma(const KernelChoice& kc, const SweepParams& p, const CUtensorMap* tmaps, int* error, int grid, cudaStream_t st);
 cudaError_t launch_stats_umma(const KernelChoice& kc, const SweepParams& p, const CUtensorMap* tmaps, int* error, int grid, cudaStream_t st);
-// Sweep of the other guided tensors (fp32 with rank > 8, rows that are not a multiple of eight elements).  tmaps: the three
-// bf16 parts of U per tensor; kc.kpad = contraction width.
+// Sweep of the other guided tensors that a tensor-core kernel serves (fp32, rank <= 8, rows that are not a multiple of eight
+// elements).  tmaps: the three bf16 parts of U per tensor; kc.kpad = contraction width.
 int tile_strip_cols();
 cudaError_t launch_sweep_tile(const KernelChoice& kc, const SweepParams& p, const CUtensorMap* tmaps, int* error, int grid, cudaStream_t st);
 // Rebuild of the row-major operand copies of U for a device-resident list of tensors in one launch (grid.y = job).

@@ -15,7 +15,7 @@
 //
 // One launch does all of it (basis_kernel): every CTA keeps its rows in shared memory as doubles through both passes, the
 // partial Gram matrices meet in global memory (L2) between barriers, and each CTA factors the r x r sum for itself, since
-// that is cheaper than another barrier.  Up to about a thousand rows per CTA the grid is a single cluster of 8 or 16 CTAs, whose
+// that is cheaper than another barrier.  Up to 4096 rows in all at rank 16, 1024 above, the grid is a single cluster of 16 or 8 CTAs, whose
 // barrier is a hardware one and whose partials every CTA adds up directly; larger inputs use one CTA per SM, launched
 // cooperatively, with a counter barrier and the sum of the partials spread over the grid.  The job is bound by latency (a
 // 2048 x 16 input is 131 KB): the six launches, the memset and the copies of the status that it took before were 95 us a

@@ -1,5 +1,6 @@
-// Sweep with a tensor-core contraction for the guided tensors that the TMA-staged kernel (zgr_umma.cu) cannot take:
-// fp32 storage with rank > 8, and any storage whose rows are not a multiple of eight elements long.
+// Sweep with a tensor-core contraction for the guided tensors that the TMA-staged kernel (zgr_umma.cu) cannot take: fp32 storage with
+// rank > 8, any storage whose rows are not a multiple of eight elements long, and sets of rank <= 8 that are worth a
+// tensor-core kernel (tensor_core_kind in zgr_host.cu has the sizes).
 //     theta <- rnd(theta + c (a Z + b U G))            (Eq. (perturbation) applied as in Algorithm 1)
 //
 // Layout.  Generator blocks run along the flattened tensor, eight elements ("an octet") at a time, so in a tensor whose
@@ -9,7 +10,8 @@
 // tail of the octet that began in the row before.  An owned octet reaches up to 7 columns beyond the strip, so the
 // product tile is computed 144 columns wide.
 //
-// Pipeline (one CTA per SM; the first item of a CTA is its own index, the others come from a counter in global memory):
+// Pipeline (one CTA per SM; small sets give it a contiguous share of the items, otherwise its first item is its own index and
+// the others come from a counter in global memory):
 //   warp 0   hands out the items through a ring of four, TMA loads of U, 128 rows at a time, pre-split into three bf16 parts
 //   warp 1   tcgen05.mma:  D = c b U G  (128 x 144, fp32) into one of three tensor-memory buffers
 //   warps 2-17  coefficient strips c b G (three bf16 parts, K-major) into shared memory, one item ahead where two strips

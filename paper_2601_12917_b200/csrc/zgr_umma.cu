@@ -1,8 +1,9 @@
 // Blackwell-native sweep for 16-bit weights with a rank > 8 subspace:
 //     theta <- rnd(theta + c (a Z + b U G))            (Eq. (perturbation) applied as in Algorithm 1)
 //
-// The generator and the Gaussian transform alone fill about 80 % of an SM's issue slots at the rate
-// HBM can feed the weights, so everything else is taken out of the SM's instruction stream:
+// The generator and the Gaussian transform are most of what an SM has to issue at the rate HBM can feed the weights (the whole
+// kernel issues in 55 % of the cycles, special functions fill 63 % of their pipe at rank 16), so everything else is taken out of
+// the SM's instruction stream:
 //
 //   * TMA brings a 128-row x NS-column tile of theta (and the matching 128 x KP tiles of U, pre-split
 //     into fp16 hi/lo) into shared memory, and writes the finished tile back; no thread issues a
@@ -26,7 +27,8 @@
 // Warp roles: warp 0 = TMA producer (loads and stores), warp 1 = MMA issuer and owner of the tensor
 // memory allocation, warps 2.. = epilogue.  The two single-thread roles run in the lane picked by
 // elect.sync, which lets their loop state and descriptors live in uniform registers.  One CTA per SM
-// (the shared-memory footprint enforces it), persistent over a static round-robin list of work items.
+// (the shared-memory footprint enforces it), persistent over its work items: a contiguous share of small sets, every
+// gridDim.x-th item of the others.
 //
 // Every wait on an mbarrier is bounded: when a wait gives up it records where in *p.error, raises a
 // CTA-wide abort flag, and all roles fall through to the common exit, where the producer drains its
