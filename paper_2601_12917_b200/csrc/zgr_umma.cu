@@ -548,26 +548,36 @@ __global__ void __launch_bounds__(UmmaCfg<KP>::THREADS, 1) sweep_umma_kernel(con
                                               Pack16<T>::pack(acc[6], acc[7])));
               }
             } else {
-              // four octets per thread, kept independent so that their generator chains interleave (one after the other with 32
-              // random bits per normal, where an octet is two generator blocks: 3615 -> 3540 us on four LLaMA-7B-shaped layers)
+              // four octets per thread, one generator chain after the other, each beside the transform of the octet before it (see
+              // normals8_acc_linked; with 32 random bits per normal, where an octet is two generator blocks, only the order of the
+              // octets is kept: 3615 -> 3540 us on four LLaMA-7B-shaped layers)
               float acc[4][8];
+              const uint32_t zero = static_cast<uint32_t>(p.early) >> 1;      // (early is 0 or 1)
+              uint32_t link = 0;
 #pragma unroll
               for (int o = 0; o < 4; ++o)
 #pragma unroll
                 for (int i = 0; i < 8; ++i) acc[o][i] = __uint_as_float(o < 2 ? h0[8 * (o & 1) + i] : h1[8 * (o & 1) + i]);
 #pragma unroll
               for (int o = 0; o < 4; ++o) {
-                normals8_acc_pre<BITS>(p.term[0].keys, pre, oct0_lo + static_cast<uint32_t>(o), p.term[0].iso, acc[o]);
-                if (BITS == 32) asm volatile("" ::: "memory");
+                if constexpr (BITS == 32) {
+                  normals8_acc_pre<BITS>(p.term[0].keys, pre, oct0_lo + static_cast<uint32_t>(o), p.term[0].iso, acc[o]);
+                  asm volatile("" ::: "memory");
+                } else {
+                  normals8_acc_linked(p.term[0].keys, pre, oct0_lo + static_cast<uint32_t>(o), p.term[0].iso, zero, link, acc[o]);
+                }
               }
               if (MULTI) {
-                // term by term over all four octets: the keys are fetched once per term, and four chains interleave
+                // term by term over all four octets: the keys are fetched once per term
 #pragma unroll 1
                 for (int q = 1; q < p.n_terms; ++q) {
                   const PhiloxKeys& keys = p.term[q].keys;
                   const PhiloxPre pre_q = philox_pre(0u, tid, keys);
 #pragma unroll
-                  for (int o = 0; o < 4; ++o) normals8_acc_pre<BITS>(keys, pre_q, oct0_lo + static_cast<uint32_t>(o), p.term[q].iso, acc[o]);
+                  for (int o = 0; o < 4; ++o) {
+                    if constexpr (BITS == 32) normals8_acc_pre<BITS>(keys, pre_q, oct0_lo + static_cast<uint32_t>(o), p.term[q].iso, acc[o]);
+                    else normals8_acc_linked(keys, pre_q, oct0_lo + static_cast<uint32_t>(o), p.term[q].iso, zero, link, acc[o]);
+                  }
                 }
               }
 #pragma unroll
