@@ -296,7 +296,7 @@ int zgr_debug_z_tcgen05(zgr_ctx* ctx, uint64_t seed, int32_t tensor, float* dev_
  * family serves which part of which tensor.  Test hook for the planner: the items of a plan must cover
  * every element of every tensor exactly once.  path: 0 isotropic (elements [row0_or_e0, +nrows_or_count) of
  * the tensor), otherwise rows [row0_or_e0, +nrows_or_count) x columns [col0, +ncols): 1 rank <= 8,
- * 2 legacy tensor-core, 3 any shape, 4 tcgen05 with TMA-staged weights.  kpad > 8 on paths 1 and 3 is the tile kernel's contraction
+ * 2 legacy tensor-core, 3 any shape, 4 tcgen05 with TMA-staged weights.  kpad > 8 on paths 1 and 3 is the three-part tensor-core kernels' contraction
  * width (an item's last octet of a row may reach into the next strip there).  `tensors[].data / U` are only inspected for alignment and
  * null-ness.  tcgen05 != 0 plans as on a device where tensor maps can be made; multi != 0 gives the plan of
  * the multi-seed sweeps.  Up to max_items items are written to out; *n_items receives the full count.

@@ -32,7 +32,7 @@ struct Group {
   int grid = 0;
   int64_t elements = 0;                                   // weights covered by one launch
   double* d_item_stats = nullptr;                         // kStatSlots x 3 doubles per item (norm bookkeeping), allocated on first use
-  int32_t* d_sched = nullptr;                             // CUDA-core and tile kernels: two item counters (caller's stream, library's second stream)
+  int32_t* d_sched = nullptr;                             // CUDA-core and three-part kernels: two item counters (caller's stream, library's second stream)
   std::vector<int32_t> first_item;                        // per tensor l: index of its first item in `items` (size n + 1; items are in tensor order)
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> timed;  // per-launch events while profiling is on
 };
@@ -188,56 +188,92 @@ EncodeTiledFn encode_tiled_fn() {
   return fn;
 }
 
-// 2-D map over a row-major 16-bit matrix (rows x cols, row pitch = cols), box = box_cols x 128 rows,
+// 2-D map over a row-major matrix of elements of `bytes` (2 or 4) bytes, rows `pitch` elements apart, box = box_cols x box_rows,
 // swizzle matching the box's row length in bytes (32, 64 or 128).
-bool make_map_16bit(CUtensorMap* out, const void* base, int64_t rows, int64_t cols, int box_cols) {
+bool make_map(CUtensorMap* out, const void* base, int bytes, int64_t rows, int64_t cols, int64_t pitch, int box_rows, int box_cols) {
   EncodeTiledFn fn = encode_tiled_fn();
   if (!fn) return false;
   const cuuint64_t dims[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
-  const cuuint64_t strides[1] = {static_cast<cuuint64_t>(cols) * 2};
-  const cuuint32_t box[2] = {static_cast<cuuint32_t>(box_cols), 128};
+  const cuuint64_t strides[1] = {static_cast<cuuint64_t>(pitch * bytes)};
+  const cuuint32_t box[2] = {static_cast<cuuint32_t>(box_cols), static_cast<cuuint32_t>(box_rows)};
   const cuuint32_t estr[2] = {1, 1};
-  const int row_bytes = box_cols * 2;
+  const int row_bytes = box_cols * bytes;
   const CUtensorMapSwizzle sw = row_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : (row_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
-  return fn(out, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, sw,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  return fn(out, bytes == 4 ? CU_TENSOR_MAP_DATA_TYPE_UINT32 : CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, const_cast<void*>(base), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+bool make_map_16bit(CUtensorMap* out, const void* base, int64_t rows, int64_t cols, int box_cols) {
+  return make_map(out, base, 2, rows, cols, cols, 128, box_cols);
 }
 
-// Weights in rank <= 8 tensors whose rows are whole octets, by storage: the kernel that serves them depends on how many there are.
-struct LowRank {
-  int64_t f32 = 0, half = 0;
-};
+// The maps of a tensor of sweep_staged_kernel: of its weights, one per residue of the row modulo 8 if the rows are no multiple of eight
+// elements (see zgr_staged.cu), and behind them the three parts of U, rows_pad x kpad each.
+int n_weight_maps(const TensorDesc& td) { return (td.cols & 7) ? 8 : 1; }
+bool make_weight_maps(CUtensorMap* out, const TensorDesc& td, void* data, int bytes) {
+  if ((td.cols & 7) == 0) return make_map(out, data, bytes, td.rows, td.cols, td.cols, 128, 128 / bytes);
+  for (int64_t i = 0; i < 8 && i < td.rows; ++i) {      // (residues without rows have no boxes)
+    const int64_t shift = -(i * td.cols) & 7;
+    if (!make_map(out + i, static_cast<uint8_t*>(data) + (i * td.cols + shift) * bytes, bytes, (td.rows - i + 7) / 8, (td.cols - shift) & ~int64_t{7},
+                  8 * td.cols, 32, 128 / bytes))
+      return false;
+  }
+  return true;
+}
+int64_t copy_rows(const TensorDesc& td) { return td.staged && (td.cols & 7) ? (td.rows + 255) / 256 * 256 : (td.rows + 127) / 128 * 128; }
+
 bool whole_octets(const zgr_tensor& t) { return (reinterpret_cast<uintptr_t>(t.data) & 15) == 0 && (t.cols % 8 == 0); }
-LowRank low_rank(const zgr_tensor* tensors, int32_t n) {
-  LowRank lr;
-  for (int32_t l = 0; l < n; ++l)
-    if (tensors[l].rank > 0 && tensors[l].rank <= 8 && whole_octets(tensors[l])) (tensors[l].dtype == ZGR_F32 ? lr.f32 : lr.half) += tensors[l].rows * tensors[l].cols;
-  return lr;
+// Weights of a model by storage, of those kinds of tensors whose kernel depends on how many there are: rank <= 8 in whole octets, and
+// all that the kernels with three-part operands may serve.
+struct SetSizes {
+  int64_t low[2] = {0, 0}, three_part[2] = {0, 0};      // [0] 16-bit, [1] fp32
+};
+SetSizes set_sizes(const zgr_tensor* tensors, int32_t n) {
+  SetSizes s;
+  for (int32_t l = 0; l < n; ++l) {
+    const zgr_tensor& t = tensors[l];
+    if (t.rank == 0) continue;
+    const int f32 = t.dtype == ZGR_F32;
+    const bool low = t.rank <= 8 && whole_octets(t);
+    if (low) s.low[f32] += t.rows * t.cols;
+    if (low || f32 || !whole_octets(t)) s.three_part[f32] += t.rows * t.cols;
+  }
+  return s;
 }
 
-// Which tcgen05 kernel serves a tensor: 1 the TMA-staged one (16-bit weights in rows that TMA can address, rank > 8), 2 the tile
-// kernel (everything else with a subspace), 0 neither.  Small sets of rank <= 8 stay with the CUDA-core kernel, which starts
-// faster and cuts finer (a step of 2.0 M bf16 weights, rank 8: 25 us there; 4.0 M: 42, 28 on the tile kernel; 300 M: 1163, 1018).
+// Which kernel family serves a tensor: 1 the TMA-staged one with two-part operands (16-bit weights in whole octets, rank > 8), 2 those with
+// three-part operands (everything else with a subspace), 0 neither.  Small sets of rank <= 8 stay with the CUDA-core kernel, which starts
+// faster and cuts finer (a step of 2.0 M bf16 weights, rank 8: 25 us there; 4.0 M: 42, 28 on the tile kernel).
 // Rank <= 8 takes no operand copies in two fp16 parts: those hold 22 bits of entries up to 2^16 2^-ushift, and the fp32
 // multiply-adds of the CUDA-core kernel, which serves the same tensors in a smaller set, have neither limit (the TMA-staged kernel:
 // 776 us at 300 M).
-int tensor_core_kind(const zgr_tensor& t, bool guided_on, const LowRank& lr) {
+int tensor_core_kind(const zgr_tensor& t, bool guided_on, const SetSizes& sizes) {
   if (!guided_on || t.rank == 0 || t.rows >= (int64_t{1} << 31) - 256) return 0;
   const bool vec = whole_octets(t);
   if (vec && t.rank <= 8) {
-    const int64_t set = t.dtype == ZGR_F32 ? lr.f32 : lr.half;
+    const int64_t set = sizes.low[t.dtype == ZGR_F32];
     if (set < (int64_t{1} << 21)) return 0;
-    // (fp32 sets that keep every SM busy for long run at the power cap, where the kernel without tensor cores catches up, the sooner
-    // the narrower its contraction and the fewer of it are padding.  us a step on CUDA cores / on the tile kernel, 16 random bits:
-    // rank 4  24 M 151 / 140, 42 M 209 / 210;  rank 5  64 M 388 / 361, 128 M 721 / 701, 160 M 892 / 892;  rank 8  48 M 290 / 260,
-    // 64 M 361 / 361, 96 M 511 / 530, 160 M 837 / 875, 354 M 1885 / 1918; with 32 bits rank 8 48 M 332 / 298, 64 M 405 / 416)
-    const int64_t line = int64_t{1} << (t.rank <= 4 ? 25 : (t.rank == 8 ? 26 : 28));
-    if (t.dtype == ZGR_F32 && set >= line) return 0;
+    // (at rank 4 half of the contraction is padding, and on fp32 sets that keep every SM busy for long the CUDA-core kernel catches up.
+    // us a step on CUDA cores / staged, 16 random bits:  rank 4  24 M 154 / 136, 63 M 332 / 331, 126 M 629 / 635, 1.2 G 4333 / 4371;
+    // rank 8  63 M 365 / 333, 126 M 681 / 640, 354 M 1796 / 1759; with 32 bits 101 M 616 / 573)
+    if (t.dtype == ZGR_F32 && t.rank <= 4 && set >= (int64_t{1} << 26)) return 0;
     return 2;
   }
   // (the TMA-staged kernel keeps the high counter word of the generator fixed: fewer than 2^32 blocks of four elements)
   if (vec && t.dtype != ZGR_F32 && t.rows * t.cols < (int64_t{1} << 34)) return t.cols < (int64_t{1} << 31) - 256 ? 1 : 0;
   return 2;
+}
+
+// Which of the two kernels with three-part operands: 1 the staged one, 0 the tile kernel.  TMA wants the weights on a 16-byte boundary
+// and rows that hold a whole octet wherever it begins; the staged kernel keeps the high counter word of the generator fixed.
+// Small sets stay with the tile kernel, whose sixteen epilogue warps share every tile (two groups on alternate tiles leave half of
+// them idle when a CTA has one or two): us a step tile / staged, bf16 rank 8 2.4 M 26.8 / 29.6, 4.0 M 32.1 / 31.9; ragged 16-bit rank 16
+// 1.6 M 34.0 / 42.6, 2.7 M 47.0 / 45.5, 18 M 135 / 106; fp32 1.0 M 27.6 / 28.7, 3.1 M 41.4 / 39.9.  fp32 rows that are no multiple of eight
+// elements do so at any size: 96 M weights of rank 16 in rows of 1001 and 4001 469 / 479 (the accurate transform hides what the tile
+// kernel spends on its transposition, and the residues cost half-empty tiles).
+int staged_kind(const zgr_tensor& t, const SetSizes& sizes) {
+  const int f32 = t.dtype == ZGR_F32;
+  return (reinterpret_cast<uintptr_t>(t.data) & 15) == 0 && t.cols >= 16 && t.cols < (int64_t{1} << 31) - 256 && t.rows * t.cols < (int64_t{1} << 34) &&
+         !(f32 && (t.cols & 7) != 0) && sizes.three_part[f32] >= 5 * (int64_t{1} << 19);
 }
 
 bool umma_wanted() {
@@ -283,10 +319,10 @@ double share_out(const std::vector<TensorDesc>& descs, const std::vector<Member>
     if (emit) starts.assign(1, 0);
     for (const Member& m : members) {
       const TensorDesc& t = descs[m.tensor];
-      const int64_t blocks = (t.rows + 127) / 128;
+      const int64_t step = m.row_step, blocks = (t.rows + step - 1) / step;
       for (int64_t c0 = 0; c0 < t.cols; c0 += strip_cols) {
         const int ncols = static_cast<int>(std::min<int64_t>(strip_cols, t.cols - c0));
-        const double wide = (ncols + 127) / 128, begin = strip_cost * t.rank * wide + item_cost;
+        const double tiles = (ncols + 127) / 128, wide = tiles * static_cast<double>(step / 128), begin = strip_cost * t.rank * tiles + item_cost;
         for (int64_t at = 0, take; at < blocks; at += take) {
           if (room < begin + wide && room < share) {
             ++cta;
@@ -295,7 +331,7 @@ double share_out(const std::vector<TensorDesc>& descs, const std::vector<Member>
           }
           take = std::min<int64_t>(std::max<int64_t>(static_cast<int64_t>((room - begin) / wide + 1e-9), 1), blocks - at);
           room -= begin + wide * static_cast<double>(take);
-          if (emit) items.push_back(WorkItem{m.tensor, ncols, 128 * at, std::min<int64_t>(128 * take, t.rows - 128 * at), c0});
+          if (emit) items.push_back(WorkItem{m.tensor, ncols, step * at, std::min<int64_t>(step * take, t.rows - step * at), c0});
         }
       }
     }
@@ -339,7 +375,7 @@ void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>&
   const int64_t sms = sm_count;
   if (tile ? tiles < 12 * sms : g.kc.path == PATH_UMMA && tiles < 24 * sms) {
     // per 128 columns and rank about a hundredth of a tile for the strip, twice that for fp32 (anything from 1/60 to 1/200 gives the
-    // same times); an item has a pipeline to fill, which the tile kernel does ahead where two strips fit
+    // same times); an item has a pipeline to fill, which the three-part kernels do ahead where two strips fit
     const double strip_cost = g.kc.precise ? 0.02 : 0.01;
     const double item_cost = tile && g.kc.kpad < 64 ? 0.3 : 0.7;
     const int widest = members.empty() ? 128 : members[0].strip;
@@ -367,19 +403,24 @@ void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>&
   const double item_cost = 0.15 + (0.2 + 0.2 * g.kc.precise + (g.kc.precise && g.kc.bits == 32 ? 0.2 : 0.0)) * ((19 * g.kc.kpad + 511) / 512) +
                            (g.kc.kpad == 64 ? 0.3 : 0.0);
   double best = 0.0;
+  const bool spans = !members.empty() && members[0].row_step == 256;      // (one step for all tensors of a group)
+  const auto blocks_of = [&](int64_t rows) { return spans ? (rows + 255) / 256 * 2 : (rows + 127) / 128; };
+  bool even = false;                                   // (long sweeps) the best so far is even when dealt out in turn
   std::vector<WorkItem> trial;
   std::vector<double> dealt(static_cast<size_t>(sm_count)), free_at(static_cast<size_t>(sm_count));
-  for (int64_t big : {16, 12, 8, 6, 4, 3, 2, 1})
+  for (int64_t big : {16, 12, 8, 9, 6, 4, 3, 2, 1})
     for (int64_t small : {big, std::max<int64_t>(big / 4, 1)}) {
-      if (tiles >= 64 * sms && big != 8 && big != 4) continue;
-      if (best > 0.0 && (small == big ? tiles / big > 16 * sms : tiles / big > 10 * sms || big == 1)) continue;
+      // (long sweeps: eight, or nine if eight deals unevenly)
+      if (tiles >= 64 * sms ? small != big || (big != 8 && big != 9) || even : big == 9) continue;
+      if (spans && (big & 3) != 0 && big != 2) continue;      // (rows in spans of 256: nothing between two and four blocks, and six is left out)
+      if (best > 0.0 && tiles < 64 * sms && (small == big ? tiles / big > 16 * sms : tiles / big > 10 * sms || big == 1)) continue;
       // No schedule ends before the mean load: heights that cannot win are not cut into items, nor replayed to their end (the
       // search is a fourth of the time that setting up such a set takes).
       const double last = 0.5 * (static_cast<double>(small) + item_cost);
       if (best > 0.0) {
         int64_t done = 0, n_items = 0;
         for (const Member& m : members) {
-          const int64_t strips = (descs[m.tensor].cols + 127) / 128, blocks = (descs[m.tensor].rows + 127) / 128, h = 3 * done < 2 * tiles ? big : small;
+          const int64_t strips = (descs[m.tensor].cols + 127) / 128, blocks = blocks_of(descs[m.tensor].rows), h = 3 * done < 2 * tiles ? big : small;
           const int64_t chunks = (descs[m.tensor].rows + 128 * h - 1) / (128 * h), even = (blocks + chunks - 1) / chunks;
           n_items += strips * ((blocks + even - 1) / even);
           done += blocks * strips;
@@ -397,7 +438,7 @@ void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>&
       double end = 0.0;
       for (const WorkItem& w : trial) {
         if (best > 0.0 && end + last >= best) break;
-        const double at = free_at[0] + static_cast<double>((w.nrows_or_count + 127) / 128) + item_cost;
+        const double at = free_at[0] + static_cast<double>(blocks_of(w.nrows_or_count)) + item_cost;
         size_t i = 0;
         for (size_t c; (c = 2 * i + 1) < free_at.size(); i = c) {
           if (c + 1 < free_at.size() && free_at[c + 1] < free_at[c]) ++c;
@@ -414,6 +455,7 @@ void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>&
         for (size_t i = 0; i < trial.size(); ++i) dealt[i % dealt.size()] += static_cast<double>(trial[i].nrows_or_count) * trial[i].ncols;
         const double mean = std::accumulate(dealt.begin(), dealt.end(), 0.0) / static_cast<double>(dealt.size());
         if (*std::max_element(dealt.begin(), dealt.end()) > 1.025 * mean) end *= 2.0;
+        else even = true;
       }
       if (best == 0.0 || end < best) {
         best = end;
@@ -435,16 +477,16 @@ void plan(const std::vector<TensorDesc>& descs, const std::vector<int>& which, b
   int64_t target = total / (static_cast<int64_t>(sm_count) * 2 * 16);
   target = std::min<int64_t>(std::max<int64_t>(target, 16384), 524288);
 
-  std::map<std::tuple<int, int, int, int>, size_t> index;  // (path, dtype, kpad, precise) -> group
-  auto group_for = [&](int path, int real_dtype, int kpad) -> Group& {
+  std::map<std::tuple<int, int, int, int, int>, size_t> index;  // (path, dtype, kpad, precise, staged) -> group
+  auto group_for = [&](int path, int real_dtype, int kpad, int staged = 0) -> Group& {
     const int precise = real_dtype == ZGR_F32 ? 1 : 0;
     const int dtype = kernel_dtype >= 0 ? kernel_dtype : real_dtype;
-    auto key = std::make_tuple(path, dtype, kpad, precise);
+    auto key = std::make_tuple(path, dtype, kpad, precise, staged);
     auto it = index.find(key);
     if (it == index.end()) {
       index[key] = out.size();
       Group g;
-      g.kc = KernelChoice{path, dtype, kpad, bits, precise};
+      g.kc = KernelChoice{path, dtype, kpad, bits, precise, staged};
       out.push_back(std::move(g));
       return out.back();
     }
@@ -467,13 +509,14 @@ void plan(const std::vector<TensorDesc>& descs, const std::vector<int>& which, b
       continue;
     }
     const bool vec = aligned && (t.cols % 8 == 0);
-    int path, kpad, strip, row_step;
+    int path, kpad, strip, row_step, staged = 0;
     const bool umma_ok = t.umma && kernel_dtype < 0;
     const bool tile_ok = t.tile && (kernel_dtype < 0 || kernel_dtype == t.dtype);
     if (tile_ok) {
-      // fp32 with rank > 8, and rows that are not a multiple of eight elements: sweep_tile_kernel.  (The test hook that
-      // sweeps an fp32 image of a 16-bit tensor keeps the one-element-per-thread kernel below.)
-      path = vec && t.rank <= 8 ? PATH_FMA : PATH_GENERIC; kpad = t.kpad; strip = tile_strip_cols(); row_step = 128;
+      // fp32 with rank > 8, rows that are not a multiple of eight elements, and low ranks: three-part operands.  (The test hook
+      // that sweeps an fp32 image of a 16-bit tensor keeps the one-element-per-thread kernel below.)
+      path = vec && t.rank <= 8 ? PATH_FMA : PATH_GENERIC; kpad = t.kpad; strip = kTileStripCols; staged = t.staged;
+      row_step = staged && (t.cols & 7) ? 256 : 128;
     } else if (!vec || (t.rank > 8 && !umma_ok && (t.Ufrag == nullptr || multi))) {
       // (the legacy tensor-core kernel applies one term per sweep; several terms take the fallback)
       path = PATH_GENERIC; kpad = 0; strip = 64; row_step = 1;
@@ -485,7 +528,7 @@ void plan(const std::vector<TensorDesc>& descs, const std::vector<int>& which, b
       path = PATH_MMA; kpad = t.rank <= 16 ? 16 : (t.rank <= 32 ? 32 : 64);
       strip = mma_strip_cols(kpad); row_step = mma_rows_per_iter(kpad);
     }
-    Group& g = group_for(path, t.dtype, kpad);
+    Group& g = group_for(path, t.dtype, kpad, staged);
     const size_t gi = static_cast<size_t>(&g - out.data());
     if (members.size() <= gi) members.resize(gi + 1);
     members[gi].push_back(Member{l, strip, row_step});
@@ -680,8 +723,9 @@ int sweep(zgr_ctx* ctx, std::vector<Group>& groups, const TensorDesc* d_descs, i
       cudaEventRecord(e0, st);
     }
     const int rc = check(ctx, g.kc.path == PATH_UMMA ? launch_sweep_umma(g.kc, p, tmaps, ctx->d_err, grid, st)
+                              : g.kc.staged ? launch_sweep_staged(g.kc, p, ctx->d_err, grid, st)
                               : is_tile(g.kc) ? launch_sweep_tile(g.kc, p, tmaps, ctx->d_err, grid, st)
-                                                                           : launch_sweep(g.kc, p, grid, st));
+                                              : launch_sweep(g.kc, p, grid, st));
     if (rc != ZGR_OK) {
       if (e0) cudaEventDestroy(e0);
       if (e1) cudaEventDestroy(e1);
@@ -894,8 +938,8 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
   std::memset(ctx->tmaps.data(), 0, ctx->tmaps.size() * sizeof(CUtensorMap));
   const bool guided_on = ctx->b != 0.0;
   ctx->guided_at_init = guided_on;
-  const LowRank lr = low_rank(tensors, n);
-  size_t operand_bytes = 0;
+  const SetSizes sizes = set_sizes(tensors, n);
+  size_t operand_bytes = 0, n_staged_maps = 0;
   for (int32_t l = 0; l < n && rc == ZGR_OK; ++l) {
     const zgr_tensor& t = tensors[l];
     TensorDesc& td = ctx->descs[static_cast<size_t>(l)];
@@ -915,17 +959,21 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
     td.dtype = t.dtype;
     td.umma = 0;
     td.tile = 0;
+    td.staged = 0;
+    td.maps = nullptr;
     td.ushift = 0;
     for (void*& copy : td.Ucopy) copy = nullptr;
     // tcgen05 kernels: row-major copies of U in parts, and three tensor maps (those of the copies once these have their place)
-    const int kind = umma_wanted() && encode_tiled_fn() != nullptr ? tensor_core_kind(t, guided_on, lr) : 0;
+    const int kind = umma_wanted() && encode_tiled_fn() != nullptr ? tensor_core_kind(t, guided_on, sizes) : 0;
     if (kind == 2 || (kind == 1 && make_map_16bit(&ctx->tmaps[static_cast<size_t>(3 * l)], t.data, t.rows, t.cols, 64))) {
       td.kpad = t.rank <= 16 ? 16 : (t.rank <= 32 ? 32 : 64);
       // entries of an orthonormal U are about 1/sqrt(rows): scaled by 2^ushift they sit between 1 and 2 in size
       // (capped at 2^12, which leaves fp16 room for entries up to 16 in size); the bf16 parts need no scaling
       if (kind == 1) td.ushift = std::min<int32_t>(12, static_cast<int32_t>(std::ceil(0.5 * std::log2(static_cast<double>(t.rows)))));
       (kind == 1 ? td.umma : td.tile) = 1;
-      operand_bytes += (kind == 1 ? 2 : 3) * static_cast<size_t>((t.rows + 127) / 128) * 128 * static_cast<size_t>(td.kpad) * 2;
+      if (kind == 2) td.staged = staged_kind(t, sizes);
+      operand_bytes += (kind == 1 ? 2 : 3) * static_cast<size_t>(copy_rows(td)) * static_cast<size_t>(td.kpad) * 2;
+      if (td.staged) n_staged_maps += static_cast<size_t>(n_weight_maps(td)) + 3;
     }
     const bool vec = (reinterpret_cast<uintptr_t>(t.data) & 15) == 0 && (t.cols % 8 == 0);
     if (guided_on && t.rank > 8 && vec && t.dtype != ZGR_F32 && !td.umma) {
@@ -947,7 +995,10 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
     merge_small_groups(ctx);
     Tables tables;
     tables.add(&ctx->d_split_jobs, jobs.data(), jobs.size());
+    std::vector<CUtensorMap> staged_maps(n_staged_maps);
+    CUtensorMap* d_staged_maps = nullptr;
     tables.add(&ctx->d_tmaps, ctx->tmaps.data(), ctx->tmaps.size());
+    tables.add(&d_staged_maps, staged_maps.data(), staged_maps.size());
     tables.add(&ctx->d_descs, ctx->descs.data(), ctx->descs.size());
     tables.add(&ctx->d_err, static_cast<const int*>(nullptr), 1);
     tables.add(&ctx->d_stats, static_cast<const double*>(nullptr), static_cast<size_t>(3 * n));
@@ -971,18 +1022,27 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
       ctx->d_qr = qr;
       ctx->qr_bytes = scratch;
     }
+    size_t map_at = 0;
     for (int32_t l = 0; l < n && rc == ZGR_OK; ++l) {
       TensorDesc& td = ctx->descs[static_cast<size_t>(l)];
       const int32_t job = ctx->split_job[static_cast<size_t>(l)];
       if (job < 0) continue;
-      const int64_t rows_pad = ((td.rows + 127) / 128) * 128;
+      const int64_t rows_pad = copy_rows(td);
       CUtensorMap* m = &ctx->tmaps[static_cast<size_t>(3 * l)] + (td.umma ? 1 : 0);
+      if (td.staged) {
+        td.maps = d_staged_maps + map_at;
+        m = &staged_maps[map_at];
+        if (!make_weight_maps(m, td, td.data, dtype_bytes(td.dtype))) rc = check(ctx, cudaErrorUnknown);
+        m += n_weight_maps(td);
+        map_at += static_cast<size_t>(n_weight_maps(td)) + 3;
+      }
       for (int i = 0; i < (td.umma ? 2 : 3); ++i) {
         td.Ucopy[i] = at;
         if (!make_map_16bit(m + i, at, rows_pad, td.kpad, td.kpad)) rc = check(ctx, cudaErrorUnknown);
         at += static_cast<size_t>(rows_pad) * td.kpad * 2;       // (a multiple of 4096 bytes)
       }
-      jobs[static_cast<size_t>(job)] = SplitJob{td.U, {td.Ucopy[0], td.Ucopy[1], td.Ucopy[2]}, td.rows, rows_pad, td.rank, td.kpad, td.umma ? td.ushift : -1};
+      jobs[static_cast<size_t>(job)] = SplitJob{td.U, {td.Ucopy[0], td.Ucopy[1], td.Ucopy[2]}, td.rows, rows_pad, td.rank, td.kpad, td.umma ? td.ushift : -1,
+                                                  td.staged && (td.cols & 7) ? 1 : 0};
     }
     if (rc == ZGR_OK) rc = tables.copy(ctx);
     if (rc == ZGR_OK) rc = split_jobs(ctx, 0, ctx->n_split_jobs, nullptr);
@@ -1418,12 +1478,27 @@ int zgr_debug_z(zgr_ctx* ctx, uint64_t seed, int32_t tensor, float* dev_out, voi
   // a one-tensor model whose weights are the zeroed output buffer, swept once with scale 1
   std::vector<TensorDesc> one(1, ctx->descs[static_cast<size_t>(tensor)]);
   one[0].data = dev_out;
+  const size_t owned_before = ctx->owned.size();
+  int rc = ZGR_OK;
+  if (one[0].staged && one[0].dtype == ZGR_F32) {
+    // the tensor's own kernel on the image: its maps of U, and new ones of the weights
+    const size_t n_maps = static_cast<size_t>(n_weight_maps(one[0]));
+    std::vector<CUtensorMap> maps(n_maps);
+    CUtensorMap* d_maps = nullptr;
+    if ((reinterpret_cast<uintptr_t>(dev_out) & 15) != 0 || !make_weight_maps(maps.data(), one[0], dev_out, 4)) {
+      one[0].tile = 0;                 // (an image that TMA cannot address: one element per thread)
+    } else {
+      rc = dev_alloc(ctx, &d_maps, n_maps + 3);
+      if (rc == ZGR_OK) rc = check(ctx, cudaMemcpy(d_maps, maps.data(), n_maps * sizeof(CUtensorMap), cudaMemcpyHostToDevice));
+      if (rc == ZGR_OK) rc = check(ctx, cudaMemcpy(d_maps + n_maps, static_cast<const CUtensorMap*>(one[0].maps) + n_maps, 3 * sizeof(CUtensorMap), cudaMemcpyDeviceToDevice));
+      one[0].maps = d_maps;
+    }
+  }
   std::vector<Group> groups;
   const bool guided_on = ctx->guided_at_init;
   plan(one, std::vector<int>(1, 0), guided_on, ctx->cfg.bits_per_normal, ctx->sm_count, groups, ZGR_F32);
-  const size_t owned_before = ctx->owned.size();
   TensorDesc* d_one = nullptr;
-  int rc = dev_alloc(ctx, &d_one, 1);
+  if (rc == ZGR_OK) rc = dev_alloc(ctx, &d_one, 1);
   if (rc == ZGR_OK) rc = check(ctx, cudaMemcpy(d_one, one.data(), sizeof(TensorDesc), cudaMemcpyHostToDevice));
   if (rc == ZGR_OK) rc = upload_groups(ctx, groups);
   if (rc == ZGR_OK) rc = check(ctx, cudaMemsetAsync(dev_out, 0, static_cast<size_t>(one[0].rows * one[0].cols) * sizeof(float), st));
@@ -1596,7 +1671,7 @@ int zgr_debug_plan(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, 
   const int valid = validate_model(tensors, n, cfg, &d, &K);
   if (valid != ZGR_OK) return valid;
   const bool guided_on = K > 0 && cfg->alpha < 1.0;
-  const LowRank lr = low_rank(tensors, n);
+  const SetSizes sizes = set_sizes(tensors, n);
   std::vector<TensorDesc> descs(static_cast<size_t>(n));
   std::vector<int> all(static_cast<size_t>(n));
   for (int32_t l = 0; l < n; ++l) {
@@ -1610,10 +1685,11 @@ int zgr_debug_plan(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, 
       td.kpad = t.rank <= 16 ? 16 : (t.rank <= 32 ? 32 : 64);
       td.Ufrag = reinterpret_cast<const uint4*>(uintptr_t{16});   // marker only: never dereferenced by the planner
     }
-    const int kind = tcgen05 ? tensor_core_kind(t, guided_on, lr) : 0;
+    const int kind = tcgen05 ? tensor_core_kind(t, guided_on, sizes) : 0;
     if (kind != 0) {
       td.kpad = t.rank <= 16 ? 16 : (t.rank <= 32 ? 32 : 64);
       (kind == 1 ? td.umma : td.tile) = 1;
+      if (kind == 2) td.staged = staged_kind(t, sizes);
     }
     all[static_cast<size_t>(l)] = l;
   }

@@ -25,7 +25,10 @@ struct TensorDesc {
   int32_t qrows;         // rows of G taken from the codes (Sec. 3.4, proportion omega); rows beyond it are drawn from the seed
   int32_t umma;          // 1: served by the tcgen05 + TMA kernel (tensor maps and row-major hi/lo copies of U exist)
   int32_t ushift;        // the hi/lo copies hold U * 2^ushift (brings a typical entry of an orthonormal U near 1)
-  int32_t tile;          // 1: served by sweep_tile_kernel (tensor maps and the three bf16 parts of U exist)
+  int32_t tile;          // 1: served by a kernel that contracts three bf16 parts (tensor maps and the parts of U exist): sweep_tile_kernel,
+  int32_t staged;        //    or, if this is 1 too, sweep_staged_kernel
+  const void* maps;      // staged: tensor maps on the device: of the weights (one, or one per residue of the row modulo 8 if the rows are no
+                         // multiple of eight elements), then the three parts of U
   void* Ucopy[3];        // library-owned, rows_pad x kpad row-major (TMA sources): fp16 hi, lo (umma) or three bf16 parts (tile)
 };
 
@@ -79,7 +82,7 @@ struct SweepParams {
   float* zout;           // rows x cols fp32 image of the one tensor swept (test hook of the tcgen05 kernel only)
   double* item_stats;    // norm bookkeeping: kStatSlots x 3 doubles per work item of the group (partial sums per warp), or null
   int32_t item_base;     // index of items[0] in the group's full item list (layer-wise launches start in the middle)
-  int32_t* sched;        // CUDA-core and tile kernels: this launch's item counter (zero between launches), see ItemFeed
+  int32_t* sched;        // CUDA-core and three-part kernels: this launch's item counter (zero between launches), see ItemFeed
   int32_t kshift;        // tcgen05 kernel: the coefficient strips are scaled by a power of two so that sum_q |c_q| b 2^kshift
                          // is near 1 (see the operand precision note in zgr_umma.cu)
 };

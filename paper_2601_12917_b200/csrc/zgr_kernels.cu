@@ -6,11 +6,12 @@
 // in registers / shared memory and never stored.
 //
 //   sweep_iso      tensors without a subspace (1-D tensors, rank 0) or with b = 0
-//   sweep_fma      rank <= 8, small sets and large fp32 ones: U G on CUDA-core FMAs in fp32, G strip in shared memory and registers
+//   sweep_fma      rank <= 8, small sets and large fp32 ones of rank <= 4: U G on CUDA-core FMAs in fp32, G strip in shared memory and registers
 //   sweep_mma      rank  > 8, fallback of the tcgen05 kernels: mma.sync, bf16 hi/lo split operands (three products per
 //                  tile, fp32 accumulate), accumulators initialised with theta
-//   sweep_generic  any shape or alignment, one element per thread (fallback of the tile kernel)
-// The tcgen05 kernels are in zgr_umma.cu (weights staged by TMA) and zgr_tile.cu (fp32, ragged rows, rank <= 8).
+//   sweep_generic  any shape or alignment, one element per thread (fallback of the kernels with three-part operands)
+// The tcgen05 kernels are in zgr_umma.cu (16-bit weights in whole octets, rank > 8), zgr_staged.cu (fp32, ragged rows, rank <= 8; both stage the
+// weights by TMA) and zgr_tile.cu (what TMA cannot address, and small sets).
 //
 // All kernels are persistent over a device-resident list of work items, so a sweep over a model with hundreds of tensors is
 // a handful of launches.
@@ -600,7 +601,7 @@ __global__ void split_subspace_kernel(const float* __restrict__ U, int64_t rows,
 }
 
 // Row-major operand copies of U for a list of tensors: two fp16 parts of U 2^shift (TMA-staged kernel) or three bf16 parts
-// of U (tile kernel).  Rows are padded to a multiple of 128 and columns to the contraction width with zeros.
+// of U (staged and tile kernels).  Rows are padded to a multiple of 128 or 256 and columns to the contraction width with zeros.
 // A thread makes eight consecutive entries of a row: one 16-byte store per part.
 struct alignas(16) SplitRow {
   uint16_t v[8];
@@ -612,7 +613,7 @@ __global__ void __launch_bounds__(256) split_subspaces_kernel(const SplitJob* __
   const int64_t n = j.rows_pad * per_row;
   const float scale = j.shift >= 0 ? __int_as_float((127 + j.shift) << 23) : 1.0f;
   for (int64_t idx = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; idx < n; idx += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int64_t row = idx / per_row;
+    const int64_t at = idx / per_row, row = j.by_residue ? staged_row_at(at) : at;
     const int k0 = static_cast<int>(idx % per_row) * 8;
     SplitRow out[3];
 #pragma unroll
@@ -622,7 +623,7 @@ __global__ void __launch_bounds__(256) split_subspaces_kernel(const SplitJob* __
     }
 #pragma unroll
     for (int q = 0; q < 3; ++q)
-      if (q < 2 || j.shift < 0) *reinterpret_cast<SplitRow*>(static_cast<uint16_t*>(j.part[q]) + row * j.kp + k0) = out[q];
+      if (q < 2 || j.shift < 0) *reinterpret_cast<SplitRow*>(static_cast<uint16_t*>(j.part[q]) + at * j.kp + k0) = out[q];
   }
 }
 

@@ -18,16 +18,17 @@ enum Path { PATH_ISO = 0, PATH_FMA = 1, PATH_MMA = 2, PATH_GENERIC = 3, PATH_UMM
 struct KernelChoice {
   int path;   // Path
   int dtype;  // ZGR_F32 | ZGR_F16 | ZGR_BF16
-  int kpad;   // contraction width.  FMA: 4 or 8;  MMA, UMMA and the tile kernel (see is_tile): 16, 32 or 64;  otherwise 0
+  int kpad;   // contraction width.  FMA: 4 or 8;  MMA, UMMA and the three-part kernels (see is_tile): 16, 32 or 64;  otherwise 0
   int bits;   // 32 or 16 random bits per normal
   int precise;  // accurate Gaussian transform (tensors stored in fp32)
+  int staged;   // among the groups of is_tile: served by sweep_staged_kernel
 };
 
 // Resident blocks of 256 threads per SM of the isotropic kernel.  Its plain instantiation (fused transform) fits 32 registers:
 // eight blocks, whose loads then cover the DRAM latency (5.74 TB/s standalone against 5.50 with six).
 constexpr int iso_blocks_per_sm(bool precise, bool multi, bool stats) { return !precise && !multi && !stats ? 8 : 5; }
 
-// The groups that sweep_tile_kernel serves: rank <= 8 tensors in whole octets are counted under the path of the CUDA-core
+// The groups that sweep_staged_kernel and sweep_tile_kernel serve: rank <= 8 tensors in whole octets are counted under the path of the CUDA-core
 // kernel (whose own widths are 4 and 8), the others under that of the fallback kernel (whose own width is 0).
 inline bool is_tile(const KernelChoice& kc) { return (kc.path == PATH_FMA && kc.kpad == 16) || (kc.path == PATH_GENERIC && kc.kpad > 0); }
 
@@ -61,8 +62,10 @@ cudaError_t launch_sweep_umma(const KernelChoice& kc, const SweepParams& p, cons
 cudaError_t launch_debug_z_umma(const KernelChoice& kc, const SweepParams& p, const CUtensorMap* tmaps, int* error, int grid, cudaStream_t st);
 cudaError_t launch_stats_umma(const KernelChoice& kc, const SweepParams& p, const CUtensorMap* tmaps, int* error, int grid, cudaStream_t st);
 // Sweep of the other guided tensors that a tensor-core kernel serves (fp32, rank <= 8, rows that are not a multiple of eight
-// elements).  tmaps: the three bf16 parts of U per tensor; kc.kpad = contraction width.
-int tile_strip_cols();
+// elements).  kc.kpad = contraction width; strips of 128 columns.  The tile kernel takes those that TMA cannot address and small sets; tmaps: the three
+// bf16 parts of U per tensor.
+constexpr int kTileStripCols = 128;
+cudaError_t launch_sweep_staged(const KernelChoice& kc, const SweepParams& p, int* error, int grid, cudaStream_t st);
 cudaError_t launch_sweep_tile(const KernelChoice& kc, const SweepParams& p, const CUtensorMap* tmaps, int* error, int grid, cudaStream_t st);
 // Rebuild of the row-major operand copies of U for a device-resident list of tensors in one launch (grid.y = job).
 struct SplitJob {
@@ -71,7 +74,12 @@ struct SplitJob {
   int64_t rows, rows_pad;
   int32_t r, kp;
   int32_t shift;   // two fp16 parts (hi, lo) of U * 2^shift; -1: three bf16 parts of U
+  int32_t by_residue;  // rows in the order of staged_copy_row (tensors of sweep_staged_kernel whose rows are no multiple of eight elements)
 };
+// Where row m of U is kept so that the 32 rows of a quarter of a tile, m mod 8 the same, follow one another; and the row kept at c.
+// (rows in spans of 256: eight residues x 32 rows)
+__host__ __device__ inline int64_t staged_copy_row(int64_t m) { return (m & ~int64_t{255}) | ((m & 7) << 5) | ((m >> 3) & 31); }
+__host__ __device__ inline int64_t staged_row_at(int64_t c) { return (c & ~int64_t{255}) | ((c & 31) << 3) | ((c >> 5) & 7); }
 #ifdef __CUDACC__
 // The parts of one entry x of U: fp16 hi + lo of x 2^shift (22 significant bits as long as the scaled entry is not far below 1:
 // lo must stay a normal fp16 number), or three bf16 parts whose sum is x (1 + lean).
@@ -95,8 +103,9 @@ __device__ __forceinline__ void split_subspace_value(bool fp16, float x, float s
 // of themselves too small.  The third part of U makes up for it.  2-norm of the error against 64 bits, of the result's, without /
 // with it / of a chain of fp32 multiply-adds:  rank 4 4.6 / 2.9 / 4.0e-8,  16 4.8 / 3.0 / 7.6e-8,  64 7.7 / 4.9 / 14.7e-8.
 __device__ __forceinline__ float truncation_lean(int kp) { return 2.2e-8f + 5e-10f * static_cast<float>(kp); }
-// Entry `at` of the copies of job j from the value x of U; scale = 2^shift.
-__device__ __forceinline__ void split_subspace_entry(const SplitJob& j, int64_t at, float x, float scale) {
+// Entry (row, k) of the copies of job j from the value x of U; scale = 2^shift.
+__device__ __forceinline__ void split_subspace_entry(const SplitJob& j, int64_t row, int k, float x, float scale) {
+  const int64_t at = (j.by_residue ? staged_copy_row(row) : row) * j.kp + k;
   uint16_t p0, p1, p2;
   split_subspace_value(j.shift >= 0, x, scale, truncation_lean(j.kp), p0, p1, p2);
   static_cast<uint16_t*>(j.part[0])[at] = p0;

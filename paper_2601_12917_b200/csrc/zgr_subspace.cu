@@ -475,7 +475,7 @@ __global__ void __launch_bounds__(kQrThreads) basis_kernel(const BasisArgs p) {
       if (k >= r) continue;                    // (the padding of the copies is zero since zgr_init)
       const float u = static_cast<float>(X[i * LD + k]);
       p.U[(row0 + i) * r + k] = u;
-      if (c.part[0] != nullptr) split_subspace_entry(c, (row0 + i) * c.kp + k, u, scale);
+      if (c.part[0] != nullptr) split_subspace_entry(c, row0 + i, k, u, scale);
     }
   }
   // The host polls the status word: it is written once every CTA's results are visible.

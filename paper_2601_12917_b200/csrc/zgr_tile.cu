@@ -1,6 +1,6 @@
-// Sweep with a tensor-core contraction for the guided tensors that the TMA-staged kernel (zgr_umma.cu) cannot take: fp32 storage with
-// rank > 8, any storage whose rows are not a multiple of eight elements long, and sets of rank <= 8 that are worth a
-// tensor-core kernel (tensor_core_kind in zgr_host.cu has the sizes).
+// Sweep with a tensor-core contraction for the guided tensors that neither TMA-staged kernel (zgr_umma.cu, zgr_staged.cu) takes: fp32
+// rows that are no multiple of eight elements long, weights that do not begin on a 16-byte boundary, rows shorter than two
+// octets, and small sets (tensor_core_kind and staged_kind in zgr_host.cu have the sizes).
 //     theta <- rnd(theta + c (a Z + b U G))            (Eq. (perturbation) applied as in Algorithm 1)
 //
 // Layout.  Generator blocks run along the flattened tensor, eight elements ("an octet") at a time, so in a tensor whose
@@ -37,16 +37,15 @@
 
 #include "zgr_device.cuh"
 #include "zgr_kernels.h"
+#include "zgr_strip.cuh"
 #include "zgr_tcgen05.cuh"
 
 namespace zgr {
 namespace {
 
-constexpr int kTileM = 128, kStrip = 128, kTileN = 144;
+constexpr int kTileM = 128;
 constexpr int kAcc = 3;                        // accumulator buffers: 3 x 144 of the 512 tensor-memory columns
-constexpr int kEpi = 16;                       // epilogue warps: 32 rows x 32 columns of a tile each
 constexpr int kTileThreads = 32 * (2 + kEpi);
-constexpr int kParts = 3;                      // bf16 parts of an operand
 constexpr int kRing = 4;                       // items published ahead
 constexpr int kPitchMax = 42;
 constexpr int kXposeBytes = 32 * kPitchMax * 4;   // one warp's buffer
@@ -81,75 +80,6 @@ __device__ __forceinline__ void tmem_ld8_tail(uint32_t taddr, uint32_t (&v)[40])
                : "=r"(v[32]), "=r"(v[33]), "=r"(v[34]), "=r"(v[35]), "=r"(v[36]), "=r"(v[37]), "=r"(v[38]), "=r"(v[39])
                : "r"(taddr)
                : "memory");
-}
-
-__device__ __forceinline__ void sts16(uint32_t saddr, uint16_t v) { asm volatile("st.shared.b16 [%0], %1;" ::"r"(saddr), "h"(v) : "memory"); }
-
-// Compressed coefficient of row k, column c, before scale and zero point.
-__device__ __forceinline__ float code1(const TensorDesc& td, int k, int64_t c) {
-  if (td.qbits == 4) {
-    const uint32_t byte = reinterpret_cast<const uint8_t*>(td.q)[static_cast<int64_t>(k) * ((td.cols + 1) >> 1) + (c >> 1)];
-    return static_cast<float>((c & 1) ? (byte >> 4) : (byte & 15u));
-  }
-  return static_cast<float>(td.q[static_cast<int64_t>(k) * td.cols + c]);
-}
-
-// The strip  c b G[0..KP)[col0 .. col0 + 144)  as K-major bf16 operands.  One unit of work is the octet of one row k of G
-// (the octets of G start at other columns in every row when cols is no multiple of 8).
-template <int BITS, bool PRECISE, bool MULTI>
-__device__ __forceinline__ void build_strip(const TensorDesc& td, const SweepParams& p, int64_t col0, int kp, int rowb, int g_bytes, uint32_t g_dst, int et) {
-  constexpr int kOct = kTileN / 8 + 1;
-  const int kp_shift = kp == 64 ? 6 : (kp == 32 ? 5 : 4);
-  const int64_t cols = td.cols;
-  for (int idx = et; idx < (kOct << kp_shift); idx += kEpi * 32) {
-    const int k = idx & (kp - 1), o = idx >> kp_shift;      // consecutive lanes: consecutive k, i.e. neighbouring shared-memory words
-    const int64_t row_e = static_cast<int64_t>(k) * cols;
-    const int64_t e = (((row_e + col0) >> 3) + o) << 3;     // first element of the octet
-    const int64_t c_first = e - row_e;                      // its column (may lie before the strip)
-    const int j0 = static_cast<int>(c_first - col0);        // -7 .. 144
-    float g[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) g[i] = 0.0f;
-    if (k < td.rank && c_first < cols) {
-      if (td.q != nullptr && k < td.qrows && (cols & 7) == 0) {
-        guided8<BITS, PRECISE, MULTI>(td, p, k, c_first, g);      // eight codes of one row in one load
-      } else if (td.q != nullptr && k < td.qrows) {
-        float cb = p.term[0].cb;
-        if (MULTI)
-          for (int q = 1; q < p.n_terms; ++q) cb += p.term[q].cb;
-        const float lambda = td.qscale[k] * cb;
-        const float delta = td.qzero ? td.qzero[k] : 0.0f;
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-          if (c_first + i >= 0 && c_first + i < cols) g[i] = lambda * (code1(td, k, c_first + i) - delta);
-      } else {
-        normals8<BITS, PRECISE>(p.term[0].keys, static_cast<uint32_t>(td.id), 1u, static_cast<uint64_t>(e), p.unit, g);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) g[i] *= p.term[0].cb;
-        if (MULTI) {
-#pragma unroll 1
-          for (int q = 1; q < p.n_terms; ++q) {
-            float y[8];
-            normals8<BITS, PRECISE>(p.term[q].keys, static_cast<uint32_t>(td.id), 1u, static_cast<uint64_t>(e), p.unit, y);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) g[i] = fmaf(p.term[q].cb, y[i], g[i]);
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int j = j0 + i;
-      if (j >= 0 && j < kTileN) {
-        uint16_t q0, q1, q2;
-        split_subspace_value(false, c_first + i < cols ? g[i] : 0.0f, 1.0f, 0.0f, q0, q1, q2);
-        const uint32_t at = g_dst + swizzle(static_cast<uint32_t>(j * rowb + 2 * k), rowb);
-        sts16(at, q0);
-        sts16(at + g_bytes, q1);
-        sts16(at + 2 * g_bytes, q2);
-      }
-    }
-  }
 }
 
 // storage of an octet as it is loaded: 16 bytes of 16-bit weights, unpacked on use, or eight floats
@@ -334,7 +264,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
     bool ok = true;
     auto strip_for = [&](int it, int no) {
       const WorkItem w = p.items[it];
-      build_strip<BITS, PRECISE, MULTI>(p.tensors[w.tensor], p, w.col0, kp, rowb, L.g_bytes, g_s + static_cast<uint32_t>((no % GS) * kParts * L.g_bytes), et);
+      build_strip<BITS, PRECISE, MULTI>(p.tensors[w.tensor], p, w.col0, kTileN, kp, rowb, L.g_bytes, g_s + static_cast<uint32_t>((no % GS) * kParts * L.g_bytes), et);
       fence_proxy_async();
       __syncwarp();
       if (lane == 0) mbar_arrive(BAR_G(no % GS));
@@ -601,8 +531,6 @@ cudaError_t launch_tile_typed(const KernelChoice& kc, const SweepParams& p, cons
                        : launch_tile_one<T, 16, PRECISE, false, false>(kc.kpad, p, tmaps, error, grid, st);
 }
 }  // namespace
-
-int tile_strip_cols() { return kStrip; }
 
 cudaError_t launch_sweep_tile(const KernelChoice& kc, const SweepParams& p, const CUtensorMap* tmaps, int* error, int grid, cudaStream_t st) {
   static_assert(kEpi <= kStatSlots, "one bookkeeping slot per epilogue warp");

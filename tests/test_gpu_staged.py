@@ -1,0 +1,69 @@
+"""The sweep whose weights are staged by TMA and whose operands have three parts, at the sizes where it can go wrong (needs a B200):
+rows that are no multiple of eight elements long around octets, strips and spans of 256 rows, residues without rows, several tensors
+of different row lengths in one launch.  Every call against the oracle, with the tolerances of helpers.py.  A set takes this kernel from
+2.6 M weights on, hence the large first tensors."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2601_12917_b200 import zgr
+
+from helpers import Pair
+from test_plan import plan
+
+pytestmark = pytest.mark.gpu
+
+LARGE = (1300, 2051)
+# rows: fewer than eight residues, around a quarter's 32 lanes and a span; columns: two octets, one strip and one less or more, ends of rows
+# that begin or end a strip
+RAGGED = [(5, 17), (1, 143), (255, 19), (256, 127), (257, 129), (264, 135), (31, 263), (300, 385), (7, 2049)]
+
+
+@pytest.mark.parametrize("dtype,bits", [("bf16", 16), ("f16", 32)])
+@pytest.mark.parametrize("rank", [1, 16, 20, 64])
+def test_ragged_rows(rank, dtype, bits):
+    shapes = [LARGE] + RAGGED + [(1, 37)]
+    ranks = [min(rank, m) for m, _ in shapes[:-1]] + [0]
+    kinds = [{"f16": zgr.F16, "bf16": zgr.BF16}[dtype]] * len(shapes)
+    assert all(it.row0_or_e0 % 256 == 0 for it in plan(shapes, ranks, kinds, bits=bits) if it.path == 3)      # whole spans
+    p = Pair(shapes, ranks, dtype, bits=bits, seed=rank)
+    reports = p.step(seed=17, lp=2.4, lm=1.7, lr=1e-4)
+    assert all(rep["moved"] > 0.3 for call in reports[:2] for rep in call)
+    assert p.lib.device_status() == 0
+
+
+# Rows shorter than two octets, and weights that do not begin on a 16-byte boundary, stay with the tile kernel beside it.
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_whole_octets_beside_other_rows(dtype):
+    p = Pair([(1300, 2056), (40, 15), (130, 64), (129, 72), (1, 136), (257, 200), (385, 129), (1, 9)], [16 if dtype == "f32" else 8, 3, 8, 4, 1, 8, 12, 0], dtype, bits=32, seed=4)
+    p.step(seed=3, lp=1.8, lm=2.3, lr=1e-4)
+    assert p.lib.device_status() == 0
+
+
+@pytest.mark.parametrize("dtype,cols", [("bf16", 2051), ("f32", 2056)])
+@pytest.mark.parametrize("rank", [12, 40])
+def test_norms_codes_and_several_seeds(rank, dtype, cols):
+    shapes, ranks = [(1300, cols), (150, 203 if dtype == "bf16" else 200), (1, 25)], [rank, 20, 0]
+    p = Pair(shapes, ranks, dtype, bits=16, seed=8, stats=True, alpha=0.4)
+    q, sc, ze = oracle.dtc_quantise_int4(oracle.coeffs(9, 0, 16, ranks[1], shapes[1][1]))
+    p.set_dtc(1, q, sc, ze, bits=4)
+    p.step(seed=31, lp=2.2, lm=1.9, lr=1e-4)
+    got = p.lib.get_stats(31)
+    for l in range(3):
+        np.testing.assert_allclose(got[l], oracle.stats_tensor(p.oracle_tensor(l), 31, l, 16, p.a, p.b), rtol=2e-5, atol=1e-9)
+    p.lib.enable_stats(False)
+    seeds, lp, lm = [41, 42, 43], [2.1, 1.6, 2.4], [1.9, 2.0, 1.8]
+    coeffs = [oracle.update_coefficient(0.0, a, b, p.eps, 1e-4) for a, b in zip(lp, lm)]
+    p.call_and_check_multi(seeds, coeffs, lambda: p.lib.restore_update_multi(seeds, lp, lm, 1e-4), "three seeds")
+
+
+# A delivered and a constructed subspace reach the copies of U that are kept by residue.
+def test_new_subspaces_of_ragged_tensors():
+    p = Pair([LARGE, (300, 385), (1, 9)], [16, 16, 0], "bf16", bits=16, seed=6)
+    for l in (0, 1):
+        p.U[l].copy_(p.U[l].flip(0))
+    p.lib.update_subspace(0)
+    p.lib.build_subspace(1, (p.U[1].flip(1) * 3.0).contiguous())
+    p.step(seed=5, lp=2.0, lm=1.6, lr=1e-4)
+    p.lib.update_subspaces([0, 1], [p.U[0], p.U[1]])
+    p.step(seed=6, lp=2.0, lm=1.6, lr=1e-4)
