@@ -2,7 +2,7 @@
 // "Guided Perturbation Sampling on Cloud"): an orthonormal basis U (rows x r, r <= 64) of the span of the r
 // gradient directions collected for one tensor, given as the columns of A (rows x r fp32, row-major).
 //
-// Method: Cholesky QR, applied twice.  One pass forms the Gram matrix  S = A^T A  (r x r), factors it
+// Method: Cholesky QR, applied twice where one pass is not enough.  One pass forms the Gram matrix  S = A^T A  (r x r), factors it
 // S = R^T R  (R upper triangular with a positive diagonal) and returns  Q = A R^-1.  In exact arithmetic that is
 // the thin Q of the QR factorisation with R_kk > 0, i.e. the same basis, column for column, as a Householder QR
 // with that sign convention.  In floating point the first pass loses orthogonality in proportion to the
@@ -46,6 +46,13 @@ constexpr int kMaxR = 64;
 // ones.  The fp32 rounding of an exact linear combination leaves up to about 3e-8 (8e-16 here), the sums in double below 5e-16 when
 // exact; directions at 5e-8 and more give a basis that is right to 3e-8 and are accepted.
 constexpr double kPivotFloor = 2e-15;
+
+// One pass is enough when it leaves the columns orthonormal far below the fp32 rounding of the result.  Errors of the Gram matrix, |dS_kl| <=
+// g |a_k| |a_l| with g about 1e-15 (sums in double over at most some hundred rows, then over the CTAs), come out of the first pass as
+// R^-T dS R^-1, at most g (sum_k |a_k| |R^-1_kj|)^2 <= g r m_j with m_j = sum_k |a_k|^2 (R^-1)_kj^2, which the factorisation has at
+// hand.  r m_j <= 1e5 (condition numbers up to about 100 after scaling the columns to one length) keeps that near 1e-10; one fp32
+// rounding is 6e-8 of an entry.  2048 x 16, mixed Gaussian directions: r m_j is about 30.
+constexpr double kOnePass = 1e5;
 
 // Partial Gram matrix of rows [chunk*128, +128) of X (rows x r).  X is fp32 (SRC_DOUBLE = false) or double.
 template <bool SRC_DOUBLE>
@@ -403,6 +410,20 @@ __global__ void __launch_bounds__(kQrThreads) basis_kernel(const BasisArgs p) {
     }
     __syncthreads();
     if (status != 0) break;
+    if (pass == 0) {
+      // Is the second pass needed (see kOnePass)?  sum_k |a_k|^2 (R^-1)_kj^2 for every column j, by the 16 threads that hold row j of M.
+      bool again = false;
+#pragma unroll
+      for (int a = 0; a < NB; ++a) {
+        double v = 0.0;
+#pragma unroll
+        for (int b = 0; b <= a; ++b) v = fma(diag[tj + 16 * b] * m[a][b], m[a][b], v);
+#pragma unroll
+        for (int off = 8; off > 0; off >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
+        if (ti + 16 * a < r && !(v * r <= kOnePass * inv[ti + 16 * a])) again = true;
+      }
+      if (!__syncthreads_or(again)) pass = 1;      // (the same answer in every CTA: all have the same sums)
+    }
     if (tid < RC) inv[tid] = tid < r ? 1.0 / sqrt(inv[tid]) : 0.0;
     for (int idx = tid; idx < (RC - r) * RC; idx += kT) Ms[(r + idx / RC) * LD + idx % RC] = 0.0;      // rank not a multiple of 16
     __syncthreads();
