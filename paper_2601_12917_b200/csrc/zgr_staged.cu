@@ -568,18 +568,32 @@ __global__ void __launch_bounds__(kThreadsStaged, 1) sweep_staged_kernel(const _
                   float th[8], z[8];
 #pragma unroll
                   for (int i = 0; i < 8; ++i) th[i] = i >= i0 && i < i1 ? load_weight(at + i) : 0.0f;
-                  iso8<BITS, PRECISE, MULTI>(p, tid, static_cast<uint64_t>(row_e + c0), z);
+                  // (the sums in the order of whole octets: the normals go onto the product, or both apart for their norms)
+                  if constexpr (SSTATS) {
+                    iso8<BITS, PRECISE, MULTI>(p, tid, static_cast<uint64_t>(row_e + c0), z);
+                  } else {
+                    const uint32_t oct = static_cast<uint32_t>((row_e + c0) >> 3);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) z[i] = __uint_as_float(d[i]);
+                    normals8_add<BITS, PRECISE>(p.term[0].keys, pre, oct, p.term[0].iso, z);
+                    if (MULTI) {
+#pragma unroll 1
+                      for (int q = 1; q < p.n_terms; ++q)
+                        normals8_add<BITS, PRECISE>(p.term[q].keys, philox_pre(0u, tid, p.term[q].keys), oct, p.term[q].iso, z);
+                    }
+                  }
                   float f_iso = 0.0f, f_gd = 0.0f, f_z = 0.0f;
 #pragma unroll
                   for (int i = 0; i < 8; ++i)
                     if (i >= i0 && i < i1) {
-                      const float g = __uint_as_float(d[i]), step = g + z[i];
-                      if (SSTATS) {
+                      if constexpr (SSTATS) {
+                        const float g = __uint_as_float(d[i]);
                         f_iso = fmaf(z[i], z[i], f_iso);
                         f_gd = fmaf(g, g, f_gd);
-                        f_z = fmaf(step, step, f_z);
+                        z[i] += g;
+                        f_z = fmaf(z[i], z[i], f_z);
                       }
-                      Storage<T>::store1(at + i, th[i] + step);
+                      Storage<T>::store1(at + i, th[i] + z[i]);
                     }
                   s_iso += static_cast<double>(f_iso);
                   s_gd += static_cast<double>(f_gd);

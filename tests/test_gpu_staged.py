@@ -4,6 +4,7 @@ of different row lengths in one launch.  Every call against the oracle, with the
 2.6 M weights on, hence the large first tensors."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
 from paper_2601_12917_b200 import zgr
@@ -67,3 +68,26 @@ def test_new_subspaces_of_ragged_tensors():
     p.step(seed=5, lp=2.0, lm=1.6, lr=1e-4)
     p.lib.update_subspaces([0, 1], [p.U[0], p.U[1]])
     p.step(seed=6, lp=2.0, lm=1.6, lr=1e-4)
+
+
+# The same tensor alone (tile kernel) and beside a larger one (staged kernel), the sizes chosen so that the mixing scalars are the same: equal
+# bits, whole octets and ends of rows alike.  On zero weights, whose result keeps the step's own 11 bits, so that one rounding of
+# the fp32 step more or less shows (in about a dozen of the 112 000 elements at the ends).
+@pytest.mark.parametrize("bits", [16, 32])
+def test_ends_of_rows_as_in_the_tile_kernel(bits):
+    rows, cols, rank = 16000, 61, 16                                       # d / K = rows / rank = 1000 in both sets
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(3)
+    U = torch.linalg.qr(torch.randn(rows, rank, generator=gen, device="cuda"))[0].contiguous()
+    V = torch.linalg.qr(torch.randn(1000, 1, generator=gen, device="cuda"))[0].contiguous()
+    results = []
+    for beside in (False, True):
+        w, big = (torch.zeros(m, n, device="cuda", dtype=torch.float16) for m, n in ((rows, cols), (1000, 2051)))
+        z = zgr.Zgr([w, big] if beside else [w], [U, V] if beside else [U], 0.5, 1e-3, zgr.SCALE_UNIT, bits)
+        z.perturb(9, 1.0)
+        one = w.clone()
+        w.zero_()
+        z.sweep_multi([10, 11], [0.75, -1.0])
+        results.append((np.float32(z.scalars()), one, w))
+    assert (results[0][0] == results[1][0]).all()
+    assert torch.equal(results[0][1], results[1][1]) and torch.equal(results[0][2], results[1][2])
