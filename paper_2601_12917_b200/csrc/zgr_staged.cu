@@ -266,7 +266,9 @@ __global__ void __launch_bounds__(kThreadsStaged, 1) sweep_staged_kernel(const _
     };
     auto wait0 = [&](uint32_t bar, uint32_t parity, int where) -> bool {
       const bool got = lane != 0 || mbar_wait<true>(bar, parity, abort_flag, error, where);
-      return __shfl_sync(0xFFFFFFFFu, static_cast<int>(got), 0) != 0;
+      const int all = __shfl_sync(0xFFFFFFFFu, static_cast<int>(got), 0);
+      __syncwarp();        // (a shuffle orders no memory: what lane 0 has waited for is in order before the other lanes' copies)
+      return all != 0;
     };
     Ring st, ur;
     int t = 0, rb = 0;
