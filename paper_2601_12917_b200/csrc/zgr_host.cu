@@ -219,7 +219,27 @@ bool make_weight_maps(CUtensorMap* out, const TensorDesc& td, void* data, int by
   }
   return true;
 }
-int64_t copy_rows(const TensorDesc& td) { return td.staged && (td.cols & 7) ? (td.rows + 255) / 256 * 256 : (td.rows + 127) / 128 * 128; }
+// Rows of such a tensor that are no multiple of eight elements are worked on in the order of the copies of U (staged_copy_row): in spans of
+// 256 rows, residues 0-3 and 4-7 of a span a block of 128 each.
+bool by_residue(const TensorDesc& td) { return td.staged && (td.cols & 7); }
+int64_t copy_rows(const TensorDesc& td) { return by_residue(td) ? (td.rows + 255) / 256 * 256 : (td.rows + 127) / 128 * 128; }
+// Rows of the tensor in front of block `block` of that order.
+int64_t rows_before(const TensorDesc& td, int64_t block) {
+  const int64_t row0 = std::min(block / 2 * 256, td.rows), span = std::min<int64_t>(td.rows - row0, 256);
+  return row0 + (block & 1 ? span / 8 * 4 + std::min<int64_t>(span & 7, 4) : 0);
+}
+// Rows that a tensor is cut into items by: its own, or its blocks in that order that hold any.
+int64_t rows_to_cut(const TensorDesc& td) {
+  if (!by_residue(td)) return td.rows;
+  const int64_t blocks = copy_rows(td) / 128;
+  return 128 * (rows_before(td, blocks - 1) < td.rows ? blocks : blocks - 1);
+}
+// First row and number of rows of an item: of the tensor, or in that order.
+std::pair<int64_t, int64_t> item_rows(const TensorDesc& td, const WorkItem& w) {
+  if (!by_residue(td)) return {w.row0_or_e0, w.nrows_or_count};
+  const int64_t first = rows_before(td, w.row0_or_e0 / 128);
+  return {first, rows_before(td, (w.row0_or_e0 + w.nrows_or_count) / 128) - first};
+}
 
 bool whole_octets(const zgr_tensor& t) { return (reinterpret_cast<uintptr_t>(t.data) & 15) == 0 && (t.cols % 8 == 0); }
 // Weights of a model by storage, of those kinds of tensors whose kernel depends on how many there are: rank <= 8 in whole octets, and
@@ -294,33 +314,35 @@ int blocks_per_sm(const KernelChoice& kc, bool multi = false, bool stats = false
 
 struct Member {
   int tensor, strip, row_step;
+  int64_t rows;                                           // rows_to_cut
 };
 
 // Append the items of one tensor: strips of `strip` columns, each cut into even chunks of at most about nrows rows.
-void cut_tensor(const TensorDesc& t, int l, int strip, int row_step, int64_t nrows_for_strip(int64_t, int), int64_t arg, std::vector<WorkItem>& items) {
-  for (int64_t c0 = 0; c0 < t.cols; c0 += strip) {
-    const int ncols = static_cast<int>(std::min<int64_t>(strip, t.cols - c0));
+void cut_tensor(const TensorDesc& t, const Member& m, int64_t nrows_for_strip(int64_t, int), int64_t arg, std::vector<WorkItem>& items) {
+  for (int64_t c0 = 0; c0 < t.cols; c0 += m.strip) {
+    const int ncols = static_cast<int>(std::min<int64_t>(m.strip, t.cols - c0));
     int64_t nrows = std::max<int64_t>(1, nrows_for_strip(arg, ncols));
-    nrows = ((nrows + row_step - 1) / row_step) * row_step;
-    const int64_t n_chunks = (t.rows + nrows - 1) / nrows;
-    nrows = (t.rows + n_chunks - 1) / n_chunks;
-    nrows = ((nrows + row_step - 1) / row_step) * row_step;
-    for (int64_t r0 = 0; r0 < t.rows; r0 += nrows) items.push_back(WorkItem{l, ncols, r0, std::min(nrows, t.rows - r0), c0});
+    nrows = ((nrows + m.row_step - 1) / m.row_step) * m.row_step;
+    const int64_t n_chunks = (m.rows + nrows - 1) / nrows;
+    nrows = (m.rows + n_chunks - 1) / n_chunks;
+    nrows = ((nrows + m.row_step - 1) / m.row_step) * m.row_step;
+    for (int64_t r0 = 0; r0 < m.rows; r0 += nrows) items.push_back(WorkItem{m.tensor, ncols, r0, std::min(nrows, m.rows - r0), c0});
   }
 }
 
 // Small sets on the tensor-core kernels: the strips, one after the other, are cut into one contiguous share per CTA, all shares
 // costing the same (in units of a 128 x 128 tile: the tiles, `strip_cost` times the rank for every 128 columns of a strip
-// begun, `item_cost` for every item begun).  A CTA then builds one or two strips instead of one per item.  Returns the cost of a share.
-double share_out(const std::vector<TensorDesc>& descs, const std::vector<Member>& members, int strip_cols, int sm_count, double strip_cost, double item_cost,
-                 std::vector<WorkItem>& items, std::vector<int32_t>& starts) {
+// begun, `item_cost` for every item begun).  A CTA then builds one or two strips instead of one per item.  Items begin at multiples of `step`
+// rows.  Returns the cost of a share; if that is not below `limit` (0: none), nothing is written.
+double share_out(const std::vector<TensorDesc>& descs, const std::vector<Member>& members, int strip_cols, int step, int sm_count, double strip_cost, double item_cost,
+                 double limit, std::vector<WorkItem>& items, std::vector<int32_t>& starts) {
   const auto fill = [&](double share, bool emit) -> int {
     int cta = 0;
     double room = share;
     if (emit) starts.assign(1, 0);
     for (const Member& m : members) {
       const TensorDesc& t = descs[m.tensor];
-      const int64_t step = m.row_step, blocks = (t.rows + step - 1) / step;
+      const int64_t blocks = (m.rows + step - 1) / step;
       for (int64_t c0 = 0; c0 < t.cols; c0 += strip_cols) {
         const int ncols = static_cast<int>(std::min<int64_t>(strip_cols, t.cols - c0));
         const double tiles = (ncols + 127) / 128, wide = tiles * static_cast<double>(step / 128), begin = strip_cost * t.rank * tiles + item_cost;
@@ -332,7 +354,7 @@ double share_out(const std::vector<TensorDesc>& descs, const std::vector<Member>
           }
           take = std::min<int64_t>(std::max<int64_t>(static_cast<int64_t>((room - begin) / wide + 1e-9), 1), blocks - at);
           room -= begin + wide * static_cast<double>(take);
-          if (emit) items.push_back(WorkItem{m.tensor, ncols, step * at, std::min<int64_t>(step * take, t.rows - step * at), c0});
+          if (emit) items.push_back(WorkItem{m.tensor, ncols, step * at, std::min<int64_t>(step * take, m.rows - step * at), c0});
         }
       }
     }
@@ -340,8 +362,12 @@ double share_out(const std::vector<TensorDesc>& descs, const std::vector<Member>
     return cta + 1;
   };
   double tiles = 0.0;
-  for (const Member& m : members) tiles += static_cast<double>((descs[m.tensor].rows + 127) / 128 * ((descs[m.tensor].cols + 127) / 128));
+  for (const Member& m : members) tiles += static_cast<double>((m.rows + 127) / 128 * ((descs[m.tensor].cols + 127) / 128));
   double low = tiles / sm_count, high = 1.25 * low + 1.0;     // (the tiles alone take `low`)
+  if (limit > 0.0) {
+    if (limit <= low || fill(limit, false) > sm_count) return limit;
+    high = std::min(high, limit);
+  }
   while (fill(high, false) > sm_count) {
     low = high;
     high *= 1.5;
@@ -350,6 +376,7 @@ double share_out(const std::vector<TensorDesc>& descs, const std::vector<Member>
     const double mid = 0.5 * (low + high);
     (fill(mid, false) <= sm_count ? high : low) = mid;
   }
+  if (limit > 0.0 && high >= limit) return limit;
   items.clear();
   fill(high, true);
   return high;
@@ -368,7 +395,7 @@ void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>&
     for (const Member& m : members) total += descs[m.tensor].rows * descs[m.tensor].cols;
     const int64_t least = std::min<int64_t>(256 * 2 * g.kc.kpad, 16384);
     const int64_t per = std::min<int64_t>(std::max<int64_t>(total / (static_cast<int64_t>(sm_count) * 2 * 8), least), 1048576);
-    for (const Member& m : members) cut_tensor(descs[m.tensor], m.tensor, m.strip, m.row_step, by_elements, per, g.items);
+    for (const Member& m : members) cut_tensor(descs[m.tensor], m, by_elements, per, g.items);
     return;
   }
   int64_t tiles = 0;
@@ -379,21 +406,24 @@ void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>&
     // same times); an item has a pipeline to fill, which the three-part kernels do ahead where two strips fit
     const double strip_cost = g.kc.precise ? 0.02 : 0.01;
     const double item_cost = tile && g.kc.kpad < 64 ? 0.3 : 0.7;
-    const int widest = members.empty() ? 128 : members[0].strip;
-    double best = share_out(descs, members, widest, sm_count, strip_cost, item_cost, g.items, g.starts);
+    const int widest = members.empty() ? 128 : members[0].strip, step = members.empty() ? 128 : members[0].row_step;      // (the same for all of a group)
+    const double best = share_out(descs, members, widest, step, sm_count, strip_cost, item_cost, 0.0, g.items, g.starts);
     if (widest > 128) {
       std::vector<WorkItem> items;
       std::vector<int32_t> starts;
-      if (share_out(descs, members, 128, sm_count, strip_cost, item_cost, items, starts) < best) {
+      if (share_out(descs, members, 128, step, sm_count, strip_cost, item_cost, 0.0, items, starts) < best) {
         g.items.swap(items);
         g.starts.swap(starts);
       }
     }
+    // Halves of spans of 256 rows where there are more spans than SMs and the shares come out smaller by more than the search resolves: in
+    // whole spans 18 M weights in rows of 1234 and 4937 are 119 shares for 148 SMs.
+    if (step > 128 && tiles > 2 * sms) share_out(descs, members, widest, 128, sm_count, strip_cost, item_cost, 0.98 * best, g.items, g.starts);
     return;
   }
   if (!tile) {
     for (const Member& m : members)
-      cut_tensor(descs[m.tensor], m.tensor, m.strip, m.row_step, by_elements, g.kc.path == PATH_UMMA ? 2 * target : target, g.items);
+      cut_tensor(descs[m.tensor], m, by_elements, g.kc.path == PATH_UMMA ? 2 * target : target, g.items);
     return;
   }
   // Handed out by a counter to one CTA per SM.  Tall items are cheap (an item costs its 128 x 128 tiles and, per 512 octets of
@@ -421,8 +451,8 @@ void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>&
       if (best > 0.0) {
         int64_t done = 0, n_items = 0;
         for (const Member& m : members) {
-          const int64_t strips = (descs[m.tensor].cols + 127) / 128, blocks = blocks_of(descs[m.tensor].rows), h = 3 * done < 2 * tiles ? big : small;
-          const int64_t chunks = (descs[m.tensor].rows + 128 * h - 1) / (128 * h), even = (blocks + chunks - 1) / chunks;
+          const int64_t strips = (descs[m.tensor].cols + 127) / 128, blocks = blocks_of(m.rows), h = 3 * done < 2 * tiles ? big : small;
+          const int64_t chunks = (m.rows + 128 * h - 1) / (128 * h), even = (blocks + chunks - 1) / chunks;
           n_items += strips * ((blocks + even - 1) / even);
           done += blocks * strips;
         }
@@ -432,7 +462,7 @@ void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>&
       trial.clear();
       int64_t done = 0;
       for (const Member& m : members) {
-        cut_tensor(descs[m.tensor], m.tensor, m.strip, m.row_step, by_rows, 128 * (3 * done < 2 * tiles ? big : small), trial);
+        cut_tensor(descs[m.tensor], m, by_rows, 128 * (3 * done < 2 * tiles ? big : small), trial);
         done += ((descs[m.tensor].rows + 127) / 128) * ((descs[m.tensor].cols + 127) / 128);
       }
       std::fill(free_at.begin(), free_at.end(), 0.0);      // heap with the CTA that is free first at [0]
@@ -453,7 +483,7 @@ void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>&
       if (tiles >= 64 * sms) {
         // long sweeps: also even when dealt out in turn, so that neither the model nor the counter has to be right
         std::fill(dealt.begin(), dealt.end(), 0.0);
-        for (size_t i = 0; i < trial.size(); ++i) dealt[i % dealt.size()] += static_cast<double>(trial[i].nrows_or_count) * trial[i].ncols;
+        for (size_t i = 0; i < trial.size(); ++i) dealt[i % dealt.size()] += static_cast<double>(item_rows(descs[trial[i].tensor], trial[i]).second) * trial[i].ncols;
         const double mean = std::accumulate(dealt.begin(), dealt.end(), 0.0) / static_cast<double>(dealt.size());
         if (*std::max_element(dealt.begin(), dealt.end()) > 1.025 * mean) end *= 2.0;
         else even = true;
@@ -517,7 +547,7 @@ void plan(const std::vector<TensorDesc>& descs, const std::vector<int>& which, b
       // fp32 with rank > 8, rows that are not a multiple of eight elements, and low ranks: three-part operands.  (The test hook
       // that sweeps an fp32 image of a 16-bit tensor keeps the one-element-per-thread kernel below.)
       path = vec && t.rank <= 8 ? PATH_FMA : PATH_GENERIC; kpad = t.kpad; strip = kTileStripCols; staged = t.staged;
-      row_step = staged && (t.cols & 7) ? 256 : 128;
+      row_step = by_residue(t) ? 256 : 128;
     } else if (!vec || (t.rank > 8 && !umma_ok && (t.Ufrag == nullptr || multi))) {
       // (the legacy tensor-core kernel applies one term per sweep; several terms take the fallback)
       path = PATH_GENERIC; kpad = 0; strip = 64; row_step = 1;
@@ -532,14 +562,14 @@ void plan(const std::vector<TensorDesc>& descs, const std::vector<int>& which, b
     Group& g = group_for(path, t.dtype, kpad, staged);
     const size_t gi = static_cast<size_t>(&g - out.data());
     if (members.size() <= gi) members.resize(gi + 1);
-    members[gi].push_back(Member{l, strip, row_step});
+    members[gi].push_back(Member{l, strip, row_step, rows_to_cut(t)});
   }
   members.resize(out.size());
   for (size_t gi = 0; gi < out.size(); ++gi)
     if (out[gi].kc.path != PATH_ISO) plan_tiles(descs, members[gi], sm_count, target, out[gi]);
   for (Group& g : out) {
     g.elements = 0;
-    for (const WorkItem& w : g.items) g.elements += g.kc.path == PATH_ISO ? w.nrows_or_count : w.nrows_or_count * w.ncols;
+    for (const WorkItem& w : g.items) g.elements += g.kc.path == PATH_ISO ? w.nrows_or_count : item_rows(descs[w.tensor], w).second * w.ncols;
   }
   for (Group& g : out)
     g.grid = !g.starts.empty() ? static_cast<int>(g.starts.size()) - 1 : static_cast<int>(std::min<int64_t>(static_cast<int64_t>(g.items.size()), static_cast<int64_t>(sm_count) * blocks_per_sm(g.kc)));
@@ -1043,7 +1073,7 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
         at += static_cast<size_t>(rows_pad) * td.kpad * 2;       // (a multiple of 4096 bytes)
       }
       jobs[static_cast<size_t>(job)] = SplitJob{td.U, {td.Ucopy[0], td.Ucopy[1], td.Ucopy[2]}, td.rows, rows_pad, td.rank, td.kpad, td.umma ? td.ushift : -1,
-                                                  td.staged && (td.cols & 7) ? 1 : 0};
+                                                  by_residue(td) ? 1 : 0};
     }
     if (rc == ZGR_OK) rc = tables.copy(ctx);
     if (rc == ZGR_OK) rc = split_jobs(ctx, 0, ctx->n_split_jobs, nullptr);
@@ -1479,15 +1509,16 @@ int zgr_debug_z(zgr_ctx* ctx, uint64_t seed, int32_t tensor, float* dev_out, voi
   // a one-tensor model whose weights are the zeroed output buffer, swept once with scale 1
   std::vector<TensorDesc> one(1, ctx->descs[static_cast<size_t>(tensor)]);
   one[0].data = dev_out;
+  if (one[0].dtype != ZGR_F32) one[0].tile = one[0].staged = 0;      // (its kernels read 16-bit weights)
   const size_t owned_before = ctx->owned.size();
   int rc = ZGR_OK;
-  if (one[0].staged && one[0].dtype == ZGR_F32) {
+  if (one[0].staged) {
     // the tensor's own kernel on the image: its maps of U, and new ones of the weights
     const size_t n_maps = static_cast<size_t>(n_weight_maps(one[0]));
     std::vector<CUtensorMap> maps(n_maps);
     CUtensorMap* d_maps = nullptr;
     if ((reinterpret_cast<uintptr_t>(dev_out) & 15) != 0 || !make_weight_maps(maps.data(), one[0], dev_out, 4)) {
-      one[0].tile = 0;                 // (an image that TMA cannot address: one element per thread)
+      one[0].tile = one[0].staged = 0;                 // (an image that TMA cannot address: one element per thread)
     } else {
       rc = dev_alloc(ctx, &d_maps, n_maps + 3);
       if (rc == ZGR_OK) rc = check(ctx, cudaMemcpy(d_maps, maps.data(), n_maps * sizeof(CUtensorMap), cudaMemcpyHostToDevice));
@@ -1699,8 +1730,8 @@ int zgr_debug_plan(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, 
   int64_t count = 0;
   for (const Group& g : groups)
     for (const WorkItem& w : g.items) {
-      if (count < max_items)
-        out[count] = zgr_plan_item{g.kc.path, g.kc.kpad, w.tensor, w.ncols, w.row0_or_e0, w.nrows_or_count, w.col0};
+      const auto [first, rows] = g.kc.path == PATH_ISO ? std::make_pair(w.row0_or_e0, w.nrows_or_count) : item_rows(descs[w.tensor], w);
+      if (count < max_items) out[count] = zgr_plan_item{g.kc.path, g.kc.kpad, w.tensor, w.ncols, first, rows, w.col0};
       ++count;
     }
   *n_items = count;

@@ -34,7 +34,8 @@ struct TensorDesc {
 
 // One unit of work of a sweep kernel.
 //   flat items (isotropic kernel): elements [e0, e0 + count) of the tensor, e0 a multiple of 8
-//   tile items (guided kernels):   rows [row0, row0 + nrows) x columns [col0, col0 + ncols)
+//   tile items (guided kernels):   rows [row0, row0 + nrows) x columns [col0, col0 + ncols); of a ragged tensor of sweep_staged_kernel in
+//                                  whole blocks of 128 rows, numbered in the order of staged_copy_row
 struct WorkItem {
   int32_t tensor;        // index into the descriptor table
   int32_t ncols;

@@ -114,10 +114,7 @@ struct Quarter {
   }
 };
 __device__ __forceinline__ int u_map(const TensorDesc& td) { return (td.cols & 7) ? 8 : 1; }
-// row blocks of an item: its rows are whole spans of 128 or 256, but for the last of the tensor
-__device__ __forceinline__ int row_blocks(const TensorDesc& td, const WorkItem& w) {
-  return (td.cols & 7) ? 2 * static_cast<int>((w.nrows_or_count + 255) >> 8) : static_cast<int>((w.nrows_or_count + 127) >> 7);
-}
+__device__ __forceinline__ int row_blocks(const WorkItem& w) { return static_cast<int>((w.nrows_or_count + 127) >> 7); }
 
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
@@ -304,7 +301,7 @@ __global__ void __launch_bounds__(kThreadsStaged, 1) sweep_staged_kernel(const _
       const CUtensorMap* umap = maps + u_map(td) + lane;
       const uint32_t box_bytes = parts ? kBoxBytes : 4 * kBoxBytes;
       const int block0 = static_cast<int>(w.row0_or_e0 >> 7), col0 = static_cast<int>(w.col0);
-      const int blocks = row_blocks(td, w);
+      const int blocks = row_blocks(w);
       for (int r = 0; r < blocks && ok; ++r, ++rb) {
         if (rb >= US && !wait0(BAR_U_FREE(ur.i), ur.round ^ 1u, 31)) { ok = false; break; }
         if (lane == 0) mbar_arrive_expect_tx(BAR_U_FULL(ur.i), static_cast<uint32_t>(kParts * L.u_bytes));
@@ -375,7 +372,7 @@ __global__ void __launch_bounds__(kThreadsStaged, 1) sweep_staged_kernel(const _
         const uint32_t idesc = (td.cols & 7) ? idesc_parts : idesc_whole;
         const int g = item_no % GS;
         if (!mbar_wait<true>(BAR_G(g), (item_no / GS) & 1, abort_flag, error, 34)) break;
-        const int blocks = row_blocks(td, w);
+        const int blocks = row_blocks(w);
         for (int r = 0; r < blocks && ok; ++r) {
           const int u = ur.i;
           if (!mbar_wait<true>(BAR_U_FULL(u), ur.round, abort_flag, error, 35)) { ok = false; break; }
@@ -455,7 +452,7 @@ __global__ void __launch_bounds__(kThreadsStaged, 1) sweep_staged_kernel(const _
       T* const base = static_cast<T*>(td.data);
       const PhiloxPre pre = philox_pre(0u, tid, p.term[0].keys);     // (tensors of 2^34 elements and more are not served here)
       const int block0 = static_cast<int>(w.row0_or_e0 >> 7), col0 = static_cast<int>(w.col0), ncols = w.ncols;
-      const int blocks = row_blocks(td, w);
+      const int blocks = row_blocks(w);
       double s_iso = 0.0, s_gd = 0.0, s_z = 0.0;             // SSTATS only
       for (int r = 0; r < blocks && ok; ++r) {
         // the strip of the next item goes into the other buffer before this item's last row block, so that its products run

@@ -10,7 +10,7 @@ import oracle
 from paper_2601_12917_b200 import zgr
 
 from helpers import Pair
-from test_plan import plan
+from test_plan import HALVES, plan
 
 pytestmark = pytest.mark.gpu
 
@@ -56,6 +56,24 @@ def test_norms_codes_and_several_seeds(rank, dtype, cols):
     seeds, lp, lm = [41, 42, 43], [2.1, 1.6, 2.4], [1.9, 2.0, 1.8]
     coeffs = [oracle.update_coefficient(0.0, a, b, p.eps, 1e-4) for a, b in zip(lp, lm)]
     p.call_and_check_multi(seeds, coeffs, lambda: p.lib.restore_update_multi(seeds, lp, lm, 1e-4), "three seeds")
+
+
+# Shares that begin and end in the middle of a span, in last spans of every kind: one seed with norms and without, several seeds.
+@pytest.mark.parametrize("rank,bits", [(16, 16), (64, 32)])
+def test_shares_in_halves_of_spans(rank, bits):
+    ranks = [min(rank, m) for m, _ in HALVES]
+    assert any(it.row0_or_e0 % 256 for it in plan(HALVES, ranks, [zgr.BF16] * len(HALVES), bits=bits))
+    p = Pair(HALVES, ranks, "bf16", bits=bits, seed=rank, stats=True)
+    p.step(seed=21, lp=2.2, lm=1.9, lr=1e-4)
+    got = p.lib.get_stats(21)
+    for l in range(len(HALVES)):
+        np.testing.assert_allclose(got[l], oracle.stats_tensor(p.oracle_tensor(l), 21, l, bits, p.a, p.b), rtol=2e-5, atol=1e-9)
+    p.lib.enable_stats(False)
+    p.call_and_check(22, 1e-3, lambda: p.lib.perturb(22, 1e-3), "perturb")
+    p.call_and_check(22, -1e-3, lambda: p.lib.restore_update(22, 2.0, 2.0, 0.0), "restore")
+    coeffs = [oracle.update_coefficient(0.0, 2.1, 1.9, p.eps, 1e-4), oracle.update_coefficient(0.0, 1.6, 2.0, p.eps, 1e-4)]
+    p.call_and_check_multi([41, 42], coeffs, lambda: p.lib.restore_update_multi([41, 42], [2.1, 1.6], [1.9, 2.0], 1e-4), "two seeds")
+    assert p.lib.device_status() == 0
 
 
 # A delivered and a constructed subspace reach the copies of U that are kept by residue.

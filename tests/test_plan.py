@@ -142,6 +142,32 @@ def test_large_sets_of_the_tile_kernel(shapes, ranks, dtype, path, sm_count):
         assert {it.path for it in items if ranks[it.tensor] > 0} == {path}
 
 
+# Ragged 16-bit sets that are dealt out in shares: a share begins and ends in the middle of a span of 256 rows where that makes the
+# largest one smaller, down to one tile above the mean (which is a whole number of tiles).  Tiles of 128 rows, two to a span.
+@pytest.mark.parametrize("d,ffn,rank", [(1234, 4937, 16), (871, 3491, 32), (701, 2803, 64), (1534, 6137, 16), (501, 2003, 8)])
+def test_shares_of_ragged_sets_are_even(d, ffn, rank):
+    shapes = [(d, d)] * 4 + [(ffn, d), (d, ffn)]
+    tiles = sum(-(-m // 256) * 2 * -(-n // 128) for m, n in shapes)
+    assert tiles < 12 * 148 and sum(m * n for m, n in shapes) > 5 << 19
+    for multi in (0, 1):
+        items = plan(shapes, [rank] * 6, [zgr.BF16] * 6, multi=multi)
+        check_exact_cover(items, shapes)
+        assert max(-(-it.nrows_or_count // 128) for it in items) <= -(-tiles // 148)
+
+
+# Last spans of every kind: one to eight rows (residues 4-7 without rows up to four), and around a block and a span.
+HALVES = [(256 * (i % 3) + r, 263 + 16 * i) for i, r in enumerate([1, 3, 4, 5, 7, 8, 9, 127, 128, 132, 133, 252, 255, 256])] + [(2500, 1029)]
+
+
+@pytest.mark.parametrize("sm_count", [148, 100])
+def test_halves_of_last_spans_are_covered(sm_count):
+    items = plan(HALVES, [min(16, m) for m, _ in HALVES], [zgr.F16] * len(HALVES), sm_count=sm_count)
+    check_exact_cover(items, HALVES)
+    for cnt in brute_force_counts(items, HALVES):
+        assert cnt.min() == 1 and cnt.max() == 1
+    assert any(it.row0_or_e0 % 256 for it in items)
+
+
 def test_alpha_one_plans_everything_as_isotropic_and_errors_are_reported():
     items = plan([(64, 256), (1, 100)], [8, 0], [zgr.BF16, zgr.BF16], alpha=1.0)
     assert {it.path for it in items} == {0}
