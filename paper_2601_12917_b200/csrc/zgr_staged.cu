@@ -451,10 +451,13 @@ __global__ void __launch_bounds__(kThreadsStaged, 1) sweep_staged_kernel(const _
       const int block0 = static_cast<int>(w.row0_or_e0 >> 7), col0 = static_cast<int>(w.col0), ncols = w.ncols;
       const int blocks = row_blocks(w);
       double s_iso = 0.0, s_gd = 0.0, s_z = 0.0;             // SSTATS only
+      // The strip of the next item goes into the other buffer before this group's last tile of this item, so that its products run
+      // while that one is worked on: in the last row block, or where that holds one tile, the other group's, in the one before it.
+      // (16-bit matrices of a few row blocks, us a step against the last row block for both groups: 128 wide, rank 8, 8 M weights 59.2 / 57.2;
+      // 512 wide, 13 M 60.4 / 57.5; 120 M ragged 465 / 456.  Several seeds on 100 M: 552 / 562, hence not there.)
+      const int strip_at = NSUB == 2 || MULTI || GS == 1 || blocks == 1 || ((t + blocks - 1) & 1) == grp ? blocks - 1 : blocks - 2;
       for (int r = 0; r < blocks && ok; ++r) {
-        // the strip of the next item goes into the other buffer before this item's last row block, so that its products run
-        // while this one is worked on
-        if (r + 1 == blocks) {
+        if (r == strip_at) {
           it_next = take(item_no + 1);
           if (GS == 2 && it_next < p.n_items) {
             if (!products_done(before)) { ok = false; break; }
