@@ -238,9 +238,7 @@ def roofline_of(kernels, eb, peak, peak_kind):
         return None, None
     per_launch_ms = top["ms_total"] / top["launches"]
     achieved = 2 * eb * top["elements"] / (per_launch_ms * 1e-3) / 1e9
-    # groups of the CUDA-core and of the fallback path that run on the tile kernel carry its contraction width
-    tile = (top["path"] == "fma" and top["kpad"] == 16) or (top["path"] == "generic" and top["kpad"] > 0)
-    kname = f"sweep_{'tile' if tile else top['path']}_kernel(k={top['kpad']})"
+    kname = f"sweep_{top['kernel']}_kernel(k={top['kpad']})"
     return top, {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                  "peak_kind": f"of {peak_kind}", "kernel": kname, "launches": top["launches"], "ms_per_launch": per_launch_ms,
                  "algorithmic_bytes_per_launch": 2 * eb * top["elements"],

@@ -300,18 +300,22 @@ int zgr_debug_z_tcgen05(zgr_ctx* ctx, uint64_t seed, int32_t tensor, float* dev_
  * width (an item's last octet of a row may reach into the next strip there).  `tensors[].data / U` are only inspected for alignment and
  * null-ness.  tcgen05 != 0 plans as on a device where tensor maps can be made; multi != 0 gives the plan of
  * the multi-seed sweeps.  Up to max_items items are written to out; *n_items receives the full count.
- * Errors as zgr_init (ZGR_EINVAL), plus sm_count < 1 or a null n_items. */
+ * Errors as zgr_init (ZGR_EINVAL), plus sm_count < 1 or a null n_items.
+ * zgr_debug_plan_kernels: the kernel of the same plan that serves each tensor (kernels: n entries), by the numbers below. */
+enum { ZGR_KERNEL_ISO = 0, ZGR_KERNEL_FMA = 1, ZGR_KERNEL_MMA = 2, ZGR_KERNEL_GENERIC = 3, ZGR_KERNEL_UMMA = 4, ZGR_KERNEL_TILE = 5, ZGR_KERNEL_STAGED = 6 };
 typedef struct {
   int32_t path, kpad, tensor, ncols;
   int64_t row0_or_e0, nrows_or_count, col0;
 } zgr_plan_item;
 int zgr_debug_plan(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, int32_t sm_count, int32_t tcgen05, int32_t multi,
                    zgr_plan_item* out, int64_t max_items, int64_t* n_items);
+int zgr_debug_plan_kernels(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, int32_t sm_count, int32_t tcgen05, int32_t multi, int32_t* kernels);
 
 /* Per-kernel timing.  While enabled, every sweep launch is bracketed by CUDA events on its stream.
  * zgr_profile_read synchronises the device, writes one entry per kernel family that ran since the
  * last read (up to max_entries) and clears the record.  path, kpad: as in zgr_plan_item; elements = weights covered by one
- * launch.  While enabled every kernel family is launched by itself (1-D tensors of small models otherwise ride along with path 1). */
+ * launch.  zgr_profile_kernels then gives the kernel (ZGR_KERNEL_*) of each entry of the last read, where path and kpad are the same for
+ * two of them.  While enabled every kernel family is launched by itself (1-D tensors of small models otherwise ride along with path 1). */
 typedef struct {
   int32_t path, dtype, kpad, launches;
   int64_t elements;
@@ -319,6 +323,7 @@ typedef struct {
 } zgr_kernel_time;
 int zgr_profile(zgr_ctx* ctx, int32_t enable);
 int zgr_profile_read(zgr_ctx* ctx, zgr_kernel_time* out, int32_t max_entries, int32_t* n_entries);
+int zgr_profile_kernels(zgr_ctx* ctx, int32_t* kernels, int32_t max_entries, int32_t* n_entries);
 
 /* Device-side health.  The tensor-core sweep waits on hardware barriers (TMA, tensor memory) with a
  * time limit; a wait that gives up records a non-zero code, abandons the sweep and lets the kernel

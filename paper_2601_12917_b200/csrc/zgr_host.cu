@@ -126,6 +126,7 @@ struct zgr_ctx {
   int sticky = 0;                     // first CUDA failure, returned by every later call
   int64_t launches = 0;
   bool profiling = false;
+  std::vector<int32_t> profiled;      // kernel_number of the entries of the last zgr_profile_read
   CUtensorMap* d_tmaps = nullptr;     // three per tensor (theta, U hi, U lo); tcgen05 path only
   std::vector<CUtensorMap> tmaps;     // host mirror
   int* d_err = nullptr;               // set by a kernel whose bounded wait gave up
@@ -894,6 +895,39 @@ int validate_model(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, 
   }
   *d_out = d;
   *K_out = K;
+  return ZGR_OK;
+}
+
+// The plan of a sweep as zgr_init would make it, without a device.
+int plan_on_host(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, int sm_count, bool tcgen05, bool multi, std::vector<TensorDesc>& descs,
+                 std::vector<Group>& groups) {
+  int64_t d = 0, K = 0;
+  const int valid = validate_model(tensors, n, cfg, &d, &K);
+  if (valid != ZGR_OK) return valid;
+  const bool guided_on = K > 0 && cfg->alpha < 1.0;
+  const SetSizes sizes = set_sizes(tensors, n);
+  descs.resize(static_cast<size_t>(n));
+  std::vector<int> all(static_cast<size_t>(n));
+  for (int32_t l = 0; l < n; ++l) {
+    const zgr_tensor& t = tensors[l];
+    TensorDesc& td = descs[static_cast<size_t>(l)];
+    std::memset(&td, 0, sizeof(td));
+    td.data = t.data; td.U = t.U; td.rows = t.rows; td.cols = t.cols; td.rank = t.rank; td.id = l; td.dtype = t.dtype; td.qbits = 8;
+    const bool vec = (reinterpret_cast<uintptr_t>(t.data) & 15) == 0 && (t.cols % 8 == 0);
+    if (guided_on && t.rank > 8 && vec && t.dtype != ZGR_F32) {
+      // what zgr_init would have built for this tensor: operand copies for the tensor-core kernels
+      td.kpad = t.rank <= 16 ? 16 : (t.rank <= 32 ? 32 : 64);
+      td.Ufrag = reinterpret_cast<const uint4*>(uintptr_t{16});   // marker only: never dereferenced by the planner
+    }
+    const int kind = tcgen05 ? tensor_core_kind(t, guided_on, sizes) : 0;
+    if (kind != 0) {
+      td.kpad = t.rank <= 16 ? 16 : (t.rank <= 32 ? 32 : 64);
+      (kind == 1 ? td.umma : td.tile) = 1;
+      if (kind == 2) td.staged = staged_kind(t, sizes);
+    }
+    all[static_cast<size_t>(l)] = l;
+  }
+  plan(descs, all, guided_on, cfg->bits_per_normal, sm_count, groups, -1, multi);
   return ZGR_OK;
 }
 
@@ -1699,34 +1733,10 @@ int zgr_build_subspace(zgr_ctx* ctx, int32_t tensor, const float* grads, int32_t
 int zgr_debug_plan(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, int32_t sm_count, int32_t tcgen05, int32_t multi,
                    zgr_plan_item* out, int64_t max_items, int64_t* n_items) {
   if (!n_items || sm_count < 1 || max_items < 0 || (max_items > 0 && !out)) return ZGR_EINVAL;
-  int64_t d = 0, K = 0;
-  const int valid = validate_model(tensors, n, cfg, &d, &K);
-  if (valid != ZGR_OK) return valid;
-  const bool guided_on = K > 0 && cfg->alpha < 1.0;
-  const SetSizes sizes = set_sizes(tensors, n);
-  std::vector<TensorDesc> descs(static_cast<size_t>(n));
-  std::vector<int> all(static_cast<size_t>(n));
-  for (int32_t l = 0; l < n; ++l) {
-    const zgr_tensor& t = tensors[l];
-    TensorDesc& td = descs[static_cast<size_t>(l)];
-    std::memset(&td, 0, sizeof(td));
-    td.data = t.data; td.U = t.U; td.rows = t.rows; td.cols = t.cols; td.rank = t.rank; td.id = l; td.dtype = t.dtype; td.qbits = 8;
-    const bool vec = (reinterpret_cast<uintptr_t>(t.data) & 15) == 0 && (t.cols % 8 == 0);
-    if (guided_on && t.rank > 8 && vec && t.dtype != ZGR_F32) {
-      // what zgr_init would have built for this tensor: operand copies for the tensor-core kernels
-      td.kpad = t.rank <= 16 ? 16 : (t.rank <= 32 ? 32 : 64);
-      td.Ufrag = reinterpret_cast<const uint4*>(uintptr_t{16});   // marker only: never dereferenced by the planner
-    }
-    const int kind = tcgen05 ? tensor_core_kind(t, guided_on, sizes) : 0;
-    if (kind != 0) {
-      td.kpad = t.rank <= 16 ? 16 : (t.rank <= 32 ? 32 : 64);
-      (kind == 1 ? td.umma : td.tile) = 1;
-      if (kind == 2) td.staged = staged_kind(t, sizes);
-    }
-    all[static_cast<size_t>(l)] = l;
-  }
+  std::vector<TensorDesc> descs;
   std::vector<Group> groups;
-  plan(descs, all, guided_on, cfg->bits_per_normal, sm_count, groups, -1, multi != 0);
+  const int rc = plan_on_host(tensors, n, cfg, sm_count, tcgen05 != 0, multi != 0, descs, groups);
+  if (rc != ZGR_OK) return rc;
   int64_t count = 0;
   for (const Group& g : groups)
     for (const WorkItem& w : g.items) {
@@ -1735,6 +1745,17 @@ int zgr_debug_plan(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, 
       ++count;
     }
   *n_items = count;
+  return ZGR_OK;
+}
+
+int zgr_debug_plan_kernels(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, int32_t sm_count, int32_t tcgen05, int32_t multi, int32_t* kernels) {
+  if (!kernels || sm_count < 1) return ZGR_EINVAL;
+  std::vector<TensorDesc> descs;
+  std::vector<Group> groups;
+  const int rc = plan_on_host(tensors, n, cfg, sm_count, tcgen05 != 0, multi != 0, descs, groups);
+  if (rc != ZGR_OK) return rc;
+  for (const Group& g : groups)
+    for (const WorkItem& w : g.items) kernels[w.tensor] = kernel_number(g.kc);
   return ZGR_OK;
 }
 
@@ -1794,6 +1815,7 @@ int zgr_profile_read(zgr_ctx* ctx, zgr_kernel_time* out, int32_t max_entries, in
   const int rc = check(ctx, cudaDeviceSynchronize());
   if (rc != ZGR_OK) return rc;
   int32_t n = 0;
+  ctx->profiled.clear();
   for (std::vector<Group>* gs : {&ctx->groups, &ctx->groups_multi})
   for (Group& g : *gs) {
     if (g.timed.empty()) continue;
@@ -1812,11 +1834,19 @@ int zgr_profile_read(zgr_ctx* ctx, zgr_kernel_time* out, int32_t max_entries, in
       o.launches = static_cast<int32_t>(g.timed.size());
       o.elements = g.elements;
       o.ms_total = total;
+      ctx->profiled.push_back(kernel_number(g.kc));
       ++n;
     }
     g.timed.clear();
   }
   *n_entries = n;
+  return ZGR_OK;
+}
+
+int zgr_profile_kernels(zgr_ctx* ctx, int32_t* kernels, int32_t max_entries, int32_t* n_entries) {
+  if (!ctx || !kernels || !n_entries || max_entries < 0) return ZGR_EINVAL;
+  *n_entries = std::min(max_entries, static_cast<int32_t>(ctx->profiled.size()));
+  std::copy_n(ctx->profiled.begin(), *n_entries, kernels);
   return ZGR_OK;
 }
 

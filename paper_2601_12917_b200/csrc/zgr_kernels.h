@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 #include <stddef.h>
 
+#include "zgr.h"
 #include "zgr_internal.h"
 
 namespace zgr {
@@ -31,6 +32,8 @@ constexpr int iso_blocks_per_sm(bool precise, bool multi, bool stats) { return !
 // The groups that sweep_staged_kernel and sweep_tile_kernel serve: rank <= 8 tensors in whole octets are counted under the path of the CUDA-core
 // kernel (whose own widths are 4 and 8), the others under that of the fallback kernel (whose own width is 0).
 inline bool is_tile(const KernelChoice& kc) { return (kc.path == PATH_FMA && kc.kpad == 16) || (kc.path == PATH_GENERIC && kc.kpad > 0); }
+// ZGR_KERNEL_*: the paths, and behind them the two kernels that share paths with others
+inline int kernel_number(const KernelChoice& kc) { return is_tile(kc) ? (kc.staged ? ZGR_KERNEL_STAGED : ZGR_KERNEL_TILE) : kc.path; }
 
 int mma_strip_cols(int kpad);     // columns of a CTA strip on the tensor-core path
 int mma_rows_per_iter(int kpad);  // rows a CTA advances per iteration there

@@ -44,6 +44,7 @@ class ZgrKernelTime(ctypes.Structure):
 
 
 PATH_NAMES = {0: "iso", 1: "fma", 2: "mma", 3: "generic", 4: "umma"}
+KERNEL_NAMES = {**PATH_NAMES, 5: "tile", 6: "staged"}      # sweep_<name>_kernel
 
 
 class ZgrError(RuntimeError):
@@ -283,8 +284,10 @@ class Zgr:
         arr = (ZgrKernelTime * 64)()
         n = ctypes.c_int32()
         _check(lib().zgr_profile_read(self._h, arr, 64, ctypes.byref(n)), "zgr_profile_read")
-        return [{"path": PATH_NAMES.get(e.path, str(e.path)), "dtype": e.dtype, "kpad": e.kpad, "launches": e.launches,
-                 "elements": e.elements, "ms_total": e.ms_total} for e in arr[: n.value]]
+        kernels = (ctypes.c_int32 * 64)()
+        _check(lib().zgr_profile_kernels(self._h, kernels, ctypes.c_int32(64), ctypes.byref(n)), "zgr_profile_kernels")
+        return [{"path": PATH_NAMES.get(e.path, str(e.path)), "kernel": KERNEL_NAMES[k], "dtype": e.dtype, "kpad": e.kpad, "launches": e.launches,
+                 "elements": e.elements, "ms_total": e.ms_total} for e, k in zip(arr[: n.value], kernels)]
 
     def enable_stats(self, on: bool) -> None:
         """Keep the norm bookkeeping inside the first perturbation of every seed (zgr_enable_stats)."""

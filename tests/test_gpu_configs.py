@@ -196,7 +196,8 @@ def test_trajectory_statistic(name):
 
 @pytest.mark.parametrize("dtype,rows,cols,rank", [
     ("bf16", 34000, 131072, 16),     # tcgen05 kernel, 4.46e9 elements: element indices beyond 2^32
-    ("f32", 1100, 4194304, 8),       # CUDA-core kernel, 4.61e9 elements, very long rows
+    ("f32", 1100, 4194304, 8),       # staged kernel, 4.61e9 elements, very long rows
+    ("f32", 1100, 4194304, 4),       # CUDA-core kernel
     ("bf16", 1, 4400000008, 0),      # isotropic kernel on one vector of 4.4e9 elements
 ])
 def test_tensor_with_more_than_2_pow_32_elements(dtype, rows, cols, rank):

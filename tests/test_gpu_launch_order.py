@@ -49,9 +49,9 @@ def _early_reader():
     return launch
 
 
-# The last 256 words of the last matrix, i.e. of the work that a sweep comes to last, for every kernel family: TMA-staged, tile
-# (ragged, fp32), CUDA-core, isotropic, the last in one and in two launches a sweep.
-@pytest.mark.parametrize("dtype,cols,rank,alpha", [("bfloat16", 4096, 32, 0.5), ("bfloat16", 4098, 16, 0.5), ("float32", 4096, 24, 0.5), ("float32", 4096, 4, 0.5),
+# The last 256 words of the last matrix, i.e. of the work that a sweep comes to last, for every kernel family: TMA-staged in two and in three
+# parts (ragged, fp32), tile, CUDA-core, isotropic, the last in one and in two launches a sweep.
+@pytest.mark.parametrize("dtype,cols,rank,alpha", [("bfloat16", 4096, 32, 0.5), ("bfloat16", 4098, 16, 0.5), ("float32", 4096, 24, 0.5), ("float32", 4098, 24, 0.5), ("float32", 4096, 4, 0.5),
                                                    ("float16", 4096, 0, 1.0)])
 @pytest.mark.parametrize("vector", [False, True])
 def test_a_kernel_behind_a_sweep_sees_its_weights(dtype, cols, rank, alpha, vector):

@@ -190,12 +190,13 @@ def test_layerwise_sweeps_of_low_rank_tensors_on_both_streams(dtype):
     assert a.lib.device_status() == 0 and a.lib.state()[0] is False
 
 
-# Layers with more items than resident blocks (CUDA-core kernel 2 per SM, isotropic kernel 5 or 8, tile kernel 1), so that every
+# Layers with more items than resident blocks (CUDA-core kernel 2 per SM, isotropic kernel 5 or 8, staged and tile kernel 1), so that every
 # layer draws on the item counter of its stream and has to leave it at zero for the next sweep.  (Path 0 is the
-# isotropic family, 1 the CUDA-core and 3 the tile kernel; the plan says that the layers are large enough.)
+# isotropic family, 1 the CUDA-core kernel and 3 the staged one or, the last case, the tile kernel; the plan says that the layers are large enough.)
 @pytest.mark.parametrize("dtype,shapes,ranks,ends,path,blocks", [
     ("f32", [(2000, 520), (1, 3_000_000)] * 2, [4, 0] * 2, [2, 4], 1, 2), ("bf16", [(2000, 520), (1, 3_000_000)] * 2, [4, 0] * 2, [2, 4], 1, 2),
-    ("bf16", [(2000, 5001)] * 3, [16] * 3, [1, 2, 3], 3, 1), ("f32", [(1500, 10248)] * 2, [24] * 2, [1, 2], 3, 1)])
+    ("bf16", [(2000, 5001)] * 3, [16] * 3, [1, 2, 3], 3, 1), ("f32", [(1500, 10248)] * 2, [24] * 2, [1, 2], 3, 1),
+    ("f32", [(2000, 5001)] * 3, [16] * 3, [1, 2, 3], 3, 1)])
 def test_layerwise_item_counters_of_both_streams(dtype, shapes, ranks, ends, path, blocks):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     items = plan(shapes, ranks, [{"f32": zgr.F32, "bf16": zgr.BF16}[dtype]] * len(shapes), sm_count=sms)

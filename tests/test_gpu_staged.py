@@ -10,7 +10,7 @@ import oracle
 from paper_2601_12917_b200 import zgr
 
 from helpers import Pair
-from test_plan import HALVES, plan
+from test_plan import HALVES, kernels, plan
 
 pytestmark = pytest.mark.gpu
 
@@ -28,7 +28,9 @@ def test_ragged_rows(rank, dtype, bits):
     kinds = [{"f16": zgr.F16, "bf16": zgr.BF16}[dtype]] * len(shapes)
     assert all(it.row0_or_e0 % 256 == 0 for it in plan(shapes, ranks, kinds, bits=bits) if it.path == 3)      # whole spans
     p = Pair(shapes, ranks, dtype, bits=bits, seed=rank)
+    p.lib.profile(True)
     reports = p.step(seed=17, lp=2.4, lm=1.7, lr=1e-4)
+    assert {k["kernel"] for k in p.lib.profile_read()} == {"staged", "iso"}
     assert all(rep["moved"] > 0.3 for call in reports[:2] for rep in call)
     assert p.lib.device_status() == 0
 
@@ -71,6 +73,22 @@ def test_shares_in_halves_of_spans(rank, bits):
     p.lib.enable_stats(False)
     p.call_and_check(22, 1e-3, lambda: p.lib.perturb(22, 1e-3), "perturb")
     p.call_and_check(22, -1e-3, lambda: p.lib.restore_update(22, 2.0, 2.0, 0.0), "restore")
+    coeffs = [oracle.update_coefficient(0.0, 2.1, 1.9, p.eps, 1e-4), oracle.update_coefficient(0.0, 1.6, 2.0, p.eps, 1e-4)]
+    p.call_and_check_multi([41, 42], coeffs, lambda: p.lib.restore_update_multi([41, 42], [2.1, 1.6], [1.9, 2.0], 1e-4), "two seeds")
+    assert p.lib.device_status() == 0
+
+
+# Items from the counter where the accumulated norms, one strip at a time (rank above 32) and several seeds go with them.
+def test_norms_and_several_seeds_from_the_counter():
+    shapes, ranks = [(4000, 5001), (2000, 5001), (1, 77)], [64, 40, 0]
+    assert kernels(shapes, ranks, [zgr.BF16] * 3) == ["staged", "staged", "iso"]
+    assert sum(it.path == 3 for it in plan(shapes, ranks, [zgr.BF16] * 3)) > torch.cuda.get_device_properties(0).multi_processor_count
+    p = Pair(shapes, ranks, "bf16", bits=16, seed=9, stats=True)
+    p.call_and_check(3, 1e-3, lambda: p.lib.perturb(3, 1e-3), "perturb")
+    got = p.lib.get_stats(3)
+    for l in range(3):
+        np.testing.assert_allclose(got[l], oracle.stats_tensor(p.oracle_tensor(l), 3, l, 16, p.a, p.b), rtol=2e-5, atol=1e-9)
+    p.call_and_check(3, -1e-3, lambda: p.lib.restore_update(3, 2.0, 2.0, 0.0), "restore")
     coeffs = [oracle.update_coefficient(0.0, 2.1, 1.9, p.eps, 1e-4), oracle.update_coefficient(0.0, 1.6, 2.0, p.eps, 1e-4)]
     p.call_and_check_multi([41, 42], coeffs, lambda: p.lib.restore_update_multi([41, 42], [2.1, 1.6], [1.9, 2.0], 1e-4), "two seeds")
     assert p.lib.device_status() == 0

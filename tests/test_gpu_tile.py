@@ -1,5 +1,5 @@
 """The kernels that are chosen by size, type and row length, at the sizes where they can go wrong (needs a B200):
-edges of tiles and octets in the tile kernel, low ranks on the tensor-core kernels, more items than blocks, bases on
+edges of tiles and octets in the tile kernel (the staged kernel, which takes larger sets, has a file of its own), low ranks on the tensor-core kernels, more items than blocks, bases on
 either side of the cluster and grid launches.  Every call against the oracle, with the tolerances of helpers.py."""
 import numpy as np
 import pytest
@@ -9,7 +9,7 @@ import oracle
 from paper_2601_12917_b200 import synth, zgr
 
 from helpers import Pair
-from test_plan import plan
+from test_plan import kernels, plan
 
 pytestmark = pytest.mark.gpu
 
@@ -71,12 +71,14 @@ def test_tile_kernel_codes_in_whole_octets(code_bits, n_rows):
     p.call_and_check_multi(seeds, coeffs, lambda: p.lib.restore_update_multi(seeds, lp, lm, 1e-4), "two seeds")
 
 
-# Sets with more items than SMs: the tile kernel draws on its item counter (below about 29 M weights each block has a share of its own),
-# in items of the two heights that the planner chose, and puts the counter back to zero: five sweeps of one context in a row.
-@pytest.mark.parametrize("dtype,shapes,ranks", [("bf16", [(4000, 5001), (2000, 5001), (1, 77)], [16, 16, 0]),
-                                                 ("f32", [(4000, 5128), (2000, 5128), (1, 77)], [24, 24, 0])])
-def test_tile_items_from_the_counter(dtype, shapes, ranks):
+# Sets with more items than SMs: the staged and the tile kernel draw on their item counters (below about 29 M weights each block has a share of its
+# own), in items of the two heights that the planner chose, and put the counter back to zero: five sweeps of one context in a row.
+@pytest.mark.parametrize("dtype,shapes,ranks,kernel", [("bf16", [(4000, 5001), (2000, 5001), (1, 77)], [16, 16, 0], "staged"),
+                                                        ("f32", [(4000, 5128), (2000, 5128), (1, 77)], [24, 24, 0], "staged"),
+                                                        ("f32", [(4000, 5001), (2000, 5001), (1, 77)], [24, 24, 0], "tile")])
+def test_tile_items_from_the_counter(dtype, shapes, ranks, kernel):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert kernels(shapes, ranks, [{"f32": zgr.F32, "bf16": zgr.BF16}[dtype]] * 3, sm_count=sms) == [kernel, kernel, "iso"]
     items = [it for it in plan(shapes, ranks, [{"f32": zgr.F32, "bf16": zgr.BF16}[dtype]] * 3, sm_count=sms) if it.path == 3]
     assert len(items) > sms and (32 + 16) * 40 >= 12 * sms        # more items than blocks, and enough tiles for the counter
     assert len({(it.nrows_or_count + 127) // 128 for it in items}) > 1
@@ -87,7 +89,7 @@ def test_tile_items_from_the_counter(dtype, shapes, ranks):
     assert p.lib.device_status() == 0
 
 
-# Low ranks: sets of 2^21 weights and more leave the CUDA-core kernel for the tile kernel, which is reported under the same path with its
+# Low ranks: sets of 2^21 weights and more leave the CUDA-core kernel for the tile kernel (larger ones for the staged one), which is reported under the same path with its
 # contraction width (narrow and ragged last strips of the CUDA-core kernel are in the parity tests).
 @pytest.mark.parametrize("dtype,path", [("bf16", "fma"), ("f16", "fma"), ("f32", "fma")])
 @pytest.mark.parametrize("rank", [1, 4, 8])
@@ -95,7 +97,9 @@ def test_low_rank_sets_of_some_size(dtype, path, rank):
     p = Pair([(1030, 2056), (1, 40), (140, 72)], [rank, 0, rank], dtype, bits=16, seed=2)
     p.lib.profile(True)
     p.step(seed=6, lp=2.0, lm=1.7, lr=1e-4)
-    assert {k["path"]: k["kpad"] for k in p.lib.profile_read()} == {path: 16, "iso": 0}
+    read = p.lib.profile_read()
+    assert {k["path"]: k["kpad"] for k in read} == {path: 16, "iso": 0}
+    assert {k["kernel"] for k in read} == {"tile", "iso"}
     assert p.lib.device_status() == 0
 
 

@@ -33,6 +33,18 @@ def plan(shapes, ranks, dtypes, bits=16, sm_count=148, tcgen05=1, multi=0, alpha
     return list(items)
 
 
+def kernels(shapes, ranks, dtypes, bits=16, sm_count=148, multi=0, misalign=()):
+    """Name of the kernel that serves each tensor (zgr_debug_plan_kernels)."""
+    n = len(shapes)
+    arr = (zgr.ZgrTensor * n)()
+    for l, ((m, c), r, dt) in enumerate(zip(shapes, ranks, dtypes)):
+        arr[l] = zgr.ZgrTensor(0x100000 * (l + 1) + (4 if l in misalign else 0), m, c, dt, r, 0x40000000 if r else None)
+    cfg = zgr.ZgrConfig(0.5, 1e-3, zgr.SCALE_UNIT, bits)
+    out = (ctypes.c_int32 * n)()
+    assert zgr.lib().zgr_debug_plan_kernels(arr, n, ctypes.byref(cfg), ctypes.c_int32(sm_count), ctypes.c_int32(1), ctypes.c_int32(multi), out) == zgr.OK
+    return [zgr.KERNEL_NAMES[k] for k in out]
+
+
 def check_exact_cover(items, shapes):
     per_tensor = {}
     for it in items:
@@ -140,6 +152,17 @@ def test_large_sets_of_the_tile_kernel(shapes, ranks, dtype, path, sm_count):
         items = plan(shapes, ranks, [dtype] * len(shapes), sm_count=sm_count, multi=multi)
         check_exact_cover(items, shapes)
         assert {it.path for it in items if ranks[it.tensor] > 0} == {path}
+
+
+# Both kernels with three-part operands carry the path of what they stand in for; what tells them apart.
+@pytest.mark.parametrize("shapes,ranks,dtype,misalign,expected", [
+    ([(1300, 2051), (40, 15), (1, 9)], [16, 8, 0], zgr.BF16, (), ["staged", "tile", "iso"]), ([(300, 2051)], [16], zgr.F16, (), ["tile"]),
+    ([(1300, 2051), (500, 2051)], [16, 16], zgr.F16, (1,), ["staged", "tile"]), ([(4000, 5001), (2000, 5128)], [24, 24], zgr.F32, (), ["tile", "staged"]),
+    ([(1300, 2056)], [8], zgr.BF16, (), ["staged"]), ([(500, 2056)], [8], zgr.BF16, (), ["fma"]), ([(1300, 2056)], [9], zgr.BF16, (), ["umma"]),
+    ([(8192, 10240)], [4], zgr.F32, (), ["fma"])])
+def test_kernel_of_each_tensor(shapes, ranks, dtype, misalign, expected):
+    assert kernels(shapes, ranks, [dtype] * len(shapes), misalign=misalign) == expected
+    assert zgr.lib().zgr_debug_plan_kernels(None, 0, None, ctypes.c_int32(148), ctypes.c_int32(1), ctypes.c_int32(0), None) == zgr.EINVAL
 
 
 # Ragged 16-bit sets that are dealt out in shares: a share begins and ends in the middle of a span of 256 rows where that makes the
