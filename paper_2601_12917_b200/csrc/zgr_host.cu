@@ -229,11 +229,11 @@ int64_t rows_before(const TensorDesc& td, int64_t block) {
   const int64_t row0 = std::min(block / 2 * 256, td.rows), span = std::min<int64_t>(td.rows - row0, 256);
   return row0 + (block & 1 ? span / 8 * 4 + std::min<int64_t>(span & 7, 4) : 0);
 }
+// Blocks of a tensor of so many rows that hold any: residues 4-7 of the last span may be empty.
+int64_t blocks_in_spans(int64_t rows) { return rows / 256 * 2 + ((rows & 255) > 4 ? 2 : (rows & 255) > 0); }
 // Rows that a tensor is cut into items by: its own, or its blocks in that order that hold any.
 int64_t rows_to_cut(const TensorDesc& td) {
-  if (!by_residue(td)) return td.rows;
-  const int64_t blocks = copy_rows(td) / 128;
-  return 128 * (rows_before(td, blocks - 1) < td.rows ? blocks : blocks - 1);
+  return by_residue(td) ? 128 * blocks_in_spans(td.rows) : td.rows;
 }
 // First row and number of rows of an item: of the tensor, or in that order.
 std::pair<int64_t, int64_t> item_rows(const TensorDesc& td, const WorkItem& w) {
@@ -247,6 +247,9 @@ bool whole_octets(const zgr_tensor& t) { return (reinterpret_cast<uintptr_t>(t.d
 // all that the kernels with three-part operands may serve.
 struct SetSizes {
   int64_t low[2] = {0, 0}, three_part[2] = {0, 0};      // [0] 16-bit, [1] fp32
+  // of the latter those in whole octets, the tiles of 128 x 128 that they fill and the strips of these, and the tiles of ragged 16-bit rows on the tile
+  // kernel and, in spans of 256 rows, on the staged one
+  int64_t octets[2] = {0, 0}, octet_tiles[2] = {0, 0}, octet_strips[2] = {0, 0}, ragged_tiles[2] = {0, 0};
 };
 SetSizes set_sizes(const zgr_tensor* tensors, int32_t n) {
   SetSizes s;
@@ -256,9 +259,29 @@ SetSizes set_sizes(const zgr_tensor* tensors, int32_t n) {
     const int f32 = t.dtype == ZGR_F32;
     const bool low = t.rank <= 8 && whole_octets(t);
     if (low) s.low[f32] += t.rows * t.cols;
-    if (low || f32 || !whole_octets(t)) s.three_part[f32] += t.rows * t.cols;
+    if (!low && !f32 && whole_octets(t)) continue;
+    s.three_part[f32] += t.rows * t.cols;
+    const int64_t strips = (t.cols + 127) / 128, tiles = (t.rows + 127) / 128 * strips;
+    if (whole_octets(t)) {
+      s.octets[f32] += t.rows * t.cols;
+      s.octet_tiles[f32] += tiles;
+      s.octet_strips[f32] += strips;
+    } else if (!f32) {
+      s.ragged_tiles[0] += tiles;
+      s.ragged_tiles[1] += blocks_in_spans(t.rows) * strips;
+    }
   }
   return s;
+}
+// What the ragged 16-bit tensors of a set take on the staged kernel, in tiles of the busiest SM on the tile kernel: a tile of the staged one is
+// shorter, the less so the more seeds share it, but spans of 256 rows may cost some more.
+bool ragged_on_staged(const SetSizes& sizes, int sm_count, int n_terms) {
+  const auto busiest = [&](int64_t tiles) {
+    const double mean = static_cast<double>(tiles) / sm_count;
+    return mean < 12.0 ? std::ceil(mean) : mean;
+  };
+  const double tile = n_terms == 1 ? 0.75 : (n_terms == 2 ? 0.85 : (n_terms == 3 ? 0.88 : 0.94));
+  return tile * busiest(sizes.ragged_tiles[1]) <= busiest(sizes.ragged_tiles[0]);
 }
 
 // Which kernel family serves a tensor: 1 the TMA-staged one with two-part operands (16-bit weights in whole octets, rank > 8), 2 those with
@@ -288,14 +311,25 @@ int tensor_core_kind(const zgr_tensor& t, bool guided_on, const SetSizes& sizes)
 // Which of the two kernels with three-part operands: 1 the staged one, 0 the tile kernel.  TMA wants the weights on a 16-byte boundary
 // and rows that hold a whole octet wherever it begins; the staged kernel keeps the high counter word of the generator fixed.
 // Small sets stay with the tile kernel, whose sixteen epilogue warps share every tile (two groups on alternate tiles leave half of
-// them idle when a CTA has one or two): us a step tile / staged, bf16 rank 8 2.4 M 26.8 / 29.6, 4.0 M 32.1 / 31.9; ragged 16-bit rank 16
-// 1.6 M 34.0 / 42.6, 2.7 M 47.0 / 45.5, 18 M 135 / 106; fp32 1.0 M 27.6 / 28.7, 3.1 M 41.4 / 39.9.  fp32 rows that are no multiple of eight
+// them idle when a CTA has one or two): us a step tile / staged, bf16 rank 8 2.4 M 26.8 / 29.6, 4.0 M 32.1 / 31.7, 8 M 59.8 / 57.5; ragged 16-bit
+// rank 16 1.6 M 34.0 / 42.6, 2.7 M 47.0 / 45.5, 3.0 M 48.5 / 44.6, 18 M 135 / 95; fp32 up to rank 16 3.1 M 38.4 / 39.0, 5.9 M 58.1 / 59.7,
+// 6.3 M 49.9 / 51.4, 7.1 M 49.2 / 48.8, 19 M 106 / 101, above 3.9 M 49.2 / 47.9, 4.9 M 57.2 / 54.3, 6.3 M 70.2 / 63.7.  fp32 rows that are no multiple of eight
 // elements do so at any size: 96 M weights of rank 16 in rows of 1001 and 4001 469 / 479 (the accurate transform hides what the tile
 // kernel spends on its transposition, and the residues cost half-empty tiles).
-int staged_kind(const zgr_tensor& t, const SetSizes& sizes) {
+//
+// Tiles that are not full cost the staged kernel more (its groups take full and half-empty ones in turn): whole octets stay with the tile kernel
+// below 0.7 of the tiles' area, in fp32 up to rank 16 (16-bit matrices of 136 and 4 x 136, 40 layers: .38 99 / 107; 192: .68 115 / 128;
+// 320: .78 162 / 161; 448: .84 111 / 106.  fp32 168: .52 148 / 156; 200: .67 156 / 165; 320: .78 193 / 186; rank 64 192: 207 / 190).  So do
+// 16-bit sets of many items (from the counter) in strips of under four tiles (matrices of 256 and 4 x 256: 2.7 146 / 152; 320: 3.8 253 / 264;
+// 384: 4.0 141 / 132).  Ragged rows: ragged_on_staged (matrices of 125: 20 tiles a layer against 12  86 / 105; 261: 114 against 90  191 / 171).
+int staged_kind(const zgr_tensor& t, const SetSizes& sizes, int sm_count) {
   const int f32 = t.dtype == ZGR_F32;
-  return (reinterpret_cast<uintptr_t>(t.data) & 15) == 0 && t.cols >= 16 && t.cols < (int64_t{1} << 31) - 256 && t.rows * t.cols < (int64_t{1} << 34) &&
-         !(f32 && (t.cols & 7) != 0) && sizes.three_part[f32] >= 5 * (int64_t{1} << 19);
+  if ((reinterpret_cast<uintptr_t>(t.data) & 15) != 0 || t.cols < 16 || t.cols >= (int64_t{1} << 31) - 256 || t.rows * t.cols >= (int64_t{1} << 34)) return 0;
+  if ((t.cols & 7) != 0) return !f32 && sizes.three_part[0] >= 5 * (int64_t{1} << 19) && ragged_on_staged(sizes, sm_count, 1);
+  const double full = static_cast<double>(sizes.octets[f32]) / (16384.0 * static_cast<double>(sizes.octet_tiles[f32]));
+  if (f32) return sizes.three_part[1] >= (t.rank <= 16 ? 13 : 5) * (int64_t{1} << 19) && (t.rank > 16 || full >= 0.7);
+  const bool short_items = sizes.octet_tiles[0] >= 12 * sm_count && sizes.octet_tiles[0] < 4 * sizes.octet_strips[0];
+  return sizes.three_part[0] >= 5 * (int64_t{1} << 19) && full >= 0.7 && !short_items;
 }
 
 bool umma_wanted() {
@@ -923,7 +957,7 @@ int plan_on_host(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, in
     if (kind != 0) {
       td.kpad = t.rank <= 16 ? 16 : (t.rank <= 32 ? 32 : 64);
       (kind == 1 ? td.umma : td.tile) = 1;
-      if (kind == 2) td.staged = staged_kind(t, sizes);
+      if (kind == 2) td.staged = staged_kind(t, sizes, sm_count);
     }
     all[static_cast<size_t>(l)] = l;
   }
@@ -1036,7 +1070,7 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
       // (capped at 2^12, which leaves fp16 room for entries up to 16 in size); the bf16 parts need no scaling
       if (kind == 1) td.ushift = std::min<int32_t>(12, static_cast<int32_t>(std::ceil(0.5 * std::log2(static_cast<double>(t.rows)))));
       (kind == 1 ? td.umma : td.tile) = 1;
-      if (kind == 2) td.staged = staged_kind(t, sizes);
+      if (kind == 2) td.staged = staged_kind(t, sizes, ctx->sm_count);
       operand_bytes += (kind == 1 ? 2 : 3) * static_cast<size_t>(copy_rows(td)) * static_cast<size_t>(td.kpad) * 2;
       if (td.staged) n_staged_maps += static_cast<size_t>(n_weight_maps(td)) + 3;
     }

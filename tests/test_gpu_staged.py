@@ -1,7 +1,7 @@
 """The sweep whose weights are staged by TMA and whose operands have three parts, at the sizes where it can go wrong (needs a B200):
 rows that are no multiple of eight elements long around octets, strips and spans of 256 rows, residues without rows, several tensors
 of different row lengths in one launch.  Every call against the oracle, with the tolerances of helpers.py.  A set takes this kernel from
-2.6 M weights on, hence the large first tensors."""
+2.6 M weights on (fp32 up to rank 16: 6.8 M), hence the large first tensors."""
 import numpy as np
 import pytest
 import torch
@@ -35,15 +35,16 @@ def test_ragged_rows(rank, dtype, bits):
     assert p.lib.device_status() == 0
 
 
-# Rows shorter than two octets, and weights that do not begin on a 16-byte boundary, stay with the tile kernel beside it.
-@pytest.mark.parametrize("dtype", ["bf16", "f32"])
-def test_whole_octets_beside_other_rows(dtype):
-    p = Pair([(1300, 2056), (40, 15), (130, 64), (129, 72), (1, 136), (257, 200), (385, 129), (1, 9)], [16 if dtype == "f32" else 8, 3, 8, 4, 1, 8, 12, 0], dtype, bits=32, seed=4)
+# Rows shorter than two octets, and weights that do not begin on a 16-byte boundary, stay with the tile kernel beside it; the smaller fp32 set does
+# altogether.
+@pytest.mark.parametrize("dtype,cols", [("bf16", 2056), ("f32", 2056), ("f32", 5304)])
+def test_whole_octets_beside_other_rows(dtype, cols):
+    p = Pair([(1300, cols), (40, 15), (130, 64), (129, 72), (1, 136), (257, 200), (385, 129), (1, 9)], [16 if dtype == "f32" else 8, 3, 8, 4, 1, 8, 12, 0], dtype, bits=32, seed=4)
     p.step(seed=3, lp=1.8, lm=2.3, lr=1e-4)
     assert p.lib.device_status() == 0
 
 
-@pytest.mark.parametrize("dtype,cols", [("bf16", 2051), ("f32", 2056)])
+@pytest.mark.parametrize("dtype,cols", [("bf16", 2051), ("f32", 2056), ("f32", 5304)])
 @pytest.mark.parametrize("rank", [12, 40])
 def test_norms_codes_and_several_seeds(rank, dtype, cols):
     shapes, ranks = [(1300, cols), (150, 203 if dtype == "bf16" else 200), (1, 25)], [rank, 20, 0]

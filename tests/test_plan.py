@@ -165,6 +165,17 @@ def test_kernel_of_each_tensor(shapes, ranks, dtype, misalign, expected):
     assert zgr.lib().zgr_debug_plan_kernels(None, 0, None, ctypes.c_int32(148), ctypes.c_int32(1), ctypes.c_int32(0), None) == zgr.EINVAL
 
 
+# The lines between the two, which depend on the whole set: small fp32 sets, tiles that are not full, short items from the counter, ragged
+# rows whose spans of 256 cost too many tiles.
+@pytest.mark.parametrize("d,layers,rank,dtype,expected", [
+    (512, 2, 16, zgr.F32, "tile"), (768, 1, 16, zgr.F32, "staged"), (512, 1, 20, zgr.F32, "staged"), (192, 40, 16, zgr.F32, "tile"), (192, 40, 64, zgr.F32, "staged"),
+    (320, 20, 4, zgr.F32, "staged"), (136, 40, 8, zgr.BF16, "tile"), (192, 40, 8, zgr.F16, "tile"), (320, 10, 8, zgr.BF16, "staged"), (320, 40, 8, zgr.BF16, "tile"), (256, 40, 8, zgr.BF16, "tile"),
+    (256, 10, 8, zgr.BF16, "staged"), (384, 20, 8, zgr.BF16, "staged"), (125, 40, 16, zgr.BF16, "tile"), (261, 20, 16, zgr.BF16, "staged"), (141, 40, 16, zgr.F16, "staged")])
+def test_lines_between_staged_and_tile_kernel(d, layers, rank, dtype, expected):
+    shapes = [(d, d), (4 * d, d), (d, d), (d, 4 * d), (d, d), (d, d)] * layers
+    assert set(kernels(shapes, [rank] * len(shapes), [dtype] * len(shapes))) == {expected}
+
+
 # Ragged 16-bit sets that are dealt out in shares: a share begins and ends in the middle of a span of 256 rows where that makes the
 # largest one smaller, down to one tile above the mean (which is a whole number of tiles).  Tiles of 128 rows, two to a span.
 @pytest.mark.parametrize("d,ffn,rank", [(1234, 4937, 16), (871, 3491, 32), (701, 2803, 64), (1534, 6137, 16), (501, 2003, 8)])
