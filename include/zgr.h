@@ -299,7 +299,7 @@ int zgr_debug_z_tcgen05(zgr_ctx* ctx, uint64_t seed, int32_t tensor, float* dev_
  * 2 legacy tensor-core, 3 any shape, 4 tcgen05 with TMA-staged weights.  kpad > 8 on paths 1 and 3 is the three-part tensor-core kernels' contraction
  * width (an item's last octet of a row may reach into the next strip there).  `tensors[].data / U` are only inspected for alignment and
  * null-ness.  tcgen05 != 0 plans as on a device where tensor maps can be made; multi != 0 gives the plan of
- * the multi-seed sweeps.  Up to max_items items are written to out; *n_items receives the full count.
+ * the sweeps of four seeds and more.  Up to max_items items are written to out; *n_items receives the full count.
  * Errors as zgr_init (ZGR_EINVAL), plus sm_count < 1 or a null n_items.
  * zgr_debug_plan_kernels: the kernel of the same plan that serves each tensor (kernels: n entries), by the numbers below. */
 enum { ZGR_KERNEL_ISO = 0, ZGR_KERNEL_FMA = 1, ZGR_KERNEL_MMA = 2, ZGR_KERNEL_GENERIC = 3, ZGR_KERNEL_UMMA = 4, ZGR_KERNEL_TILE = 5, ZGR_KERNEL_STAGED = 6 };

@@ -121,8 +121,9 @@ struct zgr_ctx {
   std::vector<SplitJob> split_jobs;   // the same on the host
   std::vector<int32_t> split_job;     // per tensor: its job, or -1
   int n_split_jobs = 0;
-  std::vector<Group> groups_multi;    // plan of multi-seed sweeps when it differs from `groups` (legacy tensor-core path only)
-  bool multi_planned = false;
+  std::vector<Group> groups_multi;    // plan of sweeps with several terms where it differs from `groups` (multi_groups)
+  bool multi_planned = false;         // (of the legacy tensor-core path, on first use)
+  int many_terms = 0;                 // from how many terms on ragged tensors of the staged kernel go to the tile kernel; 0: never
   int sticky = 0;                     // first CUDA failure, returned by every later call
   int64_t launches = 0;
   bool profiling = false;
@@ -206,6 +207,20 @@ bool make_map(CUtensorMap* out, const void* base, int bytes, int64_t rows, int64
 bool make_map_16bit(CUtensorMap* out, const void* base, int64_t rows, int64_t cols, int box_cols) {
   return make_map(out, base, 2, rows, cols, cols, 128, box_cols);
 }
+// Map over a part of U kept in the order of staged_copy_row whose boxes are 128 rows in their own order: a box takes 16 rows of each of a
+// span's eight residues, residue by residue within a row of eight.
+bool make_map_in_order(CUtensorMap* out, const void* base, int64_t rows_pad, int kpad) {
+  EncodeTiledFn fn = encode_tiled_fn();
+  if (!fn) return false;
+  const cuuint64_t row = static_cast<cuuint64_t>(kpad) * 2;
+  const cuuint64_t dims[4] = {static_cast<cuuint64_t>(kpad), 8, 32, static_cast<cuuint64_t>(rows_pad / 256)};
+  const cuuint64_t strides[3] = {32 * row, row, 256 * row};
+  const cuuint32_t box[4] = {static_cast<cuuint32_t>(kpad), 8, 16, 1};
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  const CUtensorMapSwizzle sw = kpad == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : (kpad == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
+  return fn(out, CU_TENSOR_MAP_DATA_TYPE_UINT16, 4, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, sw,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 
 // The maps of a tensor of sweep_staged_kernel: of its weights, one per residue of the row modulo 8 if the rows are no multiple of eight
 // elements (see zgr_staged.cu), and behind them the three parts of U, rows_pad x kpad each.
@@ -231,13 +246,9 @@ int64_t rows_before(const TensorDesc& td, int64_t block) {
 }
 // Blocks of a tensor of so many rows that hold any: residues 4-7 of the last span may be empty.
 int64_t blocks_in_spans(int64_t rows) { return rows / 256 * 2 + ((rows & 255) > 4 ? 2 : (rows & 255) > 0); }
-// Rows that a tensor is cut into items by: its own, or its blocks in that order that hold any.
-int64_t rows_to_cut(const TensorDesc& td) {
-  return by_residue(td) ? 128 * blocks_in_spans(td.rows) : td.rows;
-}
-// First row and number of rows of an item: of the tensor, or in that order.
-std::pair<int64_t, int64_t> item_rows(const TensorDesc& td, const WorkItem& w) {
-  if (!by_residue(td)) return {w.row0_or_e0, w.nrows_or_count};
+// First row and number of rows of an item: of the tensor, or, on the staged kernel, in that order.
+std::pair<int64_t, int64_t> item_rows(const TensorDesc& td, const KernelChoice& kc, const WorkItem& w) {
+  if (!kc.staged || !by_residue(td)) return {w.row0_or_e0, w.nrows_or_count};
   const int64_t first = rows_before(td, w.row0_or_e0 / 128);
   return {first, rows_before(td, (w.row0_or_e0 + w.nrows_or_count) / 128) - first};
 }
@@ -349,7 +360,7 @@ int blocks_per_sm(const KernelChoice& kc, bool multi = false, bool stats = false
 
 struct Member {
   int tensor, strip, row_step;
-  int64_t rows;                                           // rows_to_cut
+  int64_t rows;                                           // to be cut: the tensor's, or its blocks in the order of the copies of U
 };
 
 // Append the items of one tensor: strips of `strip` columns, each cut into even chunks of at most about nrows rows.
@@ -518,7 +529,7 @@ void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>&
       if (tiles >= 64 * sms) {
         // long sweeps: also even when dealt out in turn, so that neither the model nor the counter has to be right
         std::fill(dealt.begin(), dealt.end(), 0.0);
-        for (size_t i = 0; i < trial.size(); ++i) dealt[i % dealt.size()] += static_cast<double>(item_rows(descs[trial[i].tensor], trial[i]).second) * trial[i].ncols;
+        for (size_t i = 0; i < trial.size(); ++i) dealt[i % dealt.size()] += static_cast<double>(item_rows(descs[trial[i].tensor], g.kc, trial[i]).second) * trial[i].ncols;
         const double mean = std::accumulate(dealt.begin(), dealt.end(), 0.0) / static_cast<double>(dealt.size());
         if (*std::max_element(dealt.begin(), dealt.end()) > 1.025 * mean) end *= 2.0;
         else even = true;
@@ -533,9 +544,10 @@ void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>&
 // Split the tensors listed in `which` into work items, grouped by the kernel that serves them.
 // The kernel family follows the tensor's own storage type (fp32 tensors take the accurate transform and
 // an exact fp32 contraction); `kernel_dtype` >= 0 overrides only the type the kernel reads and writes,
-// which lets the test hook run a 16-bit tensor's kernel family on an fp32 image.
+// which lets the test hook run a 16-bit tensor's kernel family on an fp32 image.  `ragged_on_tile`: tensors kept by residue go to the
+// tile kernel all the same.
 void plan(const std::vector<TensorDesc>& descs, const std::vector<int>& which, bool guided_on, int bits, int sm_count,
-          std::vector<Group>& out, int kernel_dtype = -1, bool multi = false) {
+          std::vector<Group>& out, int kernel_dtype = -1, bool multi = false, bool ragged_on_tile = false) {
   int64_t total = 0;
   for (int l : which) total += descs[l].rows * descs[l].cols;
   // elements per item: enough items for ~16 rounds over the resident CTAs, but large enough that the
@@ -543,16 +555,16 @@ void plan(const std::vector<TensorDesc>& descs, const std::vector<int>& which, b
   int64_t target = total / (static_cast<int64_t>(sm_count) * 2 * 16);
   target = std::min<int64_t>(std::max<int64_t>(target, 16384), 524288);
 
-  std::map<std::tuple<int, int, int, int, int>, size_t> index;  // (path, dtype, kpad, precise, staged) -> group
-  auto group_for = [&](int path, int real_dtype, int kpad, int staged = 0) -> Group& {
+  std::map<std::tuple<int, int, int, int, int, int>, size_t> index;  // (path, dtype, kpad, precise, staged, by_residue) -> group
+  auto group_for = [&](int path, int real_dtype, int kpad, int staged = 0, int by_res = 0) -> Group& {
     const int precise = real_dtype == ZGR_F32 ? 1 : 0;
     const int dtype = kernel_dtype >= 0 ? kernel_dtype : real_dtype;
-    auto key = std::make_tuple(path, dtype, kpad, precise, staged);
+    auto key = std::make_tuple(path, dtype, kpad, precise, staged, by_res);
     auto it = index.find(key);
     if (it == index.end()) {
       index[key] = out.size();
       Group g;
-      g.kc = KernelChoice{path, dtype, kpad, bits, precise, staged};
+      g.kc = KernelChoice{path, dtype, kpad, bits, precise, staged, by_res};
       out.push_back(std::move(g));
       return out.back();
     }
@@ -575,14 +587,16 @@ void plan(const std::vector<TensorDesc>& descs, const std::vector<int>& which, b
       continue;
     }
     const bool vec = aligned && (t.cols % 8 == 0);
-    int path, kpad, strip, row_step, staged = 0;
+    int path, kpad, strip, row_step, staged = 0, by_res = 0;
     const bool umma_ok = t.umma && kernel_dtype < 0;
     const bool tile_ok = t.tile && (kernel_dtype < 0 || kernel_dtype == t.dtype);
     if (tile_ok) {
       // fp32 with rank > 8, rows that are not a multiple of eight elements, and low ranks: three-part operands.  (The test hook
       // that sweeps an fp32 image of a 16-bit tensor keeps the one-element-per-thread kernel below.)
-      path = vec && t.rank <= 8 ? PATH_FMA : PATH_GENERIC; kpad = t.kpad; strip = kTileStripCols; staged = t.staged;
-      row_step = by_residue(t) ? 256 : 128;
+      path = vec && t.rank <= 8 ? PATH_FMA : PATH_GENERIC; kpad = t.kpad; strip = kTileStripCols;
+      by_res = ragged_on_tile && by_residue(t);
+      staged = t.staged && !by_res;
+      row_step = staged && by_residue(t) ? 256 : 128;
     } else if (!vec || (t.rank > 8 && !umma_ok && (t.Ufrag == nullptr || multi))) {
       // (the legacy tensor-core kernel applies one term per sweep; several terms take the fallback)
       path = PATH_GENERIC; kpad = 0; strip = 64; row_step = 1;
@@ -594,17 +608,17 @@ void plan(const std::vector<TensorDesc>& descs, const std::vector<int>& which, b
       path = PATH_MMA; kpad = t.rank <= 16 ? 16 : (t.rank <= 32 ? 32 : 64);
       strip = mma_strip_cols(kpad); row_step = mma_rows_per_iter(kpad);
     }
-    Group& g = group_for(path, t.dtype, kpad, staged);
+    Group& g = group_for(path, t.dtype, kpad, staged, by_res);
     const size_t gi = static_cast<size_t>(&g - out.data());
     if (members.size() <= gi) members.resize(gi + 1);
-    members[gi].push_back(Member{l, strip, row_step, rows_to_cut(t)});
+    members[gi].push_back(Member{l, strip, row_step, staged && by_residue(t) ? 128 * blocks_in_spans(t.rows) : t.rows});
   }
   members.resize(out.size());
   for (size_t gi = 0; gi < out.size(); ++gi)
     if (out[gi].kc.path != PATH_ISO) plan_tiles(descs, members[gi], sm_count, target, out[gi]);
   for (Group& g : out) {
     g.elements = 0;
-    for (const WorkItem& w : g.items) g.elements += g.kc.path == PATH_ISO ? w.nrows_or_count : item_rows(descs[w.tensor], w).second * w.ncols;
+    for (const WorkItem& w : g.items) g.elements += g.kc.path == PATH_ISO ? w.nrows_or_count : item_rows(descs[w.tensor], g.kc, w).second * w.ncols;
   }
   for (Group& g : out)
     g.grid = !g.starts.empty() ? static_cast<int>(g.starts.size()) - 1 : static_cast<int>(std::min<int64_t>(static_cast<int64_t>(g.items.size()), static_cast<int64_t>(sm_count) * blocks_per_sm(g.kc)));
@@ -932,6 +946,15 @@ int validate_model(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, 
   return ZGR_OK;
 }
 
+// From how many terms on a sweep has the set's ragged 16-bit tensors on the tile kernel although the staged one serves single seeds.
+int many_terms_from(const std::vector<TensorDesc>& descs, const SetSizes& sizes, int sm_count) {
+  bool ragged = false;
+  for (const TensorDesc& td : descs) ragged = ragged || by_residue(td);
+  for (int n = 2; ragged && n <= 4; ++n)
+    if (!ragged_on_staged(sizes, sm_count, n)) return n;
+  return 0;
+}
+
 // The plan of a sweep as zgr_init would make it, without a device.
 int plan_on_host(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, int sm_count, bool tcgen05, bool multi, std::vector<TensorDesc>& descs,
                  std::vector<Group>& groups) {
@@ -961,7 +984,7 @@ int plan_on_host(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, in
     }
     all[static_cast<size_t>(l)] = l;
   }
-  plan(descs, all, guided_on, cfg->bits_per_normal, sm_count, groups, -1, multi);
+  plan(descs, all, guided_on, cfg->bits_per_normal, sm_count, groups, -1, multi, multi && many_terms_from(descs, sizes, sm_count) > 0);
   return ZGR_OK;
 }
 
@@ -973,10 +996,12 @@ void ledger_add(zgr_ctx* ctx, uint64_t seed, double c) {
   ctx->last_seed = seed;
 }
 
-// Plan used by sweeps with several terms: the sweep plan itself unless it contains the legacy
-// tensor-core kernel, which applies one term per sweep; those tensors are re-planned onto the fallback.
-std::vector<Group>& multi_groups(zgr_ctx* ctx, int* rc) {
+// Plan used by sweeps with n terms, n > 1: the sweep plan itself unless it contains the legacy
+// tensor-core kernel, which applies one term per sweep (those tensors are re-planned onto the fallback), or so many terms
+// are better off with the tile kernel.
+std::vector<Group>& multi_groups(zgr_ctx* ctx, int n, int* rc) {
   *rc = ZGR_OK;
+  if (ctx->many_terms > 0 && n >= ctx->many_terms) return ctx->groups_multi;
   bool legacy = false;
   for (const Group& g : ctx->groups) legacy = legacy || (g.kc.path == PATH_MMA && !g.items.empty());
   if (!legacy) return ctx->groups;
@@ -1092,6 +1117,11 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
     plan(ctx->descs, all, guided_on, cfg->bits_per_normal, ctx->sm_count, ctx->groups);
     order_groups(ctx->descs, ctx->groups);
     merge_small_groups(ctx);
+    ctx->many_terms = many_terms_from(ctx->descs, sizes, ctx->sm_count);
+    if (ctx->many_terms > 0) {
+      plan(ctx->descs, all, guided_on, cfg->bits_per_normal, ctx->sm_count, ctx->groups_multi, -1, true, true);
+      order_groups(ctx->descs, ctx->groups_multi);
+    }
     Tables tables;
     tables.add(&ctx->d_split_jobs, jobs.data(), jobs.size());
     std::vector<CUtensorMap> staged_maps(n_staged_maps);
@@ -1102,6 +1132,7 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
     tables.add(&ctx->d_err, static_cast<const int*>(nullptr), 1);
     tables.add(&ctx->d_stats, static_cast<const double*>(nullptr), static_cast<size_t>(3 * n));
     for (Group& g : ctx->groups) tables.add(g);
+    for (Group& g : ctx->groups_multi) tables.add(g);
     if (!ctx->merged.empty()) tables.add(&ctx->d_merged, ctx->merged.data(), ctx->merged.size());
     // Scratch of zgr_build_subspace, up to 2 MB (every rank up to 32, and rank 64 in one cluster): as an allocation of its own inside the
     // first call it would be most of that call.  Its first 512 bytes are the last of the zeroed tables.
@@ -1138,6 +1169,8 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
       for (int i = 0; i < (td.umma ? 2 : 3); ++i) {
         td.Ucopy[i] = at;
         if (!make_map_16bit(m + i, at, rows_pad, td.kpad, td.kpad)) rc = check(ctx, cudaErrorUnknown);
+        if (ctx->many_terms > 0 && by_residue(td) && !make_map_in_order(&ctx->tmaps[static_cast<size_t>(3 * l + i)], at, rows_pad, td.kpad))
+          rc = check(ctx, cudaErrorUnknown);
         at += static_cast<size_t>(rows_pad) * td.kpad * 2;       // (a multiple of 4096 bytes)
       }
       jobs[static_cast<size_t>(job)] = SplitJob{td.U, {td.Ucopy[0], td.Ucopy[1], td.Ucopy[2]}, td.rows, rows_pad, td.rank, td.kpad, td.umma ? td.ushift : -1,
@@ -1214,7 +1247,7 @@ int zgr_sweep_multi(zgr_ctx* ctx, int32_t n, const uint64_t* seeds, const double
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int rc = flush_descs(ctx, st);
   if (rc != ZGR_OK) return rc;
-  std::vector<Group>& groups = n > 1 ? multi_groups(ctx, &rc) : ctx->groups;
+  std::vector<Group>& groups = n > 1 ? multi_groups(ctx, n, &rc) : ctx->groups;
   if (rc != ZGR_OK) return rc;
   rc = sweep(ctx, groups, ctx->d_descs, n, seeds, coeffs, st);
   if (rc != ZGR_OK) return rc;
@@ -1241,7 +1274,7 @@ int zgr_restore_update_multi(zgr_ctx* ctx, int32_t n, const uint64_t* seeds, con
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int rc = flush_descs(ctx, st);
   if (rc != ZGR_OK) return rc;
-  std::vector<Group>& groups = n > 1 ? multi_groups(ctx, &rc) : ctx->groups;
+  std::vector<Group>& groups = n > 1 ? multi_groups(ctx, n, &rc) : ctx->groups;
   if (rc != ZGR_OK) return rc;
   rc = sweep(ctx, groups, ctx->d_descs, n, seeds, c, st);
   if (rc != ZGR_OK) return rc;
@@ -1774,7 +1807,7 @@ int zgr_debug_plan(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, 
   int64_t count = 0;
   for (const Group& g : groups)
     for (const WorkItem& w : g.items) {
-      const auto [first, rows] = g.kc.path == PATH_ISO ? std::make_pair(w.row0_or_e0, w.nrows_or_count) : item_rows(descs[w.tensor], w);
+      const auto [first, rows] = g.kc.path == PATH_ISO ? std::make_pair(w.row0_or_e0, w.nrows_or_count) : item_rows(descs[w.tensor], g.kc, w);
       if (count < max_items) out[count] = zgr_plan_item{g.kc.path, g.kc.kpad, w.tensor, w.ncols, first, rows, w.col0};
       ++count;
     }

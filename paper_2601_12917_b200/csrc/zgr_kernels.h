@@ -23,6 +23,7 @@ struct KernelChoice {
   int bits;   // 32 or 16 random bits per normal
   int precise;  // accurate Gaussian transform (tensors stored in fp32)
   int staged;   // among the groups of is_tile: served by sweep_staged_kernel
+  int by_residue;  // tile kernel: copies of U in the order of staged_copy_row, behind 4-D maps
 };
 
 // Resident blocks of 256 threads per SM of the isotropic kernel.  Its plain instantiation (fused transform) fits 32 registers:

@@ -116,7 +116,7 @@ struct RawOct<float> {
 
 template <typename T, int BITS, bool PRECISE, bool MULTI, bool SSTATS>
 __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __grid_constant__ SweepParams p, const CUtensorMap* __restrict__ tmaps,
-                                                                     int* __restrict__ error, const int kp) {
+                                                                     int* __restrict__ error, const int kp, const int by_residue) {
   extern __shared__ uint8_t smem_raw[];
   const TileSmem L = tile_smem(kp);
   const int US = L.u_stages, GS = L.g_stages, rowb = L.rowb;
@@ -202,7 +202,11 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
           if (t >= US && !mbar_wait<true>(BAR_U_FREE(u), ((t / US) - 1) & 1, abort_flag, error, 21)) { ok = false; break; }
           const uint32_t dst = smem_u32(u_base + u * kParts * L.u_bytes);
           mbar_arrive_expect_tx(BAR_U_FULL(u), static_cast<uint32_t>(kParts * L.u_bytes));
-          for (int i = 0; i < kParts; ++i) tma_load_2d(dst + i * L.u_bytes, tm + i, 0, row0, BAR_U_FULL(u));
+          // (rows kept by residue for the staged kernel: the map puts them back in order, eight residues x 16)
+          for (int i = 0; i < kParts; ++i) {
+            if (by_residue) tma_load_4d(dst + i * L.u_bytes, tm + i, 0, 0, (row0 & 255) >> 3, row0 >> 8, BAR_U_FULL(u));
+            else tma_load_2d(dst + i * L.u_bytes, tm + i, 0, row0, BAR_U_FULL(u));
+          }
         }
       }
       // let the last loads land before the CTA gives up its shared memory
@@ -512,23 +516,23 @@ __global__ void __launch_bounds__(kTileThreads, 1) sweep_tile_kernel(const __gri
 
 namespace {
 template <typename T, int BITS, bool PRECISE, bool MULTI, bool SSTATS>
-cudaError_t launch_tile_one(int kp, const SweepParams& p, const CUtensorMap* tmaps, int* error, int grid, cudaStream_t st) {
+cudaError_t launch_tile_one(int kp, int by_residue, const SweepParams& p, const CUtensorMap* tmaps, int* error, int grid, cudaStream_t st) {
   auto k = sweep_tile_kernel<T, BITS, PRECISE, MULTI, SSTATS>;
   const int smem = tile_smem(kp).total;
   const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, tile_smem(64).total);
   if (e != cudaSuccess) return e;
-  return launch_sweep_kernel(k, grid, kTileThreads, static_cast<size_t>(smem), st, p, tmaps, error, kp);
+  return launch_sweep_kernel(k, grid, kTileThreads, static_cast<size_t>(smem), st, p, tmaps, error, kp, by_residue);
 }
 template <typename T, bool PRECISE>
 cudaError_t launch_tile_typed(const KernelChoice& kc, const SweepParams& p, const CUtensorMap* tmaps, int* error, int grid, cudaStream_t st) {
   if (p.n_terms > 1)
-    return kc.bits == 32 ? launch_tile_one<T, 32, PRECISE, true, false>(kc.kpad, p, tmaps, error, grid, st)
-                         : launch_tile_one<T, 16, PRECISE, true, false>(kc.kpad, p, tmaps, error, grid, st);
+    return kc.bits == 32 ? launch_tile_one<T, 32, PRECISE, true, false>(kc.kpad, kc.by_residue, p, tmaps, error, grid, st)
+                         : launch_tile_one<T, 16, PRECISE, true, false>(kc.kpad, kc.by_residue, p, tmaps, error, grid, st);
   if (p.item_stats != nullptr)
-    return kc.bits == 32 ? launch_tile_one<T, 32, PRECISE, false, true>(kc.kpad, p, tmaps, error, grid, st)
-                         : launch_tile_one<T, 16, PRECISE, false, true>(kc.kpad, p, tmaps, error, grid, st);
-  return kc.bits == 32 ? launch_tile_one<T, 32, PRECISE, false, false>(kc.kpad, p, tmaps, error, grid, st)
-                       : launch_tile_one<T, 16, PRECISE, false, false>(kc.kpad, p, tmaps, error, grid, st);
+    return kc.bits == 32 ? launch_tile_one<T, 32, PRECISE, false, true>(kc.kpad, kc.by_residue, p, tmaps, error, grid, st)
+                         : launch_tile_one<T, 16, PRECISE, false, true>(kc.kpad, kc.by_residue, p, tmaps, error, grid, st);
+  return kc.bits == 32 ? launch_tile_one<T, 32, PRECISE, false, false>(kc.kpad, kc.by_residue, p, tmaps, error, grid, st)
+                       : launch_tile_one<T, 16, PRECISE, false, false>(kc.kpad, kc.by_residue, p, tmaps, error, grid, st);
 }
 }  // namespace
 

@@ -95,6 +95,26 @@ def test_norms_and_several_seeds_from_the_counter():
     assert p.lib.device_status() == 0
 
 
+# Ragged sets whose spans cost a tile of the busiest SM (four tiles against three): one seed on the staged kernel, several on the tile kernel,
+# which reads the copies of U kept by residue in the order of the rows.  A new subspace reaches both.
+@pytest.mark.parametrize("rank,dtype,bits", [(16, "f16", 16), (20, "bf16", 32), (64, "bf16", 16)])
+def test_several_seeds_on_the_tile_kernel(rank, dtype, bits):
+    shapes, ranks = [(6917, 131)] * 4 + [(1, 9)], [rank, rank, rank, 9, 0]
+    p = Pair(shapes, ranks, dtype, bits=bits, seed=rank)
+    p.lib.profile(True)
+    p.step(seed=3, lp=1.8, lm=2.3, lr=1e-4)
+    assert {k["kernel"] for k in p.lib.profile_read()} == {"staged", "iso"}
+    seeds, lp, lm = [41, 42, 43, 44], [2.1, 1.6, 2.4, 1.7], [1.9, 2.0, 1.8, 2.2]
+    coeffs = [oracle.update_coefficient(0.0, a, b, p.eps, 1e-4) for a, b in zip(lp, lm)]
+    p.call_and_check_multi(seeds, coeffs, lambda: p.lib.restore_update_multi(seeds, lp, lm, 1e-4), "four seeds")
+    assert {k["kernel"] for k in p.lib.profile_read()} == {"tile", "iso"}
+    p.U[1].copy_(p.U[1].flip(0))
+    p.lib.update_subspace(1)
+    p.call_and_check_multi(seeds, coeffs, lambda: p.lib.restore_update_multi(seeds, lp, lm, 1e-4), "four seeds, new subspace")
+    p.step(seed=4, lp=1.8, lm=2.3, lr=1e-4)
+    assert p.lib.device_status() == 0
+
+
 # A delivered and a constructed subspace reach the copies of U that are kept by residue.
 def test_new_subspaces_of_ragged_tensors():
     p = Pair([LARGE, (300, 385), (1, 9)], [16, 16, 0], "bf16", bits=16, seed=6)

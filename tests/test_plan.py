@@ -176,6 +176,16 @@ def test_lines_between_staged_and_tile_kernel(d, layers, rank, dtype, expected):
     assert set(kernels(shapes, [rank] * len(shapes), [dtype] * len(shapes))) == {expected}
 
 
+# Ragged sets whose spans cost a tile of the busiest SM: many seeds have the tile kernel, one the staged one.
+@pytest.mark.parametrize("shapes,multi_kernel", [([(6917, 131)] * 4, "tile"), ([(1234, 1234)] * 4 + [(4937, 1234), (1234, 4937)], "tile"),
+                                                  ([(1534, 1534)] * 4 + [(6137, 1534), (1534, 6137)], "staged")])
+def test_kernel_of_many_seeds(shapes, multi_kernel):
+    n = len(shapes)
+    assert set(kernels(shapes, [16] * n, [zgr.BF16] * n)) == {"staged"}
+    assert set(kernels(shapes, [16] * n, [zgr.BF16] * n, multi=1)) == {multi_kernel}
+    check_exact_cover(plan(shapes, [16] * n, [zgr.BF16] * n, multi=1), shapes)
+
+
 # Ragged 16-bit sets that are dealt out in shares: a share begins and ends in the middle of a span of 256 rows where that makes the
 # largest one smaller, down to one tile above the mean (which is a whole number of tiles).  Tiles of 128 rows, two to a span.
 @pytest.mark.parametrize("d,ffn,rank", [(1234, 4937, 16), (871, 3491, 32), (701, 2803, 64), (1534, 6137, 16), (501, 2003, 8)])
