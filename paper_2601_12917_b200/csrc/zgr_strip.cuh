@@ -31,7 +31,7 @@ __device__ __forceinline__ void build_strip(const TensorDesc& td, const SweepPar
                                             int et) {
   const int kp_shift = kp == 64 ? 6 : (kp == 32 ? 5 : 4);
   const int64_t cols = td.cols;
-  const int n_oct = (cols & 7) == 0 ? width / 8 : width / 8 + 1;
+  const int n_oct = width == kTileN || (cols & 7) != 0 ? width / 8 + 1 : width / 8;      // (a constant in the tile kernel)
   for (int idx = et; idx < (n_oct << kp_shift); idx += kEpi * 32) {
     const int k = idx & (kp - 1), o = idx >> kp_shift;      // consecutive lanes: consecutive k, i.e. neighbouring shared-memory words
     const int64_t row_e = static_cast<int64_t>(k) * cols;
