@@ -482,13 +482,35 @@ void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>&
   double best = 0.0;
   const bool spans = !members.empty() && members[0].row_step == 256;      // (one step for all tensors of a group)
   const auto blocks_of = [&](int64_t rows) { return spans ? (rows + 255) / 256 * 2 : (rows + 127) / 128; };
-  bool even = false;                                   // (long sweeps) the best so far is even when dealt out in turn
   std::vector<WorkItem> trial;
-  std::vector<double> dealt(static_cast<size_t>(sm_count)), free_at(static_cast<size_t>(sm_count));
+  std::vector<double> free_at(static_cast<size_t>(sm_count));
+  if (tiles >= 64 * sms) {
+    // Long sweeps: even also when dealt out in turn, so that neither the model below nor the counter has to be right: eight tiles, or nine
+    // where that is even and eight is not (rows of 50265).  Sets that neither deals evenly are replayed with both, in spans with eight.
+    // us a step with 8 / 9 / 6 / 4 tiles: RoBERTa-shaped fp32 rank 8 1732 / 1722 / 1776 / 1778, 13 layers of 1024 822 / 824 / 839 / 830, fp32 rank 32
+    // of 1152 1142 / 1157 / 1131 / 1170, 16-bit rank 8 of 2048 1200 / 1205 / 1245 / 1277: eight or nine makes no difference beyond 1 %, lower ones cost.
+    for (int64_t height : {8, 9}) {
+      if (spans && height == 9) continue;
+      trial.clear();
+      for (const Member& m : members) cut_tensor(descs[m.tensor], m, by_rows, 128 * height, trial);
+      std::fill(free_at.begin(), free_at.end(), 0.0);
+      double total = 0.0;
+      size_t cta = 0;
+      for (const WorkItem& w : trial) {
+        const double weights = static_cast<double>(item_rows(descs[w.tensor], g.kc, w).second) * w.ncols;
+        total += weights;
+        free_at[cta] += weights;
+        if (++cta == free_at.size()) cta = 0;
+      }
+      if (*std::max_element(free_at.begin(), free_at.end()) <= 1.025 * total / static_cast<double>(sm_count)) {
+        g.items.swap(trial);
+        return;
+      }
+    }
+  }
   for (int64_t big : {16, 12, 8, 9, 6, 4, 3, 2, 1})
     for (int64_t small : {big, std::max<int64_t>(big / 4, 1)}) {
-      // (long sweeps: eight, or nine if eight deals unevenly)
-      if (tiles >= 64 * sms ? small != big || (big != 8 && big != 9) || even : big == 9) continue;
+      if (tiles >= 64 * sms ? small != big || (big != 8 && big != 9) : big == 9) continue;
       if (spans && (big & 3) != 0 && big != 2) continue;      // (rows in spans of 256: nothing between two and four blocks, and six is left out)
       if (best > 0.0 && tiles < 64 * sms && (small == big ? tiles / big > 16 * sms : tiles / big > 10 * sms || big == 1)) continue;
       // No schedule ends before the mean load: heights that cannot win are not cut into items, nor replayed to their end (the
@@ -498,8 +520,8 @@ void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>&
         int64_t done = 0, n_items = 0;
         for (const Member& m : members) {
           const int64_t strips = (descs[m.tensor].cols + 127) / 128, blocks = blocks_of(m.rows), h = 3 * done < 2 * tiles ? big : small;
-          const int64_t chunks = (m.rows + 128 * h - 1) / (128 * h), even = (blocks + chunks - 1) / chunks;
-          n_items += strips * ((blocks + even - 1) / even);
+          const int64_t chunks = (m.rows + 128 * h - 1) / (128 * h), tall = (blocks + chunks - 1) / chunks;
+          n_items += strips * ((blocks + tall - 1) / tall);
           done += blocks * strips;
         }
         const double load = static_cast<double>(tiles) + static_cast<double>(n_items) * item_cost;
@@ -526,14 +548,6 @@ void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>&
         end = std::max(end, at);
       }
       end += last;
-      if (tiles >= 64 * sms) {
-        // long sweeps: also even when dealt out in turn, so that neither the model nor the counter has to be right
-        std::fill(dealt.begin(), dealt.end(), 0.0);
-        for (size_t i = 0; i < trial.size(); ++i) dealt[i % dealt.size()] += static_cast<double>(item_rows(descs[trial[i].tensor], g.kc, trial[i]).second) * trial[i].ncols;
-        const double mean = std::accumulate(dealt.begin(), dealt.end(), 0.0) / static_cast<double>(dealt.size());
-        if (*std::max_element(dealt.begin(), dealt.end()) > 1.025 * mean) end *= 2.0;
-        else even = true;
-      }
       if (best == 0.0 || end < best) {
         best = end;
         g.items = trial;
