@@ -67,9 +67,10 @@ typedef struct {
   void* data;       /* device; rows*cols elements of `dtype`, row-major, contiguous, updated in place.
                        Must be aligned to the element size.  16-bit storage with rank > 8, 16-byte alignment
                        and cols a multiple of eight elements is staged in whole tiles; all else with a
-                       subspace, except small sets of rank <= 8 and large fp32 ones, is served by a tile
-                       kernel that works on octets across row ends (tensor-core contraction with three bf16
-                       parts per operand, as accurate as fp32 multiply-adds) */
+                       subspace, except small sets of rank <= 8 and large fp32 ones of rank <= 4, is served by
+                       kernels with a tensor-core contraction of three bf16 parts per operand, as accurate as
+                       fp32 multiply-adds for entries up to 3.39e38 in size (an infinite entry gives NaN, not
+                       infinity, in its row) */
   int64_t rows;     /* m_l >= 1 */
   int64_t cols;     /* n_l >= 1 */
   int32_t dtype;    /* ZGR_F32 | ZGR_F16 | ZGR_BF16 */

@@ -405,9 +405,9 @@ __device__ __forceinline__ void normals8_acc_pre(const PhiloxKeys& keys, const P
 // octet before it have ended (`link` carries the last word from one to the next; `zero` is a zero that the compiler cannot see
 // through, so the link is real but changes nothing), and run beside the transform of the octet before.  Left to itself the compiler
 // runs the rounds of all octets first and then issues their special functions in one burst, during which the warp cannot issue
-// anything else.  One logic instruction an octet.  In the TMA-staged sweep, 16 random bits per normal: LLaMA-7B-shaped bf16
-// rank 32, four queries 71.1 -> 70.1 ms, OPT-1.3B-shaped fp16 rank 16 3404 -> 3379 us, rank 64 with int8 codes 10683 -> 10560 us,
-// eight seeds 6418 -> 6326 us; with 32 bits, where an octet is two blocks of its own, 3564 -> 3650 us.
+// anything else.  One logic instruction an octet.  In the TMA-staged sweep, 16 random bits per normal: eight
+// seeds on the OPT-1.3B-shaped fp16 set 6418 -> 6326 us, every time; single seeds 0.9 to 1.6 % less, which is within what repeated runs of one
+// side differ by; with 32 bits, where an octet is two blocks of its own, 3564 -> 3650 us.
 __device__ __forceinline__ void normals8_acc_linked(const PhiloxKeys& keys, const PhiloxPre& pre, uint32_t oct_lo, const NormalScale& ns, uint32_t zero,
                                                     uint32_t& link, float (&acc)[8]) {
   uint32_t x[4];

@@ -307,9 +307,9 @@ int tensor_core_kind(const zgr_tensor& t, bool guided_on, const SetSizes& sizes)
   if (vec && t.rank <= 8) {
     const int64_t set = sizes.low[t.dtype == ZGR_F32];
     if (set < (int64_t{1} << 21)) return 0;
-    // (at rank 4 half of the contraction is padding, and on fp32 sets that keep every SM busy for long the CUDA-core kernel catches up.
+    // (at rank 4 three quarters of the contraction are padding, and on fp32 sets that keep every SM busy for long the CUDA-core kernel catches up.
     // us a step on CUDA cores / staged, 16 random bits:  rank 4  24 M 154 / 136, 63 M 332 / 331, 126 M 629 / 635, 1.2 G 4333 / 4371;
-    // rank 8  63 M 365 / 333, 126 M 681 / 640, 354 M 1796 / 1759; with 32 bits 101 M 616 / 573)
+    // rank 8  63 M 365 / 333, 126 M 681 / 640, 354 M 1796 / 1759; with 32 bits 101 M 616 / 573; ranks 2 and 3 were not timed and go with rank 4)
     // Rank 1 leaves at 2^25 already: its one multiply-add is exact to a rounding, 2.5e-8 against 2.95e-8 of the six products.
     if (t.dtype == ZGR_F32 && t.rank <= 4 && set >= (int64_t{1} << (t.rank == 1 ? 25 : 26))) return 0;
     return 2;

@@ -27,8 +27,9 @@
 // Against sweep_tile_kernel, which loads the weights from global memory an octet per thread and turns the products round through
 // shared memory, the address arithmetic, the transposition and the exposed loads are gone.
 //
-// Operand precision.  An fp32 number is the sum of three bf16 numbers (8 bits each) without error and without range
-// limits; six of the nine products are formed, the others are below 2^-24 of the result.  With the copies of U leaning against
+// Operand precision.  An fp32 number is the sum of three bf16 numbers (8 bits each) without error, up to the largest bf16 number in size
+// (3.39e38; beyond it, and for infinities, the parts that follow the first are not numbers, and neither is what they are multiplied into);
+// six of the nine products are formed, the others are below 2^-24 of the result.  With the copies of U leaning against
 // the truncation of the tensor cores (truncation_lean) the contraction is as accurate as a chain of fp32 multiply-adds, from
 // rank 2 on more so.  The perturbation is summed on its own scale and added to the weight once.
 #include <cuda_bf16.h>
