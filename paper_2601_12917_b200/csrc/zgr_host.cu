@@ -291,7 +291,7 @@ bool ragged_on_staged(const SetSizes& sizes, int sm_count, int n_terms) {
     const double mean = static_cast<double>(tiles) / sm_count;
     return mean < 12.0 ? std::ceil(mean) : mean;
   };
-  const double tile = n_terms == 1 ? 0.75 : (n_terms == 2 ? 0.85 : (n_terms == 3 ? 0.88 : 0.94));
+  const double tile = n_terms == 1 ? 0.75 : (n_terms == 2 ? 0.85 : (n_terms == 3 ? 0.88 : 0.98));
   return tile * busiest(sizes.ragged_tiles[1]) <= busiest(sizes.ragged_tiles[0]);
 }
 
