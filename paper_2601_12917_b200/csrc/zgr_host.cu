@@ -123,7 +123,7 @@ struct zgr_ctx {
   int n_split_jobs = 0;
   std::vector<Group> groups_multi;    // plan of sweeps with several terms where it differs from `groups` (multi_groups)
   bool multi_planned = false;         // (of the legacy tensor-core path, on first use)
-  int many_terms = 0;                 // from how many terms on ragged tensors of the staged kernel go to the tile kernel; 0: never
+  int many_terms = 0;                 // from how many terms on (many_terms_from); 0: never
   int sticky = 0;                     // first CUDA failure, returned by every later call
   int64_t launches = 0;
   bool profiling = false;
@@ -260,7 +260,7 @@ struct SetSizes {
   int64_t low[2] = {0, 0}, three_part[2] = {0, 0};      // [0] 16-bit, [1] fp32
   // of the latter those in whole octets, the tiles of 128 x 128 that they fill and the strips of these, and the tiles of ragged 16-bit rows on the tile
   // kernel and, in spans of 256 rows, on the staged one
-  int64_t octets[2] = {0, 0}, octet_tiles[2] = {0, 0}, octet_strips[2] = {0, 0}, ragged_tiles[2] = {0, 0};
+  int64_t octets[2] = {0, 0}, octet_tiles[2] = {0, 0}, octet_strips[2] = {0, 0}, ragged_tiles[2] = {0, 0}, ragged_strips = 0;
 };
 SetSizes set_sizes(const zgr_tensor* tensors, int32_t n) {
   SetSizes s;
@@ -280,19 +280,18 @@ SetSizes set_sizes(const zgr_tensor* tensors, int32_t n) {
     } else if (!f32) {
       s.ragged_tiles[0] += tiles;
       s.ragged_tiles[1] += blocks_in_spans(t.rows) * strips;
+      s.ragged_strips += strips;
     }
   }
   return s;
 }
-// What the ragged 16-bit tensors of a set take on the staged kernel, in tiles of the busiest SM on the tile kernel: a tile of the staged one is
-// shorter, the less so the more seeds share it, but spans of 256 rows may cost some more.
+// Do the ragged 16-bit tensors of a set take less time on the staged kernel?  Its tile is shorter, the less so the more seeds share it, but spans
+// of 256 rows may cost some more of them on the busiest SM: 8.04 tiles a mean against 7.97 are nine against eight in shares (18 M weights in
+// rows of 1234 and 4937, tile kernel / staged: one seed 135 / 95 us, three 61.5 / 60.2, four 71.7 / 74.5, eight 123.5 / 131.8).
 bool ragged_on_staged(const SetSizes& sizes, int sm_count, int n_terms) {
-  const auto busiest = [&](int64_t tiles) {
-    const double mean = static_cast<double>(tiles) / sm_count;
-    return mean < 12.0 ? std::ceil(mean) : mean;
-  };
-  const double tile = n_terms == 1 ? 0.75 : (n_terms == 2 ? 0.85 : (n_terms == 3 ? 0.88 : 0.98));
-  return tile * busiest(sizes.ragged_tiles[1]) <= busiest(sizes.ragged_tiles[0]);
+  const double tile = n_terms == 1 ? 0.75 : (n_terms == 2 ? 0.85 : (n_terms == 3 ? 0.88 : 0.94));
+  const double on_tile = static_cast<double>(sizes.ragged_tiles[0]) / sm_count, on_staged = static_cast<double>(sizes.ragged_tiles[1]) / sm_count;
+  return on_staged < 12.0 ? tile * std::ceil(on_staged) <= std::ceil(on_tile) : tile * on_staged <= on_tile;      // (dealt out whole in shares)
 }
 
 // Which kernel family serves a tensor: 1 the TMA-staged one with two-part operands (16-bit weights in whole octets, rank > 8), 2 those with
@@ -430,7 +429,8 @@ double share_out(const std::vector<TensorDesc>& descs, const std::vector<Member>
 
 // Work items of one group.  An item is a strip of columns x a range of rows; it costs its tiles and, once, its coefficient
 // strip, so few tall items are cheap but divide badly over the SMs.  `target`: elements per item for about 16 rounds.
-void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>& members, int sm_count, int64_t target, Group& g) {
+// In shares below `shares_below` tiles per SM on the three-part kernels.
+void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>& members, int sm_count, int64_t target, int shares_below, Group& g) {
   const auto by_elements = [](int64_t elements, int ncols) { return elements / ncols; };
   const auto by_rows = [](int64_t rows, int) { return rows; };
   const bool tile = is_tile(g.kc);
@@ -447,7 +447,7 @@ void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>&
   int64_t tiles = 0;
   for (const Member& m : members) tiles += ((descs[m.tensor].rows + 127) / 128) * ((descs[m.tensor].cols + 127) / 128);
   const int64_t sms = sm_count;
-  if (tile ? tiles < 12 * sms : g.kc.path == PATH_UMMA && tiles < 24 * sms) {
+  if (tile ? tiles < shares_below * sms : g.kc.path == PATH_UMMA && tiles < 24 * sms) {
     // per 128 columns and rank about a hundredth of a tile for the strip, twice that for fp32 (anything from 1/60 to 1/200 gives the
     // same times); an item has a pipeline to fill, which the three-part kernels do ahead where two strips fit
     const double strip_cost = g.kc.precise ? 0.02 : 0.01;
@@ -555,13 +555,15 @@ void plan_tiles(const std::vector<TensorDesc>& descs, const std::vector<Member>&
     }
 }
 
+// What sweeps of many terms do with tensors kept by residue: as with one term; on the tile kernel all the same; in shares up to 24 tiles per SM.
+enum Many { MANY_AS_ONE = 0, MANY_ON_TILE = 1, MANY_IN_SHARES = 2 };
+
 // Split the tensors listed in `which` into work items, grouped by the kernel that serves them.
 // The kernel family follows the tensor's own storage type (fp32 tensors take the accurate transform and
 // an exact fp32 contraction); `kernel_dtype` >= 0 overrides only the type the kernel reads and writes,
-// which lets the test hook run a 16-bit tensor's kernel family on an fp32 image.  `ragged_on_tile`: tensors kept by residue go to the
-// tile kernel all the same.
+// which lets the test hook run a 16-bit tensor's kernel family on an fp32 image.
 void plan(const std::vector<TensorDesc>& descs, const std::vector<int>& which, bool guided_on, int bits, int sm_count,
-          std::vector<Group>& out, int kernel_dtype = -1, bool multi = false, bool ragged_on_tile = false) {
+          std::vector<Group>& out, int kernel_dtype = -1, bool multi = false, Many many = MANY_AS_ONE) {
   int64_t total = 0;
   for (int l : which) total += descs[l].rows * descs[l].cols;
   // elements per item: enough items for ~16 rounds over the resident CTAs, but large enough that the
@@ -608,7 +610,7 @@ void plan(const std::vector<TensorDesc>& descs, const std::vector<int>& which, b
       // fp32 with rank > 8, rows that are not a multiple of eight elements, and low ranks: three-part operands.  (The test hook
       // that sweeps an fp32 image of a 16-bit tensor keeps the one-element-per-thread kernel below.)
       path = vec && t.rank <= 8 ? PATH_FMA : PATH_GENERIC; kpad = t.kpad; strip = kTileStripCols;
-      by_res = ragged_on_tile && by_residue(t);
+      by_res = many == MANY_ON_TILE && by_residue(t);
       staged = t.staged && !by_res;
       row_step = staged && by_residue(t) ? 256 : 128;
     } else if (!vec || (t.rank > 8 && !umma_ok && (t.Ufrag == nullptr || multi))) {
@@ -629,7 +631,8 @@ void plan(const std::vector<TensorDesc>& descs, const std::vector<int>& which, b
   }
   members.resize(out.size());
   for (size_t gi = 0; gi < out.size(); ++gi)
-    if (out[gi].kc.path != PATH_ISO) plan_tiles(descs, members[gi], sm_count, target, out[gi]);
+    if (out[gi].kc.path != PATH_ISO)
+      plan_tiles(descs, members[gi], sm_count, target, many == MANY_IN_SHARES && !members[gi].empty() && members[gi][0].row_step == 256 ? 24 : 12, out[gi]);
   for (Group& g : out) {
     g.elements = 0;
     for (const WorkItem& w : g.items) g.elements += g.kc.path == PATH_ISO ? w.nrows_or_count : item_rows(descs[w.tensor], g.kc, w).second * w.ncols;
@@ -960,12 +963,21 @@ int validate_model(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, 
   return ZGR_OK;
 }
 
-// From how many terms on a sweep has the set's ragged 16-bit tensors on the tile kernel although the staged one serves single seeds.
-int many_terms_from(const std::vector<TensorDesc>& descs, const SetSizes& sizes, int sm_count) {
+// From how many terms on a sweep treats the set's ragged 16-bit tensors otherwise than single seeds, which the staged kernel serves, and how; 0:
+// never.  Either on the tile kernel, or, where items from the counter are few and tall, in shares: they need not be cut as low as for one seed,
+// whose layer-wise sweeps share the items out again, and the hand-out of tiles that many terms make long ends unevenly (us a pass from the
+// counter / in shares: 64 M weights in rows of 1411 four seeds 212 / 182, eight of rank 40 399 / 334; 36 M of 999 rank 48 three seeds 130 / 108;
+// 39 M of 683 eight 249 / 242; but strips of four tiles, 35 M of 384 at rank 8, four seeds 114 / 118).
+int many_terms_from(const std::vector<TensorDesc>& descs, const SetSizes& sizes, int sm_count, Many* many) {
   bool ragged = false;
   for (const TensorDesc& td : descs) ragged = ragged || by_residue(td);
+  *many = MANY_ON_TILE;
   for (int n = 2; ragged && n <= 4; ++n)
     if (!ragged_on_staged(sizes, sm_count, n)) return n;
+  *many = MANY_IN_SHARES;
+  const int64_t tiles = sizes.ragged_tiles[1];
+  if (ragged && tiles >= 12 * sm_count && tiles < 24 * sm_count && tiles >= 6 * sizes.ragged_strips) return 2;
+  *many = MANY_AS_ONE;
   return 0;
 }
 
@@ -998,7 +1010,9 @@ int plan_on_host(const zgr_tensor* tensors, int32_t n, const zgr_config* cfg, in
     }
     all[static_cast<size_t>(l)] = l;
   }
-  plan(descs, all, guided_on, cfg->bits_per_normal, sm_count, groups, -1, multi, multi && many_terms_from(descs, sizes, sm_count) > 0);
+  Many many = MANY_AS_ONE;
+  if (multi) many_terms_from(descs, sizes, sm_count, &many);
+  plan(descs, all, guided_on, cfg->bits_per_normal, sm_count, groups, -1, multi, many);
   return ZGR_OK;
 }
 
@@ -1012,7 +1026,7 @@ void ledger_add(zgr_ctx* ctx, uint64_t seed, double c) {
 
 // Plan used by sweeps with n terms, n > 1: the sweep plan itself unless it contains the legacy
 // tensor-core kernel, which applies one term per sweep (those tensors are re-planned onto the fallback), or so many terms
-// are better off with the tile kernel.
+// have a plan of their own.
 std::vector<Group>& multi_groups(zgr_ctx* ctx, int n, int* rc) {
   *rc = ZGR_OK;
   if (ctx->many_terms > 0 && n >= ctx->many_terms) return ctx->groups_multi;
@@ -1131,9 +1145,10 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
     plan(ctx->descs, all, guided_on, cfg->bits_per_normal, ctx->sm_count, ctx->groups);
     order_groups(ctx->descs, ctx->groups);
     merge_small_groups(ctx);
-    ctx->many_terms = many_terms_from(ctx->descs, sizes, ctx->sm_count);
+    Many many;
+    ctx->many_terms = many_terms_from(ctx->descs, sizes, ctx->sm_count, &many);
     if (ctx->many_terms > 0) {
-      plan(ctx->descs, all, guided_on, cfg->bits_per_normal, ctx->sm_count, ctx->groups_multi, -1, true, true);
+      plan(ctx->descs, all, guided_on, cfg->bits_per_normal, ctx->sm_count, ctx->groups_multi, -1, true, many);
       order_groups(ctx->descs, ctx->groups_multi);
     }
     Tables tables;
@@ -1183,7 +1198,7 @@ int zgr_init(zgr_ctx** out, const zgr_tensor* tensors, int32_t n, const zgr_conf
       for (int i = 0; i < (td.umma ? 2 : 3); ++i) {
         td.Ucopy[i] = at;
         if (!make_map_16bit(m + i, at, rows_pad, td.kpad, td.kpad)) rc = check(ctx, cudaErrorUnknown);
-        if (ctx->many_terms > 0 && by_residue(td) && !make_map_in_order(&ctx->tmaps[static_cast<size_t>(3 * l + i)], at, rows_pad, td.kpad))
+        if (many == MANY_ON_TILE && by_residue(td) && !make_map_in_order(&ctx->tmaps[static_cast<size_t>(3 * l + i)], at, rows_pad, td.kpad))
           rc = check(ctx, cudaErrorUnknown);
         at += static_cast<size_t>(rows_pad) * td.kpad * 2;       // (a multiple of 4096 bytes)
       }

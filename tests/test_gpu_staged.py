@@ -115,6 +115,19 @@ def test_several_seeds_on_the_tile_kernel(rank, dtype, bits):
     assert p.lib.device_status() == 0
 
 
+# Sets between 12 and 24 tiles per SM: items from the counter for one seed, another plan in shares for several, in turn.
+def test_several_seeds_in_shares_of_their_own():
+    shapes, ranks = [(25600, 131)] * 5 + [(1, 9)], [16, 16, 9, 16, 16, 0]
+    dtypes = [zgr.BF16] * 6
+    assert len(plan(shapes, ranks, dtypes)) != len(plan(shapes, ranks, dtypes, multi=1)) and kernels(shapes, ranks, dtypes, multi=1)[0] == "staged"
+    p = Pair(shapes, ranks, "bf16", bits=16, seed=7)
+    coeffs = [oracle.update_coefficient(0.0, 2.1, 1.9, p.eps, 1e-4), oracle.update_coefficient(0.0, 1.6, 2.0, p.eps, 1e-4)]
+    for seed in (3, 4):
+        p.step(seed=seed, lp=1.8, lm=2.3, lr=1e-4)
+        p.call_and_check_multi([41, 42], coeffs, lambda: p.lib.restore_update_multi([41, 42], [2.1, 1.6], [1.9, 2.0], 1e-4), "two seeds")
+    assert p.lib.device_status() == 0
+
+
 # A delivered and a constructed subspace reach the copies of U that are kept by residue.
 def test_new_subspaces_of_ragged_tensors():
     p = Pair([LARGE, (300, 385), (1, 9)], [16, 16, 0], "bf16", bits=16, seed=6)

@@ -186,6 +186,18 @@ def test_kernel_of_many_seeds(shapes, multi_kernel):
     check_exact_cover(plan(shapes, [16] * n, [zgr.BF16] * n, multi=1), shapes)
 
 
+# Ragged sets between 12 and 24 tiles per SM: from the counter with one seed, in shares with many, unless their strips are short.
+@pytest.mark.parametrize("d,ffn,layers,shares", [(1411, 5643, 2, True), (999, 3999, 3, True), (441, 1765, 12, False), (2051, 8203, 2, False)])
+def test_shares_of_many_seeds(d, ffn, layers, shares):
+    shapes = ([(d, d)] * 4 + [(ffn, d), (d, ffn)]) * layers
+    one, many = (plan(shapes, [16] * len(shapes), [zgr.BF16] * len(shapes), multi=m) for m in (0, 1))
+    check_exact_cover(many, shapes)
+    assert ([(it.tensor, it.row0_or_e0, it.col0) for it in one] != [(it.tensor, it.row0_or_e0, it.col0) for it in many]) == shares
+    tiles = sum(-(-m // 256) * 2 * -(-n // 128) for m, n in shapes)
+    if shares:
+        assert max(-(-it.nrows_or_count // 128) for it in many) <= -(-tiles // 148) and len(many) < len(one)
+
+
 # Ragged 16-bit sets that are dealt out in shares: a share begins and ends in the middle of a span of 256 rows where that makes the
 # largest one smaller, down to one tile above the mean (which is a whole number of tiles).  Tiles of 128 rows, two to a span.
 @pytest.mark.parametrize("d,ffn,rank", [(1234, 4937, 16), (871, 3491, 32), (701, 2803, 64), (1534, 6137, 16), (501, 2003, 8)])
