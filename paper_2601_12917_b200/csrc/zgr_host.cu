@@ -321,23 +321,26 @@ int tensor_core_kind(const zgr_tensor& t, bool guided_on, const SetSizes& sizes)
 // Which of the two kernels with three-part operands: 1 the staged one, 0 the tile kernel.  TMA wants the weights on a 16-byte boundary
 // and rows that hold a whole octet wherever it begins; the staged kernel keeps the high counter word of the generator fixed.
 // Small sets stay with the tile kernel, whose sixteen epilogue warps share every tile (two groups on alternate tiles leave half of
-// them idle when a CTA has one or two): us a step tile / staged, bf16 rank 8 2.4 M 26.8 / 29.6, 4.0 M 32.1 / 31.7, 8 M 59.8 / 57.5; ragged 16-bit
-// rank 16 1.6 M 34.0 / 42.6, 2.7 M 47.0 / 45.5, 3.0 M 48.5 / 44.6, 18 M 135 / 95; fp32 up to rank 16 3.1 M 38.4 / 39.0, 5.9 M 58.1 / 59.7,
-// 6.3 M 49.9 / 51.4, 7.1 M 49.2 / 48.8, 19 M 106 / 101, above 3.9 M 49.2 / 47.9, 4.9 M 57.2 / 54.3, 6.3 M 70.2 / 63.7.  fp32 rows that are no multiple of eight
-// elements do so at any size: 96 M weights of rank 16 in rows of 1001 and 4001 469 / 479 (the accurate transform hides what the tile
-// kernel spends on its transposition, and the residues cost half-empty tiles).
+// them idle when a CTA has one or two): us a step tile / staged, bf16 rank 8 2.4 M 26.8 / 29.6, 4.0 M 32.1 / 31.7, 8 M 59.8 / 57.5; ragged
+// 16-bit rank 16 1.6 M 34.0 / 42.6, 2.7 M 47.0 / 45.5, 3.0 M 48.5 / 44.6, 18 M 135 / 95; fp32 up to rank 16 3.1 M 38.4 / 39.0, 5.9 M 58.1 / 59.7,
+// 6.3 M 49.9 / 51.4, 7.1 M 49.2 / 48.8, 19 M 106 / 101; fp32 above rank 16 3.9 M 49.2 / 47.9, 4.9 M 57.2 / 54.3, 6.3 M 70.2 / 63.7.
+// fp32 rows that are no multiple of eight elements do so at any size: 96 M weights of rank 16 in rows of 1001 and 4001 469 / 479 (the accurate
+// transform hides what the tile kernel spends on its transposition, and the residues cost half-empty tiles).
 //
-// Tiles that are not full cost the staged kernel more (its groups take full and half-empty ones in turn): whole octets stay with the tile kernel
-// below 0.7 of the tiles' area, in fp32 up to rank 16 (16-bit matrices of 136 and 4 x 136, 40 layers: .38 99 / 107; 192: .68 115 / 128;
-// 320: .78 162 / 161; 448: .84 111 / 106.  fp32 168: .52 148 / 156; 200: .67 156 / 165; 320: .78 193 / 186; rank 64 192: 207 / 190).  So do
-// 16-bit sets of many items (from the counter) in strips of under four tiles (matrices of 256 and 4 x 256: 2.7 146 / 152; 320: 3.8 253 / 264;
-// 384: 4.0 141 / 132).  Ragged rows: ragged_on_staged (matrices of 125: 20 tiles a layer against 12  86 / 105; 261: 114 against 90  191 / 171).
+// Tiles that are not full cost the staged kernel more (its groups take full and half-empty ones in turn), so whole octets stay with the tile
+// kernel where less than 0.7 of the tiles' area is filled; in fp32 up to rank 16 only, there also below 0.83 in strips of under 3.5 tiles.  16-bit
+// rank 8, matrices of d and 4 d, 40 or 20 layers: d = 136, .38 99 / 107; 192, .68 115 / 128; 320, .78 162 / 161; 448, .84 111 / 106.  fp32 rank 4 to 16:
+// 168, .52 148 / 156; 200, .67 156 / 165; 320, .78 193 / 186; 337 x 1424, .81 153 / 154, and beside ragged tensors 592 / 612; 337 x 1408, .88
+// 129 / 123; fp32 rank 64, 192, .68 207 / 190.
+// So do 16-bit sets of many items (from the counter) in strips of under four tiles: d = 256, 2.7 146 / 152; 320, 3.8 253 / 264; 384, 4.0 141 / 132.
+// Ragged rows: ragged_on_staged (d = 125, 20 tiles a layer against 12, 86 / 105; 261, 114 against 90, 191 / 171).
 int staged_kind(const zgr_tensor& t, const SetSizes& sizes, int sm_count) {
   const int f32 = t.dtype == ZGR_F32;
   if ((reinterpret_cast<uintptr_t>(t.data) & 15) != 0 || t.cols < 16 || t.cols >= (int64_t{1} << 31) - 256 || t.rows * t.cols >= (int64_t{1} << 34)) return 0;
   if ((t.cols & 7) != 0) return !f32 && sizes.three_part[0] >= 5 * (int64_t{1} << 19) && ragged_on_staged(sizes, sm_count, 1);
   const double full = static_cast<double>(sizes.octets[f32]) / (16384.0 * static_cast<double>(sizes.octet_tiles[f32]));
-  if (f32) return sizes.three_part[1] >= (t.rank <= 16 ? 13 : 5) * (int64_t{1} << 19) && (t.rank > 16 || full >= 0.7);
+  if (f32 && t.rank > 16) return sizes.three_part[1] >= 5 * (int64_t{1} << 19);
+  if (f32) return sizes.three_part[1] >= 13 * (int64_t{1} << 19) && full >= (2 * sizes.octet_tiles[1] < 7 * sizes.octet_strips[1] ? 0.83 : 0.7);
   const bool short_items = sizes.octet_tiles[0] >= 12 * sm_count && sizes.octet_tiles[0] < 4 * sizes.octet_strips[0];
   return sizes.three_part[0] >= 5 * (int64_t{1} << 19) && full >= 0.7 && !short_items;
 }

@@ -176,6 +176,11 @@ def test_lines_between_staged_and_tile_kernel(d, layers, rank, dtype, expected):
     assert set(kernels(shapes, [rank] * len(shapes), [dtype] * len(shapes))) == {expected}
 
 
+def test_short_strips_that_are_not_full():
+    for cols, expected in ((1424, "tile"), (1408, "staged")):
+        assert set(kernels([(337, cols)] * 40, [4] * 40, [zgr.F32] * 40)) == {expected}
+
+
 # Ragged sets whose spans cost a tile of the busiest SM: many seeds have the tile kernel, one the staged one.
 @pytest.mark.parametrize("shapes,multi_kernel", [([(6917, 131)] * 4, "tile"), ([(1234, 1234)] * 4 + [(4937, 1234), (1234, 4937)], "tile"),
                                                   ([(1534, 1534)] * 4 + [(6137, 1534), (1534, 6137)], "staged")])
